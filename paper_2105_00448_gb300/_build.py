@@ -32,6 +32,8 @@ UNITS = {
     "noalloc.cu": [],
     "net.cu": [],
     "mg.cu": [],
+    "march.cu": [],
+    "coarse.cu": [],
 }
 
 

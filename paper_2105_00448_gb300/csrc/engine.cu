@@ -39,8 +39,12 @@ void launch_vcycle(const Ctx& c, int which, bool fp64, const MGHost& H, int part
 int vcycle_launches(const MGHost& H, bool scale);
 int vcycle_part_launches(const MGHost& H, int part, bool scale);
 void mg_coop_config(MGHost& H, bool fp64, int sm_count, long long smem_bytes);
-void mg_zmarch_config(MGHost& H, const RepDesc& rd, int sm_count, const float* r, const float* w,
-                      const int* lv_dims);
+int cluster_plan(const MGLevel* lv, int nl, int from, int cs, long long smem, MGCluster* R);
+bool cluster_init(const MGHost& H);
+bool march_init();
+void march_tile(MGLevel& L);
+int march_threads(const std::vector<MGLevel*>& lv);
+void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, std::vector<int4>& out);
 }  // namespace hca
 
 using hca::Ctx;
@@ -1191,6 +1195,8 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
           L.nx = nx;
           L.ny = ny;
           L.nz = nz;
+          // FP32: rows are padded to whole 4-site groups (padding holds 0), as the lattice's are
+          L.pitch = h->fp64 ? nx : (nx + 3) / 4 * 4;
           L.n = nn;
           L.cscale = cs;
           L.cscale32 = (float)cs;
@@ -1213,24 +1219,29 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
             goto fail;
           }
       for (int l = 1; l < H.nlev; ++l) {
-        long long tot = 0;
+        long long tot = 0, elems = 0;
+        std::vector<long long> first(n, 0);   // first element (16-byte aligned for FP32)
         for (int i = 0; i < n; ++i) {
           start[(size_t)l * (n + 1) + i] = tot;
-          if (l < rep[i].x) tot += lv[(size_t)i * hca::MG_MAXLEV + l].n;
+          if (l >= rep[i].x) continue;
+          const hca::MGLevel& L = lv[(size_t)i * hca::MG_MAXLEV + l];
+          tot += L.n;
+          first[i] = elems;
+          elems += ((long long)L.pitch * L.ny * L.nz + 3) / 4 * 4;
         }
         start[(size_t)l * (n + 1) + n] = tot;
         H.ntot[l] = tot;
         char* arr[5];
-        for (int k = 0; k < 5; ++k) ALLOC(arr[k], es * (size_t)std::max(1LL, tot));
+        for (int k = 0; k < 5; ++k) ALLOC(arr[k], es * (size_t)std::max(1LL, elems));
         for (int k = 0; k < 5; ++k)
-          if (cudaMemsetAsync(arr[k], 0, es * (size_t)std::max(1LL, tot), c.stream)) {
+          if (cudaMemsetAsync(arr[k], 0, es * (size_t)std::max(1LL, elems), c.stream)) {
             rc = HCA_ERR_CUDA;
             goto fail;
           }
         for (int i = 0; i < n; ++i) {
           if (l >= rep[i].x) continue;
           hca::MGLevel& L = lv[(size_t)i * hca::MG_MAXLEV + l];
-          const size_t o = es * (size_t)start[(size_t)l * (n + 1) + i];
+          const size_t o = es * (size_t)first[i];
           L.x = arr[0] + o;
           L.t = arr[1] + o;
           L.rhs = arr[2] + o;
@@ -1289,15 +1300,98 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
       }
       ALLOC(c.r, fbytes);
       ALLOC(c.mg_t0, fbytes);
-      ALLOC(c.mg_w, fbytes);
-      if (n == 1 && !h->fp64) {
-        int dims[3 * hca::MG_MAXLEV] = {};
-        for (int l = 0; l < hca::MG_MAXLEV; ++l) {
-          dims[3 * l] = lv[l].nx;
-          dims[3 * l + 1] = lv[l].ny;
-          dims[3 * l + 2] = lv[l].nz;
+      if (h->fp64 || H.nlev == 1) ALLOC(c.mg_w, fbytes);
+      if (!h->fp64 && H.nlev > 1) {
+        // the plane-marching sweeps of the lattice and the grid levels
+        if (!hca::march_init()) {
+          rc = HCA_ERR_CUDA;
+          goto fail;
         }
-        hca::mg_zmarch_config(H, h->reps_h[0], c.sm_count, (const float*)c.r, (const float*)c.mg_w, dims);
+        // the coarse levels from rep[i].y on run in a cluster of blocks per
+        // replicate: as many blocks as leave every cluster resident, at most 16
+        std::vector<hca::MGCluster> clus(n);
+        int cs = 16;
+        while (cs > 1 && n * cs > c.sm_count) cs /= 2;
+        const char* cse = std::getenv("HCA_MG_CLUSTER");   // another size (results do not depend on it)
+        if (cse && std::atoi(cse) >= 1 && std::atoi(cse) <= 16) cs = std::atoi(cse);
+        for (;; cs /= 2) {
+          H.cl_size = cs;
+          H.cl_smem = 0;
+          H.small = 0;
+          bool ok = true;
+          for (int i = 0; i < n && ok; ++i) {
+            const hca::MGLevel* lv_i = &lv[(size_t)i * hca::MG_MAXLEV];
+            int from = 1;   // levels of at most kClusterSites sites per block
+            while (from < rep[i].x - 1 && lv_i[from].n > hca::kClusterSites * cs) ++from;
+            const int lc = hca::cluster_plan(lv_i, rep[i].x, from, cs, 223 * 1024, &clus[i]);
+            ok = lc > 0;
+            rep[i].y = lc;
+            H.small = std::max(H.small, lc);
+            H.cl_smem = std::max(H.cl_smem, clus[i].smem);
+          }
+          if (ok && hca::cluster_init(H)) break;
+          if (cs == 1) {
+            rc = HCA_ERR_CUDA;
+            goto fail;
+          }
+        }
+        hca::MGCluster* clus_d;
+        ALLOC(clus_d, sizeof(hca::MGCluster) * (size_t)n);
+        if (cudaMemcpyAsync(clus_d, clus.data(), sizeof(hca::MGCluster) * (size_t)n, cudaMemcpyHostToDevice, c.stream) ||
+            cudaStreamSynchronize(c.stream)) {
+          rc = HCA_ERR_CUDA;
+          goto fail;
+        }
+        c.mgc = clus_d;
+        long long slots = 0;
+        std::vector<int4> blocks;
+        for (int l = 0; l < H.small; ++l) {
+          std::vector<hca::MGLevel*> set;
+          std::vector<int> ids;
+          for (int i = 0; i < n; ++i) {
+            if (l >= rep[i].y) continue;   // this replicate runs level l in its cluster
+            hca::MGLevel& L = lv[(size_t)i * hca::MG_MAXLEV + l];
+            if (l == 0) {
+              const RepDesc& r0 = h->reps_h[i];
+              L.nx = r0.nx;
+              L.ny = r0.ny;
+              L.nz = r0.nz;
+              L.pitch = r0.nxp;
+              L.n = (long long)r0.nx * r0.ny * r0.nz;
+              L.cscale = 1.0;
+              L.cscale32 = 1.f;
+              L.x = (float*)c.z + r0.off;
+              L.t = (float*)c.mg_t0 + r0.off;
+              L.rhs = (float*)c.r + r0.off;
+              L.d = (float*)c.d + r0.off;
+              L.w = nullptr;
+            }
+            hca::march_tile(L);
+            if (l == 0) {
+              L.slot0 = (int)slots;
+              slots += (long long)L.tx * L.ty * L.nseg;
+            }
+            set.push_back(&L);
+            ids.push_back(i);
+          }
+          H.mb_off[l] = (int)blocks.size();
+          H.mb_nt[l] = hca::march_threads(set);
+          hca::march_blocks(set, ids, c.sm_count, blocks);
+          H.mb_n[l] = (int)blocks.size() - H.mb_off[l];
+        }
+        int4* blocks_d;
+        ALLOC(blocks_d, sizeof(int4) * blocks.size());
+        ALLOC(c.mslot, sizeof(double) * (size_t)std::max(1LL, slots));
+        ALLOC(c.mcnt, sizeof(int) * (size_t)n);
+        if (cudaMemcpyAsync(blocks_d, blocks.data(), sizeof(int4) * blocks.size(), cudaMemcpyHostToDevice, c.stream) ||
+            cudaMemsetAsync(c.mcnt, 0, sizeof(int) * (size_t)n, c.stream) || cudaStreamSynchronize(c.stream)) {
+          rc = HCA_ERR_CUDA;
+          goto fail;
+        }
+        c.mblk = blocks_d;
+        c.lazy_scale = 1;
+        H.march = 1;
+        H.launches = hca::vcycle_launches(H, false);
       }
       hca::MGLevel* lv_d;
       long long* start_d;

@@ -18,7 +18,6 @@
 
 #include <utility>
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -278,13 +277,38 @@ namespace hca {
 
 // Device pointers and launch parameters of one handle, passed by value to
 // every kernel.  Field pointers are typed per precision by the kernels.
-// One coarse level of the multigrid hierarchy (dense, x fastest).
+// One level of the multigrid hierarchy (x fastest; entry 0, the lattice, is
+// filled for FP32 fields).
 struct MGLevel {
-  int nx, ny, nz, pad;
+  int nx, ny, nz;
+  int pitch;                // elements between rows (nx; whole 4-site groups on the grid levels of FP32 fields)
   long long n;
   void *x, *t, *rhs, *d, *w;   // iterate, second iterate, right-hand side, diagonal, 1 / diagonal
   double cscale;            // coupling of this level / coupling of the lattice (2^level)
   float cscale32;           // the same in FP32 (exact)
+  // plane-marching sweeps (FP32): patch columns and row pairs of a tile with
+  // its halo (one group and one row pair on each side), groups and rows of
+  // its interior, tiles, planes per reduction segment, segments along z, first
+  // slot, blocks
+  int cols, pairs, ox, oy, tx, ty, seg, nseg, slot0, nblk;
+};
+
+// The coarse levels a thread-block cluster holds (FP32; coarse.cu): level i of
+// the cluster is hierarchy level lc + i.
+struct MGClusterLevel {
+  int nx, nr, no, gpr;          // sites per row, rows per plane, planes, 4-site groups per row
+  int oa, ob, orr, od;          // float offsets in a block's shared memory (orr, od: -1 = global memory)
+  int p0[17];                   // first plane of each block (distributed levels)
+  float cscale;
+  int grow, gplane;             // global strides of rows and planes
+  unsigned mg, mr;              // reciprocals of gpr and nr (div_small)
+  const float *grhs, *gd;
+  float* gx;
+};
+struct MGCluster {
+  int lc, nl, ndist, zp;        // first level, levels, distributed levels, planes along z
+  int smem, pad;
+  MGClusterLevel lev[12];
 };
 
 // multigrid constants (the FP64 reference uses the same).  Above the
@@ -301,6 +325,7 @@ constexpr int MG_NU_COARSE = 16;
 constexpr long long MG_MIN_SITES = 512;     // coarsening stops at or below this size
 constexpr long long MG_SMALL_SITES = 4096;  // levels this small run inside one block
 
+constexpr long long kClusterSites = 4096;   // most sites per block of a cluster's first level
 constexpr int MG_MAXLEV = 16;
 constexpr int kVcycleParts = 6;   // launch groups of a V-cycle (see launch_vcycle)
 
@@ -327,20 +352,11 @@ struct MGHost {
   unsigned rows_ok = 0;          // bit l: every replicate's level-l rows are whole 4-site groups
   long long post_items[MG_MAXLEV] = {};   // row-kernel items per level over the replicates
   long long restr_items[MG_MAXLEV] = {};
-  // the lattice's pre-sweeps in plane-marching form (one FP32 lattice; 0 =
-  // row form): slabs along z, planes per slab, tiles along x and y
-  int zm_slabs = 0;
-  int zm_zs = 0;
-  int zm_tx = 0, zm_ty = 0;
-  int zm_mode = 0;               // 2: TMA-staged planes (default), 1: planes prefetched into registers
-  // grid levels' pre-sweeps and last post-sweep in plane-marching form
-  // (0 slabs: row form): slabs, planes per slab, tiles along x and y
-  int zl_slabs[MG_MAXLEV] = {};
-  int zl_zs[MG_MAXLEV] = {};
-  int zl_tx[MG_MAXLEV] = {}, zl_ty[MG_MAXLEV] = {};
-  // TMA tensor maps of r and 1/d over the lattice (x extent nx: the copy
-  // engine fills sites outside the lattice with zeros)
-  CUtensorMap zm_map_r, zm_map_w;
+  // FP32: the grid levels' plane-marching sweeps (march.cu): blocks of level
+  // l, their first entry in the block table and threads per block
+  int march = 0;
+  int cl_size = 0, cl_smem = 0;  // blocks and shared memory of the coarse levels' clusters
+  int mb_n[MG_MAXLEV] = {}, mb_off[MG_MAXLEV] = {}, mb_nt[MG_MAXLEV] = {};
 };
 
 struct Ctx {
@@ -373,7 +389,12 @@ struct Ctx {
   void* r;
   void* mg_t0;
   void* mg_w;         // 1 / d on the lattice (0 where d = 0)
-  const void* mg_lv;  // device MGLevel[n_reps][MG_MAXLEV] (level 0 unused)
+  const void* mg_lv;  // device MGLevel[n_reps][MG_MAXLEV] (level 0 filled for FP32 fields)
+  const int4* mblk;   // blocks of the marching sweeps: (replicate, tile, first plane, end plane)
+  double* mslot;      // their segment sums
+  int* mcnt;          // [rep] blocks done
+  const MGCluster* mgc;   // [rep] coarse levels in a cluster
+  int lazy_scale;     // 1: the first inner iteration's kernels scale r as they read it
   const long long* mg_start;  // [MG_MAXLEV][n_reps + 1] prefix sums of each level's sites over the replicates
   const int2* mg_rep;         // per replicate: (levels, first single-block level)
   const long long* mg_rowstart;  // [n_reps + 1] prefix of level-1 rows x lattice groups per row

@@ -1,0 +1,662 @@
+// Plane-marching multigrid sweeps for FP32 fields: everything a V-cycle does
+// on one grid level (the lattice or a coarse grid level, single lattices and
+// batches) in two kernels,
+//
+//   k_mg_down  both pre-sweeps, the residual, its restriction and the part of
+//              the first post-sweep that does not need the coarse correction;
+//   k_mg_up    the prolongation and both post-sweeps (on the lattice also
+//              rho = r.z and beta).
+//
+// With w = 1 / d, c the level's coupling and W1, W2 the Chebyshev weights:
+//   u  = W1 w r                                  first sweep (from zero)
+//   v  = u + W2 w (r - A u) = K u + W2 c w S(u)   second sweep, d u = W1 r,
+//                                                K = 1 + W2 (1 - W1) / W1
+//   res = r + c S(v) - d v,  rhs of the next level = its sum over children
+//   v' = v + W2 w res
+//   y  = v' + (1 - W2) p + W2 c w S(p)            first post-sweep of v + p,
+//                                                p = P x_coarse
+//   x  = (1 - W1) y + W1 w (r + c S(y))           second post-sweep
+// with S the sum over the in-box neighbours.  Algorithmic traffic per site:
+// down reads r, d, writes v' and 1/8 of a coarse site (12.5 B); up reads v',
+// r, d and 1/8 of a coarse site and writes x (16.5 B): 29 B a V-cycle.
+//
+// Form.  A block of kMT threads owns a tile of 4-site groups by row pairs (a
+// thread holds a 4 x 2 patch) and walks up z through a slab of planes.  The
+// tile includes the halo the fused sweeps need (one group in x, two rows in
+// y, where the level is wider than the tile; two planes in z), so every
+// thread runs the same code and only interior threads write.  Each plane's
+// inputs arrive by per-thread cp.async copies (zero fill outside the level)
+// into a shared-memory ring, two planes ahead; z neighbours stay in
+// registers (the loop body is unrolled by three, so nothing is rotated), y
+// neighbours go through shared memory (one barrier per plane), x neighbours
+// through lane shuffles.  Bound: shared-memory and shuffle traffic and the
+// latency a barrier a plane exposes at 16 warps per multiprocessor (ncu, down
+// at 256^3: 44 % of issue slots, 46 % of the shared-memory pipe).  Measured
+// at 256^3 (FP32): down 74 us and up 92 us a launch, against 110 us for the
+// pre-sweep and restriction kernels and 118 us for the two post-sweep kernels
+// they replaced (28.5 B a site each); on 16 uneven replicates (59 M sites)
+// 139 and 175 us (of the whole batch), against 449 and 495 us.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+#include <vector>
+
+#include "hca_internal.cuh"
+
+namespace hca {
+
+namespace {
+
+constexpr int kMT = 256;              // most threads per block (instances: 64, 128, 256)
+constexpr int kDownRing = 5;          // planes k - 2 .. k + 2 of r and d
+constexpr int kUpRing = 3;            // planes k .. k + 2 of v' and d, k - 1 .. k + 1 of r
+constexpr int kMaxSeg = 32;           // z segments of a slab (reduction slots)
+constexpr float kW1 = (float)MG_W1, kW2 = (float)MG_W2;
+constexpr float kK = (float)(1.0 + MG_W2 * (1.0 - MG_W1) / MG_W1);
+constexpr float k1W1 = (float)(1.0 - MG_W1), k1W2 = (float)(1.0 - MG_W2);
+constexpr size_t down_smem(int nt) { return (size_t)(kDownRing * 4 + 2 * 2 + 2 * 2) * nt * 16; }
+constexpr size_t up_smem(int nt) { return (size_t)(kUpRing * 6 + 2 * 2 + 2) * nt * 16 + (size_t)kMaxSeg * (nt / 32) * 8; }
+constexpr int blocks_per_sm(int nt) { return nt >= 256 ? 2 : 512 / nt; }
+
+__device__ __forceinline__ void cp16(unsigned sdst, const float* gsrc, int n) {   // n = 0: zero fill
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sdst), "l"(gsrc), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp4(unsigned sdst, const float* gsrc, int n) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sdst), "l"(gsrc), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// The patch's 4 x 2 values on one plane as pairs along x: the sums and
+// products below use the two-wide FP32 instructions (one issue for two
+// sites; every product and sum rounded as in the scalar form).
+struct P8 {
+  float2 v[2][2];   // [row][sites 0, 1 | 2, 3]
+};
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ void get_row(float2 (&v)[2], const float4* s) {
+  const float4 q = *s;
+  v[0] = make_float2(q.x, q.y);
+  v[1] = make_float2(q.z, q.w);
+}
+
+// 1 / d (0 where d = 0: padding, outside the level, an isolated empty site);
+// a smoothing weight, so the hardware reciprocal (1 ulp) serves
+__device__ __forceinline__ float inv_d(float d) {
+  float w;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(d));
+  return d > 0.f ? w : 0.f;
+}
+__device__ __forceinline__ float2 inv_d(float2 d) { return make_float2(inv_d(d.x), inv_d(d.y)); }
+
+// This thread's place in its block's tile.  Every tile carries its halo, also
+// at the level's edges (zeros there), so no neighbour needs a bounds check;
+// neighbours beyond the tile (of outermost halo patches, unused) read the
+// thread's own values.
+struct Patch {
+  int tid, lane, x0, y0;   // first site of the patch
+  int nx, nz;
+  int im, ip;          // row buffer slots of the rows below and above the patch
+  bool l0, l31;        // the x neighbour is in another warp
+  bool rok[2];         // the patch's rows inside the level (and the group)
+  bool out;            // the patch belongs to the tile's interior
+  bool part;           // the group has padding sites
+  unsigned e, sy, sz;  // element of (x0, y0, plane 0), strides (a field has fewer than 2^32 elements)
+};
+
+template <int NT>
+__device__ __forceinline__ Patch patch_of(const MGLevel& L, int4 b) {
+  Patch p;
+  p.tid = threadIdx.x;
+  p.lane = p.tid & 31;
+  const int cols = L.cols, pairs = L.pairs;
+  const int pr = p.tid / cols, col = p.tid - pr * cols;
+  p.nx = L.nx;
+  p.nz = L.nz;
+  const int ty = b.y / L.tx, tx = b.y - ty * L.tx;
+  const int g = tx * L.ox - 1 + col;
+  p.x0 = 4 * g;
+  p.y0 = ty * L.oy - 2 + 2 * pr;
+  const bool gok = g >= 0 && p.x0 < p.nx && pr < pairs;
+  p.rok[0] = gok && p.y0 >= 0 && p.y0 < L.ny;
+  p.rok[1] = gok && p.y0 >= 0 && p.y0 + 1 < L.ny;
+  p.out = p.rok[0] && col >= 1 && col <= L.ox && pr >= 1 && 2 * pr < 2 + L.oy;
+  p.part = p.x0 + 4 > p.nx;
+  p.im = NT + p.tid - (pr > 0 ? cols : 0);
+  p.ip = p.tid + (pr < pairs - 1 ? cols : 0);
+  p.l0 = p.lane == 0 && p.tid > 0;
+  p.l31 = p.lane == 31 && p.tid + 1 < NT;
+  p.sy = (unsigned)L.pitch;
+  p.sz = (unsigned)L.pitch * (unsigned)L.ny;
+  p.e = gok && p.y0 >= 0 ? (unsigned)p.x0 + p.sy * (unsigned)p.y0 : 0u;
+  return p;
+}
+
+// The sum over the neighbours of the patch on its own plane and the one
+// below: uc the plane (its rows also in row buffer B: [row of the
+// pair][thread]), um the plane below; S may be um.
+template <int NT>
+__device__ __forceinline__ void nb_patch(const Patch& p, const float4* __restrict__ B, const P8& uc, const P8& um,
+                                         P8& S) {
+  const float4 ym = B[p.im], yp = B[p.ip];
+  const float2 ymv[2] = {make_float2(ym.x, ym.y), make_float2(ym.z, ym.w)};
+  const float2 ypv[2] = {make_float2(yp.x, yp.y), make_float2(yp.z, yp.w)};
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const float2 u0 = uc.v[a][0], u1 = uc.v[a][1];
+    float lft = __shfl_up_sync(0xffffffffu, u1.y, 1), rgt = __shfl_down_sync(0xffffffffu, u0.x, 1);
+    const float* Bf = reinterpret_cast<const float*>(B + a * NT + p.tid);
+    if (p.l0) lft = Bf[-1];
+    if (p.l31) rgt = Bf[4];
+    const float2 x[2] = {make_float2(lft + u0.y, u0.x + u1.x), make_float2(u0.y + u1.y, u1.x + rgt)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 m = a == 0 ? __fadd2_rn(ymv[h], uc.v[1][h]) : __fadd2_rn(uc.v[0][h], ypv[h]);
+      S.v[a][h] = __fadd2_rn(__fadd2_rn(x[h], m), um.v[a][h]);
+    }
+  }
+}
+
+template <int NT>
+__device__ __forceinline__ void put_patch(const Patch& p, float4* __restrict__ B, const P8& u) {
+#pragma unroll
+  for (int a = 0; a < 2; ++a) B[a * NT + p.tid] = make_float4(u.v[a][0].x, u.v[a][0].y, u.v[a][1].x, u.v[a][1].y);
+}
+
+__device__ __forceinline__ void zero_patch(P8& u) {
+#pragma unroll
+  for (int a = 0; a < 2; ++a) u.v[a][0] = u.v[a][1] = make_float2(0.f, 0.f);
+}
+
+// The coupling of level l of the operator: the lattice's FP32 coupling times
+// the level's scale.
+__device__ __forceinline__ float level_coupling(const Ctx& c, int rep, int which, const MGLevel& L) {
+  return c.reps[rep].cpl32[which] * L.cscale32;
+}
+
+// On the first application of a rescaled inner solve the stored residual is
+// still unscaled: the factor the lattice kernels apply to r as they read it.
+__device__ __forceinline__ float r_scale(const RepSolve& sv) { return sv.iters == 0 ? (float)sv.scale : 1.f; }
+
+// The end of a marching kernel that sums into slots: the last block of the
+// replicate (nblk blocks) to arrive adds its n slots in an order that is the
+// same whatever the launch (64 lanes take every 64th slot, then a fixed
+// tree) and hands the sum to fin, called by one thread.
+template <class Fin>
+__device__ __forceinline__ void march_finish(const Ctx& c, int rep, int nblk, const double* slots, int n, Fin fin) {
+  __shared__ int s_last;
+  __shared__ double s_half[2];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&c.mcnt[rep], 1) == nblk - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (threadIdx.x < 64) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n; i += 64) t += __ldcg(&slots[i]);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) s_half[threadIdx.x >> 5] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    fin(s_half[0] + s_half[1]);
+    c.mcnt[rep] = 0;
+  }
+}
+
+// ------------------------------------------------------------------ down --
+template <bool LAT, int NT>
+__global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int which, int l, const int4* __restrict__ blocks) {
+  extern __shared__ __align__(16) float4 msm[];
+  const int4 b = blocks[blockIdx.x];
+  const int rep = b.x;
+  const MGLevel& L = ((const MGLevel*)c.mg_lv)[rep * MG_MAXLEV + l];
+  const MGLevel& C = (&L)[1];
+  const Patch p = patch_of<NT>(L, b);
+  const int zb = b.z, ze = b.w;
+  const float cpl = level_coupling(c, rep, which, L);
+  const float2 w2c = dup(kW2 * cpl);
+  const float* __restrict__ rr = (const float*)L.rhs;
+  const float* __restrict__ dd = (const float*)L.d;
+  float* __restrict__ vv = (float*)L.t;
+  float* __restrict__ rc = (float*)C.rhs;
+  const bool two = p.x0 / 2 + 1 < C.nx;
+  const unsigned cel = (unsigned)(p.x0 / 2) + (unsigned)C.pitch * (unsigned)(p.y0 / 2), csz = (unsigned)C.pitch * (unsigned)C.ny;
+  HCA_VC_ENTRY(c);
+  float sc = 1.f;
+  if (c.skip_idle && !c.solve[rep].active) return;   // this replicate's solve has ended
+  if (LAT) sc = r_scale(c.solve[rep]);
+  const float2 w1s = dup(LAT ? kW1 * sc : kW1);
+  float4* ring = msm + p.tid;                  // [plane mod kDownRing][r0, r1, d0, d1][thread]
+  float4* ub = msm + kDownRing * 4 * NT;       // [plane & 1][row][thread]
+  float4* vb = ub + 4 * NT;
+  const unsigned sring = smem_addr(ring);
+  const int n0 = p.rok[0] ? 16 : 0, n1 = p.rok[1] ? 16 : 0;
+  auto fetch = [&](int k, int slot) {
+    const bool zok = k >= 0 && k < p.nz;
+    const unsigned sa = sring + (unsigned)slot * (4 * NT * 16);
+    const unsigned e = zok ? p.e + (unsigned)k * p.sz : 0u;
+    const unsigned e0 = n0 ? e : 0u, e1 = zok && n1 ? e + p.sy : 0u;
+    const int m0 = zok ? n0 : 0, m1 = zok ? n1 : 0;
+    cp16(sa, rr + e0, m0);
+    cp16(sa + NT * 16, rr + e1, m1);
+    cp16(sa + 2 * NT * 16, dd + e0, m0);
+    cp16(sa + 3 * NT * 16, dd + e1, m1);
+  };
+  P8 u[3], v[3], w[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    zero_patch(u[i]);
+    zero_patch(v[i]);
+    zero_patch(w[i]);
+  }
+  float2 acc = make_float2(0.f, 0.f);
+  const int k0 = zb - 2, k1 = ze + 1;   // planes whose u is formed
+  fetch(k0, 0);
+  cp_commit();
+  fetch(k0 + 1, 1);
+  cp_commit();
+  int slot = 0;
+  // one plane: u of plane k, v of plane k - 1, the residual of plane k - 2
+  auto step = [&](auto ph, int k) {
+    constexpr int P0 = decltype(ph)::value, P1 = (P0 + 2) % 3, P2 = (P0 + 1) % 3;   // planes k, k - 1, k - 2
+    if (k + 2 <= k1) fetch(k + 2, slot + 2 >= kDownRing ? slot + 2 - kDownRing : slot + 2);
+    cp_commit();
+    cp_wait<2>();
+    float4* U0 = ub + (k & 1) * 2 * NT;
+    const float4* U1 = ub + ((k & 1) ^ 1) * 2 * NT;
+    float4* V1 = vb + ((k & 1) ^ 1) * 2 * NT;
+    const float4* V2 = vb + (k & 1) * 2 * NT;
+    // every read of shared memory and every lane exchange first: they depend
+    // on nothing formed in this step (the sums still lack the plane above)
+    const float4* rs = ring + slot * 4 * NT;
+    float2 r[2][2], d[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      get_row(r[a], rs + a * NT);
+      get_row(d[a], rs + (2 + a) * NT);
+    }
+    nb_patch<NT>(p, U1, u[P1], u[P2], u[P2]);
+    nb_patch<NT>(p, V2, v[P2], v[P0], v[P0]);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        w[P0].v[a][h] = inv_d(d[a][h]);
+        u[P0].v[a][h] = __fmul2_rn(__fmul2_rn(w1s, w[P0].v[a][h]), r[a][h]);
+      }
+    put_patch<NT>(p, U0, u[P0]);
+    {
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          v[P1].v[a][h] = __ffma2_rn(__fmul2_rn(w2c, w[P1].v[a][h]), __fadd2_rn(u[P2].v[a][h], u[P0].v[a][h]),
+                                     __fmul2_rn(dup(kK), u[P1].v[a][h]));
+      put_patch<NT>(p, V1, v[P1]);
+      // the residual of plane k - 2
+      if (k >= zb + 2) {
+        const int z = k - 2;
+        if (p.out) {
+          const float4* rz = ring + (slot >= 2 ? slot - 2 : slot - 2 + kDownRing) * 4 * NT;
+          const unsigned e = p.e + (unsigned)z * p.sz;
+          float2 pl = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int a = 0; a < 2; ++a) {
+            float2 r[2], d[2], o[2], res[2];
+            get_row(r, rz + a * NT);
+            get_row(d, rz + (2 + a) * NT);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float2 vc = v[P2].v[a][h];
+              const float2 rn = __ffma2_rn(dup(cpl), __fadd2_rn(v[P0].v[a][h], v[P1].v[a][h]),
+                                           LAT ? __fmul2_rn(r[h], dup(sc)) : r[h]);
+              res[h] = __ffma2_rn(make_float2(-d[h].x, -d[h].y), vc, rn);
+              o[h] = __ffma2_rn(__fmul2_rn(dup(kW2), w[P2].v[a][h]), res[h], vc);
+            }
+            if (p.part) {   // padding sites are no children
+              if (p.x0 + 1 >= p.nx) res[0].y = 0.f;
+              if (p.x0 + 2 >= p.nx) res[1].x = 0.f;
+              if (p.x0 + 3 >= p.nx) res[1].y = 0.f;
+            }
+            if (a == 0 || p.rok[1]) {
+              const float2 pr = make_float2(res[0].x + res[0].y, res[1].x + res[1].y);
+              pl = a == 0 ? pr : __fadd2_rn(pl, pr);
+              *reinterpret_cast<float4*>(vv + e + a * p.sy) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+            }
+          }
+          // the children's sum: rows, then planes
+          if (z & 1) pl = __fadd2_rn(acc, pl);
+          else acc = pl;
+          if ((z & 1) || z == p.nz - 1) {
+            float* q = rc + (cel + (unsigned)(z >> 1) * csz);
+            q[0] = pl.x;
+            if (two) q[1] = pl.y;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    slot = slot + 1 == kDownRing ? 0 : slot + 1;
+  };
+  for (int k = k0; k <= k1; k += 3) {
+    step(std::integral_constant<int, 0>{}, k);
+    if (k + 1 <= k1) step(std::integral_constant<int, 1>{}, k + 1);
+    if (k + 2 <= k1) step(std::integral_constant<int, 2>{}, k + 2);
+  }
+}
+
+// -------------------------------------------------------------------- up --
+template <bool LAT, int NT>
+__global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int which, int l, const int4* __restrict__ blocks) {
+  extern __shared__ __align__(16) float4 msm[];
+  const int4 b = blocks[blockIdx.x];
+  const int rep = b.x;
+  const MGLevel& L = ((const MGLevel*)c.mg_lv)[rep * MG_MAXLEV + l];
+  const MGLevel& C = (&L)[1];
+  const Patch p = patch_of<NT>(L, b);
+  const int zb = b.z, ze = b.w;
+  const float cpl = level_coupling(c, rep, which, L);
+  const float2 w2c = dup(kW2 * cpl);
+  const float* __restrict__ vv = (const float*)L.t;
+  const float* __restrict__ rr = (const float*)L.rhs;
+  const float* __restrict__ dd = (const float*)L.d;
+  const float* __restrict__ xc = (const float*)C.x;
+  float* __restrict__ xo = (float*)L.x;
+  const int cnz = C.nz;
+  const bool two = p.x0 / 2 + 1 < C.nx;
+  const unsigned csz = (unsigned)C.pitch * (unsigned)C.ny;
+  const unsigned cel = p.rok[0] ? (unsigned)(p.x0 / 2) + (unsigned)C.pitch * (unsigned)(p.y0 / 2) : 0u;
+  HCA_VC_ENTRY(c);
+  float sc = 1.f;
+  if (c.skip_idle && !c.solve[rep].active) return;
+  if (LAT) sc = r_scale(c.solve[rep]);
+  float4* ring = msm + p.tid;               // [phase][v0, v1, d0, d1, r0, r1 (of the plane before)][thread]
+  float4* yb = msm + kUpRing * 6 * NT;      // [plane & 1][row][thread]
+  float2* cells = reinterpret_cast<float2*>(yb + 4 * NT);   // [coarse plane & 3][thread]: the patch's two coarse cells
+  float2* segs = cells + 4 * NT;
+  const unsigned sring = smem_addr(ring), scell = smem_addr(cells + p.tid);
+  const int n0 = p.rok[0] ? 16 : 0, n1 = p.rok[1] ? 16 : 0;
+  // v' and d of plane k, r of plane k - 1 (used one step later)
+  auto fetch = [&](int k, int slot) {
+    const bool zok = k >= 0 && k < p.nz, z1 = k >= 1 && k <= p.nz;
+    const unsigned sa = sring + (unsigned)slot * (6 * NT * 16);
+    const unsigned ek = p.e + (unsigned)k * p.sz;
+    const int m0 = zok ? n0 : 0, m1 = zok ? n1 : 0, q0 = z1 ? n0 : 0, q1 = z1 ? n1 : 0;
+    const unsigned e0 = m0 ? ek : 0u, e1 = m1 ? ek + p.sy : 0u;
+    const unsigned f0 = q0 ? ek - p.sz : 0u, f1 = q1 ? ek - p.sz + p.sy : 0u;
+    cp16(sa, vv + e0, m0);
+    cp16(sa + NT * 16, vv + e1, m1);
+    cp16(sa + 2 * NT * 16, dd + e0, m0);
+    cp16(sa + 3 * NT * 16, dd + e1, m1);
+    cp16(sa + 4 * NT * 16, rr + f0, q0);
+    cp16(sa + 5 * NT * 16, rr + f1, q1);
+  };
+  auto fetch_cells = [&](int Z) {
+    const bool ok = p.rok[0] && Z >= 0 && Z < cnz;
+    const unsigned sa = scell + (unsigned)(Z & 3) * (NT * 8);
+    const unsigned e = ok ? cel + (unsigned)Z * csz : 0u;
+    cp4(sa, xc + e, ok ? 4 : 0);
+    cp4(sa + 4, xc + (two && ok ? e + 1 : 0u), two && ok ? 4 : 0);
+  };
+  P8 y[3], w[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    zero_patch(y[i]);
+    zero_patch(w[i]);
+  }
+  FF acc{0.f, 0.f};
+  const int k0 = zb - 1, k1 = ze;   // planes whose y is formed (k0 odd: zb is even)
+  // coarse planes k0 / 2 - 1 .. k0 / 2 + 1 before the first step (-1 below the level: zeros)
+  const int Z0 = k0 >> 1;
+  fetch(k0, 0);
+  fetch_cells(Z0);
+  fetch_cells(Z0 + 1);
+  cp_commit();
+  fetch(k0 + 1, 1);
+  fetch_cells(Z0 + 2);
+  cp_commit();
+  // cell slots of the neighbours (clamped for outermost halo patches)
+  const int cm = p.im - NT, cp = p.ip, cl = p.tid > 0 ? p.tid - 1 : 0, cr = p.tid + 1 < NT ? p.tid + 1 : p.tid;
+  const bool yin = p.rok[1];
+  float2 cur = make_float2(0.f, 0.f), below = cur;   // the patch's cells of the current coarse plane and of the one below
+  cp_wait<1>();
+  __syncthreads();
+  int seg = 0;
+  const int seglen = L.seg;
+  auto step = [&](auto ph, int k) {
+    constexpr int P0 = decltype(ph)::value, P1 = (P0 + 2) % 3, P2 = (P0 + 1) % 3;
+    const bool odd = k & 1;
+    const int Z = k >> 1;
+    if (k + 2 <= k1) {
+      fetch(k + 2, P1);
+      if (!odd) fetch_cells(Z + 2);
+    }
+    cp_commit();
+    cp_wait<2>();
+    const float2* cz = cells + (Z & 3) * NT;
+    if (!odd || k == k0) {
+      below = cur;
+      cur = cz[p.tid];
+    }
+    // y of plane k - 1: its neighbours but the plane above
+    nb_patch<NT>(p, yb + ((k & 1) ^ 1) * 2 * NT, y[P1], y[P2], y[P2]);
+    // the coarse cells around the patch: in x, in the coarse rows below and
+    // above, and along z: in its own cells, or the coarse plane below (even
+    // planes) or above (odd planes)
+    const float xl = cz[cl].y, xr = cz[cr].x;
+    const float2 co = odd ? cells[((Z + 1) & 3) * NT + p.tid] : below;
+    const float2 zn = (odd || k + 1 < p.nz) ? __fadd2_rn(co, cur) : co;
+    // the row's y neighbours: one coarse row outside the cells, one inside
+    const float2 t[2] = {__fadd2_rn(yin ? __fadd2_rn(cz[cm], cur) : cz[cm], zn), __fadd2_rn(__fadd2_rn(cz[cp], cur), zn)};
+    const float both = cur.x + cur.y;
+    float2 xs[2] = {make_float2(xl + cur.x, both), make_float2(both, cur.y + xr)};
+    if (p.part) {   // no neighbour to the right of the level's last site
+      if (p.x0 + 1 == p.nx) xs[0].x = xl;
+      if (p.x0 + 2 == p.nx) xs[0].y = cur.x;
+      if (p.x0 + 3 == p.nx) xs[1].x = cur.x;
+    }
+    const float2 pw[2] = {__fmul2_rn(dup(k1W2), dup(cur.x)), __fmul2_rn(dup(k1W2), dup(cur.y))};
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      float2 vp[2], d[2];
+      get_row(vp, ring + (P0 * 6 + a) * NT);
+      get_row(d, ring + (P0 * 6 + 2 + a) * NT);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 S = __fadd2_rn(xs[h], dup(h ? t[a].y : t[a].x));
+        w[P0].v[a][h] = inv_d(d[h]);
+        const float2 yv = __ffma2_rn(__fmul2_rn(w2c, w[P0].v[a][h]), S, __fadd2_rn(pw[h], vp[h]));
+        y[P0].v[a][h] = make_float2(d[h].x > 0.f ? yv.x : 0.f, d[h].y > 0.f ? yv.y : 0.f);
+      }
+    }
+    put_patch<NT>(p, yb + (k & 1) * 2 * NT, y[P0]);
+    if (k > zb) {
+      const int z = k - 1;
+      if (p.out) {
+        const unsigned e = p.e + (unsigned)z * p.sz;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          float2 r[2], o[2], rz = make_float2(0.f, 0.f);
+          get_row(r, ring + (P0 * 6 + 4 + a) * NT);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float2 rs = LAT ? __fmul2_rn(r[h], dup(sc)) : r[h];
+            const float2 rn = __ffma2_rn(dup(cpl), __fadd2_rn(y[P2].v[a][h], y[P0].v[a][h]), rs);
+            o[h] = __ffma2_rn(__fmul2_rn(dup(kW1), w[P1].v[a][h]), rn, __fmul2_rn(dup(k1W1), y[P1].v[a][h]));
+            if (LAT) rz = __ffma2_rn(rs, o[h], rz);
+          }
+          if (a == 0 || p.rok[1]) {
+            *reinterpret_cast<float4*>(xo + e + a * p.sy) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+            if (LAT) acc = ff_add(acc, rz.x + rz.y);
+          }
+        }
+      }
+      if (LAT && (((z + 1) % seglen) == 0 || z == ze - 1)) {
+        // the segment's sum over this warp's patches (fixed lane order)
+        const FF s = row_reduce_ff(acc, 32);
+        if (p.lane == 0) segs[seg * (NT / 32) + (p.tid >> 5)] = make_float2(s.hi, s.lo);
+        acc = FF{0.f, 0.f};
+        ++seg;
+      }
+    }
+    __syncthreads();
+  };
+  for (int k = k0; k <= k1; k += 3) {
+    step(std::integral_constant<int, 0>{}, k);
+    if (k + 1 <= k1) step(std::integral_constant<int, 1>{}, k + 1);
+    if (k + 2 <= k1) step(std::integral_constant<int, 2>{}, k + 2);
+  }
+  if (!LAT) return;
+  // the block's segment sums to their slots (warps in order), then the
+  // replicate's last block adds all slots in a fixed order
+  double* slots = c.mslot + L.slot0 + (long long)b.y * L.nseg + zb / seglen;
+  for (int s = threadIdx.x; s < seg; s += NT) {
+    double t = 0.0;
+    for (int q = 0; q < NT / 32; ++q) {
+      const float2 f = segs[s * (NT / 32) + q];
+      t += (double)f.x + (double)f.y;
+    }
+    slots[s] = t;
+  }
+  march_finish(c, rep, L.nblk, c.mslot + L.slot0, L.tx * L.ty * L.nseg, [&](double rz) {
+    RepSolve& s = c.solve[rep];
+    if (!s.active) return;
+    if (!(rz > 0.0) || !isfinite(rz)) {
+      if (!isfinite(rz)) c.sync->error = 1;
+      s.active = 0;
+      return;
+    }
+    s.beta = s.iters == 0 ? 0.0 : rz / s.rho;
+    s.rho = rz;
+  });
+}
+
+}  // namespace
+
+// ---------------------------------------------------------- configuration --
+// Tiling of a level: the fewest tiles of kMT patches (every halo patch is
+// redundant work).  It depends on the level's shape alone, as do the segment
+// sums, so results do not depend on slabs, batches or launch forms.
+void march_tile(MGLevel& L) {
+  const int gpr = (L.nx + 3) / 4, np = (L.ny + 1) / 2;   // groups per row, row pairs
+  long long best = -1;
+  for (int n = 1; n <= gpr; ++n) {
+    const int ox = (gpr + n - 1) / n, cols = ox + 2, most = kMT / cols - 2;   // row pairs of the interior
+    if (most < 1) continue;
+    const int op = (np + (np + most - 1) / most - 1) / ((np + most - 1) / most);   // even shares
+    const int tx = (gpr + ox - 1) / ox, ty = (np + op - 1) / op;
+    const long long cost = (long long)tx * ty;
+    if (best < 0 || cost < best) {
+      best = cost;
+      L.cols = cols;
+      L.pairs = op + 2;
+      L.ox = ox;
+      L.oy = 2 * op;
+      L.tx = tx;
+      L.ty = ty;
+    }
+    if (cols <= 6) break;
+  }
+  // planes per reduction segment (even, so a slab starts on a coarse plane)
+  L.seg = L.nz > 256 ? 16 : L.nz > 128 ? 8 : L.nz > 64 ? 4 : 2;
+  L.nseg = (L.nz + L.seg - 1) / L.seg;
+}
+
+// The blocks (replicate, tile, slab) of one level's launches over the
+// replicates that sweep it on the grid: slabs of whole segments, as thick as
+// balances the planes of a slab's halo against idle multiprocessors.
+void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, std::vector<int4>& out) {
+  const long long resident = 2LL * sm_count;
+  auto slab = [](const MGLevel& L, int zs) { return std::min(L.nz, (zs + L.seg - 1) / L.seg * L.seg); };
+  int best_zs = 0;
+  double best = -1;
+  for (int zs = 2; zs <= 1024; zs = zs < 64 ? zs + 2 : zs + 8) {
+    long long nb = 0;
+    double work = 0, longest = 0;
+    bool ok = true, more = false;
+    for (MGLevel* L : lv) {
+      const int z = slab(*L, zs), ns = (L->nz + z - 1) / z;
+      if (z / L->seg > kMaxSeg) ok = false;
+      if (z < L->nz) more = true;
+      nb += (long long)ns * L->tx * L->ty;
+      work += (double)ns * L->tx * L->ty * (z + 6);
+      longest = std::max(longest, z + 6.0);
+    }
+    if (!ok) break;
+    // whole waves while there are few, an even share plus a tail beyond
+    const double waves = (double)nb / resident;
+    const double t = waves <= 4 ? std::max(1.0, std::ceil(waves)) * longest : work / resident + 0.5 * longest;
+    if (best < 0 || t < best) {
+      best = t;
+      best_zs = zs;
+    }
+    if (!more) break;
+  }
+  for (size_t i = 0; i < lv.size(); ++i) {
+    MGLevel& L = *lv[i];
+    const int z = slab(L, best_zs);
+    L.nblk = 0;
+    for (int zb = 0; zb < L.nz; zb += z)
+      for (int ty = 0; ty < L.ty; ++ty)
+        for (int tx = 0; tx < L.tx; ++tx) {
+          out.push_back(make_int4(reps[i], ty * L.tx + tx, zb, std::min(L.nz, zb + z)));
+          ++L.nblk;
+        }
+  }
+}
+
+namespace {
+template <int NT>
+bool march_init_t() {
+  const void* fn[4] = {(const void*)k_mg_down<true, NT>, (const void*)k_mg_down<false, NT>,
+                       (const void*)k_mg_up<true, NT>, (const void*)k_mg_up<false, NT>};
+  for (int i = 0; i < 4; ++i)
+    if (cudaFuncSetAttribute(fn[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(i < 2 ? down_smem(NT) : up_smem(NT))) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return false;
+    }
+  return true;
+}
+
+template <int NT>
+void launch_march_t(const Ctx& c, int which, const MGHost& H, int l, bool down) {
+  const dim3 g(H.mb_n[l]), t(NT);
+  const int4* bl = c.mblk + H.mb_off[l];
+  const bool pdl = c.pdl != 0;
+  if (down && l == 0) launch_k(pdl, k_mg_down<true, NT>, g, t, down_smem(NT), c.stream, c, which, l, bl);
+  else if (down) launch_k(pdl, k_mg_down<false, NT>, g, t, down_smem(NT), c.stream, c, which, l, bl);
+  else if (l == 0) launch_k(pdl, k_mg_up<true, NT>, g, t, up_smem(NT), c.stream, c, which, l, bl);
+  else launch_k(pdl, k_mg_up<false, NT>, g, t, up_smem(NT), c.stream, c, which, l, bl);
+}
+}  // namespace
+
+// Dynamic shared memory of the marching kernels in the current context.
+bool march_init() { return march_init_t<64>() && march_init_t<128>() && march_init_t<256>(); }
+
+// Threads per block for a set of tilings.
+int march_threads(const std::vector<MGLevel*>& lv) {
+  int n = 64;
+  for (const MGLevel* L : lv)
+    while (n < L->cols * L->pairs) n *= 2;
+  return n;
+}
+
+// k_mg_down (down) or k_mg_up on grid level l.
+void launch_march(const Ctx& c, int which, const MGHost& H, int l, bool down) {
+  if (H.mb_n[l] == 0) return;
+  switch (H.mb_nt[l]) {
+    case 64: launch_march_t<64>(c, which, H, l, down); break;
+    case 128: launch_march_t<128>(c, which, H, l, down); break;
+    default: launch_march_t<256>(c, which, H, l, down); break;
+  }
+}
+
+}  // namespace hca

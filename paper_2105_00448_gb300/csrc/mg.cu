@@ -32,11 +32,12 @@
 
 #include "hca_internal.cuh"
 #include "row_ops.cuh"
-#include "tc.cuh"
 
 namespace hca {
 
 int persist_grid(const void* fn, int threads, int sm_count);
+void launch_march(const Ctx& c, int which, const MGHost& H, int l, bool down);
+void launch_mg_cluster(const Ctx& c, int which, const MGHost& H);
 
 namespace {
 
@@ -100,8 +101,8 @@ __device__ __forceinline__ View<T> view(const Ctx& c, int which, int r, int l) {
   v.ny = L.ny;
   v.nz = L.nz;
   v.off = 0;
-  v.sy = L.nx;
-  v.sz = (long long)L.nx * L.ny;
+  v.sy = L.pitch;
+  v.sz = (long long)L.pitch * L.ny;
   v.x = (T*)L.x;
   v.t = (T*)L.t;
   v.rhs = (T*)L.rhs;
@@ -388,28 +389,9 @@ __global__ void __launch_bounds__(kMgThreads) k_mg_diag(Ctx c, int which, int l)
 }
 
 // The defect-correction residual is stored unscaled: on the first
-// application of a rescaled inner solve, r *= scale (elementwise, in place);
-// replicates past that return at once.
-template <typename T>
-__global__ void __launch_bounds__(kMgThreads) k_mg_scale0(Ctx c, int which) {
-  HCA_VC_ENTRY(c);
-  RepCursor<T> k;
-  bool skip = true;
-  T sc = T(1);
-  HCA_MG_FOR_SITES(0) {
-    if (k.at(c, which, 0, q, false)) {
-      const RepSolve& sv = c.solve[k.r];
-      skip = sv.iters != 0 || sv.scale == 1.0;
-      sc = (T)sv.scale;
-    }
-    if (skip) continue;
-    int X, Y, Z;
-    k.F.coords(q - k.lo, X, Y, Z);
-    k.F.rhs[k.F.at(X, Y, Z)] *= sc;
-  }
-}
-
-// k_mg_scale0 for one lattice as a stream of four-site groups (row-major,
+// application of a rescaled inner solve r *= scale (in place).  For a lattice
+// that is its own coarsest level; the marching sweeps scale r as they read it.
+// A stream of four-site groups (row-major,
 // vector loads and stores; padding sites are left as they are).
 template <typename T>
 __global__ void __launch_bounds__(256) k_mg_scale0_rows(Ctx c) {
@@ -840,423 +822,6 @@ __global__ void __launch_bounds__(128, 5) k_mg_pre0(Ctx c, int which, T* __restr
         st4(dst + eb + off[a], VO);
       }
     }
-  }
-}
-
-// Plane-marching form of k_mg_pre0 for one FP32 lattice.  A block owns a
-// tile of kZmG four-site groups by kZmY rows and a slab of planes, and walks
-// up z: each thread keeps its group's u on planes z - 1, z and z + 1 in
-// registers, and u on plane z of the tile with a one-site halo goes to
-// shared memory (two buffers, one barrier per plane) for the x and y
-// neighbours.  So r and 1/d are read once per site (the halo's from L2), and
-// the loads of plane z + 2 are in flight during plane z's arithmetic.
-// Threads 0 .. 2 kZmG - 1 also load the two halo rows (groups), the next
-// 2 kZmY threads the halo sites at the tile's x ends.  Per site the
-// arithmetic is k_mg_pre0's (pre0_site, same neighbour order).
-constexpr int kZmG = 8, kZmY = 16, kZmThreads = kZmG * kZmY;
-constexpr int kZmPitch = 4 * kZmG + 8;   // tile row in shared memory: left halo at 3, groups from 4, right halo at 4 + 4 kZmG
-
-__global__ void __launch_bounds__(kZmThreads, 7) k_mg_pre0_z(Ctx c, int which, float* __restrict__ dst, int zs) {
-  HCA_VC_ENTRY(c);
-  __shared__ __align__(16) float ub[2][kZmY + 2][kZmPitch];
-  const RepDesc& rd = c.reps[0];
-  const float* __restrict__ rr = (const float*)c.r;
-  const float* __restrict__ ww = (const float*)c.mg_w;
-  const float cpl = op_coupling_t<float>(rd, which);
-  const int t = threadIdx.x, g = t % kZmG, ty = t / kZmG;
-  const int G = blockIdx.x * kZmG + g, y = blockIdx.y * kZmY + ty;
-  const int x0 = 4 * G;
-  const bool own = G < rd.gpr && y < rd.ny;
-  const long long sy = rd.nxp, sz = (long long)rd.nxp * rd.ny;
-  const long long eo = rd.off + x0 + sy * y;
-  // halo role: 1 a group of halo row y0 - 1 or y0 + kZmY, 2 a site at x0 - 1 or x0 + 4 kZmG
-  int hrole = 0, hrow = 0, hcol = 0, hx = 0;
-  bool hok = false;
-  long long he = 0;
-  if (t < 2 * kZmG) {
-    hrole = 1;
-    const int hy = blockIdx.y * kZmY + (t < kZmG ? -1 : kZmY), hg = blockIdx.x * kZmG + t % kZmG;
-    hok = hy >= 0 && hy < rd.ny && hg < rd.gpr;
-    he = rd.off + 4LL * hg + sy * hy;
-    hx = 4 * hg;
-    hrow = t < kZmG ? 0 : kZmY + 1;
-    hcol = 4 + 4 * (t % kZmG);
-  } else if (t < 2 * kZmG + 2 * kZmY) {
-    hrole = 2;
-    const int k = t - 2 * kZmG, side = k / kZmY, row = k % kZmY;
-    hx = side ? 4 * kZmG * (blockIdx.x + 1) : 4 * kZmG * blockIdx.x - 1;
-    const int hy = blockIdx.y * kZmY + row;
-    hok = hx >= 0 && hx < rd.nx && hy < rd.ny;
-    he = rd.off + hx + sy * hy;
-    hrow = row + 1;
-    hcol = side ? 4 + 4 * kZmG : 3;
-  }
-  const int zb = blockIdx.z * zs, ze = min(rd.nz, zb + zs);
-  auto ld_own = [&](int z, V4<float>& R, V4<float>& W) {
-    const bool ok = own && z >= 0 && z < rd.nz;
-    R = ld4_if(rr + eo + sz * z, ok);
-    W = ld4_if(ww + eo + sz * z, ok);
-  };
-  auto ld_halo = [&](int z, V4<float>& R, V4<float>& W) {
-    const bool ok = hok && z >= 0 && z < rd.nz;
-    if (hrole == 1) {
-      R = ld4_if(rr + he + sz * z, ok);
-      W = ld4_if(ww + he + sz * z, ok);
-    } else {
-      R.a[0] = (hrole == 2 && ok) ? rr[he + sz * z] : 0.f;
-      W.a[0] = (hrole == 2 && ok) ? ww[he + sz * z] : 0.f;
-    }
-  };
-  auto u_of = [&](const V4<float>& R, const V4<float>& W, int xb) {
-    V4<float> U;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) U.a[e] = (xb + e < rd.nx) ? pre0_u(R.a[e], W.a[e]) : 0.f;
-    return U;
-  };
-  // u of plane z (own group and halo role) into buffer z & 1
-  auto put = [&](int z, const V4<float>& U, const V4<float>& HR, const V4<float>& HW) {
-    float* row = &ub[z & 1][ty + 1][4 + 4 * g];
-    *reinterpret_cast<float4*>(row) = make_float4(U.a[0], U.a[1], U.a[2], U.a[3]);
-    if (hrole == 1) {
-      const V4<float> H = u_of(HR, HW, hx);
-      *reinterpret_cast<float4*>(&ub[z & 1][hrow][hcol]) = make_float4(H.a[0], H.a[1], H.a[2], H.a[3]);
-    } else if (hrole == 2) {
-      ub[z & 1][hrow][hcol] = pre0_u(HR.a[0], HW.a[0]);
-    }
-  };
-  V4<float> Rc, Wc, Rn, Wn, HRn, HWn, up, uc;
-  {
-    V4<float> Rp, Wp, HRc, HWc;
-    ld_own(zb - 1, Rp, Wp);
-    ld_own(zb, Rc, Wc);
-    ld_halo(zb, HRc, HWc);
-    ld_own(zb + 1, Rn, Wn);
-    ld_halo(zb + 1 < ze ? zb + 1 : -1, HRn, HWn);
-    up = u_of(Rp, Wp, x0);
-    uc = u_of(Rc, Wc, x0);
-    put(zb, uc, HRc, HWc);
-  }
-  __syncthreads();
-  for (int z = zb; z < ze; ++z) {
-    V4<float> Rnn, Wnn, HRnn, HWnn;
-    ld_own(z + 2 <= ze ? z + 2 : -1, Rnn, Wnn);
-    ld_halo(z + 2 < ze ? z + 2 : -1, HRnn, HWnn);
-    const V4<float> un = u_of(Rn, Wn, x0);   // plane z + 1 (zero above the lattice)
-    if (z + 1 < ze) put(z + 1, un, HRn, HWn);
-    const float* mid = &ub[z & 1][ty + 1][4 + 4 * g];
-    const float4 ym = *reinterpret_cast<const float4*>(mid - kZmPitch);
-    const float4 yp = *reinterpret_cast<const float4*>(mid + kZmPitch);
-    const float lft = mid[-1], rgt = mid[4];
-    if (own) {
-      const float ymv[4] = {ym.x, ym.y, ym.z, ym.w}, ypv[4] = {yp.x, yp.y, yp.z, yp.w};
-      V4<float> VO = zero4<float>();   // zero on padding
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int x = x0 + e;
-        if (x >= rd.nx) continue;
-        const float left = e == 0 ? lft : uc.a[e - 1];
-        const float right = e == 3 ? rgt : uc.a[e + 1];
-        const float nb = (x > 0 ? left : 0.f) + (x < rd.nx - 1 ? right : 0.f) + ymv[e] + ypv[e] + up.a[e] + un.a[e];
-        VO.a[e] = pre0_site(Rc.a[e], Wc.a[e], uc.a[e], cpl, nb);
-      }
-      st4(dst + eo + sz * z, VO);
-    }
-    up = uc;
-    uc = un;
-    Rc = Rn;
-    Wc = Wn;
-    Rn = Rnn;
-    Wn = Wnn;
-    HRn = HRnn;
-    HWn = HWnn;
-    __syncthreads();
-  }
-}
-
-// Plane-marching form of k_mg_smooth_rows<float, MODE> on grid level l >= 1
-// of one FP32 lattice: the fused pre-sweeps (SM_PRE: u = (W1 / d) rhs formed
-// at every site, x = u + (W2 / d)(rhs - A u)), the prolongation fused with
-// the first post-sweep (SM_POST: u = x + P x_C formed at every site, t = u +
-// (W2 / d)(rhs - A u)) and the last post-sweep (SM_LAST: u = t, x = t +
-// (W1 / d)(rhs - A t)).  The tiles, slabs, halo
-// roles and register prefetch of k_mg_pre0_z; the level's rows are whole
-// four-site groups.  Per site the row form's arithmetic: the neighbours'
-// u summed in the order x - 1, x + 1, y - 1, y + 1, z - 1, z + 1 (only those
-// inside the level), resid and one fused multiply-add.
-template <int MODE>
-__global__ void __launch_bounds__(kZmThreads, 7) k_mg_smooth_z(Ctx c, int which, int l, int zs) {
-  HCA_VC_ENTRY(c);
-  __shared__ __align__(16) float ub[2][kZmY + 2][kZmPitch];
-  const View<float> F = view<float>(c, which, 0, l);
-  const int gpr = F.nx >> 2;
-  const int t = threadIdx.x, g = t % kZmG, ty = t / kZmG;
-  const int G = blockIdx.x * kZmG + g, y = blockIdx.y * kZmY + ty;
-  const int x0 = 4 * G;
-  const bool own = G < gpr && y < F.ny;
-  const long long sy = F.sy, sz = F.sz;
-  const long long eo = x0 + sy * y;
-  // u's source: rhs (with 1/d), x (plus the coarse correction) or t
-  const float* __restrict__ ua = MODE == SM_PRE ? F.rhs : MODE == SM_POST ? F.x : F.t;
-  const View<float> C = view<float>(c, which, 0, MODE == SM_POST ? l + 1 : l);
-  // the coarse correction P x_C at fine (x, y, z): level l + 1's value of its cell
-  auto pxc = [&](int x, int yy, int z) {
-    return C.x[(x >> 1) + (long long)C.nx * ((yy >> 1) + (long long)C.ny * (z >> 1))];
-  };
-  int hrole = 0, hrow = 0, hcol = 0, hx = 0, hy = 0;
-  bool hok = false;
-  long long he = 0;
-  if (t < 2 * kZmG) {
-    hrole = 1;
-    hy = blockIdx.y * kZmY + (t < kZmG ? -1 : kZmY);
-    const int hg = blockIdx.x * kZmG + t % kZmG;
-    hok = hy >= 0 && hy < F.ny && hg < gpr;
-    hx = 4 * hg;
-    he = 4LL * hg + sy * hy;
-    hrow = t < kZmG ? 0 : kZmY + 1;
-    hcol = 4 + 4 * (t % kZmG);
-  } else if (t < 2 * kZmG + 2 * kZmY) {
-    hrole = 2;
-    const int k = t - 2 * kZmG, side = k / kZmY, row = k % kZmY;
-    hx = side ? 4 * kZmG * (blockIdx.x + 1) : 4 * kZmG * blockIdx.x - 1;
-    hy = blockIdx.y * kZmY + row;
-    hok = hx >= 0 && hx < F.nx && hy < F.ny;
-    he = hx + sy * hy;
-    hrow = row + 1;
-    hcol = side ? 4 + 4 * kZmG : 3;
-  }
-  const int zb = blockIdx.z * zs, ze = min(F.nz, zb + zs);
-  auto u_of = [&](const V4<float>& A, const V4<float>& W) {
-    if (MODE != SM_PRE) return A;
-    V4<float> U;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) U.a[e] = mul_rn(wt(MG_W1, W.a[e]), A.a[e]);
-    return U;
-  };
-  // u of a group (x0 = 4 G, row yy) with both of its coarse cells
-  auto u_post = [&](const V4<float>& A, int xg, int yy, int z, bool ok) {
-    V4<float> U = zero4<float>();
-    if (ok) {
-      const float c0 = pxc(xg, yy, z), c1 = pxc(xg + 2, yy, z);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) U.a[e] = A.a[e] + (e < 2 ? c0 : c1);
-    }
-    return U;
-  };
-  // u of the own group on plane z (0 outside the level)
-  auto u_own = [&](int z) {
-    const bool ok = own && z >= 0 && z < F.nz;
-    const V4<float> A = ld4_if(ua + eo + sz * z, ok);
-    if (MODE == SM_POST) return u_post(A, x0, y, z, ok);
-    const V4<float> W = MODE == SM_PRE ? ld4_if(F.w + eo + sz * z, ok) : A;
-    return u_of(A, W);
-  };
-  auto u_halo = [&](int z) {
-    const bool ok = hok && z >= 0 && z < ze;
-    V4<float> A = zero4<float>(), W = zero4<float>();
-    if (hrole == 1) {
-      A = ld4_if(ua + he + sz * z, ok);
-      if (MODE == SM_POST) return u_post(A, hx, hy, z, ok);
-      if (MODE == SM_PRE) W = ld4_if(F.w + he + sz * z, ok);
-    } else if (hrole == 2 && ok) {
-      A.a[0] = ua[he + sz * z];
-      if (MODE == SM_POST) A.a[0] = A.a[0] + pxc(hx, hy, z);
-      if (MODE == SM_PRE) W.a[0] = F.w[he + sz * z];
-    }
-    if (MODE == SM_POST) return A;
-    return u_of(A, W);
-  };
-  auto put = [&](int z, const V4<float>& U, const V4<float>& H) {
-    *reinterpret_cast<float4*>(&ub[z & 1][ty + 1][4 + 4 * g]) = make_float4(U.a[0], U.a[1], U.a[2], U.a[3]);
-    if (hrole == 1) *reinterpret_cast<float4*>(&ub[z & 1][hrow][hcol]) = make_float4(H.a[0], H.a[1], H.a[2], H.a[3]);
-    else if (hrole == 2) ub[z & 1][hrow][hcol] = H.a[0];
-  };
-  auto ld_site = [&](const float* a, int z) { return ld4_if(a + eo + sz * z, own && z < ze); };
-  V4<float> up = u_own(zb - 1), uc = u_own(zb), un = u_own(zb + 1);
-  V4<float> Rc = ld_site(F.rhs, zb), Dc = ld_site(F.d, zb), Wc = ld_site(F.w, zb);
-  V4<float> Hn = u_halo(zb + 1);
-  put(zb, uc, u_halo(zb));
-  __syncthreads();
-  for (int z = zb; z < ze; ++z) {
-    const V4<float> unn = u_own(z + 2 <= ze ? z + 2 : -1);
-    const V4<float> Hnn = u_halo(z + 2);
-    const V4<float> Rn = ld_site(F.rhs, z + 1), Dn = ld_site(F.d, z + 1), Wn = ld_site(F.w, z + 1);
-    if (z + 1 < ze) put(z + 1, un, Hn);
-    if (own) {
-      const float* mid = &ub[z & 1][ty + 1][4 + 4 * g];
-      const float4 a = *reinterpret_cast<const float4*>(mid - kZmPitch);
-      const float4 b = *reinterpret_cast<const float4*>(mid + kZmPitch);
-      const float ym[4] = {a.x, a.y, a.z, a.w}, yp[4] = {b.x, b.y, b.z, b.w};
-      const float lft = mid[-1], rgt = mid[4];
-      V4<float> Xo;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int x = x0 + k;
-        float nb = 0.f;
-        if (x > 0) nb += k > 0 ? uc.a[k - 1] : lft;
-        if (x < F.nx - 1) nb += k < 3 ? uc.a[k + 1] : rgt;
-        if (y > 0) nb += ym[k];
-        if (y < F.ny - 1) nb += yp[k];
-        if (z > 0) nb += up.a[k];
-        if (z < F.nz - 1) nb += un.a[k];
-        const float u0 = uc.a[k];
-        const float res = resid(Rc.a[k], Dc.a[k], u0, F.c, nb);
-        Xo.a[k] = fmaf(wt(MODE == SM_LAST ? MG_W1 : MG_W2, Wc.a[k]), res, u0);
-      }
-      *reinterpret_cast<V4<float>*>((MODE == SM_POST ? F.t : F.x) + eo + sz * z) = Xo;
-    }
-    up = uc;
-    uc = un;
-    un = unn;
-    Rc = Rn;
-    Dc = Dn;
-    Wc = Wn;
-    Hn = Hnn;
-    __syncthreads();
-  }
-}
-
-// TMA form of the plane-marching pre-sweeps (same tiles, slabs and
-// per-site arithmetic as k_mg_pre0_z).  One thread issues, per plane, two
-// tensor copies (r and 1/d) of the box x0 - 4 .. x0 + 4 kZmG + 3 by
-// y0 - 1 .. y0 + kZmY into one of kTmStages shared-memory stages, completing
-// on the stage's mbarrier; the copy engine fills sites outside the lattice
-// with zeros, so the halo needs no bounds checks.  A plane is consumed
-// kTmStages - 2 planes after its copy was issued; a stage is refilled after
-// the block barrier that follows its last use.  Waits are bounded: on a
-// timeout the block records SYNC_ERR_TIMEOUT, waits (bounded) for its copies
-// in flight and returns.
-constexpr int kTmW = 4 * kZmG + 8, kTmH = kZmY + 2;
-constexpr int kTmPlane = kTmW * kTmH;                      // floats per array and plane
-constexpr int kTmPlaneF = ((kTmPlane * 4 + 127) / 128) * 32;  // stage slot in floats (128-byte multiple)
-constexpr int kTmStages = 4;
-constexpr int kTmSmem = kTmStages * 2 * kTmPlaneF * 4 + 128;
-constexpr int kTmWaitLimit = 1 << 20;
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(float* sdst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
-          "r"(tc::smem_u32(sdst)),
-      "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(tc::smem_u32(bar))
-      : "memory");
-}
-
-__global__ void __launch_bounds__(kZmThreads, 7)
-    k_mg_pre0_t(Ctx c, int which, float* __restrict__ dst, int zs, const __grid_constant__ CUtensorMap tm_r,
-                const __grid_constant__ CUtensorMap tm_w) {
-  HCA_VC_ENTRY(c);
-  extern __shared__ __align__(128) float tsm_raw[];
-  __shared__ __align__(8) uint64_t bar[kTmStages];
-  // stage slots start on a 128-byte boundary (the launch adds 128 bytes)
-  float* tsm = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(tsm_raw) + 127) & ~uintptr_t(127));
-  const RepDesc& rd = c.reps[0];
-  const float cpl = op_coupling_t<float>(rd, which);
-  const int t = threadIdx.x, g = t % kZmG, ty = t / kZmG;
-  const int G = blockIdx.x * kZmG + g, y = blockIdx.y * kZmY + ty;
-  const int x0 = 4 * G;
-  const bool own = G < rd.gpr && y < rd.ny;
-  const long long sy = rd.nxp, sz = (long long)rd.nxp * rd.ny;
-  const long long eo = rd.off + x0 + sy * y;
-  const int zb = blockIdx.z * zs, ze = min(rd.nz, zb + zs);
-  const int bx = 4 * kZmG * blockIdx.x - 4, by = kZmY * blockIdx.y - 1;
-  const int nk = ze - zb + 2;   // planes zb - 1 .. ze, plane p at k = p - zb + 1
-  if (t == 0) {
-    for (int s = 0; s < kTmStages; ++s) tc::mbar_init(&bar[s], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  __syncthreads();
-  auto slot = [&](int k, int a) { return tsm + (2 * (k % kTmStages) + a) * kTmPlaneF; };
-  auto issue = [&](int k) {
-    uint64_t* b = &bar[k % kTmStages];
-    mbar_expect_tx(b, 2 * kTmPlane * 4);
-    tma_load_3d(slot(k, 0), &tm_r, bx, by, zb - 1 + k, b);
-    tma_load_3d(slot(k, 1), &tm_w, bx, by, zb - 1 + k, b);
-  };
-  auto ready = [&](int k) { return tc::mbar_wait(&bar[k % kTmStages], (uint32_t)((k / kTmStages) & 1), kTmWaitLimit); };
-  int issued = min(kTmStages, nk);
-  if (t == 0)
-    for (int k = 0; k < issued; ++k) issue(k);
-  // own group in a box: row ty + 1, columns 4 + 4 g ..
-  const int oc = (ty + 1) * kTmW + 4 + 4 * g;
-  auto own4 = [&](int k, int a) {
-    const float4 v = *reinterpret_cast<const float4*>(slot(k, a) + oc);
-    V4<float> r;
-    r.a[0] = v.x;
-    r.a[1] = v.y;
-    r.a[2] = v.z;
-    r.a[3] = v.w;
-    return r;
-  };
-  auto u_of = [&](const V4<float>& R, const V4<float>& W) {
-    V4<float> U;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) U.a[e] = (x0 + e < rd.nx) ? pre0_u(R.a[e], W.a[e]) : 0.f;
-    return U;
-  };
-  bool ok = ready(0);
-  ok = ready(1) && ok;
-  V4<float> up, uc, Rc, Wc;
-  if (ok) {
-    up = u_of(own4(0, 0), own4(0, 1));
-    Rc = own4(1, 0);
-    Wc = own4(1, 1);
-    uc = u_of(Rc, Wc);
-  }
-  bool failed = false;   // the same in every thread of the block
-  for (int z = zb;; ++z) {
-    const bool more = z < ze;
-    if (more && ok) ok = ready(z - zb + 2);
-    // one decision per block: every thread stops together on a timeout
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
-    if (!more) break;
-    const int k = z - zb + 1;
-    // every thread is past plane z - 1: its stage takes plane k - 1 + kTmStages
-    if (t == 0 && k - 1 + kTmStages < nk) {
-      issue(k - 1 + kTmStages);
-      issued = k + kTmStages;
-    }
-    const V4<float> Rn = own4(k + 1, 0), Wn = own4(k + 1, 1);
-    const V4<float> un = u_of(Rn, Wn);   // plane z + 1 (zero above the lattice)
-    if (own) {
-      const float* br = slot(k, 0) + oc;
-      const float* bw = slot(k, 1) + oc;
-      const float4 ymr = *reinterpret_cast<const float4*>(br - kTmW), ymw = *reinterpret_cast<const float4*>(bw - kTmW);
-      const float4 ypr = *reinterpret_cast<const float4*>(br + kTmW), ypw = *reinterpret_cast<const float4*>(bw + kTmW);
-      const float ymv[4] = {pre0_u(ymr.x, ymw.x), pre0_u(ymr.y, ymw.y), pre0_u(ymr.z, ymw.z), pre0_u(ymr.w, ymw.w)};
-      const float ypv[4] = {pre0_u(ypr.x, ypw.x), pre0_u(ypr.y, ypw.y), pre0_u(ypr.z, ypw.z), pre0_u(ypr.w, ypw.w)};
-      const float lft = pre0_u(br[-1], bw[-1]), rgt = pre0_u(br[4], bw[4]);
-      V4<float> VO = zero4<float>();   // zero on padding
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int x = x0 + e;
-        if (x >= rd.nx) continue;
-        const float left = e == 0 ? lft : uc.a[e - 1];
-        const float right = e == 3 ? rgt : uc.a[e + 1];
-        const float nb = (x > 0 ? left : 0.f) + (x < rd.nx - 1 ? right : 0.f) + ymv[e] + ypv[e] + up.a[e] + un.a[e];
-        VO.a[e] = pre0_site(Rc.a[e], Wc.a[e], uc.a[e], cpl, nb);
-      }
-      st4(dst + eo + sz * z, VO);
-    }
-    up = uc;
-    uc = un;
-    Rc = Rn;
-    Wc = Wn;
-  }
-  if (failed) {
-    // a copy did not complete in time: record it, and let this block's
-    // copies in flight land before its shared memory is released
-    if (t == 0) {
-      c.sync->error = SYNC_ERR_TIMEOUT;
-      for (int k = max(0, issued - kTmStages); k < issued; ++k) (void)ready(k);
-    }
-    __syncthreads();
   }
 }
 
@@ -1758,19 +1323,12 @@ void launch_post0(const Ctx& c, int which, const MGHost& H, const T* src, T om) 
   }
 }
 
-// Level l >= 1 sweeps in plane-marching form (one FP32 lattice; configured
-// by mg_zmarch_config).
-template <typename T>
-bool zlevel(const MGHost& H, int l) {
-  return std::is_same<T, float>::value && l < MG_MAXLEV && H.zl_slabs[l] > 0 && (H.rows_ok >> l & 1u);
-}
-
-// part: -1 = whole cycle; 0 = r scaling (only with `scale`: right after a
-// residual was formed, i.e. at the start of a solve or a defect-correction
-// sweep); 1 = the lattice's pre-sweeps; 2 = its restriction; 3 = the coarse
-// levels; 4 = the lattice's prolongation and first post-sweep; 5 = its last
-// post-sweep with r.z.  A lattice that is the coarsest level runs its sweeps
-// as part 3.
+// part: -1 = whole cycle; 0 = r scaling (FP32 lattice that is its own
+// coarsest level, only with `scale`: right after a residual was formed); 1 =
+// the lattice's pre-sweeps; 2 = its restriction (FP32: both, k_mg_down); 3 =
+// the coarse levels; 4 = the lattice's prolongation and first post-sweep
+// (FP32: both post-sweeps, k_mg_up); 5 = its last post-sweep with r.z.  A
+// lattice that is the coarsest level runs its sweeps as part 3.
 template <typename T>
 void vcycle_t(const Ctx& c, int which, const MGHost& H, int part, bool scale) {
   cudaStream_t s = c.stream;
@@ -1778,13 +1336,10 @@ void vcycle_t(const Ctx& c, int which, const MGHost& H, int part, bool scale) {
   T* z = (T*)c.z;
   const bool all = part < 0;
   const bool multi = c.n_reps > 1;
-  if (scale && (all || part == 0)) {
-    if (c.n_reps == 1)
-      launch_k(c.pdl != 0, k_mg_scale0_rows<T>, dim3(grid_for(H.ntot[0] / 4 + 1)), dim3(kMgThreads), 0, s, c);
-    else
-      launch_k(c.pdl != 0, k_mg_scale0<T>, dim3(grid_for(H.ntot[0])), dim3(kMgThreads), 0, s, c, which);
-  }
+  const bool pdl = c.pdl != 0;
   if (H.nlev == 1) {
+    if (scale && (all || part == 0))
+      launch_k(pdl, k_mg_scale0_rows<T>, dim3(grid_for(H.ntot[0] / 4 + 1)), dim3(kMgThreads), 0, s, c);
     if (!all && part != 3) return;
     // the lattice is the coarsest level (single replicate): MG_NU_COARSE
     // sweeps, the last one in post0
@@ -1797,90 +1352,76 @@ void vcycle_t(const Ctx& c, int which, const MGHost& H, int part, bool scale) {
     k_mg_post0<T, false, 0><<<c.n_chunks, c.threads, 0, s>>>(c, which, src, (T)MG_OMEGA_COARSE);
     return;
   }
-  // 128 threads: the lattice kernels keep ~20-28 vector loads per thread in flight
-  const int nb = (int)std::max(1LL, std::min((H.nrowitems + 127) / 128, 152LL * 16));
-  // register budgets (blocks per SM): 5 for the pre-sweeps (a few spilled
-  // registers; measured 71.4 -> 67.6 us at 256^3), 4 for the restriction
-  // (61.4 us; 65.5 us with 5)
-  const bool pdl = c.pdl != 0;
-  if (all || part == 1) {
-    if constexpr (std::is_same<T, float>::value) {
-      if (H.zm_slabs > 0 && H.zm_mode == 2) {
-        launch_k(pdl, k_mg_pre0_t, dim3(H.zm_tx, H.zm_ty, H.zm_slabs), dim3(kZmThreads), (size_t)kTmSmem, s, c, which,
-                 z, H.zm_zs, H.zm_map_r, H.zm_map_w);
-      } else if (H.zm_slabs > 0) {
-        launch_k(pdl, k_mg_pre0_z, dim3(H.zm_tx, H.zm_ty, H.zm_slabs), dim3(kZmThreads), 0, s, c, which, z, H.zm_zs);
-      } else {
-        launch_k(pdl, k_mg_pre0<T>, dim3(nb), dim3(128), 0, s, c, which, z);
-      }
-    } else {
-      launch_k(pdl, k_mg_pre0<T>, dim3(nb), dim3(128), 0, s, c, which, z);
+  if constexpr (std::is_same<T, float>::value) {
+    if (all || part == 2) launch_march(c, which, H, 0, true);
+    if (all || part == 3) {
+      for (int l = 1; l < H.small; ++l) launch_march(c, which, H, l, true);
+      launch_mg_cluster(c, which, H);
+      for (int l = H.small - 1; l >= 1; --l) launch_march(c, which, H, l, false);
     }
+    if (all || part == 4) launch_march(c, which, H, 0, false);
+  } else {
+    // 128 threads: the lattice kernels keep ~20-28 vector loads per thread in
+    // flight; register budgets (blocks per SM): 5 for the pre-sweeps, 4 for
+    // the restriction
+    const int nb = (int)std::max(1LL, std::min((H.nrowitems + 127) / 128, 152LL * 16));
+    if (all || part == 1) launch_k(pdl, k_mg_pre0<T>, dim3(nb), dim3(128), 0, s, c, which, z);
+    if (all || part == 2) launch_k(pdl, k_mg_restrict0_rows<T>, dim3(nb), dim3(128), 0, s, c, which, (const T*)z);
+    if (all || part == 3) {
+      // levels 1 .. lo-1 by per-level kernels, lo .. nlev-1 in the cooperative
+      // launch when there is one (lo = small: no level in it but the
+      // single-block ones, which then run in their own kernel)
+      const bool coop = H.coop_blocks > 0 && H.coop_from < H.small;
+      const int lo = coop ? H.coop_from : H.small;
+      for (int l = 1; l < lo; ++l) {
+        if (H.rows_ok >> l & 1u) {
+          launch_k(pdl, k_mg_smooth_rows<T, SM_PRE>, dim3(grid_for(H.post_items[l])), dim3(kMgThreads), 0, s, c, which, l);
+          // 128 threads: ~12 vector loads per thread in flight
+          launch_k(pdl, k_mg_restrict_rows<T>, dim3((int)std::min((H.restr_items[l] + 127) / 128, 152LL * 16)),
+                   dim3(128), 0, s, c, which, l);
+        } else if (multi) {
+          launch_k(pdl, k_mg_smooth<T, true, SM_PRE>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
+          launch_k(pdl, k_mg_restrict<T, true>, dim3(grid_for(H.ntot[l + 1])), dim3(kMgThreads), 0, s, c, which, l);
+        } else {
+          launch_k(pdl, k_mg_smooth<T, false, SM_PRE>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
+          launch_k(pdl, k_mg_restrict<T, false>, dim3(grid_for(H.ntot[l + 1])), dim3(kMgThreads), 0, s, c, which, l);
+        }
+      }
+      if (coop) {
+        Ctx cc = c;
+        int wh = which, l0 = lo, sm = H.small, use = H.small_smem > 0;
+        unsigned rows = H.rows_ok;
+        void* args[] = {&cc, &wh, &l0, &sm, &rows, &use};
+        (void)cudaLaunchCooperativeKernel(coarse_fn<T>(H.coop_cfg), dim3(H.coop_blocks),
+                                          dim3(coarse_threads(H.coop_cfg)), args, (size_t)H.small_smem, s);
+      } else if (H.small_smem > 0 && H.small_smem_ok) {
+        launch_k(pdl, k_mg_small_smem<T>, dim3(c.n_reps), dim3(kSmallThreads), (size_t)H.small_smem, s, c, which);
+      } else {
+        launch_k(pdl, k_mg_small<T>, dim3(c.n_reps), dim3(kSmallThreads), 0, s, c, which);
+      }
+      for (int l = lo - 1; l >= 1; --l) {
+        if (H.rows_ok >> l & 1u) {
+          launch_k(pdl, k_mg_smooth_rows<T, SM_POST>, dim3(grid_for(H.post_items[l])), dim3(kMgThreads), 0, s, c, which, l);
+          launch_k(pdl, k_mg_smooth_rows<T, SM_LAST>, dim3(grid_for(H.post_items[l])), dim3(kMgThreads), 0, s, c, which, l);
+        } else if (multi) {
+          launch_k(pdl, k_mg_smooth<T, true, SM_POST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
+          launch_k(pdl, k_mg_smooth<T, true, SM_LAST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
+        } else {
+          launch_k(pdl, k_mg_smooth<T, false, SM_POST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
+          launch_k(pdl, k_mg_smooth<T, false, SM_LAST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
+        }
+      }
+    }
+    if (all || part == 4) launch_post0<T, true>(c, which, H, nullptr, T(0));
+    if (all || part == 5) launch_post0<T, false>(c, which, H, t0, (T)MG_W1);
   }
-  if (all || part == 2) launch_k(pdl, k_mg_restrict0_rows<T>, dim3(nb), dim3(128), 0, s, c, which, (const T*)z);
-  if (all || part == 3) {
-    // levels 1 .. lo-1 by per-level kernels, lo .. nlev-1 in the cooperative
-    // launch when there is one (lo = small: no level in it but the
-    // single-block ones, which then run in their own kernel)
-    const bool coop = H.coop_blocks > 0 && H.coop_from < H.small;
-    const int lo = coop ? H.coop_from : H.small;
-    for (int l = 1; l < lo; ++l) {
-      if (zlevel<T>(H, l)) {
-        launch_k(pdl, k_mg_smooth_z<SM_PRE>, dim3(H.zl_tx[l], H.zl_ty[l], H.zl_slabs[l]), dim3(kZmThreads), 0, s, c,
-                 which, l, H.zl_zs[l]);
-        launch_k(pdl, k_mg_restrict_rows<T>, dim3((int)std::min((H.restr_items[l] + 127) / 128, 152LL * 16)), dim3(128),
-                 0, s, c, which, l);
-      } else if (H.rows_ok >> l & 1u) {
-        launch_k(pdl, k_mg_smooth_rows<T, SM_PRE>, dim3(grid_for(H.post_items[l])), dim3(kMgThreads), 0, s, c, which, l);
-        // 128 threads: ~12 vector loads per thread in flight
-        launch_k(pdl, k_mg_restrict_rows<T>, dim3((int)std::min((H.restr_items[l] + 127) / 128, 152LL * 16)), dim3(128),
-                 0, s, c, which, l);
-      } else if (multi) {
-        launch_k(pdl, k_mg_smooth<T, true, SM_PRE>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
-        launch_k(pdl, k_mg_restrict<T, true>, dim3(grid_for(H.ntot[l + 1])), dim3(kMgThreads), 0, s, c, which, l);
-      } else {
-        launch_k(pdl, k_mg_smooth<T, false, SM_PRE>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
-        launch_k(pdl, k_mg_restrict<T, false>, dim3(grid_for(H.ntot[l + 1])), dim3(kMgThreads), 0, s, c, which, l);
-      }
-    }
-    if (coop) {
-      Ctx cc = c;
-      int wh = which, l0 = lo, sm = H.small, use = H.small_smem > 0;
-      unsigned rows = H.rows_ok;
-      void* args[] = {&cc, &wh, &l0, &sm, &rows, &use};
-      (void)cudaLaunchCooperativeKernel(coarse_fn<T>(H.coop_cfg), dim3(H.coop_blocks),
-                                        dim3(coarse_threads(H.coop_cfg)), args, (size_t)H.small_smem, s);
-    } else if (H.small_smem > 0 && H.small_smem_ok) {
-      launch_k(pdl, k_mg_small_smem<T>, dim3(c.n_reps), dim3(kSmallThreads), (size_t)H.small_smem, s, c, which);
-    } else {
-      launch_k(pdl, k_mg_small<T>, dim3(c.n_reps), dim3(kSmallThreads), 0, s, c, which);
-    }
-    for (int l = lo - 1; l >= 1; --l) {
-      if (zlevel<T>(H, l)) {
-        launch_k(pdl, k_mg_smooth_z<SM_POST>, dim3(H.zl_tx[l], H.zl_ty[l], H.zl_slabs[l]), dim3(kZmThreads), 0, s, c,
-                 which, l, H.zl_zs[l]);
-        launch_k(pdl, k_mg_smooth_z<SM_LAST>, dim3(H.zl_tx[l], H.zl_ty[l], H.zl_slabs[l]), dim3(kZmThreads), 0, s, c,
-                 which, l, H.zl_zs[l]);
-      } else if (H.rows_ok >> l & 1u) {
-        launch_k(pdl, k_mg_smooth_rows<T, SM_POST>, dim3(grid_for(H.post_items[l])), dim3(kMgThreads), 0, s, c, which, l);
-        launch_k(pdl, k_mg_smooth_rows<T, SM_LAST>, dim3(grid_for(H.post_items[l])), dim3(kMgThreads), 0, s, c, which, l);
-      } else if (multi) {
-        launch_k(pdl, k_mg_smooth<T, true, SM_POST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
-        launch_k(pdl, k_mg_smooth<T, true, SM_LAST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
-      } else {
-        launch_k(pdl, k_mg_smooth<T, false, SM_POST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
-        launch_k(pdl, k_mg_smooth<T, false, SM_LAST>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, s, c, which, l);
-      }
-    }
-  }
-  if (all || part == 4) launch_post0<T, true>(c, which, H, nullptr, T(0));
-  if (all || part == 5) launch_post0<T, false>(c, which, H, t0, (T)MG_W1);
 }
 
 template <typename T>
 void mg_setup_t(const Ctx& c, int which, const MGHost& H, bool w_done) {
   const bool pdl = c.pdl != 0;
-  if (!w_done) launch_k(pdl, k_mg_w0<T>, dim3(grid_for(H.ntot[0])), dim3(kMgThreads), 0, c.stream, c, which);
+  // the marching sweeps form the lattice's 1 / d from d as they go
+  if (!w_done && !H.march) launch_k(pdl, k_mg_w0<T>, dim3(grid_for(H.ntot[0])), dim3(kMgThreads), 0, c.stream, c, which);
   for (int l = 1; l < H.nlev; ++l)
     launch_k(pdl, k_mg_diag<T>, dim3(grid_for(H.ntot[l])), dim3(kMgThreads), 0, c.stream, c, which, l);
 }
@@ -1957,97 +1498,8 @@ void mg_coop_config(MGHost& H, bool fp64, int sm_count, long long smem_bytes) {
     return;
   }
   if (fp64) coop_config_t<double>(H, sm_count, smem_bytes);
-  else coop_config_t<float>(H, sm_count, smem_bytes);
 }
 // (H.small: the deepest grid-kernel level + 1 over the batch)
-
-// A 3-D tensor map over one lattice array (x extent nx, rows nxp apart),
-// box kTmW x kTmH x 1, zero fill outside.  False if the driver entry point is
-// missing or the encoding is refused.
-bool lattice_map(CUtensorMap* m, const float* base, const RepDesc& rd) {
-  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static Encode enc = nullptr;
-  if (!enc) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn) {
-      (void)cudaGetLastError();
-      return false;
-    }
-    enc = (Encode)fn;
-  }
-  const float* p = base + rd.off;
-  if ((reinterpret_cast<uintptr_t>(p) & 15u) || (rd.nxp * 4) % 16) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)rd.nx, (cuuint64_t)rd.ny, (cuuint64_t)rd.nz};
-  const cuuint64_t strides[2] = {(cuuint64_t)rd.nxp * 4, (cuuint64_t)rd.nxp * rd.ny * 4};
-  const cuuint32_t box[3] = {(cuuint32_t)kTmW, (cuuint32_t)kTmH, 1};
-  const cuuint32_t es[3] = {1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(p), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Form and geometry of the lattice's pre-sweeps on one FP32 lattice rd
-// (arrays r and w): the plane-marching kernel with its planes staged by TMA
-// tensor copies (default; the register-prefetch form when the tensor maps
-// cannot be made or HCA_MG_ZMARCH=1), or the row form (HCA_MG_ZMARCH=0).
-// Tiles of kZmG groups by kZmY rows; the planes split into slabs so that
-// the grid is a whole number of waves of resident blocks, at most
-// HCA_MG_ZM_WAVES (default 1 for the TMA form, 2 for the register form:
-// measured best at 256^3).
-void mg_zmarch_config(MGHost& H, const RepDesc& rd, int sm_count, const float* r, const float* w,
-                      const int* lv_dims) {
-  H.zm_slabs = 0;
-  const char* e = std::getenv("HCA_MG_ZMARCH");
-  if ((e && e[0] == '0') || H.nlev <= 1) return;
-  H.zm_mode = (e && e[0] == '1') ? 1 : 2;
-  if (H.zm_mode == 2 && !(lattice_map(&H.zm_map_r, r, rd) && lattice_map(&H.zm_map_w, w, rd))) H.zm_mode = 1;
-  const void* fn = H.zm_mode == 2 ? (const void*)k_mg_pre0_t : (const void*)k_mg_pre0_z;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kZmThreads, H.zm_mode == 2 ? kTmSmem : 0) !=
-          cudaSuccess ||
-      per_sm < 1) {
-    (void)cudaGetLastError();
-    return;
-  }
-  const char* wv = std::getenv("HCA_MG_ZM_WAVES");
-  const double waves = wv ? std::max(0.05, std::atof(wv)) : (H.zm_mode == 2 ? 1.0 : 2.0);
-  H.zm_tx = (rd.gpr + kZmG - 1) / kZmG;
-  H.zm_ty = (rd.ny + kZmY - 1) / kZmY;
-  const double tiles = (double)H.zm_tx * H.zm_ty;
-  const long long want = (long long)(waves * sm_count * per_sm / tiles);   // whole waves at most
-  const int slabs = (int)std::max(1LL, std::min((long long)rd.nz, want));
-  H.zm_zs = (rd.nz + slabs - 1) / slabs;
-  H.zm_slabs = (rd.nz + H.zm_zs - 1) / H.zm_zs;
-  // grid levels with whole-group rows: the same tiles, slabs for at most
-  // HCA_MG_ZL_WAVES waves (default 1); HCA_MG_ZLEVELS=0 keeps their row form
-  const char* zl = std::getenv("HCA_MG_ZLEVELS");
-  if (zl && zl[0] == '0') return;
-  int per_sm_l = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_l, (const void*)k_mg_smooth_z<SM_PRE>, kZmThreads, 0) !=
-          cudaSuccess ||
-      per_sm_l < 1) {
-    (void)cudaGetLastError();
-    return;
-  }
-  const char* lw = std::getenv("HCA_MG_ZL_WAVES");
-  const double lwaves = lw ? std::max(0.05, std::atof(lw)) : 1.0;
-  for (int l = 1; l < std::min(H.small, MG_MAXLEV); ++l) {
-    if (!(H.rows_ok >> l & 1u)) continue;
-    const int nx = lv_dims[3 * l], ny = lv_dims[3 * l + 1], nz = lv_dims[3 * l + 2];
-    if (nx % 4) continue;
-    H.zl_tx[l] = (nx / 4 + kZmG - 1) / kZmG;
-    H.zl_ty[l] = (ny + kZmY - 1) / kZmY;
-    const double tl = (double)H.zl_tx[l] * H.zl_ty[l];
-    const long long wl = (long long)(lwaves * sm_count * per_sm_l / tl);
-    const int sl = (int)std::max(1LL, std::min((long long)nz, wl));
-    H.zl_zs[l] = (nz + sl - 1) / sl;
-    H.zl_slabs[l] = (nz + H.zl_zs[l] - 1) / H.zl_zs[l];
-  }
-}
 
 // w_done: the lattice's 1/d is already in place (the first defect-correction
 // residual sweep of an FP32 solve forms it).
@@ -2062,8 +1514,9 @@ void launch_vcycle(const Ctx& c, int which, bool fp64, const MGHost& H, int part
 }
 
 int vcycle_part_launches(const MGHost& H, int part, bool scale) {
-  if (part == 0) return scale ? 1 : 0;
-  if (H.nlev == 1) return part == 3 ? MG_NU_COARSE : 0;
+  if (H.nlev == 1) return part == 0 ? (scale ? 1 : 0) : part == 3 ? MG_NU_COARSE : 0;
+  if (H.march) return part == 2 || part == 4 ? 1 : part == 3 ? 2 * (H.small - 1) + 1 : 0;
+  if (part == 0) return 0;
   if (part == 3) {
     const int lo = H.coop_blocks > 0 && H.coop_from < H.small ? H.coop_from : H.small;
     return 4 * (lo - 1) + 1;

@@ -351,7 +351,7 @@ __global__ void __maxnreg__(REGS) k_pass_b(Ctx c, int which, void* xfield, CondA
     const T* __restrict__ qq = (const T*)c.q;
     T* __restrict__ xx = (T*)xfield;
     const T alpha = (T)sv.alpha;
-    const T zs = (sv.iters == 0 && !mg) ? (T)sv.scale : T(1);
+    const T zs = (sv.iters == 0 && (!mg || c.lazy_scale)) ? (T)sv.scale : T(1);
     const RowIter it = row_iter(rd);
     auto row = [&](int chunk, int rl, bool row_ok, int j) {
       const RowGeo geo = row_geo(rd, j);
@@ -378,7 +378,7 @@ __global__ void __maxnreg__(REGS) k_pass_b(Ctx c, int which, void* xfield, CondA
               const T q = Q.a[k];
               X.a[k] += alpha * P.a[k];
               if (mg) {
-                Z.a[k] -= alpha * q;
+                Z.a[k] = zs * Z.a[k] - alpha * q;   // zs: a power of two
                 g_rr += Z.a[k] * Z.a[k];
               } else {
                 Z.a[k] = zs * Z.a[k] - alpha * (q / D.a[k]);
@@ -794,7 +794,7 @@ __global__ void __launch_bounds__(512) __maxnreg__(REGS) k_dc_residual(Ctx c, in
             }
             st4(dd + e, D);
             st4(aa + e, AR);
-            if (MG) {   // 1/d for the V-cycle's sweeps (0 where d = 0), as k_mg_w0 forms it
+            if (MG && c.mg_w) {   // 1/d for the sweeps of a lattice without coarse levels (0 where d = 0), as k_mg_w0 forms it
               V4<float> Wv;
 #pragma unroll
               for (int k = 0; k < 4; ++k) Wv.a[k] = D.a[k] != 0.f ? 1.f / D.a[k] : 0.f;
