@@ -33,6 +33,7 @@ UNITS = {
     "net.cu": [],
     "mg.cu": [],
     "march.cu": [],
+    "cg.cu": [],
     "coarse.cu": [],
 }
 

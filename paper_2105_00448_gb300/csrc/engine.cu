@@ -14,8 +14,11 @@
 
 namespace hca {
 void launch_setup(const Ctx& c, int which, bool fp64, CondArg cnd);
-void launch_pass_a(const Ctx& c, int which, bool fp64);
-void launch_pass_b(const Ctx& c, int which, void* xfield, bool fp64, CondArg cnd);
+void launch_pass_a(const Ctx& c, int which, bool fp64, bool defer);
+void launch_pass_b(const Ctx& c, int which, void* xfield, bool fp64, bool defer, CondArg cnd);
+bool cg_init();
+long long cg_plan(const std::vector<RepDesc>& reps, int sm_count, std::vector<MGLevel>& lv, std::vector<int4>& ablk,
+                  std::vector<int4>& bblk, std::vector<int4>& bgeo, int* a_nt);
 void launch_true_residual(const Ctx& c, int which, void* xfield, bool fp64);
 void launch_apply(const Ctx& c, int which, int rep, const void* u, void* out, bool fp64);
 void launch_diff_norms(const Ctx& c, const void* a, const void* b, bool fp64);
@@ -42,9 +45,10 @@ void mg_coop_config(MGHost& H, bool fp64, int sm_count, long long smem_bytes);
 int cluster_plan(const MGLevel* lv, int nl, int from, int cs, long long smem, MGCluster* R);
 bool cluster_init(const MGHost& H);
 bool march_init();
-void march_tile(MGLevel& L);
+void march_tile(MGLevel& L, int halo_rows);
 int march_threads(const std::vector<MGLevel*>& lv);
-void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, std::vector<int4>& out);
+void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, int extra,
+                  std::vector<int4>& out);
 }  // namespace hca
 
 using hca::Ctx;
@@ -419,10 +423,13 @@ void* field_ptr(hca_handle* h, uint32_t bit) {
 
 constexpr hca::CondArg kNoCond{0ull, 0};
 
-void pass_a(hca_handle* h, int which) { hca::launch_pass_a(h->ctx, which, h->fp64); }
+// A defect correction's inner solve: FP32 fields with max_outer sweeps.
+bool dc_solve(const hca_handle* h) { return !h->fp64 && h->max_outer > 0; }
+
+void pass_a(hca_handle* h, int which) { hca::launch_pass_a(h->ctx, which, h->fp64, dc_solve(h)); }
 
 void pass_b(hca_handle* h, int which, void* x, hca::CondArg cnd) {
-  hca::launch_pass_b(h->ctx, which, x, h->fp64, cnd);
+  hca::launch_pass_b(h->ctx, which, x, h->fp64, dc_solve(h), cnd);
 }
 
 // z = M r (V-cycle); also sets rho and beta for the next pass A.  first: the
@@ -905,16 +912,14 @@ int check_convergence(hca_handle* h) {
   return HCA_OK;
 }
 
-// Launch-shape autotuner: times the oxygen CG passes (the hot pair) for each
-// candidate block size (and register cap of the FP32 passes) on the handle's
-// own lattices, best of three timed runs each, and keeps the fastest.  It runs at creation, on the solver's
-// scratch vectors (x = aux), before anything depends on them; the reductions
-// sum by rows in a fixed order, so results do not depend on the choice.
-int autotune(hca_handle* h, bool tune_regs) {
+// Launch-shape autotuner (FP64 handles): times the oxygen CG passes (the hot
+// pair) for each candidate block size on the handle's own lattices, best of
+// three timed runs each, and keeps the fastest.  It runs at creation, on the
+// solver's scratch vectors (x = aux), before anything depends on them; the
+// reductions sum by rows in a fixed order, so results do not depend on the
+// choice.
+int autotune(hca_handle* h) {
   Ctx& c = h->ctx;
-  const int cand_t[3] = {128, 256, 512};
-  const int cand_r[4] = {64, 80, 96, 128};
-  const int nr = (tune_regs && !h->fp64) ? 4 : 1;
   constexpr int kIters = 8, kReps = 3;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   HCA_TRY(cudaEventCreate(&e0));
@@ -923,50 +928,43 @@ int autotune(hca_handle* h, bool tune_regs) {
     return HCA_ERR_CUDA;
   }
   float best = 1e30f;
-  int bt = c.threads, br = c.pass_regs;
+  int bt = c.threads;
   int rc = HCA_OK;
-  // the persistent row form runs at 128 threads: larger blocks timed faster
-  // here now and then but ran pass A ~20 % slower inside a step
-  const int nt = c.persist ? 1 : 3;
-  for (int ti = 0; ti < nt && !rc; ++ti)
-    for (int ri = 0; ri < nr && !rc; ++ri) {
-      c.threads = cand_t[ti];
-      if (nr > 1) c.pass_regs = cand_r[ri];
-      hca::launch_setup(c, 0, h->fp64, kNoCond);
-      for (int k = 0; k < 2; ++k) {   // warm-up
+  for (int threads : {128, 256, 512}) {
+    c.threads = threads;
+    hca::launch_setup(c, 0, h->fp64, kNoCond);
+    for (int k = 0; k < 2; ++k) {   // warm-up
+      pass_a(h, 0);
+      pass_b(h, 0, c.aux, kNoCond);
+    }
+    // the best of kReps timed runs (a single run is noisy enough to pick a
+    // slower shape now and then)
+    float ms = 1e30f;
+    for (int rep = 0; rep < kReps && !rc; ++rep) {
+      cudaEventRecord(e0, c.stream);
+      for (int k = 0; k < kIters; ++k) {
         pass_a(h, 0);
         pass_b(h, 0, c.aux, kNoCond);
       }
-      // the best of kReps timed runs (a single run is noisy enough to pick a
-      // slower shape now and then)
-      float ms = 1e30f;
-      for (int rep = 0; rep < kReps && !rc; ++rep) {
-        cudaEventRecord(e0, c.stream);
-        for (int k = 0; k < kIters; ++k) {
-          pass_a(h, 0);
-          pass_b(h, 0, c.aux, kNoCond);
-        }
-        cudaEventRecord(e1, c.stream);
-        float t = 0.f;
-        if (cudaGetLastError() != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-            cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) {
-          rc = HCA_ERR_CUDA;
-          break;
-        }
-        ms = std::min(ms, t);
+      cudaEventRecord(e1, c.stream);
+      float t = 0.f;
+      if (cudaGetLastError() != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+          cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) {
+        rc = HCA_ERR_CUDA;
+        break;
       }
-      if (rc) break;
-      h->launches += 1 + 2 * (kReps * kIters + 2);
-      if (ms < best) {
-        best = ms;
-        bt = c.threads;
-        br = c.pass_regs;
-      }
+      ms = std::min(ms, t);
     }
+    if (rc) break;
+    h->launches += 1 + 2 * (kReps * kIters + 2);
+    if (ms < best) {
+      best = ms;
+      bt = c.threads;
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   c.threads = bt;
-  c.pass_regs = br;
   if (rc) return rc;
   // the timed passes may have left solver flags set; the solves reset the rest
   HCA_TRY(cudaMemsetAsync(&c.sync->error, 0, sizeof(int), c.stream));
@@ -1113,14 +1111,12 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
   c.n_reps = n;
   c.n_chunks = chunk0;
   c.n_supers = super0;
-  // 128 threads per block measured fastest for the CG passes on GB300
+  // row kernels (residual, set-up, ODEs): 128 threads a block; lattices of few
+  // chunks (a flat one of 200 rows has 25) get more warps a chunk instead of
+  // idle multiprocessors (its ODEs: 0.30 ms at 128 threads, 0.13 at 512)
   c.threads = cfgs[0].threads_per_block ? cfgs[0].threads_per_block : 128;
-  c.pass_regs = 96;   // measured best at 128 threads; the autotuner may change both
-  {
-    // HCA_PASS_REGS=64|80|96|128 fixes the CG passes' register cap
-    const char* pr = std::getenv("HCA_PASS_REGS");
-    if (pr) c.pass_regs = std::atoi(pr);
-  }
+  if (!cfgs[0].threads_per_block && !h->fp64)
+    while (c.threads < 512 && (long long)chunk0 * c.threads < 512LL * c.sm_count) c.threads *= 2;
   c.stream = h->stream;
   const size_t es = elem_size(h);
   const size_t fbytes = (size_t)h->total * es;
@@ -1167,6 +1163,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
     ALLOC(c.d, fbytes);
     ALLOC(c.b, fbytes);
     ALLOC(c.aux, fbytes);
+    long long mslots = 0;   // reduction slots of the marching and streaming kernels
     if (h->mg) {
       // one hierarchy per replicate; each coarse level's arrays hold all
       // replicates back to back
@@ -1366,7 +1363,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
               L.d = (float*)c.d + r0.off;
               L.w = nullptr;
             }
-            hca::march_tile(L);
+            hca::march_tile(L, 2);
             if (l == 0) {
               L.slot0 = (int)slots;
               slots += (long long)L.tx * L.ty * L.nseg;
@@ -1376,15 +1373,14 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
           }
           H.mb_off[l] = (int)blocks.size();
           H.mb_nt[l] = hca::march_threads(set);
-          hca::march_blocks(set, ids, c.sm_count, blocks);
+          hca::march_blocks(set, ids, c.sm_count, 6, blocks);
           H.mb_n[l] = (int)blocks.size() - H.mb_off[l];
         }
         int4* blocks_d;
         ALLOC(blocks_d, sizeof(int4) * blocks.size());
-        ALLOC(c.mslot, sizeof(double) * (size_t)std::max(1LL, slots));
-        ALLOC(c.mcnt, sizeof(int) * (size_t)n);
+        mslots = std::max(mslots, slots);
         if (cudaMemcpyAsync(blocks_d, blocks.data(), sizeof(int4) * blocks.size(), cudaMemcpyHostToDevice, c.stream) ||
-            cudaMemsetAsync(c.mcnt, 0, sizeof(int) * (size_t)n, c.stream) || cudaStreamSynchronize(c.stream)) {
+            cudaStreamSynchronize(c.stream)) {
           rc = HCA_ERR_CUDA;
           goto fail;
         }
@@ -1430,6 +1426,35 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
         c.mg_restr_items = pre_d + post_pre.size();
       }
       c.mg = 1;
+    }
+    if (!h->fp64) {
+      // the FP32 CG passes: tilings, blocks and reduction slots
+      std::vector<hca::MGLevel> lv;
+      std::vector<int4> ab, bb, bg;
+      mslots = std::max(mslots, hca::cg_plan(h->reps_h, c.sm_count, lv, ab, bb, bg, &c.a_nt));
+      hca::MGLevel* lv_d;
+      int4 *ab_d, *bb_d, *bg_d;
+      ALLOC(lv_d, sizeof(hca::MGLevel) * lv.size());
+      ALLOC(ab_d, sizeof(int4) * ab.size());
+      ALLOC(bb_d, sizeof(int4) * bb.size());
+      ALLOC(bg_d, sizeof(int4) * bg.size());
+      ALLOC(c.mslot, sizeof(double) * (size_t)mslots);
+      ALLOC(c.mcnt, sizeof(int) * (size_t)n);
+      if (!hca::cg_init() ||
+          cudaMemcpyAsync(lv_d, lv.data(), sizeof(hca::MGLevel) * lv.size(), cudaMemcpyHostToDevice, c.stream) ||
+          cudaMemcpyAsync(ab_d, ab.data(), sizeof(int4) * ab.size(), cudaMemcpyHostToDevice, c.stream) ||
+          cudaMemcpyAsync(bb_d, bb.data(), sizeof(int4) * bb.size(), cudaMemcpyHostToDevice, c.stream) ||
+          cudaMemcpyAsync(bg_d, bg.data(), sizeof(int4) * bg.size(), cudaMemcpyHostToDevice, c.stream) ||
+          cudaMemsetAsync(c.mcnt, 0, sizeof(int) * (size_t)n, c.stream) || cudaStreamSynchronize(c.stream)) {
+        rc = HCA_ERR_CUDA;
+        goto fail;
+      }
+      c.cg_lv = lv_d;
+      c.ablk = ab_d;
+      c.bblk = bb_d;
+      c.bgeo = bg_d;
+      c.n_ablk = (int)ab.size();
+      c.n_bblk = (int)bb.size();
     }
     if (h->learned) {
       ALLOC(h->ws_cand, sizeof(double) * (size_t)h->total);
@@ -1563,10 +1588,11 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
       // the 27 colour sweeps of the CA in one cooperative launch (HCA_CA_COOP=0: one launch per colour)
       h->ca_coop = hca::ca_coop_blocks(h->fp64, c.sm_count);
     }
-    if (!cfgs[0].threads_per_block) {
+    // (the FP32 passes have one launch shape, chosen from the lattices)
+    if (!cfgs[0].threads_per_block && h->fp64) {
       const char* nt = std::getenv("HCA_NO_TUNE");
       if (!(nt && nt[0] == '1')) {
-        rc = autotune(h, std::getenv("HCA_PASS_REGS") == nullptr);
+        rc = autotune(h);
         if (rc) goto fail;
       }
     }
@@ -1889,7 +1915,7 @@ int hca_get_stats(hca_handle* h, int32_t rep, hca_stats* out) {
 int hca_get_launch_config(hca_handle* h, int32_t* threads_per_block, int32_t* pass_regs) {
   if (!h || !threads_per_block || !pass_regs) return HCA_ERR_ARG;
   *threads_per_block = h->ctx.threads;
-  *pass_regs = h->fp64 ? 128 : h->ctx.pass_regs;
+  *pass_regs = 128;   // every form of the passes is built for at most 128 registers
   return HCA_OK;
 }
 

@@ -106,6 +106,10 @@ struct RepSolve {
   int dc_apply;    // 1: the last inner solve's correction is to be added
   double bb_outer; // |b|^2 of the defect-corrected system (from its first sweep)
   double scale;    // power of two applied to the inner problem (1 for plain solves)
+  // FP32 inner solves of a defect correction: pass A of an iteration adds the
+  // step alpha p of the one before to dx; pend: the last step is still to be
+  // added (by the update), with p in buffer pbuf (0: p, 1: p_alt)
+  int pend, pbuf;
 };
 
 // Per-replicate statistics written by kernels; copied out by hca_get_stats.
@@ -379,7 +383,6 @@ struct Ctx {
   const void* lag;  // oxygen linearisation point (K_prev) when the solve starts elsewhere; null: the start field
   // multigrid preconditioner (single replicate): residual r (the Jacobi form
   // carries z = r / d instead), level-0 scratch, coarse level table
-  int pass_regs;    // register cap of the FP32 CG passes (64, 80, 96, 128)
   int pass_ni;      // groups per lane in a row shared by all replicates (1, 2, 4; 0 = differs)
   int mg;           // 0: Jacobi (z = r / d), 1: V-cycle (z = M r)
   int persist;         // 1: the CG passes and the lattice post-sweep run in persistent row form (one FP32 lattice)
@@ -393,6 +396,11 @@ struct Ctx {
   const int4* mblk;   // blocks of the marching sweeps: (replicate, tile, first plane, end plane)
   double* mslot;      // their segment sums
   int* mcnt;          // [rep] blocks done
+  const MGLevel* cg_lv;   // [rep] the lattice's tiling in the marching CG pass A
+  const int4* ablk;       // its blocks
+  const int4* bblk;       // blocks of the streaming pass B: (replicate, first chunk, end chunk, blocks of the replicate)
+  const int4* bgeo;       // [rep] pass B: groups, groups per chunk, chunks, first slot
+  int n_ablk, n_bblk, a_nt;
   const MGCluster* mgc;   // [rep] coarse levels in a cluster
   int lazy_scale;     // 1: the first inner iteration's kernels scale r as they read it
   const long long* mg_start;  // [MG_MAXLEV][n_reps + 1] prefix sums of each level's sites over the replicates

@@ -41,136 +41,19 @@
 #include <type_traits>
 #include <vector>
 
-#include "hca_internal.cuh"
+#include "march.cuh"
 
 namespace hca {
 
 namespace {
 
-constexpr int kMT = 256;              // most threads per block (instances: 64, 128, 256)
 constexpr int kDownRing = 5;          // planes k - 2 .. k + 2 of r and d
 constexpr int kUpRing = 3;            // planes k .. k + 2 of v' and d, k - 1 .. k + 1 of r
-constexpr int kMaxSeg = 32;           // z segments of a slab (reduction slots)
 constexpr float kW1 = (float)MG_W1, kW2 = (float)MG_W2;
 constexpr float kK = (float)(1.0 + MG_W2 * (1.0 - MG_W1) / MG_W1);
 constexpr float k1W1 = (float)(1.0 - MG_W1), k1W2 = (float)(1.0 - MG_W2);
 constexpr size_t down_smem(int nt) { return (size_t)(kDownRing * 4 + 2 * 2 + 2 * 2) * nt * 16; }
 constexpr size_t up_smem(int nt) { return (size_t)(kUpRing * 6 + 2 * 2 + 2) * nt * 16 + (size_t)kMaxSeg * (nt / 32) * 8; }
-constexpr int blocks_per_sm(int nt) { return nt >= 256 ? 2 : 512 / nt; }
-
-__device__ __forceinline__ void cp16(unsigned sdst, const float* gsrc, int n) {   // n = 0: zero fill
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sdst), "l"(gsrc), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp4(unsigned sdst, const float* gsrc, int n) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sdst), "l"(gsrc), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-// The patch's 4 x 2 values on one plane as pairs along x: the sums and
-// products below use the two-wide FP32 instructions (one issue for two
-// sites; every product and sum rounded as in the scalar form).
-struct P8 {
-  float2 v[2][2];   // [row][sites 0, 1 | 2, 3]
-};
-__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
-__device__ __forceinline__ void get_row(float2 (&v)[2], const float4* s) {
-  const float4 q = *s;
-  v[0] = make_float2(q.x, q.y);
-  v[1] = make_float2(q.z, q.w);
-}
-
-// 1 / d (0 where d = 0: padding, outside the level, an isolated empty site);
-// a smoothing weight, so the hardware reciprocal (1 ulp) serves
-__device__ __forceinline__ float inv_d(float d) {
-  float w;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(d));
-  return d > 0.f ? w : 0.f;
-}
-__device__ __forceinline__ float2 inv_d(float2 d) { return make_float2(inv_d(d.x), inv_d(d.y)); }
-
-// This thread's place in its block's tile.  Every tile carries its halo, also
-// at the level's edges (zeros there), so no neighbour needs a bounds check;
-// neighbours beyond the tile (of outermost halo patches, unused) read the
-// thread's own values.
-struct Patch {
-  int tid, lane, x0, y0;   // first site of the patch
-  int nx, nz;
-  int im, ip;          // row buffer slots of the rows below and above the patch
-  bool l0, l31;        // the x neighbour is in another warp
-  bool rok[2];         // the patch's rows inside the level (and the group)
-  bool out;            // the patch belongs to the tile's interior
-  bool part;           // the group has padding sites
-  unsigned e, sy, sz;  // element of (x0, y0, plane 0), strides (a field has fewer than 2^32 elements)
-};
-
-template <int NT>
-__device__ __forceinline__ Patch patch_of(const MGLevel& L, int4 b) {
-  Patch p;
-  p.tid = threadIdx.x;
-  p.lane = p.tid & 31;
-  const int cols = L.cols, pairs = L.pairs;
-  const int pr = p.tid / cols, col = p.tid - pr * cols;
-  p.nx = L.nx;
-  p.nz = L.nz;
-  const int ty = b.y / L.tx, tx = b.y - ty * L.tx;
-  const int g = tx * L.ox - 1 + col;
-  p.x0 = 4 * g;
-  p.y0 = ty * L.oy - 2 + 2 * pr;
-  const bool gok = g >= 0 && p.x0 < p.nx && pr < pairs;
-  p.rok[0] = gok && p.y0 >= 0 && p.y0 < L.ny;
-  p.rok[1] = gok && p.y0 >= 0 && p.y0 + 1 < L.ny;
-  p.out = p.rok[0] && col >= 1 && col <= L.ox && pr >= 1 && 2 * pr < 2 + L.oy;
-  p.part = p.x0 + 4 > p.nx;
-  p.im = NT + p.tid - (pr > 0 ? cols : 0);
-  p.ip = p.tid + (pr < pairs - 1 ? cols : 0);
-  p.l0 = p.lane == 0 && p.tid > 0;
-  p.l31 = p.lane == 31 && p.tid + 1 < NT;
-  p.sy = (unsigned)L.pitch;
-  p.sz = (unsigned)L.pitch * (unsigned)L.ny;
-  p.e = gok && p.y0 >= 0 ? (unsigned)p.x0 + p.sy * (unsigned)p.y0 : 0u;
-  return p;
-}
-
-// The sum over the neighbours of the patch on its own plane and the one
-// below: uc the plane (its rows also in row buffer B: [row of the
-// pair][thread]), um the plane below; S may be um.
-template <int NT>
-__device__ __forceinline__ void nb_patch(const Patch& p, const float4* __restrict__ B, const P8& uc, const P8& um,
-                                         P8& S) {
-  const float4 ym = B[p.im], yp = B[p.ip];
-  const float2 ymv[2] = {make_float2(ym.x, ym.y), make_float2(ym.z, ym.w)};
-  const float2 ypv[2] = {make_float2(yp.x, yp.y), make_float2(yp.z, yp.w)};
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    const float2 u0 = uc.v[a][0], u1 = uc.v[a][1];
-    float lft = __shfl_up_sync(0xffffffffu, u1.y, 1), rgt = __shfl_down_sync(0xffffffffu, u0.x, 1);
-    const float* Bf = reinterpret_cast<const float*>(B + a * NT + p.tid);
-    if (p.l0) lft = Bf[-1];
-    if (p.l31) rgt = Bf[4];
-    const float2 x[2] = {make_float2(lft + u0.y, u0.x + u1.x), make_float2(u0.y + u1.y, u1.x + rgt)};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const float2 m = a == 0 ? __fadd2_rn(ymv[h], uc.v[1][h]) : __fadd2_rn(uc.v[0][h], ypv[h]);
-      S.v[a][h] = __fadd2_rn(__fadd2_rn(x[h], m), um.v[a][h]);
-    }
-  }
-}
-
-template <int NT>
-__device__ __forceinline__ void put_patch(const Patch& p, float4* __restrict__ B, const P8& u) {
-#pragma unroll
-  for (int a = 0; a < 2; ++a) B[a * NT + p.tid] = make_float4(u.v[a][0].x, u.v[a][0].y, u.v[a][1].x, u.v[a][1].y);
-}
-
-__device__ __forceinline__ void zero_patch(P8& u) {
-#pragma unroll
-  for (int a = 0; a < 2; ++a) u.v[a][0] = u.v[a][1] = make_float2(0.f, 0.f);
-}
 
 // The coupling of level l of the operator: the lattice's FP32 coupling times
 // the level's scale.
@@ -182,34 +65,6 @@ __device__ __forceinline__ float level_coupling(const Ctx& c, int rep, int which
 // still unscaled: the factor the lattice kernels apply to r as they read it.
 __device__ __forceinline__ float r_scale(const RepSolve& sv) { return sv.iters == 0 ? (float)sv.scale : 1.f; }
 
-// The end of a marching kernel that sums into slots: the last block of the
-// replicate (nblk blocks) to arrive adds its n slots in an order that is the
-// same whatever the launch (64 lanes take every 64th slot, then a fixed
-// tree) and hands the sum to fin, called by one thread.
-template <class Fin>
-__device__ __forceinline__ void march_finish(const Ctx& c, int rep, int nblk, const double* slots, int n, Fin fin) {
-  __shared__ int s_last;
-  __shared__ double s_half[2];
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&c.mcnt[rep], 1) == nblk - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (threadIdx.x < 64) {
-    double t = 0.0;
-#pragma unroll 8
-    for (int i = threadIdx.x; i < n; i += 64) t += __ldcg(&slots[i]);
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if ((threadIdx.x & 31) == 0) s_half[threadIdx.x >> 5] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    fin(s_half[0] + s_half[1]);
-    c.mcnt[rep] = 0;
-  }
-}
-
 // ------------------------------------------------------------------ down --
 template <bool LAT, int NT>
 __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int which, int l, const int4* __restrict__ blocks) {
@@ -218,7 +73,7 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int wh
   const int rep = b.x;
   const MGLevel& L = ((const MGLevel*)c.mg_lv)[rep * MG_MAXLEV + l];
   const MGLevel& C = (&L)[1];
-  const Patch p = patch_of<NT>(L, b);
+  const Patch p = patch_of<NT, 2>(L, b);
   const int zb = b.z, ze = b.w;
   const float cpl = level_coupling(c, rep, which, L);
   const float2 w2c = dup(kW2 * cpl);
@@ -360,7 +215,7 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
   const int rep = b.x;
   const MGLevel& L = ((const MGLevel*)c.mg_lv)[rep * MG_MAXLEV + l];
   const MGLevel& C = (&L)[1];
-  const Patch p = patch_of<NT>(L, b);
+  const Patch p = patch_of<NT, 2>(L, b);
   const int zb = b.z, ze = b.w;
   const float cpl = level_coupling(c, rep, which, L);
   const float2 w2c = dup(kW2 * cpl);
@@ -544,21 +399,24 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
 // Tiling of a level: the fewest tiles of kMT patches (every halo patch is
 // redundant work).  It depends on the level's shape alone, as do the segment
 // sums, so results do not depend on slabs, batches or launch forms.
-void march_tile(MGLevel& L) {
-  const int gpr = (L.nx + 3) / 4, np = (L.ny + 1) / 2;   // groups per row, row pairs
+void march_tile(MGLevel& L, int halo_rows) {
+  const int gpr = (L.nx + 3) / 4;
   long long best = -1;
   for (int n = 1; n <= gpr; ++n) {
-    const int ox = (gpr + n - 1) / n, cols = ox + 2, most = kMT / cols - 2;   // row pairs of the interior
-    if (most < 1) continue;
-    const int op = (np + (np + most - 1) / most - 1) / ((np + most - 1) / most);   // even shares
-    const int tx = (gpr + ox - 1) / ox, ty = (np + op - 1) / op;
+    const int ox = (gpr + n - 1) / n, cols = ox + 2, pairs = kMT / cols;
+    const int most = 2 * pairs - 2 * halo_rows;   // rows of the interior
+    if (most < 2) continue;
+    int ty = (L.ny + most - 1) / most;
+    const int oy = ((L.ny + ty - 1) / ty + 1) / 2 * 2;   // even shares
+    const int tx = (gpr + ox - 1) / ox;
+    ty = (L.ny + oy - 1) / oy;
     const long long cost = (long long)tx * ty;
     if (best < 0 || cost < best) {
       best = cost;
       L.cols = cols;
-      L.pairs = op + 2;
+      L.pairs = oy / 2 + halo_rows;
       L.ox = ox;
-      L.oy = 2 * op;
+      L.oy = oy;
       L.tx = tx;
       L.ty = ty;
     }
@@ -571,8 +429,10 @@ void march_tile(MGLevel& L) {
 
 // The blocks (replicate, tile, slab) of one level's launches over the
 // replicates that sweep it on the grid: slabs of whole segments, as thick as
-// balances the planes of a slab's halo against idle multiprocessors.
-void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, std::vector<int4>& out) {
+// balances the planes of a slab's halo and start-up (extra) against idle
+// multiprocessors.
+void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, int extra,
+                  std::vector<int4>& out) {
   const long long resident = 2LL * sm_count;
   auto slab = [](const MGLevel& L, int zs) { return std::min(L.nz, (zs + L.seg - 1) / L.seg * L.seg); };
   int best_zs = 0;
@@ -586,8 +446,8 @@ void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int s
       if (z / L->seg > kMaxSeg) ok = false;
       if (z < L->nz) more = true;
       nb += (long long)ns * L->tx * L->ty;
-      work += (double)ns * L->tx * L->ty * (z + 6);
-      longest = std::max(longest, z + 6.0);
+      work += (double)ns * L->tx * L->ty * (z + extra);
+      longest = std::max(longest, z + (double)extra);
     }
     if (!ok) break;
     // whole waves while there are few, an even share plus a tail beyond

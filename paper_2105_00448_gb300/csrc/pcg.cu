@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(512) k_setup(Ctx c, int which, CondArg cnd) {
                    sv.beta = 0.0;
                    sv.scale = 1.0;
                    sv.iters = 0;
+                   sv.pend = 0;
                    sv.rtol = tol;
                    sv.maxit = rr.maxit;
                    sv.zero_b = s3[2] == 0.0;
@@ -220,14 +221,13 @@ __global__ void __launch_bounds__(512) k_setup(Ctx c, int which, CondArg cnd) {
 }
 
 // ----------------------------------------------------------------- pass A --
-// All loads of a group (own site and the four neighbour rows) are issued
-// before any value is used, so a group costs one memory round trip.
-// PERSIST: the persistent row form (one lattice, one row per warp; see
-// block_arrivals), else one block per chunk.
-template <typename T, int REGS, int NI, bool PERSIST>
-__global__ void __maxnreg__(REGS) k_pass_a(Ctx c, int which) {
+// FP64 fields (FP32: cg.cu).  All loads of a group (own site and the four
+// neighbour rows) are issued before any value is used, so a group costs one
+// memory round trip; one block per chunk.
+template <typename T>
+__global__ void __maxnreg__(128) k_pass_a(Ctx c, int which) {
   HCA_COUNT_KERNEL(c);
-  const int2 ch = PERSIST ? make_int2(0, 0) : c.chunks[blockIdx.x];
+  const int2 ch = c.chunks[blockIdx.x];
   const RepDesc& rd = c.reps[ch.x];
   const RepSolve sv = c.solve[ch.x];
   if (sv.active) {
@@ -251,11 +251,7 @@ __global__ void __maxnreg__(REGS) k_pass_a(Ctx c, int which) {
       const RowGeo geo = row_geo(rd, j);
       LaneAcc<T> acc[1];
       T carry = T(0);
-      // groups per lane in a row: a compile-time count (NI > 0) lets the
-      // compiler issue the loads of all of them before the first is used
-      const int niter = NI > 0 ? NI : it.niter;
-#pragma unroll
-      for (int itn = 0; itn < niter; ++itn) {
+      for (int itn = 0; itn < it.niter; ++itn) {
         const int g = itn * it.lpr + it.sl;
         const bool gok = row_ok && g < gpr;
         const long long e = geo.base + 4LL * g;
@@ -306,15 +302,10 @@ __global__ void __maxnreg__(REGS) k_pass_a(Ctx c, int which) {
       }
       store_rows_acc(c, chunk, rl, row_ok, it.sl, it.lpr, acc, 1);
     };
-    if (PERSIST) {
-      const int R = rd.ny * rd.nz, cr = rd.chunk_rows;
-      for (int j = persist_row_begin(R) + it.warp; j < persist_row_end(R); j += it.nw) row(j / cr, j % cr, true, j);
-    } else {
-      for (int rbase = it.warp * it.rpw; rbase < rd.chunk_rows; rbase += it.nw * it.rpw) {
-        const int rl = rbase + it.sub;
-        const bool row_ok = rl < nrows;
-        row(blockIdx.x, rl, row_ok, ch.y + (row_ok ? rl : 0));
-      }
+    for (int rbase = it.warp * it.rpw; rbase < rd.chunk_rows; rbase += it.nw * it.rpw) {
+      const int rl = rbase + it.sub;
+      const bool row_ok = rl < nrows;
+      row(blockIdx.x, rl, row_ok, ch.y + (row_ok ? rl : 0));
     }
   }
   auto fin = [&](int r, const double* s1) -> int {
@@ -328,16 +319,14 @@ __global__ void __maxnreg__(REGS) k_pass_a(Ctx c, int which) {
     s.alpha = s.rho / s1[0];
     return 1;
   };
-  // float-float row slots for FP32 fields (LaneAcc<float>)
-  if (PERSIST) block_arrivals<sizeof(T) == 4>(c, 1, fin, [](int) {});
-  else warp_epilogue<sizeof(T) == 4>(c, 1, blockIdx.x, fin);
+  warp_epilogue(c, 1, blockIdx.x, fin);
 }
 
 // ----------------------------------------------------------------- pass B --
-template <typename T, int REGS, int NI, bool PERSIST>
-__global__ void __maxnreg__(REGS) k_pass_b(Ctx c, int which, void* xfield, CondArg cnd) {
+template <typename T>
+__global__ void __maxnreg__(128) k_pass_b(Ctx c, int which, void* xfield, CondArg cnd) {
   HCA_COUNT_KERNEL(c);
-  const int2 ch = PERSIST ? make_int2(0, 0) : c.chunks[blockIdx.x];
+  const int2 ch = c.chunks[blockIdx.x];
   const RepDesc& rd = c.reps[ch.x];
   const RepSolve sv = c.solve[ch.x];
   if (sv.active) {
@@ -351,16 +340,12 @@ __global__ void __maxnreg__(REGS) k_pass_b(Ctx c, int which, void* xfield, CondA
     const T* __restrict__ qq = (const T*)c.q;
     T* __restrict__ xx = (T*)xfield;
     const T alpha = (T)sv.alpha;
-    const T zs = (sv.iters == 0 && (!mg || c.lazy_scale)) ? (T)sv.scale : T(1);
+    const T zs = (sv.iters == 0 && !mg) ? (T)sv.scale : T(1);
     const RowIter it = row_iter(rd);
     auto row = [&](int chunk, int rl, bool row_ok, int j) {
       const RowGeo geo = row_geo(rd, j);
       LaneAcc<T> acc[2];
-      // groups per lane in a row: a compile-time count (NI > 0) lets the
-      // compiler issue the loads of all of them before the first is used
-      const int niter = NI > 0 ? NI : it.niter;
-#pragma unroll
-      for (int itn = 0; itn < niter; ++itn) {
+      for (int itn = 0; itn < it.niter; ++itn) {
         const int g = itn * it.lpr + it.sl;
         const bool gok = row_ok && g < gpr;
         const long long e = geo.base + 4LL * g;
@@ -378,7 +363,7 @@ __global__ void __maxnreg__(REGS) k_pass_b(Ctx c, int which, void* xfield, CondA
               const T q = Q.a[k];
               X.a[k] += alpha * P.a[k];
               if (mg) {
-                Z.a[k] = zs * Z.a[k] - alpha * q;   // zs: a power of two
+                Z.a[k] -= alpha * q;
                 g_rr += Z.a[k] * Z.a[k];
               } else {
                 Z.a[k] = zs * Z.a[k] - alpha * (q / D.a[k]);
@@ -396,15 +381,10 @@ __global__ void __maxnreg__(REGS) k_pass_b(Ctx c, int which, void* xfield, CondA
       }
       store_rows_acc(c, chunk, rl, row_ok, it.sl, it.lpr, acc, 2);
     };
-    if (PERSIST) {
-      const int R = rd.ny * rd.nz, cr = rd.chunk_rows;
-      for (int j = persist_row_begin(R) + it.warp; j < persist_row_end(R); j += it.nw) row(j / cr, j % cr, true, j);
-    } else {
-      for (int rbase = it.warp * it.rpw; rbase < rd.chunk_rows; rbase += it.nw * it.rpw) {
-        const int rl = rbase + it.sub;
-        const bool row_ok = rl < nrows;
-        row(blockIdx.x, rl, row_ok, ch.y + (row_ok ? rl : 0));
-      }
+    for (int rbase = it.warp * it.rpw; rbase < rd.chunk_rows; rbase += it.nw * it.rpw) {
+      const int rl = rbase + it.sub;
+      const bool row_ok = rl < nrows;
+      row(blockIdx.x, rl, row_ok, ch.y + (row_ok ? rl : 0));
     }
   }
   auto fin = [&](int r, const double* s2) -> int {
@@ -436,8 +416,7 @@ __global__ void __maxnreg__(REGS) k_pass_b(Ctx c, int which, void* xfield, CondA
     }
     set_cond(cnd, go);
   };
-  if (PERSIST) block_arrivals<sizeof(T) == 4>(c, 2, fin, post);
-  else warp_epilogue<sizeof(T) == 4>(c, 2, blockIdx.x, fin, post);
+  warp_epilogue(c, 2, blockIdx.x, fin, post);
 }
 
 // ----------------------------------------------------------- true residual --
@@ -712,7 +691,6 @@ __global__ void __launch_bounds__(512) __maxnreg__(REGS) k_dc_residual(Ctx c, in
     float* __restrict__ aa = (float*)c.reac;
     float* __restrict__ zz = (float*)c.z;
     float* __restrict__ bb = (float*)c.b;
-    float* __restrict__ dxv = (float*)c.dx;
     const float* __restrict__ perf = (const float*)c.perf;
     const Coef<float> q = coef<float, KIND>(rd, which);
     const double cpl = (double)q.cpl;
@@ -869,7 +847,6 @@ __global__ void __launch_bounds__(512) __maxnreg__(REGS) k_dc_residual(Ctx c, in
           }
           if (MG) st4((float*)c.r + e, R32);
           else st4(zz + e, Z);
-          st4(dxv + e, zero4<float>());
         }
       }
 #pragma unroll
@@ -900,12 +877,14 @@ __global__ void __launch_bounds__(512) __maxnreg__(REGS) k_dc_residual(Ctx c, in
                      s.dc_apply = 0;
                      s.active = 0;
                      s.iters = 0;
+                     s.pend = 0;
                      if (c.frozen[r]) return 0;
                    } else if (!s.dc_apply) {
                      return 0;        // this replicate finished in an earlier sweep
                    }
                    st.iters[which] += s.iters;
                    st.sweeps[which] += 1;
+                   s.pend = 0;
                    // |b|^2 is summed on the first sweep only (b does not change)
                    if (FIRST) s.bb_outer = s3[1];
                    const double bb = s.bb_outer;
@@ -979,6 +958,8 @@ __global__ void __launch_bounds__(512) __maxnreg__(REGS) k_dc_residual(Ctx c, in
 }
 
 // x_hi + x_lo += dx (two-word sum), or x = 0 for a vanishing right-hand side.
+// dx is what pass A of the later iterations accumulated plus the last
+// iteration's step alpha p (0 + alpha p after a single iteration).
 __global__ void __launch_bounds__(512) k_dc_update(Ctx c, float* __restrict__ x_hi, float* __restrict__ x_lo) {
   HCA_COUNT_KERNEL(c);
   const int2 ch = c.chunks[blockIdx.x];
@@ -988,18 +969,25 @@ __global__ void __launch_bounds__(512) k_dc_update(Ctx c, float* __restrict__ x_
   const int nrows = min(rd.chunk_rows, rd.ny * rd.nz - ch.y);
   const long long base0 = rd.off + (long long)ch.y * rd.nxp;
   const int ngroups = nrows * rd.gpr;
+  const bool has_x = sv.iters - sv.pend > 0;
   const float* __restrict__ dxv = (const float*)c.dx;
+  const float* __restrict__ pv = (const float*)(sv.pbuf ? c.p_alt : c.p);
+  const float alpha = (float)sv.alpha;
   const float inv_s = (float)(1.0 / sv.scale);   // a power of two: exact
   for (int gi = threadIdx.x; gi < ngroups; gi += blockDim.x) {
-    const int rl = gi / rd.gpr, g = gi % rd.gpr;
-    const long long e = base0 + (long long)rl * rd.nxp + 4LL * g;
+    const long long e = base0 + 4LL * gi;   // rows follow each other
     if (sv.zero_b) {
       st4(x_hi + e, zero4<float>());
       st4(x_lo + e, zero4<float>());
       continue;
     }
     V4<float> H = ld4(x_hi + e), L = ld4(x_lo + e);
-    V4<float> D = ld4(dxv + e);
+    V4<float> D = ld4_if(dxv + e, has_x);
+    if (sv.pend) {
+      const V4<float> P = ld4(pv + e);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) D.a[k] = __fmaf_rn(alpha, P.a[k], D.a[k]);
+    }
 #pragma unroll
     for (int k = 0; k < 4; ++k) D.a[k] = __fmul_rn(D.a[k], inv_s);
 #pragma unroll
@@ -1093,53 +1081,19 @@ int persist_grid(const void* fn, int threads, int sm_count) {
   return per * sm_count;
 }
 
-template <int REGS, int NI>
-static void launch_ab_f32(const Ctx& c, int which, bool a, void* xfield, CondArg cnd) {
-  const bool pdl = c.pdl != 0;
-  if (NI > 0 && c.persist) {
-    if (a) {
-      const void* fn = (const void*)k_pass_a<float, REGS, NI, true>;
-      launch_k(pdl, k_pass_a<float, REGS, NI, true>, dim3(persist_grid(fn, c.threads, c.sm_count)), dim3(c.threads), 0,
-               c.stream, c, which);
-    } else {
-      const void* fn = (const void*)k_pass_b<float, REGS, NI, true>;
-      launch_k(pdl, k_pass_b<float, REGS, NI, true>, dim3(persist_grid(fn, c.threads, c.sm_count)), dim3(c.threads), 0,
-               c.stream, c, which, xfield, cnd);
-    }
-    return;
-  }
-  if (a) launch_k(pdl, k_pass_a<float, REGS, NI, false>, dim3(c.n_chunks), dim3(c.threads), 0, c.stream, c, which);
-  else launch_k(pdl, k_pass_b<float, REGS, NI, false>, dim3(c.n_chunks), dim3(c.threads), 0, c.stream, c, which, xfield, cnd);
+void launch_cg_a(const Ctx& c, int which, bool defer);
+void launch_cg_b(const Ctx& c, int which, void* xfield, bool defer, CondArg cnd);
+
+// FP32 fields: the marching pass A and streaming pass B (cg.cu); defer: the
+// solve is a defect correction's inner one, whose x += alpha p pass A carries.
+void launch_pass_a(const Ctx& c, int which, bool fp64, bool defer) {
+  if (fp64) k_pass_a<double><<<c.n_chunks, c.threads, 0, c.stream>>>(c, which);
+  else launch_cg_a(c, which, defer);
 }
 
-template <int REGS>
-static void launch_ab_f32_ni(const Ctx& c, int which, bool a, void* xfield, CondArg cnd) {
-  switch (c.pass_ni) {
-    case 1: launch_ab_f32<REGS, 1>(c, which, a, xfield, cnd); break;
-    case 2: launch_ab_f32<REGS, 2>(c, which, a, xfield, cnd); break;
-    case 4: launch_ab_f32<REGS, 4>(c, which, a, xfield, cnd); break;
-    default: launch_ab_f32<REGS, 0>(c, which, a, xfield, cnd); break;
-  }
-}
-
-static void launch_ab(const Ctx& c, int which, bool fp64, bool a, void* xfield, CondArg cnd) {
-  if (fp64) {
-    if (a) k_pass_a<double, 128, 0, false><<<c.n_chunks, c.threads, 0, c.stream>>>(c, which);
-    else k_pass_b<double, 128, 0, false><<<c.n_chunks, c.threads, 0, c.stream>>>(c, which, xfield, cnd);
-    return;
-  }
-  switch (c.pass_regs) {
-    case 64: launch_ab_f32_ni<64>(c, which, a, xfield, cnd); break;
-    case 96: launch_ab_f32_ni<96>(c, which, a, xfield, cnd); break;
-    case 128: launch_ab_f32_ni<128>(c, which, a, xfield, cnd); break;
-    default: launch_ab_f32_ni<80>(c, which, a, xfield, cnd); break;
-  }
-}
-
-void launch_pass_a(const Ctx& c, int which, bool fp64) { launch_ab(c, which, fp64, true, nullptr, CondArg{0ull, 0}); }
-
-void launch_pass_b(const Ctx& c, int which, void* xfield, bool fp64, CondArg cnd) {
-  launch_ab(c, which, fp64, false, xfield, cnd);
+void launch_pass_b(const Ctx& c, int which, void* xfield, bool fp64, bool defer, CondArg cnd) {
+  if (fp64) k_pass_b<double><<<c.n_chunks, c.threads, 0, c.stream>>>(c, which, xfield, cnd);
+  else launch_cg_b(c, which, xfield, defer, cnd);
 }
 
 void launch_true_residual(const Ctx& c, int which, void* xfield, bool fp64) {
