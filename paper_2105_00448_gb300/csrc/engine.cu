@@ -16,6 +16,9 @@ namespace hca {
 void launch_setup(const Ctx& c, int which, bool fp64, CondArg cnd);
 void launch_pass_a(const Ctx& c, int which, bool fp64, bool defer);
 void launch_pass_b(const Ctx& c, int which, void* xfield, bool fp64, bool defer, CondArg cnd);
+int cg64_plan(const std::vector<RepDesc>& reps, int sm_count, std::vector<Cg64Block>& table, int* blocks, int* large,
+              long long* slots);
+void launch_cg64(const Ctx& c, int which, void* xfield, CondArg cnd);
 bool cg_init();
 long long cg_plan(const std::vector<RepDesc>& reps, int sm_count, std::vector<MGLevel>& lv, std::vector<int4>& ablk,
                   std::vector<int4>& bblk, std::vector<int4>& bgeo, int* a_nt);
@@ -108,6 +111,7 @@ struct hca_handle {
   cudaStream_t cap[3] = {nullptr, nullptr, nullptr};
   bool graphs_ok = true;
   bool capturing = false;     // a step graph is being captured
+  int large64 = 0;            // FP64 Jacobi: replicates too large for the one-launch solve
   int ca_coop = 0;            // blocks of the cooperative 27-colour CA kernel (0: one launch per colour)
   int* h_pinned = nullptr;    // [0] active replicates, [1] error flag
   std::vector<void*> allocs;
@@ -517,9 +521,14 @@ int solve_plain(hca_handle* h, int which) {
   void* x = which == 0 ? c.K : c.G[which - 1];
   HCA_LAUNCH(h, HCA_KCLASS_SETUP, 1, hca::launch_setup(c, which, h->fp64, kNoCond));
   if (h->mg) HCA_LAUNCH(h, HCA_KCLASS_MG, h->mgh.nlev, mg_setup(h, which));
-  int rc = pcg_iterate(h, which, x, h->prev_inner[which][0], false);
-  if (rc) return rc;
-  h->prev_inner[which][0] = h->last_iters;
+  // FP64 Jacobi: the small replicates' solves in one launch, the passes for the others
+  if (c.rounds64) HCA_LAUNCH(h, HCA_KCLASS_PASS_A, 2, hca::launch_cg64(c, which, x, kNoCond));
+  int rc = HCA_OK;
+  if (!c.rounds64 || h->large64) {
+    rc = pcg_iterate(h, which, x, h->prev_inner[which][0], false);
+    if (rc) return rc;
+    h->prev_inner[which][0] = h->last_iters;
+  }
   HCA_LAUNCH(h, HCA_KCLASS_RESIDUAL, 2, hca::launch_true_residual(c, which, x, h->fp64));
   HCA_TRY(cudaMemcpyAsync(h->h_pinned, &c.sync->active_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
   HCA_TRY(cudaStreamSynchronize(c.stream));
@@ -626,12 +635,20 @@ int cap_solve(hca_handle* h, int which, cudaGraph_t G) {
   int rc;
   if (!dc) {
     void* x = which == 0 ? c.K : c.G[which - 1];
+    c.stream = S;
+    if (c.rounds64 && !h->large64) {   // every replicate's solve in one launch
+      hca::launch_setup(c, which, h->fp64, kNoCond);
+      hca::launch_cg64(c, which, x, kNoCond);
+      hca::launch_true_residual(c, which, x, h->fp64);
+      HCA_TRY(cudaGetLastError());
+      return HCA_OK;
+    }
     cudaGraphConditionalHandle H;
     HCA_TRY(cudaGraphConditionalHandleCreate(&H, G, 0, cudaGraphCondAssignDefault));
     const hca::CondArg cnd{H, 1};
-    c.stream = S;
     hca::launch_setup(c, which, h->fp64, cnd);
     if (h->mg) mg_setup(h, which);
+    if (c.rounds64) hca::launch_cg64(c, which, x, cnd);
     HCA_TRY(cudaGetLastError());
     // the V-cycle opens the loop's body, so none runs after the pass B that
     // ends the loop (the set-up leaves r unscaled: no r scaling either)
@@ -1455,6 +1472,25 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
       c.bgeo = bg_d;
       c.n_ablk = (int)ab.size();
       c.n_bblk = (int)bb.size();
+    }
+    if (h->fp64 && !h->mg) {
+      std::vector<hca::Cg64Block> t;
+      long long slots = 0;
+      c.rounds64 = hca::cg64_plan(h->reps_h, c.sm_count, t, &c.n_blk64, &h->large64, &slots);
+      if (c.rounds64) {
+        hca::Cg64Block* t_d;
+        ALLOC(t_d, sizeof(hca::Cg64Block) * t.size());
+        ALLOC(c.slot64, sizeof(ulonglong2) * (size_t)slots);
+        ALLOC(c.epoch64, sizeof(unsigned) * (size_t)n);
+        if (cudaMemcpyAsync(t_d, t.data(), sizeof(hca::Cg64Block) * t.size(), cudaMemcpyHostToDevice, c.stream) ||
+            cudaMemsetAsync(c.epoch64, 0, sizeof(unsigned) * (size_t)n, c.stream) ||
+            cudaMemsetAsync(c.slot64, 0, sizeof(ulonglong2) * (size_t)slots, c.stream) ||
+            cudaStreamSynchronize(c.stream)) {
+          rc = HCA_ERR_CUDA;
+          goto fail;
+        }
+        c.blk64 = t_d;
+      }
     }
     if (h->learned) {
       ALLOC(h->ws_cand, sizeof(double) * (size_t)h->total);

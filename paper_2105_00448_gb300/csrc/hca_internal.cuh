@@ -315,6 +315,13 @@ struct MGCluster {
   MGClusterLevel lev[12];
 };
 
+// A block's part in the one-launch FP64 solve of a small replicate (cg64.cu).
+struct Cg64Block {
+  int rep, idx, n, ng;   // replicate (-1: idle), block of its group, blocks, 2-site groups a thread
+  int nt, pad;           // threads of a block that hold sites
+  long long slot;        // the group's first reduction slot
+};
+
 // multigrid constants (the FP64 reference uses the same).  Above the
 // coarsest level a V-cycle smooths with two Jacobi sweeps before the coarse
 // correction, of weights MG_W1 then MG_W2, and two after it, MG_W2 then
@@ -401,6 +408,10 @@ struct Ctx {
   const int4* bblk;       // blocks of the streaming pass B: (replicate, first chunk, end chunk, blocks of the replicate)
   const int4* bgeo;       // [rep] pass B: groups, groups per chunk, chunks, first slot
   int n_ablk, n_bblk, a_nt;
+  const Cg64Block* blk64;   // FP64 Jacobi: [round][block] of the small replicates' one-launch solves
+  ulonglong2* slot64;       // their blocks' partial sums
+  unsigned* epoch64;        // [rep] their exchanges so far
+  int n_blk64, rounds64;
   const MGCluster* mgc;   // [rep] coarse levels in a cluster
   int lazy_scale;     // 1: the first inner iteration's kernels scale r as they read it
   const long long* mg_start;  // [MG_MAXLEV][n_reps + 1] prefix sums of each level's sites over the replicates
