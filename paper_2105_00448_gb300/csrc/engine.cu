@@ -36,7 +36,7 @@ void launch_philox_uniforms(unsigned long long seed, unsigned long long site0, l
 void launch_advance_step(const Ctx& c, long long by);
 void launch_ca_compact(const Ctx& c, bool fp64);
 void launch_ca_colour(const Ctx& c, int colour, int blocks_x, bool fp64);
-int ca_coop_blocks(bool fp64, int sm_count);
+int ca_coop_blocks(bool fp64, int sm_count, int n_reps, long long sites);
 void launch_ca_colours(const Ctx& c, int blocks, bool fp64);
 void launch_ca_sync(const Ctx& c, int blocks_x, bool fp64);
 void launch_vessels(const Ctx& c, bool fp64);
@@ -1622,7 +1622,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
       // sweep that ended every replicate's iteration) returns at once
       c.skip_idle = 1;
       // the 27 colour sweeps of the CA in one cooperative launch (HCA_CA_COOP=0: one launch per colour)
-      h->ca_coop = hca::ca_coop_blocks(h->fp64, c.sm_count);
+      h->ca_coop = hca::ca_coop_blocks(h->fp64, c.sm_count, n, h->total);
     }
     // (the FP32 passes have one launch shape, chosen from the lattices)
     if (!cfgs[0].threads_per_block && h->fp64) {
