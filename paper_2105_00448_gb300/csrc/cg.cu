@@ -13,14 +13,15 @@
 // plain FP32 solve (no defect correction) keeps x += alpha p in pass B.
 //
 // Pass A marches up z like the V-cycle's sweeps (march.cu): patches of 4 x 2
-// sites, inputs staged two planes ahead by per-thread cp.async copies, p of
+// sites, inputs staged two planes ahead by tensor copies, p of
 // the plane's rows exchanged through shared memory, z neighbours in
 // registers.  Pass B is a stream of 4-site groups through a cp.async ring.
 // Both leave the split of the L1 where the V-cycle's kernels need it: row
 // kernels that load through a large L1 ran at 77 us each at 256^3, but every
 // switch between them and those kernels cost ~12 us (with the split pinned
 // for all of them, pass A 102 us and pass B 89 us).  Measured at 256^3: pass
-// A 87 us (an average of 22 B a site), pass B 48 us; a step 15.2 -> 13.5 ms.
+// A 75 us (an average of 22 B a site; 87 with per-thread copies), pass B 48 us;
+// a step 15.2 -> 13.0 ms by the passes themselves.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -37,7 +38,7 @@ void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int s
 namespace {
 
 constexpr int kARing = 3;             // planes k .. k + 2 of z, p_old and dx, k - 1 .. k + 1 of d
-constexpr size_t a_smem(int nt) { return (size_t)(kARing * 8 + 4) * nt * 16 + (size_t)kMaxSeg * (nt / 32) * 8; }
+constexpr size_t a_smem(int nt) { return (size_t)(kARing * 8 + 4) * nt * 16 + (size_t)kMaxSeg * (nt / 32) * 8 + 128; }
 
 // ----------------------------------------------------------------- pass A --
 template <int NT, bool DEFER>
@@ -51,14 +52,16 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which
   const int zb = b.z, ze = b.w;
   const float cpl = rd.cpl32[which];
   const long long off = rd.off;
+  __shared__ __align__(8) uint64_t bar[kARing];
+  const CUtensorMap* maps = c.tmaps + L.map0;   // z, p, p_alt, dx, d
+  mbars_init(bar, kARing, maps, 5);
   HCA_COUNT_KERNEL(c);
   const RepSolve sv = c.solve[rep];
   if (!sv.active) return;
   const int par = c.sync->parity;
-  const float* __restrict__ pp = (const float*)(par ? c.p_alt : c.p) + off;
   float* __restrict__ pn = (float*)(par ? c.p : c.p_alt) + off;
-  const float* __restrict__ zz = (const float*)c.z + off;
-  const float* __restrict__ dd = (const float*)c.d + off;
+  const CUtensorMap* map_p = &maps[par ? 2 : 1];
+  const uint32_t box = 32u * (uint32_t)(L.cols * L.pairs);
   float* __restrict__ qq = (float*)c.q + off;
   float* __restrict__ xx = (float*)c.dx + off;
   const float2 beta = dup((float)sv.beta), alpha = dup((float)sv.alpha);
@@ -67,51 +70,44 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which
   // the first iteration of a rescaled inner solve starts from scale * z (the
   // V-cycle scales r itself before it forms z)
   const float2 zs = dup((sv.iters == 0 && !c.mg) ? (float)sv.scale : 1.f);
-  float4* ring = msm + p.tid;              // [phase][z0, z1, p0, p1, x0, x1, d0, d1 (of the plane before)][thread]
-  float4* pb = msm + kARing * 8 * NT;      // [plane & 1][row][thread]
+  float4* ring = align128(msm);            // [phase][z, p, x, d (of the plane before)][row][group]
+  float4* pb = ring + kARing * 8 * NT;     // [plane & 1][row of the pair][thread]
   float2* segs = reinterpret_cast<float2*>(pb + 4 * NT);
-  const unsigned sring = smem_addr(ring);
-  const int n0 = p.rok[0] ? 16 : 0, n1 = p.rok[1] ? 16 : 0;
   auto fetch = [&](int k, int slot) {
-    const bool zok = k >= 0 && k < p.nz, z1 = k >= 1 && k <= p.nz;
-    const unsigned sa = sring + (unsigned)slot * (8 * NT * 16);
-    const unsigned ek = p.e + (unsigned)k * p.sz;
-    const int m0 = zok ? n0 : 0, m1 = zok ? n1 : 0;
-    const unsigned e0 = m0 ? ek : 0u, e1 = m1 ? ek + p.sy : 0u;
-    cp16(sa, zz + e0, m0);
-    cp16(sa + NT * 16, zz + e1, m1);
-    cp16(sa + 2 * NT * 16, pp + e0, use_p ? m0 : 0);
-    cp16(sa + 3 * NT * 16, pp + e1, use_p ? m1 : 0);
-    if (DEFER) {
-      cp16(sa + 4 * NT * 16, xx + e0, use_x && p.in[0] ? m0 : 0);
-      cp16(sa + 5 * NT * 16, xx + e1, use_x && p.in[1] ? m1 : 0);
-    }
-    const int q0 = z1 && p.in[0] ? 16 : 0, q1 = z1 && p.in[1] ? 16 : 0;
-    cp16(sa + 6 * NT * 16, dd + (q0 ? ek - p.sz : 0u), q0);
-    cp16(sa + 7 * NT * 16, dd + (q1 ? ek - p.sz + p.sy : 0u), q1);
+    float4* s = ring + slot * 8 * NT;
+    mbar_expect_tx(&bar[slot], (2u + use_p + use_x) * box);
+    tma_load_3d(s, &maps[0], p.tx0, p.ty0, k, &bar[slot]);
+    if (use_p) tma_load_3d(s + 2 * NT, map_p, p.tx0, p.ty0, k, &bar[slot]);
+    if (use_x) tma_load_3d(s + 4 * NT, &maps[3], p.tx0, p.ty0, k, &bar[slot]);
+    tma_load_3d(s + 6 * NT, &maps[4], p.tx0, p.ty0, k - 1, &bar[slot]);
   };
   P8 u[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) zero_patch(u[i]);
   FF acc{0.f, 0.f};
   const int k0 = zb - 1, k1 = ze;   // planes whose p is formed
-  fetch(k0, 0);
-  cp_commit();
-  fetch(k0 + 1, 1);
-  cp_commit();
+  int issued = 2;   // (thread 0)
+  if (p.tid == 0) {
+    fetch(k0, 0);
+    fetch(k0 + 1, 1);
+  }
   int seg = 0;
+  uint32_t phase = 0;
   const int seglen = L.seg;
   auto step = [&](auto ph, int k) {
     constexpr int P0 = decltype(ph)::value, P1 = (P0 + 2) % 3, P2 = (P0 + 1) % 3;
-    if (k + 2 <= k1) fetch(k + 2, P1);
-    cp_commit();
-    cp_wait<2>();
+    if (p.tid == 0 && k + 2 <= k1) {
+      fetch(k + 2, P1);
+      ++issued;
+    }
+    const bool ok = tc::mbar_wait(&bar[P0], phase, kTmaWaitLimit);
     const float4* rs = ring + P0 * 8 * NT;
     float2 z[2][2], po[2][2];
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-      get_row(z[a], rs + a * NT);
-      get_row(po[a], rs + (2 + a) * NT);
+      get_row(z[a], rs + (a ? p.r1 : p.r0));
+      if (use_p) get_row(po[a], rs + 2 * NT + (a ? p.r1 : p.r0));
+      else po[a][0] = po[a][1] = make_float2(0.f, 0.f);
     }
     nb_patch<NT>(p, pb + ((k & 1) ^ 1) * 2 * NT, u[P1], u[P2], u[P2]);
 #pragma unroll
@@ -124,8 +120,8 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
         if (!p.in[a]) continue;
-        float2 x[2];
-        get_row(x, rs + (4 + a) * NT);
+        float2 x[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (use_x) get_row(x, rs + 4 * NT + (a ? p.r1 : p.r0));
 #pragma unroll
         for (int h = 0; h < 2; ++h) x[h] = __ffma2_rn(alpha, po[a][h], x[h]);
         *reinterpret_cast<float4*>(xx + (e + a * p.sy)) = make_float4(x[0].x, x[0].y, x[1].x, x[1].y);
@@ -137,7 +133,7 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which
       for (int a = 0; a < 2; ++a) {
         if (!p.in[a]) continue;
         float2 d[2], q[2];
-        get_row(d, rs + (6 + a) * NT);
+        get_row(d, rs + 6 * NT + (a ? p.r1 : p.r0));
         float g_s = 0.f;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -164,12 +160,15 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which
         ++seg;
       }
     }
-    __syncthreads();
+    return !__syncthreads_or(!ok);   // a copy timed out: every thread stops
   };
-  for (int k = k0; k <= k1; k += 3) {
-    step(std::integral_constant<int, 0>{}, k);
-    if (k + 1 <= k1) step(std::integral_constant<int, 1>{}, k + 1);
-    if (k + 2 <= k1) step(std::integral_constant<int, 2>{}, k + 2);
+  for (int k = k0; k <= k1; k += 3, phase ^= 1) {
+    if (!step(std::integral_constant<int, 0>{}, k) ||
+        (k + 1 <= k1 && !step(std::integral_constant<int, 1>{}, k + 1)) ||
+        (k + 2 <= k1 && !step(std::integral_constant<int, 2>{}, k + 2))) {
+      tma_abort(c, bar, kARing, k - k0, issued);
+      return;
+    }
   }
   double* slots = c.mslot + L.slot0 + (long long)b.y * L.nseg + zb / seglen;
   for (int s = threadIdx.x; s < seg; s += NT) {

@@ -48,6 +48,7 @@ void mg_coop_config(MGHost& H, bool fp64, int sm_count, long long smem_bytes);
 int cluster_plan(const MGLevel* lv, int nl, int from, int cs, long long smem, MGCluster* R);
 bool cluster_init(const MGHost& H);
 bool march_init();
+bool march_map(CUtensorMap* m, const MGLevel& L, const void* base);
 void march_tile(MGLevel& L, int halo_rows);
 int march_threads(const std::vector<MGLevel*>& lv);
 void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, int extra,
@@ -1181,6 +1182,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
     ALLOC(c.b, fbytes);
     ALLOC(c.aux, fbytes);
     long long mslots = 0;   // reduction slots of the marching and streaming kernels
+    std::vector<CUtensorMap> maps;   // their inputs
     if (h->mg) {
       // one hierarchy per replicate; each coarse level's arrays hold all
       // replicates back to back
@@ -1381,6 +1383,14 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
               L.w = nullptr;
             }
             hca::march_tile(L, 2);
+            L.map0 = (int)maps.size();
+            for (void* a : {L.rhs, L.d, L.t}) {
+              maps.emplace_back();
+              if (!hca::march_map(&maps.back(), L, a)) {
+                rc = HCA_ERR_CUDA;
+                goto fail;
+              }
+            }
             if (l == 0) {
               L.slot0 = (int)slots;
               slots += (long long)L.tx * L.ty * L.nseg;
@@ -1449,6 +1459,21 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
       std::vector<hca::MGLevel> lv;
       std::vector<int4> ab, bb, bg;
       mslots = std::max(mslots, hca::cg_plan(h->reps_h, c.sm_count, lv, ab, bb, bg, &c.a_nt));
+      for (int i = 0; i < n; ++i) {
+        hca::MGLevel& L = lv[i];
+        const long long o = h->reps_h[i].off;
+        L.map0 = (int)maps.size();
+        for (void* a : {c.z, c.p, c.p_alt, c.dx, c.d}) {
+          maps.emplace_back();
+          if (!hca::march_map(&maps.back(), L, (float*)a + o)) {
+            rc = HCA_ERR_CUDA;
+            goto fail;
+          }
+        }
+      }
+      CUtensorMap* maps_d;
+      ALLOC(maps_d, sizeof(CUtensorMap) * maps.size());
+      c.tmaps = maps_d;
       hca::MGLevel* lv_d;
       int4 *ab_d, *bb_d, *bg_d;
       ALLOC(lv_d, sizeof(hca::MGLevel) * lv.size());
@@ -1458,6 +1483,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
       ALLOC(c.mslot, sizeof(double) * (size_t)mslots);
       ALLOC(c.mcnt, sizeof(int) * (size_t)n);
       if (!hca::cg_init() ||
+          cudaMemcpyAsync(maps_d, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice, c.stream) ||
           cudaMemcpyAsync(lv_d, lv.data(), sizeof(hca::MGLevel) * lv.size(), cudaMemcpyHostToDevice, c.stream) ||
           cudaMemcpyAsync(ab_d, ab.data(), sizeof(int4) * ab.size(), cudaMemcpyHostToDevice, c.stream) ||
           cudaMemcpyAsync(bb_d, bb.data(), sizeof(int4) * bb.size(), cudaMemcpyHostToDevice, c.stream) ||

@@ -18,6 +18,7 @@
 
 #include <utility>
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -295,6 +296,7 @@ struct MGLevel {
   // its interior, tiles, planes per reduction segment, segments along z, first
   // slot, blocks
   int cols, pairs, ox, oy, tx, ty, seg, nseg, slot0, nblk;
+  int map0;                 // first tensor map of its arrays (the box: a tile's rows of one plane)
 };
 
 // The coarse levels a thread-block cluster holds (FP32; coarse.cu): level i of
@@ -401,6 +403,7 @@ struct Ctx {
   void* mg_w;         // 1 / d on the lattice (0 where d = 0)
   const void* mg_lv;  // device MGLevel[n_reps][MG_MAXLEV] (level 0 filled for FP32 fields)
   const int4* mblk;   // blocks of the marching sweeps: (replicate, tile, first plane, end plane)
+  const CUtensorMap* tmaps;   // tensor maps of the marching sweeps' inputs
   double* mslot;      // their segment sums
   int* mcnt;          // [rep] blocks done
   const MGLevel* cg_lv;   // [rep] the lattice's tiling in the marching CG pass A

@@ -23,19 +23,18 @@
 // Form.  A block of kMT threads owns a tile of 4-site groups by row pairs (a
 // thread holds a 4 x 2 patch) and walks up z through a slab of planes.  The
 // tile includes the halo the fused sweeps need (one group in x, two rows in
-// y, where the level is wider than the tile; two planes in z), so every
-// thread runs the same code and only interior threads write.  Each plane's
-// inputs arrive by per-thread cp.async copies (zero fill outside the level)
-// into a shared-memory ring, two planes ahead; z neighbours stay in
+// y; two planes in z), so every thread runs the same code and only interior
+// threads write.  Each plane's inputs arrive by tensor copies (zeros outside
+// the level) in a shared-memory ring, two planes ahead; z neighbours stay in
 // registers (the loop body is unrolled by three, so nothing is rotated), y
 // neighbours go through shared memory (one barrier per plane), x neighbours
 // through lane shuffles.  Bound: shared-memory and shuffle traffic and the
-// latency a barrier a plane exposes at 16 warps per multiprocessor (ncu, down
-// at 256^3: 44 % of issue slots, 46 % of the shared-memory pipe).  Measured
-// at 256^3 (FP32): down 74 us and up 92 us a launch, against 110 us for the
-// pre-sweep and restriction kernels and 118 us for the two post-sweep kernels
-// they replaced (28.5 B a site each); on 16 uneven replicates (59 M sites)
-// 139 and 175 us (of the whole batch), against 449 and 495 us.
+// latency a barrier a plane exposes at 16 warps per multiprocessor.  Measured
+// at 256^3 (FP32): down 64 us and up 66 us a launch (74 and 92 with a
+// per-thread cp.async of each patch), against 110 us for the pre-sweep and
+// restriction kernels and 118 us for the two post-sweep kernels they replaced
+// (28.5 B a site each); on 16 uneven replicates (59 M sites, all levels'
+// launches apart) 137 and 145 us, against 449 and 495 us.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -52,8 +51,8 @@ constexpr int kUpRing = 3;            // planes k .. k + 2 of v' and d, k - 1 ..
 constexpr float kW1 = (float)MG_W1, kW2 = (float)MG_W2;
 constexpr float kK = (float)(1.0 + MG_W2 * (1.0 - MG_W1) / MG_W1);
 constexpr float k1W1 = (float)(1.0 - MG_W1), k1W2 = (float)(1.0 - MG_W2);
-constexpr size_t down_smem(int nt) { return (size_t)(kDownRing * 4 + 2 * 2 + 2 * 2) * nt * 16; }
-constexpr size_t up_smem(int nt) { return (size_t)(kUpRing * 6 + 2 * 2 + 2) * nt * 16 + (size_t)kMaxSeg * (nt / 32) * 8; }
+constexpr size_t down_smem(int nt) { return (size_t)(kDownRing * 4 + 2 * 2 + 2 * 2) * nt * 16 + 128; }
+constexpr size_t up_smem(int nt) { return (size_t)(kUpRing * 6 + 2 * 2 + 2) * nt * 16 + (size_t)kMaxSeg * (nt / 32) * 8 + 128; }
 
 // The coupling of level l of the operator: the lattice's FP32 coupling times
 // the level's scale.
@@ -77,10 +76,12 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int wh
   const int zb = b.z, ze = b.w;
   const float cpl = level_coupling(c, rep, which, L);
   const float2 w2c = dup(kW2 * cpl);
-  const float* __restrict__ rr = (const float*)L.rhs;
-  const float* __restrict__ dd = (const float*)L.d;
+  const CUtensorMap* maps = c.tmaps + L.map0;   // r, d, v'
   float* __restrict__ vv = (float*)L.t;
   float* __restrict__ rc = (float*)C.rhs;
+  const uint32_t box = 32u * (uint32_t)(L.cols * L.pairs);
+  __shared__ __align__(8) uint64_t bar[kDownRing];
+  mbars_init(bar, kDownRing, maps, 2);
   const bool two = p.x0 / 2 + 1 < C.nx;
   const unsigned cel = (unsigned)(p.x0 / 2) + (unsigned)C.pitch * (unsigned)(p.y0 / 2), csz = (unsigned)C.pitch * (unsigned)C.ny;
   HCA_VC_ENTRY(c);
@@ -88,21 +89,13 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int wh
   if (c.skip_idle && !c.solve[rep].active) return;   // this replicate's solve has ended
   if (LAT) sc = r_scale(c.solve[rep]);
   const float2 w1s = dup(LAT ? kW1 * sc : kW1);
-  float4* ring = msm + p.tid;                  // [plane mod kDownRing][r0, r1, d0, d1][thread]
-  float4* ub = msm + kDownRing * 4 * NT;       // [plane & 1][row][thread]
+  float4* ring = align128(msm);                // [plane mod kDownRing][r, d][row][group]
+  float4* ub = ring + kDownRing * 4 * NT;      // [plane & 1][row of the pair][thread]
   float4* vb = ub + 4 * NT;
-  const unsigned sring = smem_addr(ring);
-  const int n0 = p.rok[0] ? 16 : 0, n1 = p.rok[1] ? 16 : 0;
   auto fetch = [&](int k, int slot) {
-    const bool zok = k >= 0 && k < p.nz;
-    const unsigned sa = sring + (unsigned)slot * (4 * NT * 16);
-    const unsigned e = zok ? p.e + (unsigned)k * p.sz : 0u;
-    const unsigned e0 = n0 ? e : 0u, e1 = zok && n1 ? e + p.sy : 0u;
-    const int m0 = zok ? n0 : 0, m1 = zok ? n1 : 0;
-    cp16(sa, rr + e0, m0);
-    cp16(sa + NT * 16, rr + e1, m1);
-    cp16(sa + 2 * NT * 16, dd + e0, m0);
-    cp16(sa + 3 * NT * 16, dd + e1, m1);
+    mbar_expect_tx(&bar[slot], 2 * box);
+    tma_load_3d(ring + (slot * 4) * NT, &maps[0], p.tx0, p.ty0, k, &bar[slot]);
+    tma_load_3d(ring + (slot * 4 + 2) * NT, &maps[1], p.tx0, p.ty0, k, &bar[slot]);
   };
   P8 u[3], v[3], w[3];
 #pragma unroll
@@ -113,17 +106,22 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int wh
   }
   float2 acc = make_float2(0.f, 0.f);
   const int k0 = zb - 2, k1 = ze + 1;   // planes whose u is formed
-  fetch(k0, 0);
-  cp_commit();
-  fetch(k0 + 1, 1);
-  cp_commit();
+  int issued = 2;   // (thread 0)
+  if (p.tid == 0) {
+    fetch(k0, 0);
+    fetch(k0 + 1, 1);
+  }
   int slot = 0;
-  // one plane: u of plane k, v of plane k - 1, the residual of plane k - 2
+  uint32_t par = 0;
+  // one plane: u of plane k, v of plane k - 1, the residual of plane k - 2;
+  // false when a copy timed out (the same in every thread)
   auto step = [&](auto ph, int k) {
     constexpr int P0 = decltype(ph)::value, P1 = (P0 + 2) % 3, P2 = (P0 + 1) % 3;   // planes k, k - 1, k - 2
-    if (k + 2 <= k1) fetch(k + 2, slot + 2 >= kDownRing ? slot + 2 - kDownRing : slot + 2);
-    cp_commit();
-    cp_wait<2>();
+    if (p.tid == 0 && k + 2 <= k1) {
+      fetch(k + 2, slot + 2 >= kDownRing ? slot + 2 - kDownRing : slot + 2);
+      ++issued;
+    }
+    const bool ok = tc::mbar_wait(&bar[slot], par, kTmaWaitLimit);
     float4* U0 = ub + (k & 1) * 2 * NT;
     const float4* U1 = ub + ((k & 1) ^ 1) * 2 * NT;
     float4* V1 = vb + ((k & 1) ^ 1) * 2 * NT;
@@ -134,8 +132,8 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int wh
     float2 r[2][2], d[2][2];
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-      get_row(r[a], rs + a * NT);
-      get_row(d[a], rs + (2 + a) * NT);
+      get_row(r[a], rs + (a ? p.r1 : p.r0));
+      get_row(d[a], rs + 2 * NT + (a ? p.r1 : p.r0));
     }
     nb_patch<NT>(p, U1, u[P1], u[P2], u[P2]);
     nb_patch<NT>(p, V2, v[P2], v[P0], v[P0]);
@@ -165,8 +163,8 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int wh
 #pragma unroll
           for (int a = 0; a < 2; ++a) {
             float2 r[2], d[2], o[2], res[2];
-            get_row(r, rz + a * NT);
-            get_row(d, rz + (2 + a) * NT);
+            get_row(r, rz + (a ? p.r1 : p.r0));
+            get_row(d, rz + 2 * NT + (a ? p.r1 : p.r0));
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               const float2 vc = v[P2].v[a][h];
@@ -197,13 +195,17 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_down(Ctx c, int wh
         }
       }
     }
-    __syncthreads();
     slot = slot + 1 == kDownRing ? 0 : slot + 1;
+    par ^= slot == 0;
+    return !__syncthreads_or(!ok);
   };
   for (int k = k0; k <= k1; k += 3) {
-    step(std::integral_constant<int, 0>{}, k);
-    if (k + 1 <= k1) step(std::integral_constant<int, 1>{}, k + 1);
-    if (k + 2 <= k1) step(std::integral_constant<int, 2>{}, k + 2);
+    if (!step(std::integral_constant<int, 0>{}, k) ||
+        (k + 1 <= k1 && !step(std::integral_constant<int, 1>{}, k + 1)) ||
+        (k + 2 <= k1 && !step(std::integral_constant<int, 2>{}, k + 2))) {
+      tma_abort(c, bar, kDownRing, k - k0, issued);
+      return;
+    }
   }
 }
 
@@ -219,10 +221,11 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
   const int zb = b.z, ze = b.w;
   const float cpl = level_coupling(c, rep, which, L);
   const float2 w2c = dup(kW2 * cpl);
-  const float* __restrict__ vv = (const float*)L.t;
-  const float* __restrict__ rr = (const float*)L.rhs;
-  const float* __restrict__ dd = (const float*)L.d;
+  const CUtensorMap* maps = c.tmaps + L.map0;   // r, d, v'
   const float* __restrict__ xc = (const float*)C.x;
+  const uint32_t box = 32u * (uint32_t)(L.cols * L.pairs);
+  __shared__ __align__(8) uint64_t bar[kUpRing];
+  mbars_init(bar, kUpRing, maps, 3);
   float* __restrict__ xo = (float*)L.x;
   const int cnz = C.nz;
   const bool two = p.x0 / 2 + 1 < C.nx;
@@ -232,26 +235,17 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
   float sc = 1.f;
   if (c.skip_idle && !c.solve[rep].active) return;
   if (LAT) sc = r_scale(c.solve[rep]);
-  float4* ring = msm + p.tid;               // [phase][v0, v1, d0, d1, r0, r1 (of the plane before)][thread]
-  float4* yb = msm + kUpRing * 6 * NT;      // [plane & 1][row][thread]
+  float4* ring = align128(msm);             // [phase][v', d, r (of the plane before)][row][group]
+  float4* yb = ring + kUpRing * 6 * NT;     // [plane & 1][row of the pair][thread]
   float2* cells = reinterpret_cast<float2*>(yb + 4 * NT);   // [coarse plane & 3][thread]: the patch's two coarse cells
   float2* segs = cells + 4 * NT;
-  const unsigned sring = smem_addr(ring), scell = smem_addr(cells + p.tid);
-  const int n0 = p.rok[0] ? 16 : 0, n1 = p.rok[1] ? 16 : 0;
+  const unsigned scell = smem_addr(cells + p.tid);
   // v' and d of plane k, r of plane k - 1 (used one step later)
   auto fetch = [&](int k, int slot) {
-    const bool zok = k >= 0 && k < p.nz, z1 = k >= 1 && k <= p.nz;
-    const unsigned sa = sring + (unsigned)slot * (6 * NT * 16);
-    const unsigned ek = p.e + (unsigned)k * p.sz;
-    const int m0 = zok ? n0 : 0, m1 = zok ? n1 : 0, q0 = z1 ? n0 : 0, q1 = z1 ? n1 : 0;
-    const unsigned e0 = m0 ? ek : 0u, e1 = m1 ? ek + p.sy : 0u;
-    const unsigned f0 = q0 ? ek - p.sz : 0u, f1 = q1 ? ek - p.sz + p.sy : 0u;
-    cp16(sa, vv + e0, m0);
-    cp16(sa + NT * 16, vv + e1, m1);
-    cp16(sa + 2 * NT * 16, dd + e0, m0);
-    cp16(sa + 3 * NT * 16, dd + e1, m1);
-    cp16(sa + 4 * NT * 16, rr + f0, q0);
-    cp16(sa + 5 * NT * 16, rr + f1, q1);
+    mbar_expect_tx(&bar[slot], 3 * box);
+    tma_load_3d(ring + (slot * 6) * NT, &maps[2], p.tx0, p.ty0, k, &bar[slot]);
+    tma_load_3d(ring + (slot * 6 + 2) * NT, &maps[1], p.tx0, p.ty0, k, &bar[slot]);
+    tma_load_3d(ring + (slot * 6 + 4) * NT, &maps[0], p.tx0, p.ty0, k - 1, &bar[slot]);
   };
   auto fetch_cells = [&](int Z) {
     const bool ok = p.rok[0] && Z >= 0 && Z < cnz;
@@ -270,11 +264,14 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
   const int k0 = zb - 1, k1 = ze;   // planes whose y is formed (k0 odd: zb is even)
   // coarse planes k0 / 2 - 1 .. k0 / 2 + 1 before the first step (-1 below the level: zeros)
   const int Z0 = k0 >> 1;
-  fetch(k0, 0);
+  int issued = 2;   // (thread 0)
+  if (p.tid == 0) {
+    fetch(k0, 0);
+    fetch(k0 + 1, 1);
+  }
   fetch_cells(Z0);
   fetch_cells(Z0 + 1);
   cp_commit();
-  fetch(k0 + 1, 1);
   fetch_cells(Z0 + 2);
   cp_commit();
   // cell slots of the neighbours (clamped for outermost halo patches)
@@ -285,16 +282,21 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
   __syncthreads();
   int seg = 0;
   const int seglen = L.seg;
+  uint32_t par = 0;
   auto step = [&](auto ph, int k) {
     constexpr int P0 = decltype(ph)::value, P1 = (P0 + 2) % 3, P2 = (P0 + 1) % 3;
     const bool odd = k & 1;
     const int Z = k >> 1;
     if (k + 2 <= k1) {
-      fetch(k + 2, P1);
+      if (p.tid == 0) {
+        fetch(k + 2, P1);
+        ++issued;
+      }
       if (!odd) fetch_cells(Z + 2);
     }
     cp_commit();
     cp_wait<2>();
+    const bool ok = tc::mbar_wait(&bar[P0], par, kTmaWaitLimit);
     const float2* cz = cells + (Z & 3) * NT;
     if (!odd || k == k0) {
       below = cur;
@@ -321,8 +323,8 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
       float2 vp[2], d[2];
-      get_row(vp, ring + (P0 * 6 + a) * NT);
-      get_row(d, ring + (P0 * 6 + 2 + a) * NT);
+      get_row(vp, ring + (P0 * 6) * NT + (a ? p.r1 : p.r0));
+      get_row(d, ring + (P0 * 6 + 2) * NT + (a ? p.r1 : p.r0));
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const float2 S = __fadd2_rn(xs[h], dup(h ? t[a].y : t[a].x));
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
           float2 r[2], o[2], rz = make_float2(0.f, 0.f);
-          get_row(r, ring + (P0 * 6 + 4 + a) * NT);
+          get_row(r, ring + (P0 * 6 + 4) * NT + (a ? p.r1 : p.r0));
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const float2 rs = LAT ? __fmul2_rn(r[h], dup(sc)) : r[h];
@@ -361,12 +363,15 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
         ++seg;
       }
     }
-    __syncthreads();
+    return !__syncthreads_or(!ok);
   };
-  for (int k = k0; k <= k1; k += 3) {
-    step(std::integral_constant<int, 0>{}, k);
-    if (k + 1 <= k1) step(std::integral_constant<int, 1>{}, k + 1);
-    if (k + 2 <= k1) step(std::integral_constant<int, 2>{}, k + 2);
+  for (int k = k0; k <= k1; k += 3, par ^= 1) {
+    if (!step(std::integral_constant<int, 0>{}, k) ||
+        (k + 1 <= k1 && !step(std::integral_constant<int, 1>{}, k + 1)) ||
+        (k + 2 <= k1 && !step(std::integral_constant<int, 2>{}, k + 2))) {
+      tma_abort(c, bar, kUpRing, k - k0, issued);
+      return;
+    }
   }
   if (!LAT) return;
   // the block's segment sums to their slots (warps in order), then the
@@ -403,9 +408,9 @@ void march_tile(MGLevel& L, int halo_rows) {
   const int gpr = (L.nx + 3) / 4;
   long long best = -1;
   for (int n = 1; n <= gpr; ++n) {
-    const int ox = (gpr + n - 1) / n, cols = ox + 2, pairs = kMT / cols;
+    const int ox = (gpr + n - 1) / n, cols = ox + 2, pairs = std::min(kMT / cols, 128);
     const int most = 2 * pairs - 2 * halo_rows;   // rows of the interior
-    if (most < 2) continue;
+    if (most < 2 || 4 * cols > 256) continue;   // (a tensor copy's box: at most 256 elements a side)
     int ty = (L.ny + most - 1) / most;
     const int oy = ((L.ny + ty - 1) / ty + 1) / 2 * 2;   // even shares
     const int tx = (gpr + ox - 1) / ox;
@@ -497,6 +502,29 @@ void launch_march_t(const Ctx& c, int which, const MGHost& H, int l, bool down) 
   else launch_k(pdl, k_mg_up<false, NT>, g, t, up_smem(NT), c.stream, c, which, l, bl);
 }
 }  // namespace
+
+// A tensor map of one array of a level (x extent nx, rows `pitch` apart), box a
+// tile's rows of one plane, zero fill outside.  False if the driver's entry
+// point is missing or refuses the encoding.
+bool march_map(CUtensorMap* m, const MGLevel& L, const void* base) {
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess || !fn) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  const cuuint64_t dims[3] = {(cuuint64_t)L.nx, (cuuint64_t)L.ny, (cuuint64_t)L.nz};
+  const cuuint64_t strides[2] = {(cuuint64_t)L.pitch * 4, (cuuint64_t)L.pitch * L.ny * 4};
+  const cuuint32_t box[3] = {(cuuint32_t)(4 * L.cols), (cuuint32_t)(2 * L.pairs), 1};
+  const cuuint32_t es[3] = {1, 1, 1};
+  return ((Encode)fn)(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 // Dynamic shared memory of the marching kernels in the current context.
 bool march_init() { return march_init_t<64>() && march_init_t<128>() && march_init_t<256>(); }

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "hca_internal.cuh"
+#include "tc.cuh"
 
 namespace hca {
 
@@ -13,6 +14,51 @@ constexpr int blocks_per_sm(int nt) { return nt >= 256 ? 2 : 512 / nt; }
 
 __device__ __forceinline__ void cp16(unsigned sdst, const float* gsrc, int n) {   // n = 0: zero fill
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sdst), "l"(gsrc), "r"(n) : "memory");
+}
+
+// Planes of a tile arrive by tensor copies: one thread issues, per plane and
+// input array, the box of the tile's rows (halo included, zeros outside the
+// level), completing on the stage's mbarrier.  (Per-thread 16-byte cp.async
+// copies of the patches took 14 shared-memory cycles a warp instruction: the
+// pipe the sweeps' own exchanges need.)
+constexpr int kTmaWaitLimit = 1 << 20;
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(bar)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(void* sdst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
+          "r"(tc::smem_u32(sdst)),
+      "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(tc::smem_u32(bar))
+      : "memory");
+}
+// One thread: the stages' barriers, and the maps (in global memory, written by a
+// copy at creation; the acquire also drops what the descriptor cache may hold
+// of an earlier handle at the same address).
+__device__ __forceinline__ void mbars_init(uint64_t* bar, int n, const CUtensorMap* maps, int n_maps) {
+  if (threadIdx.x == 0) {
+    for (int m = 0; m < n_maps; ++m)
+      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((unsigned long long)&maps[m])
+                   : "memory");
+    for (int s = 0; s < n; ++s) tc::mbar_init(&bar[s], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ float4* align128(void* p) {
+  return reinterpret_cast<float4*>((reinterpret_cast<uintptr_t>(p) + 127) & ~uintptr_t(127));
+}
+// A copy did not complete in time: record it and let this block's copies in
+// flight (uses n .. issued - 1 of a ring of `ring` stages) land before its
+// shared memory is released.
+__device__ __forceinline__ void tma_abort(const Ctx& c, uint64_t* bar, int ring, int n, int issued) {
+  if (threadIdx.x == 0) {
+    c.sync->error = SYNC_ERR_TIMEOUT;
+    for (int k = n; k < issued; ++k) (void)tc::mbar_wait(&bar[k % ring], (uint32_t)((k / ring) & 1), kTmaWaitLimit);
+  }
+  __syncthreads();
 }
 __device__ __forceinline__ void cp4(unsigned sdst, const float* gsrc, int n) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sdst), "l"(gsrc), "r"(n) : "memory");
@@ -52,6 +98,8 @@ __device__ __forceinline__ float2 inv_d(float2 d) { return make_float2(inv_d(d.x
 // thread's own values.
 struct Patch {
   int tid, lane, x0, y0;   // first site of the patch
+  int tx0, ty0;        // first site and row of the tile's box
+  int r0, r1;          // the patch's rows in a staged box (16-byte units)
   int nx, nz;
   int im, ip;          // row buffer slots of the rows below and above the patch
   bool l0, l31;        // the x neighbour is in another warp
@@ -78,6 +126,10 @@ __device__ __forceinline__ Patch patch_of(const MGLevel& L, int4 b) {
   const int g = tx * L.ox - 1 + col;
   p.x0 = 4 * g;
   p.y0 = ty * L.oy - HY + 2 * pr;
+  p.tx0 = 4 * (tx * L.ox - 1);
+  p.ty0 = ty * L.oy - HY;
+  p.r0 = pr < pairs ? 2 * pr * cols + col : 0;
+  p.r1 = p.r0 + (pr < pairs ? cols : 0);
   const bool gok = g >= 0 && p.x0 < p.nx && pr < pairs, cin = col >= 1 && col <= L.ox;
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
