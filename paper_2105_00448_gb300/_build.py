@@ -34,6 +34,7 @@ UNITS = {
     "mg.cu": [],
     "march.cu": [],
     "cg.cu": [],
+    "dc.cu": [],
     "cg64.cu": [],
     "coarse.cu": [],
 }

@@ -166,8 +166,8 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which
     if (!step(std::integral_constant<int, 0>{}, k) ||
         (k + 1 <= k1 && !step(std::integral_constant<int, 1>{}, k + 1)) ||
         (k + 2 <= k1 && !step(std::integral_constant<int, 2>{}, k + 2))) {
-      tma_abort(c, bar, kARing, k - k0, issued);
-      return;
+      tma_abort(c, bar, kARing, k - k0, issued);   // (goes on to its arrival)
+      break;
     }
   }
   double* slots = c.mslot + L.slot0 + (long long)b.y * L.nseg + zb / seglen;
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kBT, 4) k_cg_b(Ctx c, int which, float* __rest
   c.sync->active_count = n_active;
   c.sync->parity ^= 1;
   const int g = ++c.sync->guard;
-  bool go = n_active > 0;
+  bool go = n_active > 0 && *(volatile int*)&c.sync->error != SYNC_ERR_TIMEOUT;
   if (go && g >= c.sync->guard_limit) {
     // every replicate stops at maxit; this only guards the graph loop
     c.sync->error = 2;
@@ -426,7 +426,7 @@ long long cg_plan(const std::vector<RepDesc>& reps, int sm_count, std::vector<MG
     L.pitch = reps[i].nxp;
     march_tile(L, 1);
     L.slot0 = (int)slots;
-    slots += (long long)L.tx * L.ty * L.nseg;
+    slots += 3LL * L.tx * L.ty * L.nseg;   // (the residual sweep has three sums)
     set.push_back(&L);
     ids.push_back((int)i);
   }

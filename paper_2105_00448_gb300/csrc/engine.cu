@@ -25,8 +25,8 @@ long long cg_plan(const std::vector<RepDesc>& reps, int sm_count, std::vector<MG
 void launch_true_residual(const Ctx& c, int which, void* xfield, bool fp64);
 void launch_apply(const Ctx& c, int which, int rep, const void* u, void* out, bool fp64);
 void launch_diff_norms(const Ctx& c, const void* a, const void* b, bool fp64);
-void launch_dc_residual(const Ctx& c, int which, const void* x_hi, const void* x_lo, bool first, CondArg outer,
-                        CondArg inner);
+bool dc_init();
+void launch_dc_residual(const Ctx& c, int which, bool first, CondArg outer, CondArg inner);
 void launch_dc_update(const Ctx& c, void* x_hi, void* x_lo);
 void launch_init(const Ctx& c, const float* pc, const float* pf, const float* pv, int* err, bool fp64);
 void launch_ode(const Ctx& c, bool fp64);
@@ -546,7 +546,7 @@ int solve_dc(hca_handle* h, int which) {
   void* xl = which == 0 ? c.K_lo : c.G_lo[which - 1];
   for (int outer = 0;; ++outer) {
     HCA_LAUNCH(h, HCA_KCLASS_RESIDUAL, 1,
-               hca::launch_dc_residual(c, which, xh, xl, outer == 0, kNoCond, kNoCond));
+               hca::launch_dc_residual(c, which, outer == 0, kNoCond, kNoCond));
     if (h->mg && outer == 0) HCA_LAUNCH(h, HCA_KCLASS_MG, h->mgh.nlev - 1, mg_setup(h, which, true));
     HCA_TRY(cudaMemcpyAsync(h->h_pinned, &c.sync->active_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, c.stream));
     HCA_TRY(cudaStreamSynchronize(c.stream));
@@ -674,7 +674,7 @@ int cap_solve(hca_handle* h, int which, cudaGraph_t G) {
   HCA_TRY(cudaGraphConditionalHandleCreate(&Hi, G, 0, cudaGraphCondAssignDefault));
   const hca::CondArg co{Ho, 1}, ci{Hi, 1};
   c.stream = S;
-  hca::launch_dc_residual(c, which, xh, xl, true, co, ci);
+  hca::launch_dc_residual(c, which, true, co, ci);
   if (h->mg) mg_setup(h, which, true);
   HCA_TRY(cudaGetLastError());
   // Each loop's body opens with its V-cycle, so none runs after the residual
@@ -699,7 +699,7 @@ int cap_solve(hca_handle* h, int which, cudaGraph_t G) {
   HCA_TRY(cudaStreamEndCapture(S3, &bi));
   c.stream = S2;
   hca::launch_dc_update(c, xh, xl);
-  hca::launch_dc_residual(c, which, xh, xl, false, co, ci);
+  hca::launch_dc_residual(c, which, false, co, ci);
   HCA_TRY(cudaGetLastError());
   HCA_TRY(cudaStreamEndCapture(S2, &bo));
   c.stream = S;
@@ -1463,7 +1463,12 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
         hca::MGLevel& L = lv[i];
         const long long o = h->reps_h[i].off;
         L.map0 = (int)maps.size();
-        for (void* a : {c.z, c.p, c.p_alt, c.dx, c.d}) {
+        std::vector<void*> arrays = {c.z, c.p, c.p_alt, c.dx, c.d, c.reac, c.b, c.perf, c.Vc, c.aux, c.K, c.K_lo};
+        for (int f = 0; f < hca::MAX_FIELDS; ++f) {   // (operator f + 1; an unused one repeats oxygen's)
+          arrays.push_back(c.G[f] ? c.G[f] : c.K);
+          arrays.push_back(c.G_lo[f] ? c.G_lo[f] : c.K_lo);
+        }
+        for (void* a : arrays) {
           maps.emplace_back();
           if (!hca::march_map(&maps.back(), L, (float*)a + o)) {
             rc = HCA_ERR_CUDA;
@@ -1482,7 +1487,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
       ALLOC(bg_d, sizeof(int4) * bg.size());
       ALLOC(c.mslot, sizeof(double) * (size_t)mslots);
       ALLOC(c.mcnt, sizeof(int) * (size_t)n);
-      if (!hca::cg_init() ||
+      if (!hca::cg_init() || !hca::dc_init() ||
           cudaMemcpyAsync(maps_d, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice, c.stream) ||
           cudaMemcpyAsync(lv_d, lv.data(), sizeof(hca::MGLevel) * lv.size(), cudaMemcpyHostToDevice, c.stream) ||
           cudaMemcpyAsync(ab_d, ab.data(), sizeof(int4) * ab.size(), cudaMemcpyHostToDevice, c.stream) ||

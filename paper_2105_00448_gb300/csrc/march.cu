@@ -369,8 +369,8 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
     if (!step(std::integral_constant<int, 0>{}, k) ||
         (k + 1 <= k1 && !step(std::integral_constant<int, 1>{}, k + 1)) ||
         (k + 2 <= k1 && !step(std::integral_constant<int, 2>{}, k + 2))) {
-      tma_abort(c, bar, kUpRing, k - k0, issued);
-      return;
+      tma_abort(c, bar, kUpRing, k - k0, issued);   // (goes on to its arrival)
+      break;
     }
   }
   if (!LAT) return;

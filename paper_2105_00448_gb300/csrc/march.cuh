@@ -22,6 +22,9 @@ __device__ __forceinline__ void cp16(unsigned sdst, const float* gsrc, int n) { 
 // copies of the patches took 14 shared-memory cycles a warp instruction: the
 // pipe the sweeps' own exchanges need.)
 constexpr int kTmaWaitLimit = 1 << 20;
+// The lattice's maps, from MGLevel::map0 of its pass A tiling: z, p, p_alt, dx,
+// d; a, b, perfusion, V, K_prev; x_hi and x_lo of each operator.
+constexpr int kMapReac = 5, kMapFields = 10;
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(bar)), "r"(bytes)
                : "memory");
@@ -33,14 +36,18 @@ __device__ __forceinline__ void tma_load_3d(void* sdst, const CUtensorMap* map, 
       "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(tc::smem_u32(bar))
       : "memory");
 }
-// One thread: the stages' barriers, and the maps (in global memory, written by a
-// copy at creation; the acquire also drops what the descriptor cache may hold
-// of an earlier handle at the same address).
+// The maps are in global memory, written by a copy at creation; the acquire
+// also drops what the descriptor cache may hold of an earlier handle at the
+// same address.
+__device__ __forceinline__ void maps_acquire(const CUtensorMap* maps, int n) {
+  for (int m = 0; m < n; ++m)
+    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((unsigned long long)&maps[m])
+                 : "memory");
+}
+// The stages' barriers, and the maps the block uses (one thread).
 __device__ __forceinline__ void mbars_init(uint64_t* bar, int n, const CUtensorMap* maps, int n_maps) {
   if (threadIdx.x == 0) {
-    for (int m = 0; m < n_maps; ++m)
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((unsigned long long)&maps[m])
-                   : "memory");
+    maps_acquire(maps, n_maps);
     for (int s = 0; s < n; ++s) tc::mbar_init(&bar[s], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -31,66 +31,11 @@
 #include <cstdlib>
 
 #include "hca_internal.cuh"
+#include "reaction.cuh"
 #include "row_ops.cuh"
 
 namespace hca {
 namespace {
-
-// a + k p for the drug reaction: in FP32 rounded after the product and after
-// the sum (no fused multiply-add), so the stored FP32 coefficients of the
-// system are the plain IEEE result of these operations.
-__device__ __forceinline__ float add_prod(float a, float k, float p) { return __fadd_rn(a, __fmul_rn(k, p)); }
-__device__ __forceinline__ double add_prod(double a, double k, double p) { return a + k * p; }
-
-// The coefficients of operator `which` in the field precision, converted
-// from the handle's FP64 parameters once per thread: the conversions run on
-// the FP64 pipe (a small fraction of the FP32 rate on this GPU), and the
-// parameters sit in global memory, where the compiler cannot keep them in
-// registers across the kernel's own stores.
-template <typename T>
-struct Coef {
-  T cpl, phi_K, K1, r_K, o2_mass, base, kappa, uptake;
-};
-template <typename T, int KIND>
-__device__ __forceinline__ Coef<T> coef(const RepDesc& rd, int which) {
-  Coef<T> q;
-  q.cpl = op_coupling_t<T>(rd, which);
-  q.phi_K = q.K1 = q.r_K = q.o2_mass = q.base = q.kappa = q.uptake = T(0);
-  if (KIND == 0) {
-    q.phi_K = (T)rd.phi_K;
-    q.K1 = (T)rd.K1;
-    q.r_K = (T)rd.r_K;
-    q.o2_mass = (T)rd.o2_mass;
-  } else {
-    const int dd = which - 1;
-    q.base = (T)rd.base_drug[dd];
-    q.kappa = (T)rd.kappa[dd];
-    q.uptake = (T)rd.uptake[dd];
-  }
-  return q;
-}
-
-// Reaction coefficient a of the operator at one site (d = c n + a).
-template <typename T, int KIND>
-__device__ __forceinline__ T reaction_site(const Coef<T>& q, uint8_t s, T K_prev, T pf) {
-  T a;
-  if (KIND == 0) {
-    a = is_consumer(s) ? q.phi_K / (q.K1 + K_prev) : T(0);
-    if (is_vessel(s)) a += q.r_K;
-    a += q.o2_mass;   // 0 for the quasi-steady form
-  } else {
-    a = q.base;
-    if (is_vessel(s)) a = add_prod(a, q.kappa, pf);
-    if (is_cancer(s)) a += q.uptake;
-  }
-  return a;
-}
-
-// Diagonal of the operator at one site.
-template <typename T, int KIND>
-__device__ __forceinline__ T diag_site(const Coef<T>& q, int n_nb, uint8_t s, T K_prev, T pf) {
-  return q.cpl * (T)n_nb + reaction_site<T, KIND>(q, s, K_prev, pf);
-}
 
 // ------------------------------------------------------------------ setup --
 // r = b - A x0 with x0 the current field; writes d, z = r/d (and b for drugs
@@ -601,362 +546,6 @@ __global__ void __launch_bounds__(512) k_diff_norms(Ctx c, const T* __restrict__
                  });
 }
 
-// A sum of FP32 terms s * 2^ex kept as m * 2^e in FP32 arithmetic (the
-// terms are scaled sums of a few squares, so m stays of order one; terms more
-// than 2^126 below the running sum underflow to zero), converted to FP64 once.
-struct ScaledAcc {
-  float m = 0.f;
-  int e = 0;
-  __device__ __forceinline__ void add(float s, int ex) {
-    if (s == 0.f) return;
-    if (m == 0.f) {
-      m = s;
-      e = ex;
-    } else if (ex > e) {
-      m = scalbnf(m, e - ex) + s;
-      e = ex;
-    } else {
-      m += scalbnf(s, ex - e);
-    }
-  }
-  // m 2^e in FP64, exactly: 2^e is built from its bits when it is a normal
-  // double (two FP64-pipe instructions instead of a library ldexp)
-  __device__ __forceinline__ double value() const {
-    if (m == 0.f) return 0.0;
-    if (e < -1022 || e > 1023) return ldexp((double)m, e);
-    return (double)m * __longlong_as_double((long long)(e + 1023) << 52);
-  }
-};
-
-// The sum of a row's lane accumulators (lane segments of lpr lanes, fixed
-// xor tree: partners form the same sum, so every lane of the segment ends
-// with it) in FP32 arithmetic, converted to FP64 once per row.
-__device__ __forceinline__ double row_reduce_scaled(ScaledAcc a, int lpr) {
-  for (int o = lpr >> 1; o > 0; o >>= 1) {
-    const float bm = __shfl_xor_sync(0xffffffffu, a.m, o, 32);
-    const int be = __shfl_xor_sync(0xffffffffu, a.e, o, 32);
-    if (bm != 0.f) {
-      if (a.m == 0.f) {
-        a.m = bm;
-        a.e = be;
-      } else {
-        const int e = max(a.e, be);
-        a.m = scalbnf(a.m, a.e - e) + scalbnf(bm, be - e);
-        a.e = e;
-      }
-    }
-  }
-  return a.value();
-}
-
-// --------------------------------------------------- defect correction ---
-// FP32 storage scheme.  The solution is kept as two FP32 words, x = x_hi +
-// x_lo.  Each sweep evaluates the residual r = b - A x to about 48 bits
-// (float-float arithmetic) from the two-word solution, with the diagonal
-// rebuilt exactly as c n + a from the stored FP32 reaction coefficient a (storing d = c n + a itself in FP32 would
-// round away most digits of the small reaction part: 1/dt + psi ~ 0.03 next to
-// c n ~ 600 for a drug).  It stops the solve when |r| <= rtol |b| (FP64 norms)
-// and otherwise starts an FP32 inner CG on the correction, A32 dx = fl32(r),
-// dx0 = 0, to the inner tolerance, where A32 uses the FP32 diagonal.  The first
-// sweep of a solve (FIRST) also builds and stores a, d (and b for a drug).
-// With the multigrid preconditioner (MG) the kernel stores r for the V-cycle,
-// which forms z itself; otherwise it stores the Jacobi z = r / d and sums r.z.
-// Per site the arithmetic is FP32 and float-float (FP64 runs at a small
-// fraction of the FP32 rate on this GPU).
-// The epilogue of a row kernel in either form (block per chunk, or
-// persistent rows with block-level chunk arrivals).
-template <bool PERSIST, class Fin, class Post>
-__device__ __forceinline__ void dc_epilogue(const Ctx& c, int ndot, int chunk, Fin fin, Post post) {
-  if (PERSIST) block_arrivals(c, ndot, fin, post);
-  else warp_epilogue(c, ndot, chunk, fin, post);
-}
-
-template <int KIND, bool FIRST, bool MG, bool PERSIST = false, int REGS = 128>
-__global__ void __launch_bounds__(512) __maxnreg__(REGS) k_dc_residual(Ctx c, int which, const float* __restrict__ x_hi,
-                                                     const float* __restrict__ x_lo, CondArg outer,
-                                                     CondArg inner) {
-  HCA_COUNT_KERNEL(c);
-  __shared__ double s_G0;
-  const int2 ch = PERSIST ? make_int2(0, 0) : c.chunks[blockIdx.x];
-  const RepDesc& rd = c.reps[ch.x];
-  const RepSolve sv = c.solve[ch.x];
-  const bool live = FIRST || sv.active || sv.dc_apply;
-  if (KIND == 1 && FIRST) {
-    if (threadIdx.x == 0) s_G0 = substep_plasma(rd, which, *c.step, c.sub);
-    __syncthreads();
-  }
-  if (live) {
-    const int nrows = min(rd.chunk_rows, rd.ny * rd.nz - ch.y);
-    float* __restrict__ dd = (float*)c.d;
-    float* __restrict__ aa = (float*)c.reac;
-    float* __restrict__ zz = (float*)c.z;
-    float* __restrict__ bb = (float*)c.b;
-    const float* __restrict__ perf = (const float*)c.perf;
-    const Coef<float> q = coef<float, KIND>(rd, which);
-    const double cpl = (double)q.cpl;
-    const float G0 = KIND == 1 && FIRST ? (float)s_G0 : 0.f;
-    const bool bax = rd.bax[which] != 0;
-    const bool o2t = KIND == 0 && rd.bx[0] != 0.0;
-    const double bx = rd.bx[which];
-    // bx as an unevaluated float pair (b = bx x0 + ... is formed to ~48 bits)
-    const float bx_hi = (float)bx, bx_lo = (float)(bx - (double)bx_hi);
-    const float bvessel = (float)(bax ? 2.0 * rd.r_K * rd.K0 : rd.r_K * rd.K0);
-    const float av = (float)(bax ? 2.0 * rd.a_vegf : rd.a_vegf);
-    const RowIter it = row_iter(rd);
-    const float cpl32 = (float)cpl;
-    // one row j (chunk slot rl of `chunk`; row_ok false: a padding slot of the last chunk)
-    auto row = [&](int chunk, int rl, bool row_ok, int j) {
-      const RowGeo geo = row_geo(rd, j);
-      ScaledAcc la[NDOT];
-      float carry_h = 0.f, carry_l = 0.f;
-      for (int itn = 0; itn < it.niter; ++itn) {
-        const int g = itn * it.lpr + it.sl;
-        const bool gok = row_ok && g < rd.gpr;
-        const long long e = geo.base + 4LL * g;
-        // the two-word solution x_hi + x_lo at the group and its neighbour rows
-        const V4<float> Xh = ld4_if(x_hi + e, gok), Xl = ld4_if(x_lo + e, gok);
-        const V4<float> ymh = ld4_if(x_hi + e - geo.sy, gok && geo.ym), yml = ld4_if(x_lo + e - geo.sy, gok && geo.ym);
-        const V4<float> yph = ld4_if(x_hi + e + geo.sy, gok && geo.yp), ypl = ld4_if(x_lo + e + geo.sy, gok && geo.yp);
-        const V4<float> zmh = ld4_if(x_hi + e - geo.sz, gok && geo.zm), zml = ld4_if(x_lo + e - geo.sz, gok && geo.zm);
-        const V4<float> zph = ld4_if(x_hi + e + geo.sz, gok && geo.zp), zpl = ld4_if(x_lo + e + geo.sz, gok && geo.zp);
-        // every other load of the group is issued here too, before any value
-        // is used, so a group costs one memory round trip: the site after the
-        // group (the segment's last lane), and d, a, b (later sweeps) or the
-        // state, perfusion and Vc (the first sweep)
-        const bool last_lane = it.sl == it.lpr - 1 && gok && g + 1 < rd.gpr;
-        const float rnh = last_lane ? x_hi[e + 4] : 0.f, rnl = last_lane ? x_lo[e + 4] : 0.f;
-        const bool vegf = KIND == 1 && which == WHICH_VEGF;
-        V4<float> D = zero4<float>(), B = zero4<float>(), AR = zero4<float>(), SRC = zero4<float>();
-        V4<float> PF = zero4<float>(), VC = zero4<float>();
-        uchar4 st = make_uchar4(0, 0, 0, 0);
-        if (gok && FIRST) {
-          st = ld_state4(c.state + e);
-          if (KIND == 1) PF = ld4(perf + e);
-          if (vegf) VC = ld4((const float*)c.Vc + e);
-        } else if (gok) {
-          if (!MG) D = ld4(dd + e);
-          AR = ld4(aa + e);
-          B = ld4(bb + e);
-        }
-        float lh, rh, ll, rlo;
-        x_neighbours(Xh, g, rd.gpr, it.sl, it.lpr, gok, carry_h, lh, rh, [&] { return rnh; });
-        x_neighbours(Xl, g, rd.gpr, it.sl, it.lpr, gok, carry_l, ll, rlo, [&] { return rnl; });
-        if (gok) {
-          if (FIRST) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int xk = 4 * g + k;
-              const uint8_t s = st_at(st, k);
-              D.a[k] = 0.f;
-              B.a[k] = 0.f;
-              AR.a[k] = 0.f;
-              SRC.a[k] = 0.f;
-              if (xk < rd.nx) {
-                // x0 bx to ~48 bits, rounded once; x0 rounded to FP32
-                const FF xbx = ff_mul(FF{Xh.a[k], Xl.a[k]}, FF{bx_hi, bx_lo});
-                const float xb32 = __fadd_rn(xbx.hi, xbx.lo);
-                const float xk32 = __fadd_rn(Xh.a[k], Xl.a[k]);
-                // the operator is linearised about K_prev: the start field, or c.lag when the solve starts from another guess
-                const float lag = (KIND == 0 && c.lag) ? ((const float*)c.lag)[e + k] : xk32;
-                AR.a[k] = reaction_site<float, KIND>(q, s, lag, PF.a[k]);
-                D.a[k] = cpl32 * (float)neighbour_count(rd, geo, xk) + AR.a[k];
-                if (KIND == 0) {
-                  SRC.a[k] = is_vessel(s) ? bvessel : 0.f;
-                  B.a[k] = SRC.a[k] + (o2t ? xb32 : 0.f);
-                } else {
-                  if (vegf) SRC.a[k] = is_consumer(s) ? av * VC.a[k] : 0.f;
-                  else SRC.a[k] = is_vessel(s) ? __fmul_rn(__fmul_rn(q.kappa, PF.a[k]), G0) : 0.f;
-                  B.a[k] = __fadd_rn(xb32, SRC.a[k]);
-                }
-              }
-            }
-            st4(dd + e, D);
-            st4(aa + e, AR);
-            if (MG && c.mg_w) {   // 1/d for the sweeps of a lattice without coarse levels (0 where d = 0), as k_mg_w0 forms it
-              V4<float> Wv;
-#pragma unroll
-              for (int k = 0; k < 4; ++k) Wv.a[k] = D.a[k] != 0.f ? 1.f / D.a[k] : 0.f;
-              st4((float*)c.mg_w + e, Wv);
-            }
-          }
-          V4<float> Z, R32 = zero4<float>();
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            Z.a[k] = 0.f;
-            if (4 * g + k < rd.nx) {
-              // r = b - (d x - c sum_nb x) in float-float (~48 bits): the
-              // operator's terms cancel to the small defect; d = c n + a is
-              // formed exactly from the stored reaction a
-              const FF xv{Xh.a[k], Xl.a[k]};
-              const FF L{k == 0 ? lh : Xh.a[k - 1], k == 0 ? ll : Xl.a[k - 1]};
-              const FF Rr{k == 3 ? rh : Xh.a[k + 1], k == 3 ? rlo : Xl.a[k + 1]};
-              const FF nb = ff_add(ff_add(ff_add(L, Rr), ff_add(FF{ymh.a[k], yml.a[k]}, FF{yph.a[k], ypl.a[k]})),
-                                   ff_add(FF{zmh.a[k], zml.a[k]}, FF{zph.a[k], zpl.a[k]}));
-              const FF d = ff_add(ff_two_prod(cpl32, (float)neighbour_count(rd, geo, 4 * g + k)), AR.a[k]);
-              const FF t = ff_add(ff_mul(d, xv), ff_neg(ff_mul(nb, cpl32)));
-              // Crank-Nicolson: b = (4/h) x0 - A x0 + source, formed once from the start field
-              if (FIRST && bax) {
-                const FF bf = ff_add(ff_add(ff_mul(xv, FF{bx_hi, bx_lo}), SRC.a[k]), ff_neg(t));
-                B.a[k] = __fadd_rn(bf.hi, bf.lo);
-              }
-              const FF rf = ff_add(ff_neg(t), B.a[k]);
-              const float r32 = __fadd_rn(rf.hi, rf.lo);
-              if (!MG) Z.a[k] = D.a[k] != 0.f ? r32 / D.a[k] : 0.f;
-              R32.a[k] = r32;
-            }
-          }
-          if (FIRST) st4(bb + e, B);
-          // the group's |r|^2, r.z and |b|^2: each 4-term sum is taken in
-          // FP32 after an exact power-of-two scaling by the group's largest
-          // magnitude (a decayed field's residual, ~1e-22, would underflow
-          // when squared unscaled); the lane keeps its groups' sums as a
-          // scaled FP32 pair and enters the FP64 row sums once per row (FP64
-          // arithmetic is a small fraction of FP32's on this GPU)
-          auto scaled_sum = [](const V4<float>& v, ScaledAcc& acc) {
-            float m = 0.f;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) m = fmaxf(m, fabsf(v.a[k]));
-            if (m == 0.f) return;
-            const int ex = ilogbf(m);
-            float s2 = 0.f;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float u = scalbnf(v.a[k], -ex);
-              s2 += u * u;
-            }
-            acc.add(s2, 2 * ex);
-          };
-          scaled_sum(R32, la[0]);
-          if (FIRST) scaled_sum(B, la[1]);
-          if (!MG) {
-            // r.z with z = r / d: scale r and z by the same power (|z| may be
-            // far from |r|, so each is scaled by its own group maximum)
-            float mr = 0.f, mz = 0.f;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              mr = fmaxf(mr, fabsf(R32.a[k]));
-              mz = fmaxf(mz, fabsf(Z.a[k]));
-            }
-            if (mr > 0.f && mz > 0.f) {
-              const int er = ilogbf(mr), ez = ilogbf(mz);
-              float s = 0.f;
-#pragma unroll
-              for (int k = 0; k < 4; ++k) s += scalbnf(R32.a[k], -er) * scalbnf(Z.a[k], -ez);
-              la[2].add(s, er + ez);
-            }
-          }
-          if (MG) st4((float*)c.r + e, R32);
-          else st4(zz + e, Z);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < NDOT; ++k) {
-        const double v = row_reduce_scaled(la[k], it.lpr);
-        if (row_ok && it.sl == 0) c.rowp[((long long)chunk * CHUNK_ROWS + rl) * NDOT + k] = v;
-      }
-    };
-    if (PERSIST) {
-      const int R = rd.ny * rd.nz, cr = rd.chunk_rows;
-      for (int j = persist_row_begin(R) + it.warp; j < persist_row_end(R); j += it.nw) row(j / cr, j % cr, true, j);
-    } else {
-      for (int rbase = it.warp * it.rpw; rbase < rd.chunk_rows; rbase += it.nw * it.rpw) {
-        const int rl = rbase + it.sub;
-        const bool row_ok = rl < nrows;
-        row(blockIdx.x, rl, row_ok, ch.y + (row_ok ? rl : 0));
-      }
-    }
-  }
-  dc_epilogue<PERSIST>(c, 3, blockIdx.x,
-                 [&](int r, const double* s3) -> int {
-                   const RepDesc& rr = c.reps[r];
-                   RepSolve& s = c.solve[r];
-                   DevStats& st = c.stats[r];
-                   if (FIRST) {
-                     s.outer = 0;
-                     s.zero_b = 0;
-                     s.dc_apply = 0;
-                     s.active = 0;
-                     s.iters = 0;
-                     s.pend = 0;
-                     if (c.frozen[r]) return 0;
-                   } else if (!s.dc_apply) {
-                     return 0;        // this replicate finished in an earlier sweep
-                   }
-                   st.iters[which] += s.iters;
-                   st.sweeps[which] += 1;
-                   s.pend = 0;
-                   // |b|^2 is summed on the first sweep only (b does not change)
-                   if (FIRST) s.bb_outer = s3[1];
-                   const double bb = s.bb_outer;
-                   if (!isfinite(s3[0]) || !isfinite(bb) || !isfinite(s3[2])) {
-                     c.sync->error = 1;
-                     st.nonfinite = 1;
-                     s.active = 0;
-                     s.dc_apply = 0;
-                     return 0;
-                   }
-                   const double tol = which == 0 ? rr.rtol_o2 : rr.rtol_drug;
-                   if (bb == 0.0) {
-                     s.zero_b = 1;
-                     s.rel_true = 0.0;
-                     st.rel[which] = 0.0;
-                     s.active = 0;
-                     s.dc_apply = 0;
-                     return 0;
-                   }
-                   const double rel = sqrt(s3[0] / bb);
-                   s.rel_true = rel;
-                   st.rel[which] = rel;
-                   if (rel <= tol || s.outer >= rr.max_outer) {
-                     if (rel > tol) st.not_converged |= 1 << which;
-                     s.active = 0;
-                     s.dc_apply = 0;
-                     return 0;
-                   }
-                   // start the inner FP32 solve A dx = fl32(r), rescaled by a
-                   // power of two so that its values are O(1) per site (the
-                   // residual of a decayed field can be ~1e-22, whose FP32
-                   // squares underflow); the update divides the scale out
-                   s.outer += 1;
-                   const double n_sites = (double)rr.nx * rr.ny * rr.nz;
-                   const double rms = sqrt(s3[0] / n_sites);
-                   int e = rms > 0.0 ? -ilogb(rms) : 0;
-                   e = e < -120 ? -120 : (e > 120 ? 120 : e);
-                   const double sc = ldexp(1.0, e);
-                   s.scale = sc;
-                   s.rho = s3[2] * sc * sc;
-                   s.rnorm2 = s3[0] * sc * sc;
-                   s.bnorm2 = s3[0] * sc * sc;
-                   // inner tolerance: rtol_inner relative to this sweep's
-                   // defect, or, when the outer target is within a factor 8
-                   // of that (or looser), the reduction that reaches half the
-                   // outer target, so the last sweep neither over-solves nor
-                   // falls just short and costs another sweep
-                   const double q = 0.5 * tol / rel;
-                   s.rtol = q >= 0.125 * rr.rtol_inner ? q : rr.rtol_inner;
-                   s.maxit = rr.maxit;
-                   s.iters = 0;
-                   s.alpha = 0.0;
-                   s.beta = 0.0;
-                   s.dc_apply = 1;
-                   // the multigrid form leaves rho to the V-cycle (s3[2] = 0)
-                   s.active = (MG ? s3[0] > 0.0 : s3[2] > 0.0) ? 1 : 0;
-                   return s.active;
-                 },
-                 [&](int n_active) {
-                   c.sync->parity = 0;
-                   c.sync->guard = 0;
-                   const int g = FIRST ? (c.sync->guard_outer = 0) : ++c.sync->guard_outer;
-                   bool go = n_active > 0;
-                   if (go && g >= c.sync->guard_outer_limit) {
-                     c.sync->error = 2;
-                     go = false;
-                   }
-                   set_cond(outer, go);
-                   set_cond(inner, go);
-                 });
-}
-
 // x_hi + x_lo += dx (two-word sum), or x = 0 for a vanishing right-hand side.
 // dx is what pass A of the later iterations accumulated plus the last
 // iteration's step alpha p (0 + alpha p after a single iteration).
@@ -1009,37 +598,6 @@ __global__ void __launch_bounds__(512) k_dc_update(Ctx c, float* __restrict__ x_
 }  // namespace
 
 // ------------------------------------------------------------- launchers --
-int persist_grid(const void* fn, int threads, int sm_count);
-
-template <int KIND, bool FIRST, bool MG>
-static void launch_dc_residual_v(const Ctx& c, int which, const float* x_hi, const float* x_lo, CondArg outer,
-                                 CondArg inner) {
-  if (c.persist) {
-    // a 96-register cap: 16 -> 20 warps per SM (measured 176 -> 170 us per launch at 256^3)
-    const int g = persist_grid((const void*)k_dc_residual<KIND, FIRST, MG, true, 96>, c.threads, c.sm_count);
-    launch_k(c.pdl != 0, k_dc_residual<KIND, FIRST, MG, true, 96>, dim3(g), dim3(c.threads), 0, c.stream, c, which, x_hi,
-             x_lo, outer, inner);
-  } else {
-    launch_k(c.pdl != 0, k_dc_residual<KIND, FIRST, MG, false>, dim3(c.n_chunks), dim3(c.threads), 0, c.stream, c, which,
-             x_hi, x_lo, outer, inner);
-  }
-}
-
-template <int KIND>
-static void launch_dc_residual_t(const Ctx& c, int which, const float* x_hi, const float* x_lo, bool first,
-                                 CondArg outer, CondArg inner) {
-  if (first && c.mg) launch_dc_residual_v<KIND, true, true>(c, which, x_hi, x_lo, outer, inner);
-  else if (first) launch_dc_residual_v<KIND, true, false>(c, which, x_hi, x_lo, outer, inner);
-  else if (c.mg) launch_dc_residual_v<KIND, false, true>(c, which, x_hi, x_lo, outer, inner);
-  else launch_dc_residual_v<KIND, false, false>(c, which, x_hi, x_lo, outer, inner);
-}
-
-void launch_dc_residual(const Ctx& c, int which, const void* x_hi, const void* x_lo, bool first, CondArg outer,
-                        CondArg inner) {
-  if (which == 0) launch_dc_residual_t<0>(c, which, (const float*)x_hi, (const float*)x_lo, first, outer, inner);
-  else launch_dc_residual_t<1>(c, which, (const float*)x_hi, (const float*)x_lo, first, outer, inner);
-}
-
 void launch_dc_update(const Ctx& c, void* x_hi, void* x_lo) {
   launch_k(c.pdl != 0, k_dc_update, dim3(c.n_chunks), dim3(c.threads), 0, c.stream, c, (float*)x_hi, (float*)x_lo);
 }
