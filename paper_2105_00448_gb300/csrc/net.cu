@@ -593,13 +593,41 @@ __global__ void __launch_bounds__(kThreads) k_wgrad(const WgArgs a) {
   }
 }
 
-// dst[i] = sum_g part[g][i], g = 0 .. G-1 in order (deterministic split-K reduce)
-__global__ void k_sum_parts(const float* __restrict__ part, int G, long long n, float* __restrict__ dst) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int g = 0; g < G; ++g) s += part[(long long)g * n + i];
-    dst[i] = s;
+// dst[i] = sum_g part[g][i] (split-K reduce): 8 warps of a block take every
+// eighth partial of 32 neighbouring elements, then add their sums in order, so
+// the result does not depend on the launch.  Latency of the loads is the
+// bound; a thread per element walking all partials took 31 us for 304 x 6,912
+// values, this form 5.
+constexpr int kSumWarps = 8;
+__global__ void __launch_bounds__(32 * kSumWarps) k_sum_parts(const float* __restrict__ part, int G, long long n,
+                                                              float* __restrict__ dst) {
+  __shared__ float sb[kSumWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long i = blockIdx.x * 32LL + lane;
+  float s = 0.f;
+  if (i < n) {
+#pragma unroll 8
+    for (int g = warp; g < G; g += kSumWarps) s += part[(long long)g * n + i];
   }
+  sb[warp][lane] = s;
+  __syncthreads();
+  if (warp || i >= n) return;
+  float t = 0.f;
+#pragma unroll
+  for (int w = 0; w < kSumWarps; ++w) t += sb[w][lane];
+  dst[i] = t;
+}
+
+// The block's sum of v (fixed xor tree per warp, warps in order), in thread 0.
+template <int NT>
+__device__ __forceinline__ float block_sum(float v, float* sb) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float t = 0.f;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < NT / 32; ++w) t += sb[w];
+  return t;
 }
 
 // ------------------------------------------------------- elementwise ---
@@ -637,22 +665,27 @@ __global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int 
 
 constexpr int kEwThreads = 256;
 
-// Per-block channel sums written to part[blockIdx.x][C] in a fixed order:
-// vals[t][c] (one row of 8 channels per thread for the channel chunk j(t)).
+// Per-block channel sums written to part[blockIdx.x][C] in a fixed order: v
+// holds 8 channels of chunk threadIdx.x % (C / 8); lanes of a chunk by an xor
+// tree, then the warps in order.
 template <int C>
-__device__ __forceinline__ void block_channel_sums(float (&v)[8], int j, float* __restrict__ part, float* sbuf) {
-  // sbuf: kEwThreads * 8 floats
-#pragma unroll
-  for (int e = 0; e < 8; ++e) sbuf[threadIdx.x * 8 + e] = v[e];
-  __syncthreads();
+__device__ __forceinline__ void block_channel_sums(float (&v)[8], float* __restrict__ part, float* sbuf) {
+  // sbuf: (kEwThreads / 32) * C floats
   constexpr int NCH = C / 8;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    for (int o = 16; o >= NCH; o >>= 1) v[e] += __shfl_xor_sync(0xffffffffu, v[e], o);
+  if (lane < NCH) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) sbuf[warp * C + lane * 8 + e] = v[e];
+  }
+  __syncthreads();
   for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    const int jj = c / 8, e = c % 8;
     float s = 0.f;
-    for (int t = jj; t < (int)blockDim.x; t += NCH) s += sbuf[t * 8 + e];
+    for (int w = 0; w < kEwThreads / 32; ++w) s += sbuf[w * C + c];
     part[(long long)blockIdx.x * C + c] = s;
   }
-  (void)j;
 }
 
 // Gradient of a layer's pre-activation from the raw gradient of its output:
@@ -664,7 +697,7 @@ template <int C, int POOL>
 __global__ void __launch_bounds__(kEwThreads) k_combine(const float* __restrict__ graw, const bf16* __restrict__ y,
                                                         const bf16* skip, bf16* g, int D, int H, int W,
                                                         float* __restrict__ part) {
-  __shared__ float sbuf[kEwThreads * 8];
+  __shared__ float sbuf[(kEwThreads / 32) * C];
   constexpr int NCH = C / 8;
   const long long n = (long long)D * H * W * NCH;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -710,7 +743,7 @@ __global__ void __launch_bounds__(kEwThreads) k_combine(const float* __restrict_
     }
     *reinterpret_cast<uint4*>(g + s * C + j * 8) = o;
   }
-  block_channel_sums<C>(bs, j, part, sbuf);
+  block_channel_sums<C>(bs, part, sbuf);
 }
 
 // Head and loss: out = d0 . hw + hb was written by the last convolution.
@@ -724,7 +757,7 @@ __global__ void __launch_bounds__(kEwThreads) k_head_bwd(const bf16* __restrict_
                                                          const float* __restrict__ target, const float* __restrict__ gbuf,
                                                          const float* __restrict__ hw, long long N,
                                                          bf16* __restrict__ gd0, float* __restrict__ part) {
-  __shared__ float sbuf[kEwThreads];
+  __shared__ float sbuf[kEwThreads / 32][kHeadParts];
   float acc[kHeadParts];
 #pragma unroll
   for (int k = 0; k < kHeadParts; ++k) acc[k] = 0.f;
@@ -762,25 +795,38 @@ __global__ void __launch_bounds__(kEwThreads) k_head_bwd(const bf16* __restrict_
     reinterpret_cast<uint4*>(gd0 + s * 16)[0] = o[0];
     reinterpret_cast<uint4*>(gd0 + s * 16)[1] = o[1];
   }
+  // the block's sums: lanes by an xor tree, warps in order (a block-wide tree
+  // with two barriers a level for each of the 34 sums was most of the kernel)
+#pragma unroll
   for (int k = 0; k < kHeadParts; ++k) {
-    sbuf[threadIdx.x] = acc[k];
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) sbuf[threadIdx.x] += sbuf[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) part[(long long)blockIdx.x * kHeadParts + k] = sbuf[0];
-    __syncthreads();
+    float v = acc[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5][k] = v;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < kHeadParts; k += blockDim.x) {
+    float v = 0.f;
+    for (int w = 0; w < kEwThreads / 32; ++w) v += sbuf[w][k];
+    part[(long long)blockIdx.x * kHeadParts + k] = v;
   }
 }
 
-// Sum per-block partials part[b][k] (b = 0 .. nb-1 in order) into dst[map(k)].
-__global__ void k_scatter_parts(const float* __restrict__ part, int nb, int width, float* __restrict__ grads,
-                                const long long* __restrict__ dst_index, float* __restrict__ loss, float loss_scale) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= width) return;
+// Sum per-block partials part[b][k] over b into dst[map(k)], a block per k
+// (threads take every 128th partial, then a fixed tree; one thread per k
+// walking all of them took up to 65 us for 1,216 blocks, this form 3).
+constexpr int kScatterThreads = 128;
+__global__ void __launch_bounds__(kScatterThreads) k_scatter_parts(const float* __restrict__ part, int nb, int width,
+                                                                   float* __restrict__ grads,
+                                                                   const long long* __restrict__ dst_index,
+                                                                   float* __restrict__ loss, float loss_scale) {
+  __shared__ float sb[kScatterThreads / 32];
+  const int k = blockIdx.x;
   float s = 0.f;
-  for (int b = 0; b < nb; ++b) s += part[(long long)b * width + k];
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nb; b += kScatterThreads) s += part[(long long)b * width + k];
+  s = block_sum<kScatterThreads>(s, sb);
+  if (threadIdx.x != 0) return;
   const long long d = dst_index[k];
   if (d >= 0) grads[d] = s;
   else if (loss) *loss = s * loss_scale;
@@ -825,7 +871,7 @@ __device__ __forceinline__ float apply_scaled(const FeatureArgs& f, const float*
 __global__ void __launch_bounds__(kEwThreads) k_res_u(FeatureArgs f, const float* __restrict__ Kp,
                                                       const float* __restrict__ out, const float* __restrict__ tgt,
                                                       float* __restrict__ u, float* __restrict__ part) {
-  __shared__ float sb[kEwThreads];
+  __shared__ float sb[kEwThreads / 32];
   const long long n = (long long)f.nx * f.ny * f.nz;
   const float cpl = (float)(f.D_K / (f.dx * f.dx));
   float acc = 0.f;
@@ -834,13 +880,8 @@ __global__ void __launch_bounds__(kEwThreads) k_res_u(FeatureArgs f, const float
     u[s] = v;
     acc += v * v;
   }
-  sb[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sb[threadIdx.x] += sb[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = sb[0];
+  acc = block_sum<kEwThreads>(acc, sb);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
 // dL/dout of L = w_mse mean(e^2) + w_res mean(u^2):
@@ -849,7 +890,7 @@ __global__ void __launch_bounds__(kEwThreads) k_loss_grad(FeatureArgs f, const f
                                                           const float* __restrict__ out, const float* __restrict__ tgt,
                                                           const float* __restrict__ u, float w_mse, float w_res,
                                                           float* __restrict__ g, float* __restrict__ part) {
-  __shared__ float sb[kEwThreads];
+  __shared__ float sb[kEwThreads / 32];
   const long long n = (long long)f.nx * f.ny * f.nz;
   const float cpl = (float)(f.D_K / (f.dx * f.dx));
   const float sc = 2.0f / (float)n;
@@ -861,25 +902,23 @@ __global__ void __launch_bounds__(kEwThreads) k_loss_grad(FeatureArgs f, const f
     if (w_res != 0.f) v += w_res * sc * apply_scaled(f, Kp, u, nullptr, s, cpl);
     g[s] = v;
   }
-  sb[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sb[threadIdx.x] += sb[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = sb[0];
+  acc = block_sum<kEwThreads>(acc, sb);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// loss = sa * sum(pa[0..nb)) + sb * sum(pb[0..nb)), blocks in order
-__global__ void k_sum_loss(const float* __restrict__ pa, int nb, float sa, const float* __restrict__ pb, float sb,
-                           float* __restrict__ loss) {
-  if (threadIdx.x || blockIdx.x) return;
+// loss = sa * sum(pa[0..nb)) + sb * sum(pb[0..nb)) (one block, fixed order)
+__global__ void __launch_bounds__(kEwThreads) k_sum_loss(const float* __restrict__ pa, int nb, float sa,
+                                                         const float* __restrict__ pb, float sb,
+                                                         float* __restrict__ loss) {
+  __shared__ float sm[2][kEwThreads / 32];
   float a = 0.f, b = 0.f;
-  for (int i = 0; i < nb; ++i) {
+  for (int i = threadIdx.x; i < nb; i += kEwThreads) {
     a += pa[i];
     b += pb[i];
   }
-  *loss = sa * a + sb * b;
+  a = block_sum<kEwThreads>(a, sm[0]);
+  b = block_sum<kEwThreads>(b, sm[1]);
+  if (threadIdx.x == 0) *loss = sa * a + sb * b;
 }
 
 // Adam (Kingma & Ba 2015, Algorithm 1) with FP32 master weights.
@@ -1255,7 +1294,7 @@ void wgrad(hca_net* n, cudaStream_t s, const bf16* in, const bf16* gy, int D, in
   int G = std::max(1, std::min(n_tiles, 2 * n->sm_count / gy_blocks));
   G = (int)std::min<long long>(G, n->wpart_n / per);
   k_wgrad<CI, CO, UP><<<dim3(G, gy_blocks), kThreads, wgrad_smem_bytes<CI, CO, UP>(), s>>>(a);
-  k_sum_parts<<<ew_blocks(per, n->sm_count), kEwThreads, 0, s>>>(n->wpart, G, per, dst);
+  k_sum_parts<<<(int)((per + 31) / 32), 32 * kSumWarps, 0, s>>>(n->wpart, G, per, dst);
 }
 
 template <int C, int POOL>
@@ -1264,7 +1303,7 @@ void combine(hca_net* n, cudaStream_t s, const float* graw, const bf16* y, const
   const long long cnt = n->Ln[lvl] * (C / 8);
   const int nb = std::min(ew_blocks(cnt, n->sm_count), n->bpart_blocks);
   k_combine<C, POOL><<<nb, kEwThreads, 0, s>>>(graw, y, skip, g, n->Ld[lvl], n->Lh[lvl], n->Lw[lvl], n->bpart);
-  k_scatter_parts<<<1, 64, 0, s>>>(n->bpart, nb, C, n->grads, n->bias_index + 64 * layer, nullptr, 0.f);
+  k_scatter_parts<<<C, kScatterThreads, 0, s>>>(n->bpart, nb, C, n->grads, n->bias_index + 64 * layer, nullptr, 0.f);
 }
 
 template <int C>
@@ -1313,10 +1352,11 @@ void backward(hca_net* n, cudaStream_t s, const float* target, const float* gbuf
   const int* W = n->Lw;
   const ParamLayout& L = n->L;
   {
-    const int nb = std::min(ew_blocks(n->Ln[0], n->sm_count), n->bpart_blocks);
+    // two blocks per multiprocessor: each ends with its 34 sums
+    const int nb = std::min(std::min(ew_blocks(n->Ln[0], n->sm_count), 2 * n->sm_count), n->bpart_blocks);
     k_head_bwd<<<nb, kEwThreads, 0, s>>>(n->d0, n->out, target, gbuf, n->params + L.hw_off, n->Ln[0], n->g0,
                                          n->bpart);
-    k_scatter_parts<<<1, 64, 0, s>>>(n->bpart, nb, kHeadParts, n->grads, n->head_index, gbuf ? nullptr : n->loss,
+    k_scatter_parts<<<kHeadParts, kScatterThreads, 0, s>>>(n->bpart, nb, kHeadParts, n->grads, n->head_index, gbuf ? nullptr : n->loss,
                                      1.0f / (float)n->Ln[0]);
   }
   // dec0: input up(d1), output gradient g0
@@ -1648,7 +1688,7 @@ int hca_net_gradients(hca_net* n, const hca_config* cfg, const uint8_t* state, c
   k_res_u<<<nr, kEwThreads, 0, s>>>(f, K_prev, n->out, n->tgt, n->ru, n->bpart);
   k_loss_grad<<<nr, kEwThreads, 0, s>>>(f, K_prev, n->out, n->tgt, n->ru, (float)w_mse, (float)w_res, n->rg,
                                         n->bpart + n->bpart_blocks);
-  k_sum_loss<<<1, 32, 0, s>>>(n->bpart, nr, (float)w_res / (float)n->Ln[0], n->bpart + n->bpart_blocks,
+  k_sum_loss<<<1, kEwThreads, 0, s>>>(n->bpart, nr, (float)w_res / (float)n->Ln[0], n->bpart + n->bpart_blocks,
                               (float)w_mse / (float)n->Ln[0], n->loss);
   backward(n, s, n->tgt, n->rg);
   if (grads) NET_CUDA(cudaMemcpyAsync(grads, n->grads, n->L.total * sizeof(float), cudaMemcpyDeviceToDevice, s));
