@@ -162,159 +162,232 @@ struct ConvArgs {
   int Di, Hi, Wi;      // input lattice (D/2.. when UP)
 };
 
-template <int CI, int CO, int MT, bool UP, int EPI>
-constexpr int conv_smem_bytes() {
-  constexpr int TZ = MT;  // 4 warps x MT rows = TZ x kTY rows
-  constexpr int halo = Halo<TZ, UP>::N * CI * 2;
-  constexpr int red = EPI == EPI_DOWN ? 4 * MT * 8 * CO * 4 : 0;
-  return (halo > red ? halo : red) + 9 * CO * CI * 2;
+// 16-byte copy from global to shared memory; src_bytes = 0 writes zeros
+// (the source is not read).
+__device__ __forceinline__ void cp_async16_zfill(void* sdst, const void* gsrc, int src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(sdst)), "l"(gsrc), "r"(src_bytes)
+               : "memory");
 }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <int CI, int CO, int MT, bool UP, int EPI>
-__global__ void __launch_bounds__(kThreads) k_conv(const ConvArgs a) {
-  constexpr int TZ = MT;
-  constexpr int NT = CO / 8;        // n8 tiles
+// Geometry of a convolution block: NW warps of R tile rows each (TZ planes by
+// kTY rows), XO output sites along x, CB of the CO output channels.  Along x a
+// row is S interleaved M tiles (tile m holds sites S j + m, j = 0..15; of the
+// upsampled form: two per phase, one per output parity), so a tap's shift in x
+// turns one tile's rows into another's: the fragments of S + 2 phases serve all
+// three taps of the row.  The halo is staged with the phases apart
+// ([row][phase][j]), which keeps a fragment's rows consecutive.
+template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
+struct ConvTile {
+  static constexpr int ROWS = NW * R, TZ = ROWS / kTY, XO = (UP ? 32 : 16) * S;
+  static constexpr int M = (UP ? 2 : 1) * S;   // M tiles of a row
+  static constexpr int HZ = UP ? TZ / 2 + 2 : TZ + 2, HY = UP ? kTY / 2 + 2 : kTY + 2, HX = 16 * S + 2;
+  static constexpr int LP = (HX + S - 1) / S;  // sites of a phase
+  static constexpr int HALO = HZ * HY * S * LP * CI * 2;
+  static constexpr int RED = EPI == 3 ? ROWS * (XO / 2) * CB * 4 : 0;
+  static constexpr int WPLANE = 9 * CB * CI * 2;
+  static constexpr int SMEM = (HALO > RED ? HALO : RED) + 2 * WPLANE;
+  static constexpr int PER_SM = 232448 / (SMEM + 1024);
+  static constexpr int MIN_BLOCKS = PER_SM * NW > 16 ? 16 / NW : PER_SM;   // (128 registers at least)
+  static_assert(TZ >= 2 && TZ % 2 == 0 && CB % 16 == 0 && CO % CB == 0, "tile shape");
+  static_assert(!(UP && EPI == 3) && (EPI != 1 || CB == CO), "epilogue");
+};
+
+template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
+__global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, EPI>::MIN_BLOCKS)) k_conv(const ConvArgs a) {
+  using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
+  constexpr int NT = CB / 8;        // n8 tiles
   constexpr int KC = CI / 16;       // k16 steps per tap
-  using HL = Halo<TZ, UP>;
+  constexpr int NCH = CI / 8;
+  constexpr int M = T::M, NQ = S + 2;
+  constexpr bool HOLD = S > 1 || UP;   // fragments shared by the taps of a row
   extern __shared__ __align__(128) char smem[];
-  constexpr int kHaloBytes = conv_smem_bytes<CI, CO, MT, UP, EPI>() - 9 * CO * CI * 2;
   char* sh = smem;
-  char* sw = smem + kHaloBytes;
-
-  const int z0 = blockIdx.z * TZ, y0 = blockIdx.y * kTY, x0 = blockIdx.x * kRowX;
+  char* sw = smem + T::SMEM - 2 * T::WPLANE;
+  const int cg = blockIdx.x % (CO / CB), co0 = cg * CB;
+  const int z0 = blockIdx.z * T::TZ, y0 = blockIdx.y * kTY, x0 = (int)(blockIdx.x / (CO / CB)) * T::XO;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  stage_halo<CI, TZ, UP>(sh, a.in, a.Di, a.Hi, a.Wi, z0, y0, x0);
+  // the halo and the first plane of taps; the next plane follows while one is used
+  {
+    const int oz = UP ? (z0 >> 1) - 1 : z0 - 1, oy = UP ? (y0 >> 1) - 1 : y0 - 1, ox = UP ? (x0 >> 1) - 1 : x0 - 1;
+    for (int i = threadIdx.x; i < T::HZ * T::HY * T::HX * NCH; i += 32 * NW) {
+      const int h = i / NCH, j = i - h * NCH;
+      const int hx = h % T::HX, row = h / T::HX;
+      const int gz = oz + row / T::HY, gy = oy + row % T::HY, gx = ox + hx;
+      const bool in = gz >= 0 && gz < a.Di && gy >= 0 && gy < a.Hi && gx >= 0 && gx < a.Wi;
+      const bf16* src = in ? a.in + (((long long)gz * a.Hi + gy) * a.Wi + gx) * CI + 8 * j : a.in;
+      cp_async16_zfill(sh + 16 * chunk_pos<CI>((row * S + hx % S) * T::LP + hx / S, j), src, in ? 16 : 0);
+    }
+  }
+  auto stage_w = [&](int plane) {
+    char* dst = sw + (plane & 1) * T::WPLANE;
+    const bf16* wp = a.w + ((long long)plane * 9 * CO + co0) * CI;
+    for (int i = threadIdx.x; i < 9 * CB * NCH; i += 32 * NW) {
+      const int r = i / NCH, j = i - r * NCH;
+      cp_async16_zfill(dst + 16 * chunk_pos<CI>(r, j), wp + ((long long)(r / CB) * CO + r % CB) * CI + 8 * j, 16);
+    }
+    cp_async_commit();
+  };
+  stage_w(0);
 
-  float acc[MT][NT][4];
+  float acc[R][M][NT][4];
 #pragma unroll
-  for (int m = 0; m < MT; ++m)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int n = 0; n < NT; ++n)
+    for (int m = 0; m < M; ++m)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[r][m][n][e] = 0.f;
 
-  const uint32_t shb = smem_u32(sh), swb = smem_u32(sw);
+  const uint32_t shb = smem_u32(sh);
   const int q = lane >> 3;
   const int a_x = (lane & 7) + ((q & 1) << 3), a_j = q >> 1;        // A rows / k half
   const int b_co = (lane & 7) + ((q >> 1) << 3), b_j = q & 1;       // B rows / k half
 
-  for (int dz = -1; dz <= 1; ++dz) {
-    __syncthreads();   // previous plane's weights fully consumed (and halo staged)
-    {
-      constexpr int NCH = CI / 8;
-      const bf16* wp = a.w + (long long)(dz + 1) * 9 * CO * CI;
-      for (int i = threadIdx.x; i < 9 * CO * NCH; i += blockDim.x) {
-        const int r = i / NCH, j = i - r * NCH;
-        *reinterpret_cast<uint4*>(sw + 16 * chunk_pos<CI>(r, j)) =
-            __ldg(reinterpret_cast<const uint4*>(wp + (long long)r * CI) + j);
-      }
-    }
-    __syncthreads();
+  // taps in order (dz, dy, dx), channels within a tap: the accumulation order
 #pragma unroll 1
-    for (int t9 = 0; t9 < 9; ++t9) {
-      const int dy = t9 / 3 - 1, dx = t9 % 3 - 1;
+  for (int dz = -1; dz <= 1; ++dz) {
+    cp_async_wait<0>();
+    __syncthreads();   // this plane's taps are there, the plane before is consumed
+    if (dz < 1) stage_w(dz + 2);
+    const uint32_t swb = smem_u32(sw) + ((dz + 1) & 1) * T::WPLANE;
+#pragma unroll 1
+    for (int dy = -1; dy <= 1; ++dy) {
+      int hrow[R];   // halo row of the tile row
 #pragma unroll
-      for (int kc = 0; kc < KC; ++kc) {
-        uint32_t b[NT][2];
-#pragma unroll
-        for (int np = 0; np < NT / 2; ++np) {
-          uint32_t r[4];
-          const int row = t9 * CO + np * 16 + b_co;
-          ldsm_x4(swb + 16 * chunk_pos<CI>(row, 2 * kc + b_j), r);
-          b[2 * np][0] = r[0];
-          b[2 * np][1] = r[1];
-          b[2 * np + 1][0] = r[2];
-          b[2 * np + 1][1] = r[3];
-        }
-#pragma unroll
-        for (int m = 0; m < MT; ++m) {
-          const int rr = warp * MT + m;
-          const int tz = rr / kTY, ty = rr - tz * kTY;
-          const int h = HL::row(tz, ty, a_x, dz, dy, dx);
-          uint32_t af[4];
-          ldsm_x4(shb + 16 * chunk_pos<CI>(h, 2 * kc + a_j), af);
-#pragma unroll
-          for (int n = 0; n < NT; ++n) mma16816(acc[m][n], af, b[n][0], b[n][1]);
-        }
+      for (int r = 0; r < R; ++r) {
+        const int rr = warp * R + r, tz = rr / kTY, ty = rr - tz * kTY;
+        hrow[r] = (UP ? (((tz + dz) >> 1) + 1) * T::HY + (((ty + dy) >> 1) + 1) : (tz + dz + 1) * T::HY + (ty + dy + 1)) *
+                  (S * T::LP);
       }
+      uint32_t af[HOLD ? R : 1][HOLD ? NQ : 1][HOLD ? KC : 1][4];
+      if (HOLD) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int p = 0; p < NQ; ++p)
+#pragma unroll
+            for (int kc = 0; kc < KC; ++kc)
+              ldsm_x4(shb + 16 * chunk_pos<CI>(hrow[r] + (p % S) * T::LP + p / S + a_x, 2 * kc + a_j), af[r][p][kc]);
+      }
+#pragma unroll
+      for (int dx = -1; dx <= 1; ++dx)
+#pragma unroll
+        for (int kc = 0; kc < KC; ++kc) {
+          const int t9 = (dy + 1) * 3 + dx + 1;
+          uint32_t b[NT][2];
+#pragma unroll
+          for (int np = 0; np < NT / 2; ++np) {
+            uint32_t f[4];
+            ldsm_x4(swb + 16 * chunk_pos<CI>(t9 * CB + np * 16 + b_co, 2 * kc + b_j), f);
+            b[2 * np][0] = f[0];
+            b[2 * np][1] = f[1];
+            b[2 * np + 1][0] = f[2];
+            b[2 * np + 1][1] = f[3];
+          }
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+              if (HOLD) {
+                const int p = UP ? m / 2 + ((m % 2 + dx + 2) / 2 - 1) + 1 : m + dx + 1;
+#pragma unroll
+                for (int n = 0; n < NT; ++n) mma16816(acc[r][m][n], af[r][p][kc], b[n][0], b[n][1]);
+              } else {
+                ldsm_x4(shb + 16 * chunk_pos<CI>(hrow[r] + dx + 1 + a_x, 2 * kc + a_j), af[0][0][0]);
+#pragma unroll
+                for (int n = 0; n < NT; ++n) mma16816(acc[r][m][n], af[0][0][0], b[n][0], b[n][1]);
+              }
+            }
+        }
     }
   }
 
   // ------------------------------------------------------------ epilogue
   const int cq = (lane & 3) * 2;
+  // output x of tile m, fragment row j
+  auto site_x = [&](int m, int j) { return UP ? 2 * (S * j + m / 2) + m % 2 : S * j + m; };
   if (EPI == EPI_DOWN) {
     __syncthreads();   // halo no longer read: reuse it for the 2x2x2 sums
     float* red = reinterpret_cast<float*>(smem);
 #pragma unroll
-    for (int m = 0; m < MT; ++m) {
-      const int rr = warp * MT + m;
+    for (int r = 0; r < R; ++r) {
+      const int rr = warp * R + r;
 #pragma unroll
-      for (int n = 0; n < NT; ++n)
+      for (int m = 0; m < M; m += S > 1 ? 2 : 1)
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          // sum the x pair (lanes l and l ^ 4 hold x and x ^ 1)
-          float v0 = acc[m][n][2 * hf], v1 = acc[m][n][2 * hf + 1];
-          v0 += __shfl_xor_sync(0xffffffffu, v0, 4);
-          v1 += __shfl_xor_sync(0xffffffffu, v1, 4);
-          const int x = (lane >> 2) + 8 * hf;
-          if ((x & 1) == 0) {
-            float* p = red + ((rr * 8 + (x >> 1)) * CO) + n * 8 + cq;
-            p[0] = v0;
-            p[1] = v1;
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            const int j = (lane >> 2) + 8 * hf;
+            float v0 = acc[r][m][n][2 * hf], v1 = acc[r][m][n][2 * hf + 1];
+            if (S > 1) {   // the x pair: tiles m and m + 1
+              v0 += acc[r][m + (S > 1)][n][2 * hf];
+              v1 += acc[r][m + (S > 1)][n][2 * hf + 1];
+            } else {       // lanes l and l ^ 4 hold x and x ^ 1
+              v0 += __shfl_xor_sync(0xffffffffu, v0, 4);
+              v1 += __shfl_xor_sync(0xffffffffu, v1, 4);
+            }
+            if (S > 1 || (j & 1) == 0)
+              *reinterpret_cast<float2*>(red + (rr * (T::XO / 2) + (S * j + m) / 2) * CB + n * 8 + cq) = make_float2(v0, v1);
           }
-        }
     }
     __syncthreads();
     const int Dc = a.D >> 1, Hc = a.H >> 1, Wc = a.W >> 1;
-    constexpr int NOUT = (TZ / 2) * (kTY / 2) * 8 * CO;
-    for (int i = threadIdx.x; i < NOUT; i += blockDim.x) {
-      const int co = i % CO, xp = (i / CO) % 8, cy = (i / (CO * 8)) % (kTY / 2), cz = i / (CO * 8 * (kTY / 2));
+    constexpr int XH = T::XO / 2, NOUT = (T::TZ / 2) * (kTY / 2) * XH * CB;
+    for (int i = threadIdx.x; i < NOUT; i += 32 * NW) {
+      const int co = i % CB, xp = (i / CB) % XH, cy = (i / (CB * XH)) % (kTY / 2), cz = i / (CB * XH * (kTY / 2));
       const int r00 = (2 * cz) * kTY + 2 * cy;
-      auto R = [&](int r) { return red[(r * 8 + xp) * CO + co]; };
-      const float v = (R(r00) + R(r00 + 1)) + (R(r00 + kTY) + R(r00 + kTY + 1));
+      auto Rd = [&](int r) { return red[(r * XH + xp) * CB + co]; };
+      const float v = (Rd(r00) + Rd(r00 + 1)) + (Rd(r00 + kTY) + Rd(r00 + kTY + 1));
       const int Z = (z0 >> 1) + cz, Y = (y0 >> 1) + cy, X = (x0 >> 1) + xp;
-      if (Z < Dc && Y < Hc && X < Wc) a.out_f[(((long long)Z * Hc + Y) * Wc + X) * CO + co] = v;
+      if (Z < Dc && Y < Hc && X < Wc) a.out_f[(((long long)Z * Hc + Y) * Wc + X) * CO + co0 + co] = v;
     }
     return;
   }
 
 #pragma unroll
-  for (int m = 0; m < MT; ++m) {
-    const int rr = warp * MT + m;
+  for (int r = 0; r < R; ++r) {
+    const int rr = warp * R + r;
     const int tz = rr / kTY, ty = rr - tz * kTY;
     const int z = z0 + tz, y = y0 + ty;
 #pragma unroll
-    for (int hf = 0; hf < 2; ++hf) {
-      const int x = x0 + (lane >> 2) + 8 * hf;
-      const bool ok = z < a.D && y < a.H && x < a.W;
-      const long long site = ((long long)z * a.H + y) * a.W + x;
-      float head = 0.f;
+    for (int m = 0; m < M; ++m)
 #pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        const int co = n * 8 + cq;
-        float v0 = acc[m][n][2 * hf], v1 = acc[m][n][2 * hf + 1];
-        if (EPI == EPI_RAW) {
-          if (ok) *reinterpret_cast<float2*>(a.out_f + site * CO + co) = make_float2(v0, v1);
-          continue;
+      for (int hf = 0; hf < 2; ++hf) {
+        const int x = x0 + site_x(m, (lane >> 2) + 8 * hf);
+        const bool ok = z < a.D && y < a.H && x < a.W;
+        const long long site = ((long long)z * a.H + y) * a.W + x;
+        float head = 0.f;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          const int co = co0 + n * 8 + cq;
+          float v0 = acc[r][m][n][2 * hf], v1 = acc[r][m][n][2 * hf + 1];
+          if (EPI == EPI_RAW) {
+            if (ok) *reinterpret_cast<float2*>(a.out_f + site * CO + co) = make_float2(v0, v1);
+            continue;
+          }
+          v0 += a.bias[co];
+          v1 += a.bias[co + 1];
+          if (a.skip && ok) {
+            const __nv_bfloat162 k = *reinterpret_cast<const __nv_bfloat162*>(a.skip + site * CO + co);
+            v0 += __low2float(k);
+            v1 += __high2float(k);
+          }
+          v0 = fmaxf(v0, 0.f);
+          v1 = fmaxf(v1, 0.f);
+          if (ok && a.out) *reinterpret_cast<uint32_t*>(a.out + site * CO + co) = pack_bf2(v0, v1);
+          if (EPI == EPI_HEAD) head += bfr(v0) * a.head_w[co] + bfr(v1) * a.head_w[co + 1];
         }
-        v0 += a.bias[co];
-        v1 += a.bias[co + 1];
-        if (a.skip && ok) {
-          const __nv_bfloat162 s = *reinterpret_cast<const __nv_bfloat162*>(a.skip + site * CO + co);
-          v0 += __low2float(s);
-          v1 += __high2float(s);
+        if (EPI == EPI_HEAD) {
+          head += __shfl_xor_sync(0xffffffffu, head, 1);
+          head += __shfl_xor_sync(0xffffffffu, head, 2);
+          if (ok && (lane & 3) == 0) a.out_f[site] = head + a.head_b[0];
         }
-        v0 = fmaxf(v0, 0.f);
-        v1 = fmaxf(v1, 0.f);
-        if (ok && a.out) *reinterpret_cast<uint32_t*>(a.out + site * CO + co) = pack_bf2(v0, v1);
-        if (EPI == EPI_HEAD) head += bfr(v0) * a.head_w[co] + bfr(v1) * a.head_w[co + 1];
       }
-      if (EPI == EPI_HEAD) {
-        head += __shfl_xor_sync(0xffffffffu, head, 1);
-        head += __shfl_xor_sync(0xffffffffu, head, 2);
-        if (ok && (lane & 3) == 0) a.out_f[site] = head + a.head_b[0];
-      }
-    }
   }
 }
 
@@ -350,16 +423,6 @@ template <int CO, int TZ>
 constexpr uint32_t tc_cols() {
   return TZ * CO <= 32 ? 32u : TZ * CO <= 64 ? 64u : TZ * CO <= 128 ? 128u : TZ * CO <= 256 ? 256u : 512u;
 }
-
-// 16-byte copy from global to shared memory; src_bytes = 0 writes zeros
-// (the source is not read).
-__device__ __forceinline__ void cp_async16_zfill(void* sdst, const void* gsrc, int src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(sdst)), "l"(gsrc), "r"(src_bytes)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Start the copies of tile `tile`'s halo into sh (the tile's output origin
 // from its index over (W/8, H/16, ceil(D/TZ))).
@@ -1165,11 +1228,29 @@ int ew_blocks(long long n, int sm) {
   return (int)std::max(1LL, std::min(b, (long long)sm * 8));
 }
 
-template <int CI, int CO, int MT, bool UP, int EPI>
-int conv_attr() {
-  constexpr int sm = conv_smem_bytes<CI, CO, MT, UP, EPI>();
-  NET_CUDA(cudaFuncSetAttribute(k_conv<CI, CO, MT, UP, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
+int conv_attr_t() {
+  using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
+  NET_CUDA(cudaFuncSetAttribute(k_conv<CI, CO, CB, S, R, NW, UP, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM));
   return HCA_OK;
+}
+
+// The block shape of a layer: output channels and x phases of a block, rows of
+// a warp, warps (and the phases where the lattice is too narrow for those).
+template <int CI, int CO, bool UP>
+struct ConvShape {
+  static constexpr int CB = CI == 64 ? (UP && CO == 32 ? 32 : 16) : CO == 64 ? 32 : CO;
+  static constexpr int S = CI == 16 ? (CO == 16 ? 4 : 2) : CI == 32 && CO == 16 ? 2 : 1;
+  static constexpr int R = CI == 16 && CO == 16 ? 2 : 1;
+  static constexpr int NW = 8;
+};
+
+template <int CI, int CO, bool UP, int EPI>
+int conv_attr() {
+  using C = ConvShape<CI, CO, UP>;
+  const int rc = conv_attr_t<CI, CO, C::CB, C::S, C::R, C::NW, UP, EPI>();
+  if (rc || C::S == 1) return rc;
+  return conv_attr_t<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>();
 }
 
 template <int CI, int CO, bool UP>
@@ -1181,19 +1262,19 @@ int wgrad_attr() {
 
 int set_attributes() {
   int rc = 0;
-  if ((rc = conv_attr<16, 16, 4, false, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<16, 32, 4, false, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<32, 64, 2, false, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<64, 64, 2, false, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<64, 64, 2, true, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<64, 32, 4, true, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<32, 16, 4, true, EPI_HEAD>())) return rc;
-  if ((rc = conv_attr<16, 32, 4, false, EPI_DOWN>())) return rc;
-  if ((rc = conv_attr<32, 64, 2, false, EPI_DOWN>())) return rc;
-  if ((rc = conv_attr<64, 64, 2, false, EPI_DOWN>())) return rc;
-  if ((rc = conv_attr<64, 64, 2, false, EPI_RAW>())) return rc;
-  if ((rc = conv_attr<64, 32, 4, false, EPI_RAW>())) return rc;
-  if ((rc = conv_attr<32, 16, 4, false, EPI_RAW>())) return rc;
+  if ((rc = conv_attr<16, 16, false, EPI_FWD>())) return rc;
+  if ((rc = conv_attr<16, 32, false, EPI_FWD>())) return rc;
+  if ((rc = conv_attr<32, 64, false, EPI_FWD>())) return rc;
+  if ((rc = conv_attr<64, 64, false, EPI_FWD>())) return rc;
+  if ((rc = conv_attr<64, 64, true, EPI_FWD>())) return rc;
+  if ((rc = conv_attr<64, 32, true, EPI_FWD>())) return rc;
+  if ((rc = conv_attr<32, 16, true, EPI_HEAD>())) return rc;
+  if ((rc = conv_attr<16, 32, false, EPI_DOWN>())) return rc;
+  if ((rc = conv_attr<32, 64, false, EPI_DOWN>())) return rc;
+  if ((rc = conv_attr<64, 64, false, EPI_DOWN>())) return rc;
+  if ((rc = conv_attr<64, 64, false, EPI_RAW>())) return rc;
+  if ((rc = conv_attr<64, 32, false, EPI_RAW>())) return rc;
+  if ((rc = conv_attr<32, 16, false, EPI_RAW>())) return rc;
   if ((rc = wgrad_attr<16, 16, false>())) return rc;
   if ((rc = wgrad_attr<16, 32, false>())) return rc;
   if ((rc = wgrad_attr<32, 64, false>())) return rc;
@@ -1247,8 +1328,15 @@ void conv_tc(cudaStream_t s, int* status, const bf16* in, const bf16* w, const f
   k_conv_tc<CI, CO, TZ, UP, EPI><<<grid, 128, tc_conv_smem_bytes<CI, CO, TZ>(), s>>>(a, status);
 }
 
+template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
+void conv_launch(cudaStream_t s, const ConvArgs& a) {
+  using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
+  const dim3 grid((a.W + T::XO - 1) / T::XO * (CO / CB), (a.H + kTY - 1) / kTY, (a.D + T::TZ - 1) / T::TZ);
+  k_conv<CI, CO, CB, S, R, NW, UP, EPI><<<grid, 32 * NW, T::SMEM, s>>>(a);
+}
+
 // One convolution launch; (D, H, W) is the output lattice.
-template <int CI, int CO, int MT, bool UP, int EPI>
+template <int CI, int CO, bool UP, int EPI>
 void conv(cudaStream_t s, const bf16* in, const bf16* w, const float* bias, const bf16* skip, bf16* out,
           float* out_f, const float* hw, const float* hb, int D, int H, int W) {
   ConvArgs a;
@@ -1266,8 +1354,13 @@ void conv(cudaStream_t s, const bf16* in, const bf16* w, const float* bias, cons
   a.Di = UP ? D / 2 : D;
   a.Hi = UP ? H / 2 : H;
   a.Wi = UP ? W / 2 : W;
-  const dim3 grid((W + kRowX - 1) / kRowX, (H + kTY - 1) / kTY, (D + MT - 1) / MT);
-  k_conv<CI, CO, MT, UP, EPI><<<grid, kThreads, conv_smem_bytes<CI, CO, MT, UP, EPI>(), s>>>(a);
+  using C = ConvShape<CI, CO, UP>;
+  // interleaved tiles cover 16 S (upsampled: 32 S) sites of x: taken where
+  // rounding the row up to that costs at most an eighth
+  const int one = UP ? 32 : 16, wide = one * C::S;
+  const int pad_w = (W + wide - 1) / wide * wide, pad_1 = (W + one - 1) / one * one;
+  if (C::S > 1 && 8 * pad_w <= 9 * pad_1) conv_launch<CI, CO, C::CB, C::S, C::R, C::NW, UP, EPI>(s, a);
+  else conv_launch<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>(s, a);
 }
 
 // Weight gradient of one layer into grads[w_off ...]; (D, H, W) = output lattice.
@@ -1325,21 +1418,21 @@ void forward(hca_net* n, cudaStream_t s, bool keep_d0) {
     conv_tc<16, 16, 4, false, EPI_FWD>(s, n->tc_status, n->x, Wq(n, 0), Bias(n, 0), nullptr, n->e0, nullptr, nullptr,
                                        nullptr, D[0], H[0], W[0]);
   else
-    conv<16, 16, 4, false, EPI_FWD>(s, n->x, Wq(n, 0), Bias(n, 0), nullptr, n->e0, nullptr, nullptr, nullptr, D[0],
+    conv<16, 16, false, EPI_FWD>(s, n->x, Wq(n, 0), Bias(n, 0), nullptr, n->e0, nullptr, nullptr, nullptr, D[0],
                                     H[0], W[0]);
   pool<16>(n, s, n->e0, n->p0, 0);
-  conv<16, 32, 4, false, EPI_FWD>(s, n->p0, Wq(n, 1), Bias(n, 1), nullptr, n->e1, nullptr, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<16, 32, false, EPI_FWD>(s, n->p0, Wq(n, 1), Bias(n, 1), nullptr, n->e1, nullptr, nullptr, nullptr, D[1], H[1], W[1]);
   pool<32>(n, s, n->e1, n->p1, 1);
-  conv<32, 64, 2, false, EPI_FWD>(s, n->p1, Wq(n, 2), Bias(n, 2), nullptr, n->e2, nullptr, nullptr, nullptr, D[2], H[2], W[2]);
+  conv<32, 64, false, EPI_FWD>(s, n->p1, Wq(n, 2), Bias(n, 2), nullptr, n->e2, nullptr, nullptr, nullptr, D[2], H[2], W[2]);
   pool<64>(n, s, n->e2, n->p2, 2);
-  conv<64, 64, 2, false, EPI_FWD>(s, n->p2, Wq(n, 3), Bias(n, 3), nullptr, n->e3, nullptr, nullptr, nullptr, D[3], H[3], W[3]);
-  conv<64, 64, 2, true, EPI_FWD>(s, n->e3, Wq(n, 4), Bias(n, 4), n->e2, n->d2, nullptr, nullptr, nullptr, D[2], H[2], W[2]);
-  conv<64, 32, 4, true, EPI_FWD>(s, n->d2, Wq(n, 5), Bias(n, 5), n->e1, n->d1, nullptr, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<64, 64, false, EPI_FWD>(s, n->p2, Wq(n, 3), Bias(n, 3), nullptr, n->e3, nullptr, nullptr, nullptr, D[3], H[3], W[3]);
+  conv<64, 64, true, EPI_FWD>(s, n->e3, Wq(n, 4), Bias(n, 4), n->e2, n->d2, nullptr, nullptr, nullptr, D[2], H[2], W[2]);
+  conv<64, 32, true, EPI_FWD>(s, n->d2, Wq(n, 5), Bias(n, 5), n->e1, n->d1, nullptr, nullptr, nullptr, D[1], H[1], W[1]);
   if (n->use_tc)
     conv_tc<32, 16, 4, true, EPI_HEAD>(s, n->tc_status, n->d1, Wq(n, 6), Bias(n, 6), n->e0, keep_d0 ? n->d0 : nullptr,
                                        n->out, n->params + n->L.hw_off, n->params + n->L.hb_off, D[0], H[0], W[0]);
   else
-    conv<32, 16, 4, true, EPI_HEAD>(s, n->d1, Wq(n, 6), Bias(n, 6), n->e0, keep_d0 ? n->d0 : nullptr, n->out,
+    conv<32, 16, true, EPI_HEAD>(s, n->d1, Wq(n, 6), Bias(n, 6), n->e0, keep_d0 ? n->d0 : nullptr, n->out,
                                     n->params + n->L.hw_off, n->params + n->L.hb_off, D[0], H[0], W[0]);
 }
 
@@ -1361,27 +1454,27 @@ void backward(hca_net* n, cudaStream_t s, const float* target, const float* gbuf
   }
   // dec0: input up(d1), output gradient g0
   wgrad<32, 16, true>(n, s, n->d1, n->g0, D[0], H[0], W[0], n->grads + L.w_off[6]);
-  conv<16, 32, 4, false, EPI_DOWN>(s, n->g0, Wt(n, 6), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[0], H[0], W[0]);
+  conv<16, 32, false, EPI_DOWN>(s, n->g0, Wt(n, 6), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[0], H[0], W[0]);
   combine<32, 0>(n, s, n->graw, n->d1, nullptr, n->g1, 1, 5);
   // dec1: input up(d2)
   wgrad<64, 32, true>(n, s, n->d2, n->g1, D[1], H[1], W[1], n->grads + L.w_off[5]);
-  conv<32, 64, 2, false, EPI_DOWN>(s, n->g1, Wt(n, 5), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<32, 64, false, EPI_DOWN>(s, n->g1, Wt(n, 5), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[1], H[1], W[1]);
   combine<64, 0>(n, s, n->graw, n->d2, nullptr, n->g2, 2, 4);
   // dec2: input up(e3)
   wgrad<64, 64, true>(n, s, n->e3, n->g2, D[2], H[2], W[2], n->grads + L.w_off[4]);
-  conv<64, 64, 2, false, EPI_DOWN>(s, n->g2, Wt(n, 4), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[2], H[2], W[2]);
+  conv<64, 64, false, EPI_DOWN>(s, n->g2, Wt(n, 4), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[2], H[2], W[2]);
   combine<64, 0>(n, s, n->graw, n->e3, nullptr, n->g3, 3, 3);
   // enc3: input p2
   wgrad<64, 64, false>(n, s, n->p2, n->g3, D[3], H[3], W[3], n->grads + L.w_off[3]);
-  conv<64, 64, 2, false, EPI_RAW>(s, n->g3, Wt(n, 3), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[3], H[3], W[3]);
+  conv<64, 64, false, EPI_RAW>(s, n->g3, Wt(n, 3), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[3], H[3], W[3]);
   combine<64, 1>(n, s, n->graw, n->e2, n->g2, n->ge2, 2, 2);
   // enc2: input p1
   wgrad<32, 64, false>(n, s, n->p1, n->ge2, D[2], H[2], W[2], n->grads + L.w_off[2]);
-  conv<64, 32, 4, false, EPI_RAW>(s, n->ge2, Wt(n, 2), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[2], H[2], W[2]);
+  conv<64, 32, false, EPI_RAW>(s, n->ge2, Wt(n, 2), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[2], H[2], W[2]);
   combine<32, 1>(n, s, n->graw, n->e1, n->g1, n->ge1, 1, 1);
   // enc1: input p0
   wgrad<16, 32, false>(n, s, n->p0, n->ge1, D[1], H[1], W[1], n->grads + L.w_off[1]);
-  conv<32, 16, 4, false, EPI_RAW>(s, n->ge1, Wt(n, 1), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<32, 16, false, EPI_RAW>(s, n->ge1, Wt(n, 1), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[1], H[1], W[1]);
   combine<16, 1>(n, s, n->graw, n->e0, n->g0, n->ge0, 0, 0);
   // enc0: input x
   wgrad<16, 16, false>(n, s, n->x, n->ge0, D[0], H[0], W[0], n->grads + L.w_off[0]);
