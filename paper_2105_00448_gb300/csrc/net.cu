@@ -19,6 +19,7 @@
 // 2x upsampling of the decoder is folded into the halo gather; the sum over
 // the 2x2x2 children that its gradient needs is folded into the epilogue.
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -178,59 +179,89 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // upsampled form: two per phase, one per output parity), so a tap's shift in x
 // turns one tile's rows into another's: the fragments of S + 2 phases serve all
 // three taps of the row.  The halo is staged with the phases apart
-// ([row][phase][j]), which keeps a fragment's rows consecutive.
+// ([phase][row][j], a tensor copy per phase: every S-th site), which keeps a
+// fragment's rows consecutive; the copies' swizzle modes are chunk_pos's layout.
 template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
 struct ConvTile {
   static constexpr int ROWS = NW * R, TZ = ROWS / kTY, XO = (UP ? 32 : 16) * S;
   static constexpr int M = (UP ? 2 : 1) * S;   // M tiles of a row
-  static constexpr int HZ = UP ? TZ / 2 + 2 : TZ + 2, HY = UP ? kTY / 2 + 2 : kTY + 2, HX = 16 * S + 2;
-  static constexpr int LP = (HX + S - 1) / S;  // sites of a phase
-  static constexpr int HALO = HZ * HY * S * LP * CI * 2;
-  static constexpr int RED = EPI == 3 ? ROWS * (XO / 2) * CB * 4 : 0;
+  static constexpr int HZ = UP ? TZ / 2 + 2 : TZ + 2, HY = UP ? kTY / 2 + 2 : kTY + 2, LP = 18;   // sites of a phase row
+  static constexpr int PHASE = HZ * HY * LP;   // sites of a phase
+  static constexpr int HALO = S * PHASE * CI * 2;
+  static constexpr int RED = EPI == 3 ? (ROWS * (XO / 2) * CB * 4 + 1023) / 1024 * 1024 : 0;
   static constexpr int WPLANE = 9 * CB * CI * 2;
-  static constexpr int SMEM = (HALO > RED ? HALO : RED) + 2 * WPLANE;
+  static constexpr int SMEM = (HALO > RED ? HALO : RED) + 2 * WPLANE + 16;   // (and two barriers)
   static constexpr int PER_SM = 232448 / (SMEM + 1024);
-  static constexpr int MIN_BLOCKS = PER_SM * NW > 16 ? 16 / NW : PER_SM;   // (128 registers at least)
+  // blocks of 8 warps the accumulators and shared fragments leave registers for
+  static constexpr int LIVE = R * M * (CB / 8) * 4 + (S > 1 || UP ? R * (S + 2) * (CI / 16) * 4 : 4);
+  static constexpr int FIT = LIVE > 64 ? 2 : LIVE > 24 ? 3 : 4;
+  static constexpr int MIN_BLOCKS = PER_SM < FIT ? PER_SM : FIT;
+  static_assert(PHASE % 8 == 0, "a phase starts where the swizzle pattern does");
   static_assert(TZ >= 2 && TZ % 2 == 0 && CB % 16 == 0 && CO % CB == 0, "tile shape");
   static_assert(!(UP && EPI == 3) && (EPI != 1 || CB == CO), "epilogue");
 };
 
+// The tensor maps of a convolution's inputs: the activations by phase of x
+// (every S-th site; box: a block's halo rows of one phase) and the weights
+// (box: a plane of nine taps for CB output channels).
+struct ConvMaps {
+  CUtensorMap in[4], w;
+};
+
+// The waits for the copies are bounded; a timeout is recorded in *status and
+// ends the block.
+constexpr int kConvWaitLimit = 1 << 20;
+
+__device__ __forceinline__ void tma_box_4d(uint32_t dst, const CUtensorMap* map, int c1, int c2, int c3, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(
+          dst),
+      "l"((unsigned long long)map), "r"(0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_box_3d(uint32_t dst, const CUtensorMap* map, int c1, int c2, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"((unsigned long long)map), "r"(0), "r"(c1), "r"(c2), "r"(bar)
+      : "memory");
+}
+
 template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
-__global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, EPI>::MIN_BLOCKS)) k_conv(const ConvArgs a) {
+__global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, EPI>::MIN_BLOCKS))
+    k_conv(const ConvArgs a, const __grid_constant__ ConvMaps maps, int* status) {
   using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
   constexpr int NT = CB / 8;        // n8 tiles
   constexpr int KC = CI / 16;       // k16 steps per tap
-  constexpr int NCH = CI / 8;
   constexpr int M = T::M, NQ = S + 2;
   constexpr bool HOLD = S > 1 || UP;   // fragments shared by the taps of a row
-  extern __shared__ __align__(128) char smem[];
+  extern __shared__ __align__(1024) char smem[];
   char* sh = smem;
-  char* sw = smem + T::SMEM - 2 * T::WPLANE;
+  char* sw = smem + T::SMEM - 16 - 2 * T::WPLANE;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + T::SMEM - 16);
   const int cg = blockIdx.x % (CO / CB), co0 = cg * CB;
   const int z0 = blockIdx.z * T::TZ, y0 = blockIdx.y * kTY, x0 = (int)(blockIdx.x / (CO / CB)) * T::XO;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // the halo and the first plane of taps; the next plane follows while one is used
-  {
-    const int oz = UP ? (z0 >> 1) - 1 : z0 - 1, oy = UP ? (y0 >> 1) - 1 : y0 - 1, ox = UP ? (x0 >> 1) - 1 : x0 - 1;
-    for (int i = threadIdx.x; i < T::HZ * T::HY * T::HX * NCH; i += 32 * NW) {
-      const int h = i / NCH, j = i - h * NCH;
-      const int hx = h % T::HX, row = h / T::HX;
-      const int gz = oz + row / T::HY, gy = oy + row % T::HY, gx = ox + hx;
-      const bool in = gz >= 0 && gz < a.Di && gy >= 0 && gy < a.Hi && gx >= 0 && gx < a.Wi;
-      const bf16* src = in ? a.in + (((long long)gz * a.Hi + gy) * a.Wi + gx) * CI + 8 * j : a.in;
-      cp_async16_zfill(sh + 16 * chunk_pos<CI>((row * S + hx % S) * T::LP + hx / S, j), src, in ? 16 : 0);
-    }
-  }
+  // the halo and the first two planes of taps; the third follows the first
   auto stage_w = [&](int plane) {
-    char* dst = sw + (plane & 1) * T::WPLANE;
-    const bf16* wp = a.w + ((long long)plane * 9 * CO + co0) * CI;
-    for (int i = threadIdx.x; i < 9 * CB * NCH; i += 32 * NW) {
-      const int r = i / NCH, j = i - r * NCH;
-      cp_async16_zfill(dst + 16 * chunk_pos<CI>(r, j), wp + ((long long)(r / CB) * CO + r % CB) * CI + 8 * j, 16);
-    }
-    cp_async_commit();
+    tma_box_3d(smem_u32(sw) + (plane & 1) * T::WPLANE, &maps.w, co0, 9 * plane, smem_u32(&bar[plane & 1]));
   };
-  stage_w(0);
+  auto expect = [&](int b, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&bar[b])), "r"(bytes) : "memory");
+  };
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&bar[0], 1);
+    tc::mbar_init(&bar[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    const int oz = UP ? (z0 >> 1) - 1 : z0 - 1, oy = UP ? (y0 >> 1) - 1 : y0 - 1, ox = (UP ? x0 >> 1 : x0) / S - 1;
+    expect(0, (uint32_t)(T::HALO + T::WPLANE));
+    for (int p = 0; p < S; ++p)
+      tma_box_4d(smem_u32(sh) + p * (T::PHASE * CI * 2), &maps.in[p], ox, oy, oz, smem_u32(&bar[0]));
+    stage_w(0);
+    expect(1, (uint32_t)T::WPLANE);
+    stage_w(1);
+  }
+  __syncthreads();
 
   float acc[R][M][NT][4];
 #pragma unroll
@@ -250,9 +281,22 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
   // taps in order (dz, dy, dx), channels within a tap: the accumulation order
 #pragma unroll 1
   for (int dz = -1; dz <= 1; ++dz) {
-    cp_async_wait<0>();
-    __syncthreads();   // this plane's taps are there, the plane before is consumed
-    if (dz < 1) stage_w(dz + 2);
+    // this plane's taps are there (the same in every thread), the plane before is consumed
+    const bool ok = tc::mbar_wait(&bar[(dz + 1) & 1], dz == 1 ? 1u : 0u, kConvWaitLimit);
+    if (!__syncthreads_and(ok)) {
+      if (threadIdx.x == 0) {
+        *(volatile int*)status = 1;
+        // the copies in flight land before the block's shared memory is released
+        (void)tc::mbar_wait(&bar[0], dz == 1 ? 1u : 0u, kConvWaitLimit);
+        (void)tc::mbar_wait(&bar[1], 0u, kConvWaitLimit);
+      }
+      __syncthreads();
+      return;
+    }
+    if (dz == 0 && threadIdx.x == 0) {
+      expect(0, (uint32_t)T::WPLANE);
+      stage_w(2);
+    }
     const uint32_t swb = smem_u32(sw) + ((dz + 1) & 1) * T::WPLANE;
 #pragma unroll 1
     for (int dy = -1; dy <= 1; ++dy) {
@@ -260,8 +304,7 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int rr = warp * R + r, tz = rr / kTY, ty = rr - tz * kTY;
-        hrow[r] = (UP ? (((tz + dz) >> 1) + 1) * T::HY + (((ty + dy) >> 1) + 1) : (tz + dz + 1) * T::HY + (ty + dy + 1)) *
-                  (S * T::LP);
+        hrow[r] = (UP ? (((tz + dz) >> 1) + 1) * T::HY + (((ty + dy) >> 1) + 1) : (tz + dz + 1) * T::HY + (ty + dy + 1)) * T::LP;
       }
       uint32_t af[HOLD ? R : 1][HOLD ? NQ : 1][HOLD ? KC : 1][4];
       if (HOLD) {
@@ -271,7 +314,8 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
           for (int p = 0; p < NQ; ++p)
 #pragma unroll
             for (int kc = 0; kc < KC; ++kc)
-              ldsm_x4(shb + 16 * chunk_pos<CI>(hrow[r] + (p % S) * T::LP + p / S + a_x, 2 * kc + a_j), af[r][p][kc]);
+              ldsm_x4(shb + 16 * chunk_pos<CI>(((p + S - 1) % S) * T::PHASE + hrow[r] + (p + S - 1) / S + a_x, 2 * kc + a_j),
+                      af[r][p][kc]);
       }
 #pragma unroll
       for (int dx = -1; dx <= 1; ++dx)
@@ -501,7 +545,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(const ConvArgs a, int* status) 
       tc::commit(mbar);
     }
     const bool done = tc::mbar_wait(mbar, (uint32_t)(it & 1), 1 << 22);
-    if (!done && (t & 31) == 0) atomicExch(status, 1);
+    if (!done && (t & 31) == 0) *(volatile int*)status = 1;
     alive = __syncthreads_and(done) != 0;   // one decision for the whole block
     tc::fence_after();
     if (alive) {
@@ -1131,7 +1175,8 @@ __global__ void __launch_bounds__(kEwThreads) k_ws_norms(FeatureArgs f, const T*
   if (threadIdx.x < 3) part[blockIdx.x * 3 + threadIdx.x] = sb[threadIdx.x][0];
 }
 
-__global__ void k_ws_decide(const double* __restrict__ part, int nb, int always, WsResult* __restrict__ res) {
+__global__ void k_ws_decide(const double* __restrict__ part, int nb, int always, const int* status,
+                            WsResult* __restrict__ res) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double s[3] = {0.0, 0.0, 0.0};
   for (int b = 0; b < nb; ++b)
@@ -1139,7 +1184,8 @@ __global__ void k_ws_decide(const double* __restrict__ part, int nb, int always,
   const double bn = s[2] > 0.0 ? sqrt(s[2]) : 1.0;
   res->r0_prev = sqrt(s[0]) / bn;
   res->r0_learned = sqrt(s[1]) / bn;
-  res->used = always || ((s[1] == s[1]) && s[1] < s[0]) ? 1 : 0;
+  // (no guess from a pass that did not complete)
+  res->used = !*(volatile const int*)status && (always || ((s[1] == s[1]) && s[1] < s[0])) ? 1 : 0;
 }
 
 template <typename T>
@@ -1189,10 +1235,13 @@ struct hca_net {
   long long* bias_index = nullptr;   // device: 7 x 64 destinations of the bias partials
   bool trainable = false;
   // the full-resolution layers (enc0, dec0 + head) of the forward pass on the
-  // fifth-generation tensor cores (k_conv_tc); tc_status: set by a kernel whose
-  // completion wait timed out
+  // fifth-generation tensor cores (k_conv_tc)
   bool use_tc = false;
-  int* tc_status = nullptr;
+  // tensor maps of the convolutions' inputs (the net's own arrays): the seven
+  // layers, then the input gradients of dec0, dec1, dec2, enc3, enc2, enc1
+  ConvMaps maps[13];
+  // pinned host memory: set by a kernel whose bounded wait timed out
+  int* status = nullptr;
 };
 
 namespace {
@@ -1232,7 +1281,29 @@ template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
 int conv_attr_t() {
   using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
   NET_CUDA(cudaFuncSetAttribute(k_conv<CI, CO, CB, S, R, NW, UP, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM));
+  NET_CUDA(cudaFuncSetAttribute(k_conv<CI, CO, CB, S, R, NW, UP, EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   return HCA_OK;
+}
+
+// A tensor map of BF16 values with the channel chunks swizzled as chunk_pos
+// does (rank 3 or 4, rows of `ci` channels); false if the driver refuses it.
+bool bf16_map(CUtensorMap* m, const void* base, int rank, int ci, const cuuint64_t* dims, const cuuint64_t* strides,
+              const cuuint32_t* box) {
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess || !fn) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  const CUtensorMapSwizzle sw = ci == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : ci == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+  return ((Encode)fn)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box, es,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // The block shape of a layer: output channels and x phases of a block, rows of
@@ -1328,39 +1399,66 @@ void conv_tc(cudaStream_t s, int* status, const bf16* in, const bf16* w, const f
   k_conv_tc<CI, CO, TZ, UP, EPI><<<grid, 128, tc_conv_smem_bytes<CI, CO, TZ>(), s>>>(a, status);
 }
 
-template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
-void conv_launch(cudaStream_t s, const ConvArgs& a) {
-  using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
-  const dim3 grid((a.W + T::XO - 1) / T::XO * (CO / CB), (a.H + kTY - 1) / kTY, (a.D + T::TZ - 1) / T::TZ);
-  k_conv<CI, CO, CB, S, R, NW, UP, EPI><<<grid, 32 * NW, T::SMEM, s>>>(a);
+// Interleaved tiles cover 16 S (upsampled: 32 S) sites of x: taken where
+// rounding the row up to that costs at most an eighth.
+template <int CI, int CO, bool UP>
+bool conv_wide(int W) {
+  constexpr int S = ConvShape<CI, CO, UP>::S, one = UP ? 32 : 16, wide = one * S;
+  const int pad_w = (W + wide - 1) / wide * wide, pad_1 = (W + one - 1) / one * one;
+  return S > 1 && 8 * pad_w <= 9 * pad_1;
 }
 
-// One convolution launch; (D, H, W) is the output lattice.
+template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
+bool conv_maps(ConvMaps* m, const bf16* in, const bf16* w, int Di, int Hi, int Wi) {
+  using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
+  const cuuint64_t row = (cuuint64_t)CI * 2;
+  for (int p = 0; p < S; ++p) {   // (the lattice's dimensions are multiples of 8 at level 0, of S at the layer's)
+    const cuuint64_t dims[4] = {CI, (cuuint64_t)(Wi / S), (cuuint64_t)Hi, (cuuint64_t)Di};
+    const cuuint64_t strides[3] = {S * row, Wi * row, (cuuint64_t)Wi * Hi * row};
+    const cuuint32_t box[4] = {CI, (cuuint32_t)T::LP, (cuuint32_t)T::HY, (cuuint32_t)T::HZ};
+    if (!bf16_map(&m->in[p], in + (size_t)p * CI, 4, CI, dims, strides, box)) return false;
+  }
+  const cuuint64_t wd[3] = {CI, CO, 27}, ws[2] = {row, CO * row};
+  const cuuint32_t wb[3] = {CI, CB, 9};
+  return bf16_map(&m->w, w, 3, CI, wd, ws, wb);
+}
+
+// The maps of the convolution whose output lattice is level lvl.
 template <int CI, int CO, bool UP, int EPI>
-void conv(cudaStream_t s, const bf16* in, const bf16* w, const float* bias, const bf16* skip, bf16* out,
-          float* out_f, const float* hw, const float* hb, int D, int H, int W) {
-  ConvArgs a;
-  a.in = in;
-  a.w = w;
+bool conv_prepare(hca_net* n, int slot, const bf16* in, const bf16* w, int lvl) {
+  using C = ConvShape<CI, CO, UP>;
+  const int li = lvl + UP;   // the input's level
+  if (conv_wide<CI, CO, UP>(n->Lw[lvl]))
+    return conv_maps<CI, CO, C::CB, C::S, C::R, C::NW, UP, EPI>(&n->maps[slot], in, w, n->Ld[li], n->Lh[li], n->Lw[li]);
+  return conv_maps<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>(&n->maps[slot], in, w, n->Ld[li], n->Lh[li], n->Lw[li]);
+}
+
+template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
+void conv_launch(cudaStream_t s, const ConvArgs& a, const ConvMaps& maps, int* status) {
+  using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
+  const dim3 grid((a.W + T::XO - 1) / T::XO * (CO / CB), (a.H + kTY - 1) / kTY, (a.D + T::TZ - 1) / T::TZ);
+  k_conv<CI, CO, CB, S, R, NW, UP, EPI><<<grid, 32 * NW, T::SMEM, s>>>(a, maps, status);
+}
+
+// One convolution launch on the inputs of maps[slot]; the output lattice is level lvl.
+template <int CI, int CO, bool UP, int EPI>
+void conv(hca_net* n, cudaStream_t s, int slot, const float* bias, const bf16* skip, bf16* out, float* out_f,
+          const float* hw, const float* hb, int lvl) {
+  ConvArgs a{};
   a.bias = bias;
   a.skip = skip;
   a.out = out;
   a.out_f = out_f;
   a.head_w = hw;
   a.head_b = hb;
-  a.D = D;
-  a.H = H;
-  a.W = W;
-  a.Di = UP ? D / 2 : D;
-  a.Hi = UP ? H / 2 : H;
-  a.Wi = UP ? W / 2 : W;
+  a.D = n->Ld[lvl];
+  a.H = n->Lh[lvl];
+  a.W = n->Lw[lvl];
   using C = ConvShape<CI, CO, UP>;
-  // interleaved tiles cover 16 S (upsampled: 32 S) sites of x: taken where
-  // rounding the row up to that costs at most an eighth
-  const int one = UP ? 32 : 16, wide = one * C::S;
-  const int pad_w = (W + wide - 1) / wide * wide, pad_1 = (W + one - 1) / one * one;
-  if (C::S > 1 && 8 * pad_w <= 9 * pad_1) conv_launch<CI, CO, C::CB, C::S, C::R, C::NW, UP, EPI>(s, a);
-  else conv_launch<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>(s, a);
+  if (conv_wide<CI, CO, UP>(a.W))
+    conv_launch<CI, CO, C::CB, C::S, C::R, C::NW, UP, EPI>(s, a, n->maps[slot], n->status);
+  else
+    conv_launch<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>(s, a, n->maps[slot], n->status);
 }
 
 // Weight gradient of one layer into grads[w_off ...]; (D, H, W) = output lattice.
@@ -1409,31 +1507,47 @@ const bf16* Wq(hca_net* n, int l) { return n->wq + n->L.wq_off[l]; }
 const bf16* Wt(hca_net* n, int l) { return n->wt + n->L.wq_off[l]; }
 const float* Bias(hca_net* n, int l) { return n->params + n->L.b_off[l]; }
 
+// The tensor maps of every convolution (the net's arrays are allocated).
+bool prepare_convs(hca_net* n) {
+  const bool fwd = conv_prepare<16, 16, false, EPI_FWD>(n, 0, n->x, Wq(n, 0), 0) &&
+                   conv_prepare<16, 32, false, EPI_FWD>(n, 1, n->p0, Wq(n, 1), 1) &&
+                   conv_prepare<32, 64, false, EPI_FWD>(n, 2, n->p1, Wq(n, 2), 2) &&
+                   conv_prepare<64, 64, false, EPI_FWD>(n, 3, n->p2, Wq(n, 3), 3) &&
+                   conv_prepare<64, 64, true, EPI_FWD>(n, 4, n->e3, Wq(n, 4), 2) &&
+                   conv_prepare<64, 32, true, EPI_FWD>(n, 5, n->d2, Wq(n, 5), 1) &&
+                   conv_prepare<32, 16, true, EPI_HEAD>(n, 6, n->d1, Wq(n, 6), 0);
+  if (!fwd || !n->trainable) return fwd;
+  return conv_prepare<16, 32, false, EPI_DOWN>(n, 7, n->g0, Wt(n, 6), 0) &&
+         conv_prepare<32, 64, false, EPI_DOWN>(n, 8, n->g1, Wt(n, 5), 1) &&
+         conv_prepare<64, 64, false, EPI_DOWN>(n, 9, n->g2, Wt(n, 4), 2) &&
+         conv_prepare<64, 64, false, EPI_RAW>(n, 10, n->g3, Wt(n, 3), 3) &&
+         conv_prepare<64, 32, false, EPI_RAW>(n, 11, n->ge2, Wt(n, 2), 2) &&
+         conv_prepare<32, 16, false, EPI_RAW>(n, 12, n->ge1, Wt(n, 1), 1);
+}
+
 // Forward pass from n->x; with keep_d0 the last activation is stored (training).
 void forward(hca_net* n, cudaStream_t s, bool keep_d0) {
   const int* D = n->Ld;
   const int* H = n->Lh;
   const int* W = n->Lw;
   if (n->use_tc)
-    conv_tc<16, 16, 4, false, EPI_FWD>(s, n->tc_status, n->x, Wq(n, 0), Bias(n, 0), nullptr, n->e0, nullptr, nullptr,
+    conv_tc<16, 16, 4, false, EPI_FWD>(s, n->status, n->x, Wq(n, 0), Bias(n, 0), nullptr, n->e0, nullptr, nullptr,
                                        nullptr, D[0], H[0], W[0]);
   else
-    conv<16, 16, false, EPI_FWD>(s, n->x, Wq(n, 0), Bias(n, 0), nullptr, n->e0, nullptr, nullptr, nullptr, D[0],
-                                    H[0], W[0]);
+    conv<16, 16, false, EPI_FWD>(n, s, 0, Bias(n, 0), nullptr, n->e0, nullptr, nullptr, nullptr, 0);
   pool<16>(n, s, n->e0, n->p0, 0);
-  conv<16, 32, false, EPI_FWD>(s, n->p0, Wq(n, 1), Bias(n, 1), nullptr, n->e1, nullptr, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<16, 32, false, EPI_FWD>(n, s, 1, Bias(n, 1), nullptr, n->e1, nullptr, nullptr, nullptr, 1);
   pool<32>(n, s, n->e1, n->p1, 1);
-  conv<32, 64, false, EPI_FWD>(s, n->p1, Wq(n, 2), Bias(n, 2), nullptr, n->e2, nullptr, nullptr, nullptr, D[2], H[2], W[2]);
+  conv<32, 64, false, EPI_FWD>(n, s, 2, Bias(n, 2), nullptr, n->e2, nullptr, nullptr, nullptr, 2);
   pool<64>(n, s, n->e2, n->p2, 2);
-  conv<64, 64, false, EPI_FWD>(s, n->p2, Wq(n, 3), Bias(n, 3), nullptr, n->e3, nullptr, nullptr, nullptr, D[3], H[3], W[3]);
-  conv<64, 64, true, EPI_FWD>(s, n->e3, Wq(n, 4), Bias(n, 4), n->e2, n->d2, nullptr, nullptr, nullptr, D[2], H[2], W[2]);
-  conv<64, 32, true, EPI_FWD>(s, n->d2, Wq(n, 5), Bias(n, 5), n->e1, n->d1, nullptr, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<64, 64, false, EPI_FWD>(n, s, 3, Bias(n, 3), nullptr, n->e3, nullptr, nullptr, nullptr, 3);
+  conv<64, 64, true, EPI_FWD>(n, s, 4, Bias(n, 4), n->e2, n->d2, nullptr, nullptr, nullptr, 2);
+  conv<64, 32, true, EPI_FWD>(n, s, 5, Bias(n, 5), n->e1, n->d1, nullptr, nullptr, nullptr, 1);
   if (n->use_tc)
-    conv_tc<32, 16, 4, true, EPI_HEAD>(s, n->tc_status, n->d1, Wq(n, 6), Bias(n, 6), n->e0, keep_d0 ? n->d0 : nullptr,
+    conv_tc<32, 16, 4, true, EPI_HEAD>(s, n->status, n->d1, Wq(n, 6), Bias(n, 6), n->e0, keep_d0 ? n->d0 : nullptr,
                                        n->out, n->params + n->L.hw_off, n->params + n->L.hb_off, D[0], H[0], W[0]);
   else
-    conv<32, 16, true, EPI_HEAD>(s, n->d1, Wq(n, 6), Bias(n, 6), n->e0, keep_d0 ? n->d0 : nullptr, n->out,
-                                    n->params + n->L.hw_off, n->params + n->L.hb_off, D[0], H[0], W[0]);
+    conv<32, 16, true, EPI_HEAD>(n, s, 6, Bias(n, 6), n->e0, keep_d0 ? n->d0 : nullptr, n->out, n->params + n->L.hw_off, n->params + n->L.hb_off, 0);
 }
 
 // Backward pass after forward(keep_d0 = true): the MSE loss against target,
@@ -1454,27 +1568,27 @@ void backward(hca_net* n, cudaStream_t s, const float* target, const float* gbuf
   }
   // dec0: input up(d1), output gradient g0
   wgrad<32, 16, true>(n, s, n->d1, n->g0, D[0], H[0], W[0], n->grads + L.w_off[6]);
-  conv<16, 32, false, EPI_DOWN>(s, n->g0, Wt(n, 6), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[0], H[0], W[0]);
+  conv<16, 32, false, EPI_DOWN>(n, s, 7, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 0);
   combine<32, 0>(n, s, n->graw, n->d1, nullptr, n->g1, 1, 5);
   // dec1: input up(d2)
   wgrad<64, 32, true>(n, s, n->d2, n->g1, D[1], H[1], W[1], n->grads + L.w_off[5]);
-  conv<32, 64, false, EPI_DOWN>(s, n->g1, Wt(n, 5), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<32, 64, false, EPI_DOWN>(n, s, 8, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 1);
   combine<64, 0>(n, s, n->graw, n->d2, nullptr, n->g2, 2, 4);
   // dec2: input up(e3)
   wgrad<64, 64, true>(n, s, n->e3, n->g2, D[2], H[2], W[2], n->grads + L.w_off[4]);
-  conv<64, 64, false, EPI_DOWN>(s, n->g2, Wt(n, 4), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[2], H[2], W[2]);
+  conv<64, 64, false, EPI_DOWN>(n, s, 9, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 2);
   combine<64, 0>(n, s, n->graw, n->e3, nullptr, n->g3, 3, 3);
   // enc3: input p2
   wgrad<64, 64, false>(n, s, n->p2, n->g3, D[3], H[3], W[3], n->grads + L.w_off[3]);
-  conv<64, 64, false, EPI_RAW>(s, n->g3, Wt(n, 3), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[3], H[3], W[3]);
+  conv<64, 64, false, EPI_RAW>(n, s, 10, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 3);
   combine<64, 1>(n, s, n->graw, n->e2, n->g2, n->ge2, 2, 2);
   // enc2: input p1
   wgrad<32, 64, false>(n, s, n->p1, n->ge2, D[2], H[2], W[2], n->grads + L.w_off[2]);
-  conv<64, 32, false, EPI_RAW>(s, n->ge2, Wt(n, 2), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[2], H[2], W[2]);
+  conv<64, 32, false, EPI_RAW>(n, s, 11, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 2);
   combine<32, 1>(n, s, n->graw, n->e1, n->g1, n->ge1, 1, 1);
   // enc1: input p0
   wgrad<16, 32, false>(n, s, n->p0, n->ge1, D[1], H[1], W[1], n->grads + L.w_off[1]);
-  conv<32, 16, false, EPI_RAW>(s, n->ge1, Wt(n, 1), nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, D[1], H[1], W[1]);
+  conv<32, 16, false, EPI_RAW>(n, s, 12, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 1);
   combine<16, 1>(n, s, n->graw, n->e0, n->g0, n->ge0, 0, 0);
   // enc0: input x
   wgrad<16, 16, false>(n, s, n->x, n->ge0, D[0], H[0], W[0], n->grads + L.w_off[0]);
@@ -1496,7 +1610,12 @@ void features(hca_net* n, cudaStream_t s, const FeatureArgs& f, const T* K) {
   k_features<T><<<ew_blocks(n->Ln[0], n->sm_count), kEwThreads, 0, s>>>(f, K, n->x);
 }
 
+// A kernel's bounded wait gave up (seen by the calls that wait for the GPU,
+// and by the call after one that does not).
+int net_status(const hca_net* n) { return *(volatile const int*)n->status ? HCA_ERR_TIMEOUT : HCA_OK; }
+
 int adam_update(hca_net* n, double lr, double beta1, double beta2, double eps) {
+  if (const int rc = net_status(n)) return rc;
   n->adam_t += 1;
   const double c1 = 1.0 - std::pow(beta1, (double)n->adam_t), c2 = 1.0 - std::pow(beta2, (double)n->adam_t);
   k_adam<<<ew_blocks(n->L.total, n->sm_count), kEwThreads, 0, n->stream>>>(
@@ -1539,8 +1658,8 @@ int create_impl(int D, int H, int W, int trainable, void* stream, hca_net** out)
   NET_ALLOC(n->params, n->L.total * sizeof(float));
   NET_ALLOC(n->wq, n->L.wq_total * b2);
   NET_ALLOC(n->wt, n->L.wq_total * b2);
-  NET_ALLOC(n->tc_status, sizeof(int));
-  NET_CUDA(cudaMemset(n->tc_status, 0, sizeof(int)));
+  NET_CUDA(cudaHostAlloc((void**)&n->status, sizeof(int), cudaHostAllocDefault));
+  *n->status = 0;
   {
     // tcgen05 forward for the full-resolution layers with HCA_NET_TC=1
     // (compute capability 10.x; tiles of 8 x 16 sites).  Off by default: with
@@ -1602,6 +1721,7 @@ int create_impl(int D, int H, int W, int trainable, void* stream, hca_net** out)
     NET_CUDA(cudaMemsetAsync(n->v, 0, n->L.total * sizeof(float), n->stream));
     NET_CUDA(cudaMemsetAsync(n->grads, 0, n->L.total * sizeof(float), n->stream));
   }
+  if (!prepare_convs(n)) return HCA_ERR_CUDA;
   quantize(n, n->stream);
   NET_CUDA(cudaGetLastError());
   NET_CUDA(cudaStreamSynchronize(n->stream));
@@ -1643,7 +1763,7 @@ int ws_o2(hca_net* n, const FeatureArgs& f, bool fp64, bool always, void* K, flo
     forward(n, s, false);
     k_ws_candidate<double><<<nb, kEwThreads, 0, s>>>(f, Kd, nullptr, n->out, cand, static_cast<double*>(lag));
     k_ws_norms<double><<<nbn, kEwThreads, 0, s>>>(f, Kd, nullptr, cand, part);
-    k_ws_decide<<<1, 32, 0, s>>>(part, nbn, always ? 1 : 0, res);
+    k_ws_decide<<<1, 32, 0, s>>>(part, nbn, always ? 1 : 0, n->status, res);
     k_ws_apply<double><<<nb, kEwThreads, 0, s>>>(f, res, cand, static_cast<double*>(K), nullptr);
   } else {
     const float* Kf = static_cast<const float*>(K);
@@ -1651,7 +1771,7 @@ int ws_o2(hca_net* n, const FeatureArgs& f, bool fp64, bool always, void* K, flo
     forward(n, s, false);
     k_ws_candidate<float><<<nb, kEwThreads, 0, s>>>(f, Kf, K_lo, n->out, cand, static_cast<float*>(lag));
     k_ws_norms<float><<<nbn, kEwThreads, 0, s>>>(f, Kf, K_lo, cand, part);
-    k_ws_decide<<<1, 32, 0, s>>>(part, nbn, always ? 1 : 0, res);
+    k_ws_decide<<<1, 32, 0, s>>>(part, nbn, always ? 1 : 0, n->status, res);
     k_ws_apply<float><<<nb, kEwThreads, 0, s>>>(f, res, cand, static_cast<float*>(K), K_lo);
   }
   NET_CUDA(cudaGetLastError());
@@ -1716,7 +1836,7 @@ int hca_net_forward(hca_net* n, const hca_config* cfg, const uint8_t* state, con
   NET_CUDA(cudaMemcpyAsync(out, n->out, n->Ln[0] * sizeof(float), cudaMemcpyDeviceToDevice, n->stream));
   NET_CUDA(cudaGetLastError());
   NET_CUDA(cudaStreamSynchronize(n->stream));
-  return HCA_OK;
+  return net_status(n);
 }
 
 int hca_net_forward_x(hca_net* n, const void* x, float* out) {
@@ -1726,7 +1846,7 @@ int hca_net_forward_x(hca_net* n, const void* x, float* out) {
   NET_CUDA(cudaMemcpyAsync(out, n->out, n->Ln[0] * sizeof(float), cudaMemcpyDeviceToDevice, n->stream));
   NET_CUDA(cudaGetLastError());
   NET_CUDA(cudaStreamSynchronize(n->stream));
-  return HCA_OK;
+  return net_status(n);
 }
 
 int hca_net_read_activation(hca_net* n, int32_t which, void* dst) {
@@ -1763,7 +1883,7 @@ int hca_net_gradients_x(hca_net* n, const void* x, const float* target, float* g
   if (loss) NET_CUDA(cudaMemcpyAsync(loss, n->loss, sizeof(float), cudaMemcpyDeviceToDevice, n->stream));
   NET_CUDA(cudaGetLastError());
   NET_CUDA(cudaStreamSynchronize(n->stream));
-  return HCA_OK;
+  return net_status(n);
 }
 
 int hca_net_gradients(hca_net* n, const hca_config* cfg, const uint8_t* state, const float* perf,
@@ -1854,6 +1974,7 @@ int hca_net_destroy(hca_net* n) {
   if (!n) return HCA_OK;
   if (n->stream) cudaStreamSynchronize(n->stream);
   for (void* p : n->allocs) cudaFree(p);
+  if (n->status) cudaFreeHost(n->status);
   delete n;
   return HCA_OK;
 }
