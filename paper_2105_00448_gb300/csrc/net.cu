@@ -11,13 +11,19 @@
 // weights, and of their tap-flipped transposes for the input gradient, are
 // refreshed after every update.
 //
-// Convolutions are implicit GEMMs: M = output sites (tiles of 16 consecutive
-// x by TZ x TY rows), N = C_out, K = 27 C_in.  A block stages its input halo
-// once in shared memory (XOR-swizzled 16-byte chunks, conflict-free for
-// ldmatrix row gathers), stages the weights one z-plane of taps at a time,
-// and every warp runs mma.m16n8k16 BF16 -> FP32 over its rows.  The nearest
-// 2x upsampling of the decoder is folded into the halo gather; the sum over
-// the 2x2x2 children that its gradient needs is folded into the epilogue.
+// Convolutions are implicit GEMMs: M = output sites (tiles of 16 sites of a
+// row), N = C_out, K = 27 C_in.  A block's input halo and the weights (a z-plane
+// of taps at a time, one ahead) arrive in shared memory by tensor copies whose
+// swizzle modes leave ldmatrix's row gathers free of bank conflicts, and every
+// warp runs mma.m16n8k16 BF16 -> FP32 over its rows.  The nearest 2x upsampling
+// of the decoder is folded into the halo's coordinates; the sum over the 2x2x2
+// children that its gradient needs is folded into the epilogue.
+//
+// Bound (forward at 128^3, 135 GFLOP, 431 us): the mma.sync pipe, which peaks
+// at 600 TFLOP/s on this chip (225 us), with the halo's traffic exposed where
+// two or three blocks fit a multiprocessor: dec0 129 us, enc0 83, dec1 68.
+// (One ldmatrix of the input per tap and tile, weights staged between barriers
+// and 128-thread blocks took 192, 115 and 88 us, 585 us in all.)
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -40,8 +46,6 @@ namespace hcanet {
 using bf16 = __nv_bfloat16;
 namespace tc = hca::tc;
 
-constexpr int kThreads = 128;
-constexpr int kRowX = 16;   // sites per tile row (one m16 MMA tile)
 constexpr int kTY = 4;      // tile rows along y
 
 // conv layers: name order enc0, enc1, enc2, enc3, dec2, dec1, dec0
@@ -113,40 +117,6 @@ __device__ __forceinline__ uint32_t pack_bf2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// halo geometry of a conv tile (input coordinates)
-template <int TZ, bool UP>
-struct Halo {
-  static constexpr int HZ = UP ? TZ / 2 + 2 : TZ + 2;
-  static constexpr int HY = UP ? kTY / 2 + 2 : kTY + 2;
-  static constexpr int HX = UP ? kRowX / 2 + 2 : kRowX + 2;
-  static constexpr int N = HZ * HY * HX;
-  // halo row of tile-local output site (tz, ty, x) shifted by (dz, dy, dx)
-  __device__ __forceinline__ static int row(int tz, int ty, int x, int dz, int dy, int dx) {
-    if (UP) return ((((tz + dz) >> 1) + 1) * HY + (((ty + dy) >> 1) + 1)) * HX + (((x + dx) >> 1) + 1);
-    return ((tz + dz + 1) * HY + (ty + dy + 1)) * HX + (x + dx + 1);
-  }
-};
-
-// Stage the halo of a tile whose output origin is (z0, y0, x0) (all even).
-template <int CI, int TZ, bool UP>
-__device__ __forceinline__ void stage_halo(char* sm, const bf16* __restrict__ in, int Di, int Hi, int Wi, int z0,
-                                           int y0, int x0) {
-  using HL = Halo<TZ, UP>;
-  constexpr int NCH = CI / 8;
-  const int oz = UP ? (z0 >> 1) - 1 : z0 - 1;
-  const int oy = UP ? (y0 >> 1) - 1 : y0 - 1;
-  const int ox = UP ? (x0 >> 1) - 1 : x0 - 1;
-  for (int i = threadIdx.x; i < HL::N * NCH; i += blockDim.x) {
-    const int h = i / NCH, j = i - h * NCH;
-    const int hx = h % HL::HX, hy = (h / HL::HX) % HL::HY, hz = h / (HL::HX * HL::HY);
-    const int gz = oz + hz, gy = oy + hy, gx = ox + hx;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (gz >= 0 && gz < Di && gy >= 0 && gy < Hi && gx >= 0 && gx < Wi)
-      v = __ldg(reinterpret_cast<const uint4*>(in + (((long long)gz * Hi + gy) * Wi + gx) * CI) + j);
-    *reinterpret_cast<uint4*>(sm + 16 * chunk_pos<CI>(h, j)) = v;
-  }
-}
-
 // ----------------------------------------------------- forward / dgrad ---
 enum { EPI_FWD = 0, EPI_HEAD = 1, EPI_RAW = 2, EPI_DOWN = 3 };
 
@@ -212,11 +182,12 @@ struct ConvMaps {
 // ends the block.
 constexpr int kConvWaitLimit = 1 << 20;
 
-__device__ __forceinline__ void tma_box_4d(uint32_t dst, const CUtensorMap* map, int c1, int c2, int c3, uint32_t bar) {
+__device__ __forceinline__ void tma_box_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
+                                           uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(
           dst),
-      "l"((unsigned long long)map), "r"(0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+      "l"((unsigned long long)map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
       : "memory");
 }
 __device__ __forceinline__ void tma_box_3d(uint32_t dst, const CUtensorMap* map, int c1, int c2, uint32_t bar) {
@@ -256,7 +227,7 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
     const int oz = UP ? (z0 >> 1) - 1 : z0 - 1, oy = UP ? (y0 >> 1) - 1 : y0 - 1, ox = (UP ? x0 >> 1 : x0) / S - 1;
     expect(0, (uint32_t)(T::HALO + T::WPLANE));
     for (int p = 0; p < S; ++p)
-      tma_box_4d(smem_u32(sh) + p * (T::PHASE * CI * 2), &maps.in[p], ox, oy, oz, smem_u32(&bar[0]));
+      tma_box_4d(smem_u32(sh) + p * (T::PHASE * CI * 2), &maps.in[p], 0, ox, oy, oz, smem_u32(&bar[0]));
     stage_w(0);
     expect(1, (uint32_t)T::WPLANE);
     stage_w(1);
@@ -493,7 +464,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(const ConvArgs a, int* status) 
   constexpr int NCH = CI / 8;
   constexpr uint32_t HALO_B = tc_halo_bytes<CI, TZ>(), TAP_B = CI * CO * 2;
   constexpr uint32_t NCOL = tc_cols<CO, TZ>();
-  extern __shared__ __align__(128) char smem[];
+  extern __shared__ __align__(1024) char smem[];
   char* shb0 = smem;
   char* sw = smem + 2 * HALO_B;
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sw + 27 * TAP_B);
@@ -594,110 +565,137 @@ __global__ void __launch_bounds__(128) k_conv_tc(const ConvArgs a, int* status) 
 
 // ------------------------------------------------------------- wgrad ---
 // dW[t, co, ci] = sum over sites m of gy[m, co] x[m + off_t, ci] (x = the
-// layer input, upsampled on the fly when UP).  M = co (m16 tiles), N = ci,
-// K = sites.  A warp owns P (tap, co-tile) units with all ci; blockIdx.y picks
-// the unit group; blocks along x split the sites and write FP32 partials that
-// a second kernel sums in a fixed order.
+// layer input, upsampled on the fly when UP).  M = 16 co, N = up to 32 ci (a
+// tile per blockIdx.y), K = sites.  The nine warps of a block own one (dz, dy)
+// each with its three dx; along x the sites of a row are S interleaved groups
+// of 16 (upsampled: two per phase, one per parity), so a fragment of x serves
+// all three taps and a fragment of gy all of them.  Tiles (8 rows) arrive by
+// tensor copies, one ahead; blocks along x split them and write FP32 partials
+// that a second kernel sums in a fixed order.  Bound: the MMAs and, at the
+// coarse levels, latency.  All seven layers at 64^3:
+// 90 us (dec0's 25), against 195 (69) with fragments loaded per tap.
+template <int CI, int CO, int S, bool UP>
+struct WgTile {
+  static constexpr int CB = CI < 32 ? CI : 32;   // input channels of a block
+  static constexpr int TZ = 2, ROWS = TZ * kTY, M = (UP ? 2 : 1) * S, XO = 16 * M, LP = 18;
+  static constexpr int HZ = UP ? TZ / 2 + 2 : TZ + 2, HY = UP ? kTY / 2 + 2 : kTY + 2;
+  static constexpr int PHASE = HZ * HY * LP, HALO = S * PHASE * CB * 2;
+  static constexpr int GROUP = ROWS * 16, GY = M * GROUP * 16 * 2;   // sites, bytes
+  static constexpr int STAGE = HALO + GY, SMEM = 2 * STAGE + 16;
+  static constexpr int PER_SM = 232448 / (SMEM + 1024) < 3 ? 232448 / (SMEM + 1024) : 3;   // (registers: 72 a thread)
+  static_assert(PHASE % 8 == 0 && HALO % (16 * CB) == 0 && STAGE % (16 * CB) == 0 && HALO % 256 == 0,
+                "phases, groups and stages start where the swizzle patterns do (8 rows)");
+};
+
+// Tensor maps of a layer's weight gradient: the input by phase of x, the
+// output's gradient by site group (box: 16 channels of a tile's rows).
+struct WgMaps {
+  CUtensorMap in[2], gy[4];
+};
+
 struct WgArgs {
-  const bf16* in;
-  const bf16* gy;
   float* part;         // [gridDim.x][27][CO][CI]
-  int D, H, W, Di, Hi, Wi;
   int tiles_x, tiles_y, tiles_z;
 };
 
-constexpr int kWgMT = 2;   // 8 tile rows (TZ = 2)
+constexpr int kWgThreads = 288;
 
-template <int CI, int CO, bool UP>
-constexpr int wgrad_smem_bytes() {
-  return Halo<kWgMT, UP>::N * CI * 2 + 4 * kWgMT * kRowX * CO * 2;
-}
-
-template <int CI, int CO, bool UP>
-__global__ void __launch_bounds__(kThreads) k_wgrad(const WgArgs a) {
-  constexpr int TZ = kWgMT;
-  constexpr int ROWS = 4 * kWgMT;
-  constexpr int NT = CI / 8;
-  constexpr int P = 128 / CI;           // units per warp
-  constexpr int MTILES = CO / 16;
-  constexpr int U = 27 * MTILES;
-  using HL = Halo<TZ, UP>;
-  extern __shared__ __align__(128) char smem[];
-  char* sh = smem;
-  char* sg = smem + HL::N * CI * 2;
+template <int CI, int CO, int S, bool UP>
+__global__ void __launch_bounds__(kWgThreads, (WgTile<CI, CO, S, UP>::PER_SM))
+    k_wgrad(const WgArgs a, const __grid_constant__ WgMaps maps, int* status) {
+  using T = WgTile<CI, CO, S, UP>;
+  constexpr int CB = T::CB, NT = CB / 8, M = T::M;
+  extern __shared__ __align__(1024) char smem[];
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * T::STAGE);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int q = lane >> 3;
-
-  float acc[P][NT][4];
+  const int dz = warp / 3 - 1, dy = warp % 3 - 1, mt = blockIdx.y % (CO / 16), c0 = (int)(blockIdx.y / (CO / 16)) * CB;
+  const int n_tiles = a.tiles_x * a.tiles_y * a.tiles_z;
+  auto fetch = [&](int tile, int st) {
+    const int bx = tile % a.tiles_x, by = (tile / a.tiles_x) % a.tiles_y, bz = tile / (a.tiles_x * a.tiles_y);
+    const int z0 = bz * T::TZ, y0 = by * kTY;
+    const uint32_t b = smem_u32(&bar[st]), d = smem_u32(smem) + st * T::STAGE;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"((uint32_t)T::STAGE) : "memory");
+    const int oz = UP ? (z0 >> 1) - 1 : z0 - 1, oy = UP ? (y0 >> 1) - 1 : y0 - 1;
+    for (int p = 0; p < S; ++p)   // (the tile starts at input site 16 S bx)
+      tma_box_4d(d + p * (T::PHASE * CB * 2), &maps.in[p], c0, 16 * bx - 1, oy, oz, b);
+    for (int m = 0; m < M; ++m)
+      tma_box_4d(d + T::HALO + m * (T::GROUP * 32), &maps.gy[m], 16 * mt, 16 * bx, y0, z0, b);
+  };
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&bar[0], 1);
+    tc::mbar_init(&bar[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if ((int)blockIdx.x < n_tiles) fetch(blockIdx.x, 0);
+  }
+  float acc[3][NT][4];
 #pragma unroll
-  for (int i = 0; i < P; ++i)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][n][e] = 0.f;
-
-  const int ubase = (blockIdx.y * 4 + warp) * P;
-  const uint32_t shb = smem_u32(sh), sgb = smem_u32(sg);
-  const int n_tiles = a.tiles_x * a.tiles_y * a.tiles_z;
-  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int bx = tile % a.tiles_x, by = (tile / a.tiles_x) % a.tiles_y, bz = tile / (a.tiles_x * a.tiles_y);
-    const int z0 = bz * TZ, y0 = by * kTY, x0 = bx * kRowX;
-    __syncthreads();
-    stage_halo<CI, TZ, UP>(sh, a.in, a.Di, a.Hi, a.Wi, z0, y0, x0);
-    {
-      constexpr int NCH = CO / 8;
-      for (int i = threadIdx.x; i < ROWS * kRowX * NCH; i += blockDim.x) {
-        const int s = i / NCH, j = i - s * NCH;
-        const int x = s % kRowX, rr = s / kRowX;
-        const int z = z0 + rr / kTY, y = y0 + rr % kTY, xx = x0 + x;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (z < a.D && y < a.H && xx < a.W)
-          v = __ldg(reinterpret_cast<const uint4*>(a.gy + (((long long)z * a.H + y) * a.W + xx) * CO) + j);
-        *reinterpret_cast<uint4*>(sg + 16 * chunk_pos<CO>(s, j)) = v;
+  __syncthreads();
+  int it = 0;
+  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+    const int st = it & 1;
+    if (threadIdx.x == 0 && tile + (int)gridDim.x < n_tiles) fetch(tile + gridDim.x, st ^ 1);
+    const bool ok = tc::mbar_wait(&bar[st], (uint32_t)(it >> 1) & 1u, kConvWaitLimit);
+    if (!__syncthreads_and(ok)) {   // (the same in every thread)
+      if (threadIdx.x == 0) {
+        *(volatile int*)status = 1;
+        // the copies in flight land before the block's shared memory is released
+        (void)tc::mbar_wait(&bar[st], (uint32_t)(it >> 1) & 1u, kConvWaitLimit);
+        if (tile + (int)gridDim.x < n_tiles)
+          (void)tc::mbar_wait(&bar[st ^ 1], (uint32_t)((it + 1) >> 1) & 1u, kConvWaitLimit);
       }
+      __syncthreads();
+      return;
     }
-    __syncthreads();
+    const uint32_t shb = smem_u32(smem) + st * T::STAGE, sgb = shb + T::HALO;
 #pragma unroll 1
-    for (int rr = 0; rr < ROWS; ++rr) {
+    for (int rr = 0; rr < T::ROWS; ++rr) {
       const int tz = rr / kTY, ty = rr - tz * kTY;
+      const int h = (UP ? (((tz + dz) >> 1) + 1) * T::HY + (((ty + dy) >> 1) + 1) : (tz + dz + 1) * T::HY + (ty + dy + 1)) *
+                        T::LP + (lane & 7) + ((q & 1) << 3);
+      uint32_t af[M][4];
 #pragma unroll
-      for (int i = 0; i < P; ++i) {
-        const int u = ubase + i;
-        if (u >= U) break;
-        const int tap = u / MTILES, mt = u - tap * MTILES;
-        const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-        uint32_t af[4];
-        {
-          const int s = rr * kRowX + (lane & 7) + ((q >> 1) << 3);
-          ldsm_x4_t(sgb + 16 * chunk_pos<CO>(s, 2 * mt + (q & 1)), af);
-        }
-        const int h = HL::row(tz, ty, (lane & 7) + ((q & 1) << 3), dz, dy, dx);
+      for (int m = 0; m < M; ++m)
+        ldsm_x4_t(sgb + 16 * chunk_pos<16>(m * T::GROUP + rr * 16 + (lane & 7) + ((q >> 1) << 3), q & 1), af[m]);
+#pragma unroll
+      for (int p = 0; p < S + 2; ++p) {
 #pragma unroll
         for (int np = 0; np < NT / 2; ++np) {
           uint32_t r[4];
-          ldsm_x4_t(shb + 16 * chunk_pos<CI>(h, 2 * np + (q >> 1)), r);
-          mma16816(acc[i][2 * np], af, r[0], r[1]);
-          mma16816(acc[i][2 * np + 1], af, r[2], r[3]);
+          ldsm_x4_t(shb + 16 * chunk_pos<CB>(((p + S - 1) % S) * T::PHASE + h + (p + S - 1) / S, 2 * np + (q >> 1)), r);
+#pragma unroll
+          for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int dx = -1; dx <= 1; ++dx) {
+              const int pm = UP ? m / 2 + (m % 2 + dx + 2) / 2 : m + dx + 1;   // the phase tap dx of group m reads
+              if (pm == p) {
+                mma16816(acc[dx + 1][2 * np], af[m], r[0], r[1]);
+                mma16816(acc[dx + 1][2 * np + 1], af[m], r[2], r[3]);
+              }
+            }
         }
       }
     }
+    __syncthreads();   // this stage is free
   }
   float* part = a.part + (long long)blockIdx.x * 27 * CO * CI;
   const int cq = (lane & 3) * 2;
 #pragma unroll
-  for (int i = 0; i < P; ++i) {
-    const int u = ubase + i;
-    if (u >= U) break;
-    const int tap = u / MTILES, mt = u - tap * MTILES;
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
-        const int co = mt * 16 + (lane >> 2) + 8 * hf, ci = n * 8 + cq;
-        *reinterpret_cast<float2*>(part + ((long long)tap * CO + co) * CI + ci) =
+        const int co = mt * 16 + (lane >> 2) + 8 * hf, ci = c0 + n * 8 + cq;
+        *reinterpret_cast<float2*>(part + ((long long)(warp * 3 + i) * CO + co) * CI + ci) =
             make_float2(acc[i][n][2 * hf], acc[i][n][2 * hf + 1]);
       }
-  }
 }
 
 // dst[i] = sum_g part[g][i] (split-K reduce): 8 warps of a block take every
@@ -1240,6 +1238,7 @@ struct hca_net {
   // tensor maps of the convolutions' inputs (the net's own arrays): the seven
   // layers, then the input gradients of dec0, dec1, dec2, enc3, enc2, enc1
   ConvMaps maps[13];
+  WgMaps wmaps[7];   // of the layers' weight gradients
   // pinned host memory: set by a kernel whose bounded wait timed out
   int* status = nullptr;
 };
@@ -1324,10 +1323,16 @@ int conv_attr() {
   return conv_attr_t<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>();
 }
 
+// Phases of a weight gradient's tiles (the lattice of a layer's input has a
+// multiple of that many sites in x).
+template <int CI, int CO, bool UP>
+constexpr int wgrad_phases() { return CI == 16 || (CI == 32 && UP) ? 2 : 1; }
+
 template <int CI, int CO, bool UP>
 int wgrad_attr() {
-  constexpr int sm = wgrad_smem_bytes<CI, CO, UP>();
-  NET_CUDA(cudaFuncSetAttribute(k_wgrad<CI, CO, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+  constexpr int S = wgrad_phases<CI, CO, UP>(), sm = WgTile<CI, CO, S, UP>::SMEM;
+  NET_CUDA(cudaFuncSetAttribute(k_wgrad<CI, CO, S, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+  NET_CUDA(cudaFuncSetAttribute(k_wgrad<CI, CO, S, UP>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   return HCA_OK;
 }
 
@@ -1461,30 +1466,43 @@ void conv(hca_net* n, cudaStream_t s, int slot, const float* bias, const bf16* s
     conv_launch<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>(s, a, n->maps[slot], n->status);
 }
 
-// Weight gradient of one layer into grads[w_off ...]; (D, H, W) = output lattice.
+// The maps of layer `layer`'s weight gradient; lvl: the output's level.
 template <int CI, int CO, bool UP>
-void wgrad(hca_net* n, cudaStream_t s, const bf16* in, const bf16* gy, int D, int H, int W, float* dst) {
+bool wgrad_prepare(hca_net* n, int layer, const bf16* in, const bf16* gy, int lvl) {
+  constexpr int S = wgrad_phases<CI, CO, UP>();
+  using T = WgTile<CI, CO, S, UP>;
+  WgMaps& m = n->wmaps[layer];
+  auto by_phase = [&](CUtensorMap* map, const bf16* base, int c, int phases, int l, int bc, int bx, int by, int bz) {
+    const cuuint64_t row = (cuuint64_t)c * 2, W = n->Lw[l], H = n->Lh[l], D = n->Ld[l];
+    const cuuint64_t dims[4] = {(cuuint64_t)c, W / phases, H, D}, strides[3] = {phases * row, W * row, W * H * row};
+    const cuuint32_t box[4] = {(cuuint32_t)bc, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
+    for (int p = 0; p < phases; ++p)
+      if (!bf16_map(&map[p], base + (size_t)p * c, 4, bc, dims, strides, box)) return false;
+    return true;
+  };
+  return by_phase(m.in, in, CI, S, lvl + UP, T::CB, T::LP, T::HY, T::HZ) && by_phase(m.gy, gy, CO, T::M, lvl, 16, 16, kTY, T::TZ);
+}
+
+// Weight gradient of one layer into dst (27, CO, CI); the output lattice is level lvl.
+template <int CI, int CO, bool UP>
+void wgrad(hca_net* n, cudaStream_t s, int layer, int lvl, float* dst) {
+  constexpr int S = wgrad_phases<CI, CO, UP>();
+  using T = WgTile<CI, CO, S, UP>;
   WgArgs a;
-  a.in = in;
-  a.gy = gy;
   a.part = n->wpart;
-  a.D = D;
-  a.H = H;
-  a.W = W;
-  a.Di = UP ? D / 2 : D;
-  a.Hi = UP ? H / 2 : H;
-  a.Wi = UP ? W / 2 : W;
-  a.tiles_x = (W + kRowX - 1) / kRowX;
-  a.tiles_y = (H + kTY - 1) / kTY;
-  a.tiles_z = (D + kWgMT - 1) / kWgMT;
-  constexpr int P = 128 / CI;
-  constexpr int U = 27 * (CO / 16);
-  const int gy_blocks = (U + 4 * P - 1) / (4 * P);
+  a.tiles_x = (n->Lw[lvl] + T::XO - 1) / T::XO;
+  a.tiles_y = (n->Lh[lvl] + kTY - 1) / kTY;
+  a.tiles_z = (n->Ld[lvl] + T::TZ - 1) / T::TZ;
+  constexpr int mts = CO / 16 * (CI / T::CB);   // tiles of the gradient
   const int n_tiles = a.tiles_x * a.tiles_y * a.tiles_z;
   const long long per = 27LL * CO * CI;
-  int G = std::max(1, std::min(n_tiles, 2 * n->sm_count / gy_blocks));
+  // one wave of blocks (every further block is a partial to sum), each with
+  // the same number of tiles but for a remainder
+  int G = std::max(1, std::min(n_tiles, T::PER_SM * n->sm_count / mts));
   G = (int)std::min<long long>(G, n->wpart_n / per);
-  k_wgrad<CI, CO, UP><<<dim3(G, gy_blocks), kThreads, wgrad_smem_bytes<CI, CO, UP>(), s>>>(a);
+  const int rounds = (n_tiles + G - 1) / G;
+  G = (n_tiles + rounds - 1) / rounds;
+  k_wgrad<CI, CO, S, UP><<<dim3(G, mts), kWgThreads, T::SMEM, s>>>(a, n->wmaps[layer], n->status);
   k_sum_parts<<<(int)((per + 31) / 32), 32 * kSumWarps, 0, s>>>(n->wpart, G, per, dst);
 }
 
@@ -1522,7 +1540,14 @@ bool prepare_convs(hca_net* n) {
          conv_prepare<64, 64, false, EPI_DOWN>(n, 9, n->g2, Wt(n, 4), 2) &&
          conv_prepare<64, 64, false, EPI_RAW>(n, 10, n->g3, Wt(n, 3), 3) &&
          conv_prepare<64, 32, false, EPI_RAW>(n, 11, n->ge2, Wt(n, 2), 2) &&
-         conv_prepare<32, 16, false, EPI_RAW>(n, 12, n->ge1, Wt(n, 1), 1);
+         conv_prepare<32, 16, false, EPI_RAW>(n, 12, n->ge1, Wt(n, 1), 1) &&
+         wgrad_prepare<32, 16, true>(n, 6, n->d1, n->g0, 0) &&
+         wgrad_prepare<64, 32, true>(n, 5, n->d2, n->g1, 1) &&
+         wgrad_prepare<64, 64, true>(n, 4, n->e3, n->g2, 2) &&
+         wgrad_prepare<64, 64, false>(n, 3, n->p2, n->g3, 3) &&
+         wgrad_prepare<32, 64, false>(n, 2, n->p1, n->ge2, 2) &&
+         wgrad_prepare<16, 32, false>(n, 1, n->p0, n->ge1, 1) &&
+         wgrad_prepare<16, 16, false>(n, 0, n->x, n->ge0, 0);
 }
 
 // Forward pass from n->x; with keep_d0 the last activation is stored (training).
@@ -1554,9 +1579,6 @@ void forward(hca_net* n, cudaStream_t s, bool keep_d0) {
 // or (gbuf != null) the output gradient in gbuf; fills n->grads (and n->loss
 // for the MSE loss).
 void backward(hca_net* n, cudaStream_t s, const float* target, const float* gbuf) {
-  const int* D = n->Ld;
-  const int* H = n->Lh;
-  const int* W = n->Lw;
   const ParamLayout& L = n->L;
   {
     // two blocks per multiprocessor: each ends with its 34 sums
@@ -1567,31 +1589,31 @@ void backward(hca_net* n, cudaStream_t s, const float* target, const float* gbuf
                                      1.0f / (float)n->Ln[0]);
   }
   // dec0: input up(d1), output gradient g0
-  wgrad<32, 16, true>(n, s, n->d1, n->g0, D[0], H[0], W[0], n->grads + L.w_off[6]);
+  wgrad<32, 16, true>(n, s, 6, 0, n->grads + L.w_off[6]);
   conv<16, 32, false, EPI_DOWN>(n, s, 7, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 0);
   combine<32, 0>(n, s, n->graw, n->d1, nullptr, n->g1, 1, 5);
   // dec1: input up(d2)
-  wgrad<64, 32, true>(n, s, n->d2, n->g1, D[1], H[1], W[1], n->grads + L.w_off[5]);
+  wgrad<64, 32, true>(n, s, 5, 1, n->grads + L.w_off[5]);
   conv<32, 64, false, EPI_DOWN>(n, s, 8, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 1);
   combine<64, 0>(n, s, n->graw, n->d2, nullptr, n->g2, 2, 4);
   // dec2: input up(e3)
-  wgrad<64, 64, true>(n, s, n->e3, n->g2, D[2], H[2], W[2], n->grads + L.w_off[4]);
+  wgrad<64, 64, true>(n, s, 4, 2, n->grads + L.w_off[4]);
   conv<64, 64, false, EPI_DOWN>(n, s, 9, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 2);
   combine<64, 0>(n, s, n->graw, n->e3, nullptr, n->g3, 3, 3);
   // enc3: input p2
-  wgrad<64, 64, false>(n, s, n->p2, n->g3, D[3], H[3], W[3], n->grads + L.w_off[3]);
+  wgrad<64, 64, false>(n, s, 3, 3, n->grads + L.w_off[3]);
   conv<64, 64, false, EPI_RAW>(n, s, 10, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 3);
   combine<64, 1>(n, s, n->graw, n->e2, n->g2, n->ge2, 2, 2);
   // enc2: input p1
-  wgrad<32, 64, false>(n, s, n->p1, n->ge2, D[2], H[2], W[2], n->grads + L.w_off[2]);
+  wgrad<32, 64, false>(n, s, 2, 2, n->grads + L.w_off[2]);
   conv<64, 32, false, EPI_RAW>(n, s, 11, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 2);
   combine<32, 1>(n, s, n->graw, n->e1, n->g1, n->ge1, 1, 1);
   // enc1: input p0
-  wgrad<16, 32, false>(n, s, n->p0, n->ge1, D[1], H[1], W[1], n->grads + L.w_off[1]);
+  wgrad<16, 32, false>(n, s, 1, 1, n->grads + L.w_off[1]);
   conv<32, 16, false, EPI_RAW>(n, s, 12, nullptr, nullptr, nullptr, n->graw, nullptr, nullptr, 1);
   combine<16, 1>(n, s, n->graw, n->e0, n->g0, n->ge0, 0, 0);
   // enc0: input x
-  wgrad<16, 16, false>(n, s, n->x, n->ge0, D[0], H[0], W[0], n->grads + L.w_off[0]);
+  wgrad<16, 16, false>(n, s, 0, 0, n->grads + L.w_off[0]);
 }
 
 void quantize(hca_net* n, cudaStream_t s) {
