@@ -40,20 +40,20 @@ WORKLOAD = dict(precision="f32", n_drugs=2, seed=1, rtol_o2=1e-8, rtol_drug=1e-8
                 dose_interval=21, preconditioner=1)     # 1 = HCA_PC_MG
 CORR_LEN = 8.0
 # algorithmic HBM bytes per site of each kernel class (FP32):
-#   pass A reads z, p_old, d and writes p_new and q = A p_new; pass B reads p, q, x, r and
-#   writes x, r;
-#   defect-correction residual (later sweeps) reads x_hi, x_lo, d, a, b and writes z, dx, r;
-#   multigrid on the lattice, four kernels per V-cycle: the two pre-sweeps read r, 1/d and
-#   write the pre-smoothed iterate v (12 B); the restriction reads v, r, d and writes
-#   v' = v + (W2/d)(r - A v) and the 1/8-size coarse right-hand side (16.5 B); the prolongation
-#   + first post-sweep reads v', 1/d and the 1/8-size coarse correction and writes y (12.5 B);
-#   the last post-sweep reads y, r, 1/d and writes z (16 B); ODE reads state, K and
-#   updates phi, P, Vc
-BYTES_PER_SITE = {"pass_a": 20, "pass_b": 24, "setup": 17, "residual": 24, "ode": 29,
-                  "mg_pre0": 12, "mg_restrict0": 16.5, "mg_post0": 12.5, "mg_last0": 16}
-# the method's minimum per site where this design moves more: CG pass A reads
-# z, d, p_old and writes p (16 B); storing q = A p for pass B adds 4 B
-BYTES_MIN_PER_SITE = {**BYTES_PER_SITE, "pass_a": 16}
+#   pass A reads z, d and writes p and q = A p (16 B) in a solve's first iteration, reads p_old and
+#   writes x too in the second (24 B) and reads x too from then on (28 B): 22 B on this workload;
+#   pass B reads r, q and writes r;
+#   defect-correction residual (later sweeps) reads x_hi, x_lo, a, b and writes r;
+#   multigrid on the lattice, two kernels per V-cycle: the way down (mg_restrict0: pre-sweeps,
+#   residual, restriction, the part of the first post-sweep that needs no correction) reads r, d
+#   and writes v' and the 1/8-size coarse right-hand side (12.5 B); the way up (mg_post0:
+#   prolongation, both post-sweeps, r.z) reads v', d, r and the 1/8-size coarse correction and
+#   writes z (16.5 B); ODE reads state, K and updates phi, P, Vc
+BYTES_PER_SITE = {"pass_a": 22, "pass_b": 12, "setup": 17, "residual": 20, "ode": 29,
+                  "mg_restrict0": 12.5, "mg_post0": 16.5}
+# the method's minimum per site where this design moves more: storing q = A p
+# for pass B adds 4 B to pass A
+BYTES_MIN_PER_SITE = {**BYTES_PER_SITE, "pass_a": 18}
 # step-level algorithmic bytes per lattice site (FP32 storage): set-up and
 # solve start-up, ODE and CA 70 B, 13 B per defect-correction residual sweep,
 # 40 B per CG iteration (two-pass minimum), plus per V-cycle the lattice's
@@ -63,10 +63,10 @@ BYTES_MIN_PER_SITE = {**BYTES_PER_SITE, "pass_a": 16}
 # number of sweeps when they are fused) and the coarse levels (33 B per
 # coarse site, by the same count)
 STEP_FIXED_B, STEP_DC_B, STEP_IT_B, VCYCLE_LATTICE_B, VCYCLE_COARSE_B = 70, 13, 40, 29, 33
-# the bytes this design's kernels move per CG iteration (pass A also stores
-# q: 44 B) and per V-cycle (the four lattice kernels: 57 B; per coarse site the
-# four coarse kernels, fused pre-sweeps 16, restriction 12.5, fused first
-# post-sweep 20.5, last sweep 20 B: 69 B)
+# yardstick of records taken before the V-cycle's sweeps were fused and x += alpha p
+# moved into pass A: 44 B per CG iteration, 57 B per V-cycle on the lattice (four
+# kernels), 69 B per coarse site; today's kernels move 34 B per iteration and the
+# minimum above per V-cycle
 STEP_IT_DESIGN_B, VCYCLE_LATTICE_DESIGN_B, VCYCLE_COARSE_DESIGN_B = 44, 57, 69
 
 
@@ -165,7 +165,7 @@ def traffic_record(kernel: str):
             rec = json.load(f)[kernel]
     except Exception:
         return None
-    if rec.get("source_sha") != kernel_source_sha():
+    if rec.get("source_sha") != kernel_source_sha() or rec.get("kernel_sha") != hot_kernel_sha():
         return None
     return rec.get("dram_bytes_per_site")
 
@@ -182,13 +182,22 @@ def code_lines(text: str):
     return out
 
 
-def kernel_source_sha(root: str = ROOT) -> str:
-    """Fingerprint of the hot kernels' code, matched against profiles/traffic.json."""
+def _sha(root: str, names) -> str:
     h = hashlib.sha256()
-    for name in ("hca_internal.cuh", "row_ops.cuh", "pcg.cu", "mg.cu"):
+    for name in names:
         with open(os.path.join(root, "paper_2105_00448_gb300", "csrc", name), encoding="utf-8") as f:
             h.update("\n".join(code_lines(f.read())).encode())
     return h.hexdigest()[:16]
+
+
+def kernel_source_sha(root: str = ROOT) -> str:
+    """Fingerprint of the solver's shared code, matched against profiles/traffic.json."""
+    return _sha(root, ("hca_internal.cuh", "row_ops.cuh", "pcg.cu", "mg.cu"))
+
+
+def hot_kernel_sha(root: str = ROOT) -> str:
+    """Fingerprint of the FP32 solver's kernels, matched against profiles/traffic.json."""
+    return _sha(root, ("march.cuh", "march.cu", "cg.cu", "dc.cu", "coarse.cu"))
 
 
 # ------------------------------------------------------------ oracle ---
@@ -287,8 +296,8 @@ def step_roofline(prof, steps: int, sites: int, ms_per_step: float, level_fracti
             "frac_design_bytes": design * sites / (ms_per_step * 1e-3) / 1e9 / peak,
             "formula": "70 + 13 n_dc + 40 n_it + n_vc (29 + 33 f_coarse) B/site x sites / step time; f_coarse = "
                        "coarse-level sites per lattice site; 29 and 33 B are the V-cycle's minimum with its sweeps "
-                       "fused; frac_design_bytes counts what the kernels move (44 B per iteration, "
-                       "57 + 69 f_coarse B per V-cycle)"}
+                       "fused; frac_design_bytes: the bytes of the unfused kernels (44 B per iteration, "
+                       "57 + 69 f_coarse B per V-cycle), for comparison with earlier records"}
 
 
 def run_reference(args):
@@ -417,10 +426,8 @@ def run_gpu(args):
     achieved = bytes_per_launch / (avg_ms * 1e-3) / 1e9
     design_bytes = BYTES_PER_SITE[dom] * sites
     tr = traffic_record(dom)
-    kernel_names = {"pass_a": "k_pass_a<float>", "pass_b": "k_pass_b<float>", "setup": "k_setup<float>",
-                    "residual": "k_dc_residual", "ode": "k_ode<float>", "mg_pre0": "k_mg_pre0<float>",
-                    "mg_restrict0": "k_mg_restrict0_rows<float>", "mg_post0": "k_mg_post0<float, true>",
-                    "mg_last0": "k_mg_post0<float, false>"}
+    kernel_names = {"pass_a": "k_cg_a", "pass_b": "k_cg_b", "setup": "k_setup<float>", "residual": "k_dc_residual",
+                    "ode": "k_ode<float>", "mg_restrict0": "k_mg_down", "mg_post0": "k_mg_up"}
     roofline = {"bound": "hbm", "kernel": kernel_names[dom], "achieved": achieved, "peak": peak,
                 "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": tr * sites if tr is not None else None,

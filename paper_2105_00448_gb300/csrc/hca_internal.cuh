@@ -394,7 +394,6 @@ struct Ctx {
   // carries z = r / d instead), level-0 scratch, coarse level table
   int pass_ni;      // groups per lane in a row shared by all replicates (1, 2, 4; 0 = differs)
   int mg;           // 0: Jacobi (z = r / d), 1: V-cycle (z = M r)
-  int persist;         // 1: the CG passes and the lattice post-sweep run in persistent row form (one FP32 lattice)
   int pdl;             // 1: the CG and V-cycle kernels launch with programmatic dependent launch
   int skip_idle;       // 1 (solves): a V-cycle's kernels return at once when the set-up, residual
                        // sweep or pass B before it left no replicate iterating (nothing reads its z)

@@ -35,7 +35,6 @@
 
 namespace hca {
 
-int persist_grid(const void* fn, int threads, int sm_count);
 void launch_march(const Ctx& c, int which, const MGHost& H, int l, bool down);
 void launch_mg_cluster(const Ctx& c, int which, const MGHost& H);
 
@@ -1142,10 +1141,10 @@ __global__ void __launch_bounds__(NT, MINB) k_mg_coarse(Ctx c, int which, int lo
 // level): reads u, r and 1/d, 16 B per site with the write; then rho = r.z with the fixed-order reductions
 // of the CG passes and beta = rho / rho_old (0 on the first application of a
 // solve).
-template <typename T, bool PROLONG, int NI, bool PERSIST = false>
+template <typename T, bool PROLONG, int NI>
 __global__ void __maxnreg__(64) k_mg_post0(Ctx c, int which, const T* __restrict__ src, T om) {
   HCA_VC_ENTRY(c);
-  const int2 ch = PERSIST ? make_int2(0, 0) : c.chunks[blockIdx.x];
+  const int2 ch = c.chunks[blockIdx.x];
   const RepDesc& rd = c.reps[ch.x];
   const int nrows = min(rd.chunk_rows, rd.ny * rd.nz - ch.y);
   const T* __restrict__ rr = (const T*)c.r;
@@ -1253,15 +1252,10 @@ __global__ void __maxnreg__(64) k_mg_post0(Ctx c, int which, const T* __restrict
     }
     if (!PROLONG) store_rows_acc(c, chunk, rl, row_ok, it.sl, it.lpr, acc, 1);
   };
-  if (PERSIST) {
-    const int R = rd.ny * rd.nz, cr = rd.chunk_rows;
-    for (int j = persist_row_begin(R) + it.warp; j < persist_row_end(R); j += it.nw) row(j / cr, j % cr, true, j);
-  } else {
-    for (int rbase = it.warp * it.rpw; rbase < rd.chunk_rows; rbase += it.nw * it.rpw) {
-      const int rl = rbase + it.sub;
-      const bool row_ok = rl < nrows;
-      row(blockIdx.x, rl, row_ok, ch.y + (row_ok ? rl : 0));
-    }
+  for (int rbase = it.warp * it.rpw; rbase < rd.chunk_rows; rbase += it.nw * it.rpw) {
+    const int rl = rbase + it.sub;
+    const bool row_ok = rl < nrows;
+    row(blockIdx.x, rl, row_ok, ch.y + (row_ok ? rl : 0));
   }
   if (PROLONG) return;
   auto fin = [&](int r, const double* s1) -> int {
@@ -1277,8 +1271,7 @@ __global__ void __maxnreg__(64) k_mg_post0(Ctx c, int which, const T* __restrict
     return 1;
   };
   // float-float row slots for FP32 fields (LaneAcc<float>)
-  if (PERSIST) block_arrivals<sizeof(T) == 4>(c, 1, fin, [](int) {});
-  else warp_epilogue<sizeof(T) == 4>(c, 1, blockIdx.x, fin);
+  warp_epilogue<sizeof(T) == 4>(c, 1, blockIdx.x, fin);
 }
 
 // Launch shapes of the cooperative coarse-level kernel: 0 = 256 threads with
@@ -1296,24 +1289,11 @@ int grid_for(long long n) {
   return (int)std::max(1LL, std::min(b, 152LL * 16));
 }
 
-// One of the lattice's post-sweep kernels (k_mg_post0), in the persistent
-// row form when the handle uses it.
+// One of the lattice's post-sweep kernels (k_mg_post0).
 template <typename T, bool PROLONG>
 void launch_post0(const Ctx& c, int which, const MGHost& H, const T* src, T om) {
   cudaStream_t s = c.stream;
   const bool pdl = c.pdl != 0;
-  if (c.persist && (H.ni == 1 || H.ni == 2 || H.ni == 4)) {
-    const void* fn = H.ni == 1   ? (const void*)k_mg_post0<T, PROLONG, 1, true>
-                     : H.ni == 2 ? (const void*)k_mg_post0<T, PROLONG, 2, true>
-                                 : (const void*)k_mg_post0<T, PROLONG, 4, true>;
-    const dim3 g(persist_grid(fn, c.threads, c.sm_count));
-    switch (H.ni) {
-      case 1: launch_k(pdl, k_mg_post0<T, PROLONG, 1, true>, g, dim3(c.threads), 0, s, c, which, src, om); break;
-      case 2: launch_k(pdl, k_mg_post0<T, PROLONG, 2, true>, g, dim3(c.threads), 0, s, c, which, src, om); break;
-      default: launch_k(pdl, k_mg_post0<T, PROLONG, 4, true>, g, dim3(c.threads), 0, s, c, which, src, om); break;
-    }
-    return;
-  }
   const dim3 g(c.n_chunks);
   switch (H.ni) {
     case 1: launch_k(pdl, k_mg_post0<T, PROLONG, 1>, g, dim3(c.threads), 0, s, c, which, src, om); break;

@@ -25,7 +25,6 @@
 // update would let one block read a neighbour row another block has already
 // overwritten); a parity bit in device memory, flipped by pass B, names the
 // current buffer, so the same two kernels form the body of a graph loop.
-#include <mutex>
 #include <vector>
 
 #include <cstdlib>
@@ -616,27 +615,6 @@ static void launch_setup_t(const Ctx& c, int which, CondArg cnd) {
 void launch_setup(const Ctx& c, int which, bool fp64, CondArg cnd) {
   if (fp64) launch_setup_t<double>(c, which, cnd);
   else launch_setup_t<float>(c, which, cnd);
-}
-
-// Blocks of a persistent row kernel: every block resident at once (its
-// occupancy at `threads` per block times the SM count), cached per kernel.
-int persist_grid(const void* fn, int threads, int sm_count) {
-  struct Entry {
-    const void* fn;
-    int threads, sm, grid;
-  };
-  static std::mutex mu;
-  static std::vector<Entry> cache;
-  std::lock_guard<std::mutex> lock(mu);
-  for (const Entry& e : cache)
-    if (e.fn == fn && e.threads == threads && e.sm == sm_count) return e.grid;
-  int per = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, 0) != cudaSuccess || per < 1) {
-    (void)cudaGetLastError();
-    per = 1;
-  }
-  cache.push_back({fn, threads, sm_count, per * sm_count});
-  return per * sm_count;
 }
 
 void launch_cg_a(const Ctx& c, int which, bool defer);
