@@ -1339,7 +1339,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
             const hca::MGLevel* lv_i = &lv[(size_t)i * hca::MG_MAXLEV];
             int from = 1;   // levels of at most kClusterSites sites per block
             while (from < rep[i].x - 1 && lv_i[from].n > hca::kClusterSites * cs) ++from;
-            const int lc = hca::cluster_plan(lv_i, rep[i].x, from, cs, 223 * 1024, &clus[i]);
+            const int lc = hca::cluster_plan(lv_i, rep[i].x, from, cs, hca::kClusterSmem, &clus[i]);
             ok = lc > 0;
             rep[i].y = lc;
             H.small = std::max(H.small, lc);

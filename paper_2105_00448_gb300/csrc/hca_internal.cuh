@@ -301,9 +301,11 @@ struct MGLevel {
 
 // The coarse levels a thread-block cluster holds (FP32; coarse.cu): level i of
 // the cluster is hierarchy level lc + i.
+constexpr int kClusterSmem = 215 * 1024;   // dynamic shared memory of a cluster's block at most (12 KB are static)
 struct MGClusterLevel {
   int nx, nr, no, gpr;          // sites per row, rows per plane, planes, 4-site groups per row
   int oa, ob, orr, od;          // float offsets in a block's shared memory (orr, od: -1 = global memory)
+  int few;                      // a block's slab is at most two groups a thread
   int p0[17];                   // first plane of each block (distributed levels)
   float cscale;
   int grow, gplane;             // global strides of rows and planes
