@@ -735,6 +735,15 @@ __device__ __forceinline__ float block_sum(float v, float* sb) {
   return t;
 }
 
+// Site s of an (nz, ny, nx) lattice (at most 2^27 sites: 32-bit divisions; the
+// 64-bit ones cost more than the rest of these kernels).
+__device__ __forceinline__ void site_xyz(long long s, int nx, int ny, int& x, int& y, int& z) {
+  const unsigned u = (unsigned)s, row = u / (unsigned)nx;
+  x = (int)(u - row * (unsigned)nx);
+  z = (int)(row / (unsigned)ny);
+  y = (int)(row - (unsigned)z * (unsigned)ny);
+}
+
 // ------------------------------------------------------- elementwise ---
 // 2x2x2 average pooling, children summed in a fixed order.
 template <int C>
@@ -745,7 +754,8 @@ __global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int 
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int j = (int)(i % NCH);
     const long long s = i / NCH;
-    const int X = (int)(s % Wc), Y = (int)((s / Wc) % Hc), Z = (int)(s / ((long long)Wc * Hc));
+    int X, Y, Z;
+    site_xyz(s, Wc, Hc, X, Y, Z);
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
@@ -817,7 +827,8 @@ __global__ void __launch_bounds__(kEwThreads) k_combine(const float* __restrict_
     const __nv_bfloat162* py = reinterpret_cast<const __nv_bfloat162*>(&yv);
     float gv[8];
     if (POOL) {
-      const int x = (int)(s % W), yy = (int)((s / W) % H), z = (int)(s / ((long long)W * H));
+      int x, yy, z;
+      site_xyz(s, W, H, x, yy, z);
       const long long ps = (((long long)(z >> 1) * (H >> 1) + (yy >> 1)) * (W >> 1) + (x >> 1));
       const float4 g0 = *reinterpret_cast<const float4*>(graw + ps * C + j * 8);
       const float4 g1 = *reinterpret_cast<const float4*>(graw + ps * C + j * 8 + 4);
@@ -944,21 +955,30 @@ __global__ void k_target(const float* __restrict__ Kp, const float* __restrict__
     t[i] = scale * (Kn[i] - Kp[i]);
 }
 
+// The parameters in FP32, converted on the host: a thread of these kernels has
+// a site or two, and its FP64 conversions and division took longer than both.
+struct FeatureF {
+  float cpl, phi_K, K1, r_K, K0, b;
+};
+inline FeatureF feature_f(const FeatureArgs& f) {
+  return FeatureF{(float)(f.D_K / (f.dx * f.dx)), (float)f.phi_K, (float)f.K1, (float)f.r_K, (float)f.K0, (float)(f.r_K * f.K0)};
+}
+
 // Residual loss L = mean(u^2), u = A e / c, e = out - target, A the oxygen
 // operator lagged at K_prev (dense lattice), c = D_K / dx^2.
-__device__ __forceinline__ float o2_diag(const FeatureArgs& f, const float* __restrict__ Kp, long long e, int cnt,
-                                         float cpl) {
+__device__ __forceinline__ float o2_diag(const FeatureArgs& f, const FeatureF& c, const float* __restrict__ Kp, long long e,
+                                         int cnt) {
   const uint8_t st = f.state[e];
   const bool consumer = st == HCA_PROLIF || st == HCA_QUIESC || st == HCA_STROMA;
-  const float reac = (consumer ? (float)f.phi_K / ((float)f.K1 + Kp[e]) : 0.f) + (st == HCA_VESSEL ? (float)f.r_K : 0.f);
-  return cpl * (float)cnt + reac;
+  const float reac = (consumer ? c.phi_K / (c.K1 + Kp[e]) : 0.f) + (st == HCA_VESSEL ? c.r_K : 0.f);
+  return c.cpl * (float)cnt + reac;
 }
 
 // v = (A w) / c on the dense lattice, w = a - b (b may be null).
-__device__ __forceinline__ float apply_scaled(const FeatureArgs& f, const float* __restrict__ Kp,
-                                              const float* __restrict__ a, const float* __restrict__ b, long long s,
-                                              float cpl) {
-  const int xx = (int)(s % f.nx), yy = (int)((s / f.nx) % f.ny), zz = (int)(s / ((long long)f.nx * f.ny));
+__device__ __forceinline__ float apply_scaled(const FeatureArgs& f, const FeatureF& c, const float* __restrict__ Kp,
+                                              const float* __restrict__ a, const float* __restrict__ b, long long s) {
+  int xx, yy, zz;
+  site_xyz(s, f.nx, f.ny, xx, yy, zz);
   const long long sy = f.nx, sz = (long long)f.nx * f.ny;
   auto w = [&](long long i) { return b ? a[i] - b[i] : a[i]; };
   float nb = 0.f;
@@ -969,19 +989,18 @@ __device__ __forceinline__ float apply_scaled(const FeatureArgs& f, const float*
   if (yy < f.ny - 1) { nb += w(s + sy); ++cnt; }
   if (zz > 0) { nb += w(s - sz); ++cnt; }
   if (zz < f.nz - 1) { nb += w(s + sz); ++cnt; }
-  const float d = o2_diag(f, Kp, s, cnt, cpl);
-  return (d * w(s) - cpl * nb) / cpl;
+  const float d = o2_diag(f, c, Kp, s, cnt);
+  return (d * w(s) - c.cpl * nb) / c.cpl;
 }
 
-__global__ void __launch_bounds__(kEwThreads) k_res_u(FeatureArgs f, const float* __restrict__ Kp,
+__global__ void __launch_bounds__(kEwThreads) k_res_u(FeatureArgs f, FeatureF c, const float* __restrict__ Kp,
                                                       const float* __restrict__ out, const float* __restrict__ tgt,
                                                       float* __restrict__ u, float* __restrict__ part) {
   __shared__ float sb[kEwThreads / 32];
   const long long n = (long long)f.nx * f.ny * f.nz;
-  const float cpl = (float)(f.D_K / (f.dx * f.dx));
   float acc = 0.f;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-    const float v = apply_scaled(f, Kp, out, tgt, s, cpl);
+    const float v = apply_scaled(f, c, Kp, out, tgt, s);
     u[s] = v;
     acc += v * v;
   }
@@ -991,20 +1010,19 @@ __global__ void __launch_bounds__(kEwThreads) k_res_u(FeatureArgs f, const float
 
 // dL/dout of L = w_mse mean(e^2) + w_res mean(u^2):
 //   2 w_mse e / N + 2 w_res (A u) / (c N); per-block sums of e^2 into part.
-__global__ void __launch_bounds__(kEwThreads) k_loss_grad(FeatureArgs f, const float* __restrict__ Kp,
+__global__ void __launch_bounds__(kEwThreads) k_loss_grad(FeatureArgs f, FeatureF c, const float* __restrict__ Kp,
                                                           const float* __restrict__ out, const float* __restrict__ tgt,
                                                           const float* __restrict__ u, float w_mse, float w_res,
                                                           float* __restrict__ g, float* __restrict__ part) {
   __shared__ float sb[kEwThreads / 32];
   const long long n = (long long)f.nx * f.ny * f.nz;
-  const float cpl = (float)(f.D_K / (f.dx * f.dx));
   const float sc = 2.0f / (float)n;
   float acc = 0.f;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
     const float e = out[s] - tgt[s];
     acc += e * e;
     float v = w_mse * sc * e;
-    if (w_res != 0.f) v += w_res * sc * apply_scaled(f, Kp, u, nullptr, s, cpl);
+    if (w_res != 0.f) v += w_res * sc * apply_scaled(f, c, Kp, u, nullptr, s);
     g[s] = v;
   }
   acc = block_sum<kEwThreads>(acc, sb);
@@ -1068,12 +1086,12 @@ __global__ void k_quantize(const float* __restrict__ params, QuantTable T, bf16*
 // lagged at K_prev (7-point stencil, homogeneous Neumann), zeros.  Fields are
 // read with a row pitch (the solver's padded layout or dense); x is dense.
 template <typename T>
-__global__ void k_features(FeatureArgs f, const T* __restrict__ K, bf16* __restrict__ x) {
+__global__ void k_features(FeatureArgs f, FeatureF c, const T* __restrict__ K, bf16* __restrict__ x) {
   const long long n = (long long)f.nx * f.ny * f.nz;
   const long long sy = f.pitch, sz = (long long)f.pitch * f.ny;
-  const float cpl = (float)(f.D_K / (f.dx * f.dx));
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-    const int xx = (int)(s % f.nx), yy = (int)((s / f.nx) % f.ny), zz = (int)(s / ((long long)f.nx * f.ny));
+    int xx, yy, zz;
+    site_xyz(s, f.nx, f.ny, xx, yy, zz);
     const long long e = f.base + xx + sy * yy + sz * zz;
     const uint8_t st = f.state[e];
     const float k = (float)K[e];
@@ -1087,17 +1105,17 @@ __global__ void k_features(FeatureArgs f, const T* __restrict__ K, bf16* __restr
     if (zz < f.nz - 1) { nb += (float)K[e + sz]; ++cnt; }
     const bool consumer = st == HCA_PROLIF || st == HCA_QUIESC || st == HCA_STROMA;
     const bool vessel = st == HCA_VESSEL;
-    const float reac = (consumer ? (float)f.phi_K / ((float)f.K1 + k) : 0.f) + (vessel ? (float)f.r_K : 0.f);
-    const float d = cpl * (float)cnt + reac;
-    const float b = vessel ? (float)(f.r_K * f.K0) : 0.f;
-    const float r = b - (d * k - cpl * nb);
-    const float ch8 = d != 0.f ? (float)kNetScale * r / (d * (float)f.K0) : 0.f;
+    const float reac = (consumer ? c.phi_K / (c.K1 + k) : 0.f) + (vessel ? c.r_K : 0.f);
+    const float d = c.cpl * (float)cnt + reac;
+    const float b = vessel ? c.b : 0.f;
+    const float r = b - (d * k - c.cpl * nb);
+    const float ch8 = d != 0.f ? (float)kNetScale * r / (d * c.K0) : 0.f;
     uint4 o[2];
     uint32_t* po = reinterpret_cast<uint32_t*>(o);
     po[0] = pack_bf2(st == 0 ? 1.f : 0.f, st == 1 ? 1.f : 0.f);
     po[1] = pack_bf2(st == 2 ? 1.f : 0.f, st == 3 ? 1.f : 0.f);
     po[2] = pack_bf2(st == 4 ? 1.f : 0.f, st == 5 ? 1.f : 0.f);
-    po[3] = pack_bf2((float)static_cast<const T*>(f.perf)[e], k / (float)f.K0);
+    po[3] = pack_bf2((float)static_cast<const T*>(f.perf)[e], k / c.K0);
     po[4] = pack_bf2(ch8, 0.f);
     po[5] = po[6] = po[7] = 0u;
     reinterpret_cast<uint4*>(x + s * 16)[0] = o[0];
@@ -1114,7 +1132,8 @@ __global__ void k_ws_candidate(FeatureArgs f, const T* __restrict__ K, const flo
   const long long n = (long long)f.nx * f.ny * f.nz;
   const long long sy = f.pitch, sz = (long long)f.pitch * f.ny;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-    const int xx = (int)(s % f.nx), yy = (int)((s / f.nx) % f.ny), zz = (int)(s / ((long long)f.nx * f.ny));
+    int xx, yy, zz;
+    site_xyz(s, f.nx, f.ny, xx, yy, zz);
     const long long e = f.base + xx + sy * yy + sz * zz;
     const double kp = (double)K[e] + (K_lo ? (double)K_lo[e] : 0.0);
     cand[e] = kp + f.K0 / kNetScale * (double)out[s];
@@ -1135,7 +1154,8 @@ __global__ void __launch_bounds__(kEwThreads) k_ws_norms(FeatureArgs f, const T*
   double a0 = 0.0, a1 = 0.0, a2 = 0.0;
   auto kp = [&](long long e) { return (double)K[e] + (K_lo ? (double)K_lo[e] : 0.0); };
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-    const int xx = (int)(s % f.nx), yy = (int)((s / f.nx) % f.ny), zz = (int)(s / ((long long)f.nx * f.ny));
+    int xx, yy, zz;
+    site_xyz(s, f.nx, f.ny, xx, yy, zz);
     const long long e = f.base + xx + sy * yy + sz * zz;
     const uint8_t st = f.state[e];
     const double k = kp(e);
@@ -1193,7 +1213,8 @@ __global__ void k_ws_apply(FeatureArgs f, const WsResult* __restrict__ res, cons
   const long long n = (long long)f.nx * f.ny * f.nz;
   const long long sy = f.pitch, sz = (long long)f.pitch * f.ny;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-    const int xx = (int)(s % f.nx), yy = (int)((s / f.nx) % f.ny), zz = (int)(s / ((long long)f.nx * f.ny));
+    int xx, yy, zz;
+    site_xyz(s, f.nx, f.ny, xx, yy, zz);
     const long long e = f.base + xx + sy * yy + sz * zz;
     const double c = cand[e];
     const T hi = (T)c;
@@ -1629,7 +1650,7 @@ void quantize(hca_net* n, cudaStream_t s) {
 
 template <typename T>
 void features(hca_net* n, cudaStream_t s, const FeatureArgs& f, const T* K) {
-  k_features<T><<<ew_blocks(n->Ln[0], n->sm_count), kEwThreads, 0, s>>>(f, K, n->x);
+  k_features<T><<<ew_blocks(n->Ln[0], n->sm_count), kEwThreads, 0, s>>>(f, feature_f(f), K, n->x);
 }
 
 // A kernel's bounded wait gave up (seen by the calls that wait for the GPU,
@@ -1920,8 +1941,8 @@ int hca_net_gradients(hca_net* n, const hca_config* cfg, const uint8_t* state, c
   features<float>(n, s, f, K_prev);
   k_target<<<nb, kEwThreads, 0, s>>>(K_prev, K_new, n->Ln[0], (float)(kNetScale / cfg->K0), n->tgt);
   forward(n, s, true);
-  k_res_u<<<nr, kEwThreads, 0, s>>>(f, K_prev, n->out, n->tgt, n->ru, n->bpart);
-  k_loss_grad<<<nr, kEwThreads, 0, s>>>(f, K_prev, n->out, n->tgt, n->ru, (float)w_mse, (float)w_res, n->rg,
+  k_res_u<<<nr, kEwThreads, 0, s>>>(f, feature_f(f), K_prev, n->out, n->tgt, n->ru, n->bpart);
+  k_loss_grad<<<nr, kEwThreads, 0, s>>>(f, feature_f(f), K_prev, n->out, n->tgt, n->ru, (float)w_mse, (float)w_res, n->rg,
                                         n->bpart + n->bpart_blocks);
   k_sum_loss<<<1, kEwThreads, 0, s>>>(n->bpart, nr, (float)w_res / (float)n->Ln[0], n->bpart + n->bpart_blocks,
                               (float)w_mse / (float)n->Ln[0], n->loss);
