@@ -14,17 +14,18 @@
 // MG_NU_COARSE sweeps of weight MG_OMEGA_COARSE on the coarsest level), so M
 // is symmetric.
 //
-// Level 0 is the solver's padded field layout: rhs = r, diagonal = d, 1/d in
-// mg_w; z holds the pre-smoothed iterate v between the pre-sweep kernel and
-// the restriction, mg_t0 the part v' of the first post-sweep that the
-// restriction leaves for the post-sweep kernels (or the iterate when the
-// lattice is the coarsest level); coarser levels are dense arrays, the replicates of a batch
-// concatenated per level (each replicate has its own hierarchy; a per-level
-// prefix table maps a flattened site index to its replicate).  Levels of at
-// most MG_SMALL_SITES sites run inside one block per replicate (block
-// barriers between sweeps).  The last kernel, the last post-sweep on level 0,
-// also forms rho = r.z with the fixed-order reductions of the CG passes and
-// sets beta, per replicate.
+// Level 0 is the solver's padded field layout; coarser levels are dense arrays
+// with rows of whole 4-site groups, the replicates of a batch concatenated per
+// level (each replicate has its own hierarchy).  FP32 hierarchies run in the
+// marching kernels (march.cu) and the coarse-level clusters (coarse.cu); here
+// are the diagonals of both precisions, the FP64 sweeps, and the FP32 lattice
+// that is its own coarsest level.  FP64: z holds the pre-smoothed iterate v
+// between the pre-sweep kernel and the restriction, mg_t0 the part v' of the
+// first post-sweep that the restriction leaves for the post-sweep kernels; a
+// per-level prefix table maps a flattened site index to its replicate; levels
+// of at most MG_SMALL_SITES sites run inside one block per replicate; the last
+// post-sweep on level 0 also forms rho = r.z with the fixed-order reductions
+// of the CG passes and sets beta, per replicate.
 
 #include <algorithm>
 #include <cstdlib>

@@ -17,9 +17,10 @@
 // swizzle modes leave ldmatrix's row gathers free of bank conflicts, and every
 // warp runs mma.m16n8k16 BF16 -> FP32 over its rows.  The nearest 2x upsampling
 // of the decoder is folded into the halo's coordinates; the sum over the 2x2x2
-// children that its gradient needs is folded into the epilogue.
+// children that its gradient needs and the encoder's 2x2x2 pooling are folded
+// into the epilogue.
 //
-// Bound (forward at 128^3, 135 GFLOP, 431 us): the mma.sync pipe, which peaks
+// Bound (forward at 128^3, 135 GFLOP, 414 us): the mma.sync pipe, which peaks
 // at 600 TFLOP/s on this chip (225 us), with the halo's traffic exposed where
 // two or three blocks fit a multiprocessor: dec0 129 us, enc0 83, dec1 68.
 // (One ldmatrix of the input per tap and tile, weights staged between barriers
@@ -118,14 +119,32 @@ __device__ __forceinline__ uint32_t pack_bf2(float lo, float hi) {
 }
 
 // ----------------------------------------------------- forward / dgrad ---
-enum { EPI_FWD = 0, EPI_HEAD = 1, EPI_RAW = 2, EPI_DOWN = 3 };
+enum { EPI_FWD = 0, EPI_HEAD = 1, EPI_RAW = 2, EPI_DOWN = 3, EPI_POOL = 4 };   // EPI_POOL: EPI_FWD and its 2x2x2 means
+
+// Adds 8 BF16 values; a 2x2x2 mean of 8 channels.
+__device__ __forceinline__ void add_bf8(float (&acc)[8], uint4 v) {
+  const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    acc[2 * e] += __low2float(p[e]);
+    acc[2 * e + 1] += __high2float(p[e]);
+  }
+}
+__device__ __forceinline__ uint4 mean_bf8(const float (&acc)[8]) {
+  uint4 o;
+  uint32_t* po = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) po[e] = pack_bf2(acc[2 * e] * 0.125f, acc[2 * e + 1] * 0.125f);
+  return o;
+}
 
 struct ConvArgs {
   const bf16* in;      // input (Di, Hi, Wi, CI)
   const bf16* w;       // weights (27, CO, CI)
   const float* bias;   // CO (EPI_FWD / EPI_HEAD)
   const bf16* skip;    // (D, H, W, CO) or null
-  bf16* out;           // (D, H, W, CO) (EPI_FWD; EPI_HEAD: optional)
+  bf16* out;           // (D, H, W, CO) (EPI_FWD, EPI_POOL; EPI_HEAD: optional)
+  bf16* out_p;         // (D/2, H/2, W/2, CO) (EPI_POOL)
   float* out_f;        // EPI_HEAD: (D, H, W); EPI_RAW: (D, H, W, CO); EPI_DOWN: (D/2, H/2, W/2, CO)
   const float* head_w; // 16 (EPI_HEAD)
   const float* head_b; // 1 (EPI_HEAD)
@@ -160,6 +179,7 @@ struct ConvTile {
   static constexpr int HALO = S * PHASE * CI * 2;
   static constexpr int RED = EPI == 3 ? (ROWS * (XO / 2) * CB * 4 + 1023) / 1024 * 1024 : 0;
   static constexpr int WPLANE = 9 * CB * CI * 2;
+  static_assert(EPI != 4 || ROWS * XO * CB * 2 <= HALO, "the outputs to be pooled fit the halo's place");
   static constexpr int SMEM = (HALO > RED ? HALO : RED) + 2 * WPLANE + 16;   // (and two barriers)
   static constexpr int PER_SM = 232448 / (SMEM + 1024);
   // blocks of 8 warps the accumulators and shared fragments leave registers for
@@ -168,7 +188,7 @@ struct ConvTile {
   static constexpr int MIN_BLOCKS = PER_SM < FIT ? PER_SM : FIT;
   static_assert(PHASE % 8 == 0, "a phase starts where the swizzle pattern does");
   static_assert(TZ >= 2 && TZ % 2 == 0 && CB % 16 == 0 && CO % CB == 0, "tile shape");
-  static_assert(!(UP && EPI == 3) && (EPI != 1 || CB == CO), "epilogue");
+  static_assert(!(UP && (EPI == 3 || EPI == 4)) && (EPI != 1 || CB == CO), "epilogue");
 };
 
 // The tensor maps of a convolution's inputs: the activations by phase of x
@@ -364,6 +384,9 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
     return;
   }
 
+  // EPI_POOL: the block's outputs, [row][tile][j][channel], over the halo
+  char* pool = smem;
+  if (EPI == EPI_POOL) __syncthreads();   // (the halo is no longer read)
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int rr = warp * R + r;
@@ -394,7 +417,10 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
           }
           v0 = fmaxf(v0, 0.f);
           v1 = fmaxf(v1, 0.f);
-          if (ok && a.out) *reinterpret_cast<uint32_t*>(a.out + site * CO + co) = pack_bf2(v0, v1);
+          const uint32_t packed = pack_bf2(v0, v1);
+          if (ok && a.out) *reinterpret_cast<uint32_t*>(a.out + site * CO + co) = packed;
+          if (EPI == EPI_POOL)
+            *reinterpret_cast<uint32_t*>(pool + (((rr * M + m) * 16 + (lane >> 2) + 8 * hf) * CB + n * 8 + cq) * 2) = packed;
           if (EPI == EPI_HEAD) head += bfr(v0) * a.head_w[co] + bfr(v1) * a.head_w[co + 1];
         }
         if (EPI == EPI_HEAD) {
@@ -403,6 +429,25 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
           if (ok && (lane & 3) == 0) a.out_f[site] = head + a.head_b[0];
         }
       }
+  }
+  if (EPI != EPI_POOL) return;
+  // 2x2x2 means of the BF16 outputs, children summed in the order of k_pool
+  __syncthreads();
+  constexpr int XH = T::XO / 2, PC = CB / 8, NPOOL = (T::TZ / 2) * (kTY / 2) * XH * PC;
+  const int Dc = a.D >> 1, Hc = a.H >> 1, Wc = a.W >> 1;
+  for (int i = threadIdx.x; i < NPOOL; i += 32 * NW) {
+    const int ch = i % PC, xp = (i / PC) % XH, cy = (i / (PC * XH)) % (kTY / 2), cz = i / (PC * XH * (kTY / 2));
+    const int Z = (z0 >> 1) + cz, Y = (y0 >> 1) + cy, X = (x0 >> 1) + xp;
+    if (Z >= Dc || Y >= Hc || X >= Wc) continue;
+    float sum[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) sum[e] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int rr = (2 * cz + (c >> 2)) * kTY + 2 * cy + ((c >> 1) & 1), x = 2 * xp + (c & 1);
+      add_bf8(sum, *reinterpret_cast<const uint4*>(pool + (((rr * M + x % S) * 16 + x / S) * CB + ch * 8) * 2));
+    }
+    *reinterpret_cast<uint4*>(a.out_p + (((long long)Z * Hc + Y) * Wc + X) * CO + co0 + ch * 8) = mean_bf8(sum);
   }
 }
 
@@ -762,19 +807,9 @@ __global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int 
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       const int z = 2 * Z + (c >> 2), y = 2 * Y + ((c >> 1) & 1), x = 2 * X + (c & 1);
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(in + (((long long)z * H + y) * W + x) * C) + j);
-      const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        acc[2 * e] += __low2float(p[e]);
-        acc[2 * e + 1] += __high2float(p[e]);
-      }
+      add_bf8(acc, __ldg(reinterpret_cast<const uint4*>(in + (((long long)z * H + y) * W + x) * C) + j));
     }
-    uint4 o;
-    uint32_t* po = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) po[e] = pack_bf2(acc[2 * e] * 0.125f, acc[2 * e + 1] * 0.125f);
-    *reinterpret_cast<uint4*>(out + s * C + j * 8) = o;
+    *reinterpret_cast<uint4*>(out + s * C + j * 8) = mean_bf8(acc);
   }
 }
 
@@ -1359,9 +1394,9 @@ int wgrad_attr() {
 
 int set_attributes() {
   int rc = 0;
-  if ((rc = conv_attr<16, 16, false, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<16, 32, false, EPI_FWD>())) return rc;
-  if ((rc = conv_attr<32, 64, false, EPI_FWD>())) return rc;
+  if ((rc = conv_attr<16, 16, false, EPI_POOL>())) return rc;
+  if ((rc = conv_attr<16, 32, false, EPI_POOL>())) return rc;
+  if ((rc = conv_attr<32, 64, false, EPI_POOL>())) return rc;
   if ((rc = conv_attr<64, 64, false, EPI_FWD>())) return rc;
   if ((rc = conv_attr<64, 64, true, EPI_FWD>())) return rc;
   if ((rc = conv_attr<64, 32, true, EPI_FWD>())) return rc;
@@ -1469,11 +1504,12 @@ void conv_launch(cudaStream_t s, const ConvArgs& a, const ConvMaps& maps, int* s
 // One convolution launch on the inputs of maps[slot]; the output lattice is level lvl.
 template <int CI, int CO, bool UP, int EPI>
 void conv(hca_net* n, cudaStream_t s, int slot, const float* bias, const bf16* skip, bf16* out, float* out_f,
-          const float* hw, const float* hb, int lvl) {
+          const float* hw, const float* hb, int lvl, bf16* out_p = nullptr) {
   ConvArgs a{};
   a.bias = bias;
   a.skip = skip;
   a.out = out;
+  a.out_p = out_p;
   a.out_f = out_f;
   a.head_w = hw;
   a.head_b = hb;
@@ -1548,9 +1584,9 @@ const float* Bias(hca_net* n, int l) { return n->params + n->L.b_off[l]; }
 
 // The tensor maps of every convolution (the net's arrays are allocated).
 bool prepare_convs(hca_net* n) {
-  const bool fwd = conv_prepare<16, 16, false, EPI_FWD>(n, 0, n->x, Wq(n, 0), 0) &&
-                   conv_prepare<16, 32, false, EPI_FWD>(n, 1, n->p0, Wq(n, 1), 1) &&
-                   conv_prepare<32, 64, false, EPI_FWD>(n, 2, n->p1, Wq(n, 2), 2) &&
+  const bool fwd = conv_prepare<16, 16, false, EPI_POOL>(n, 0, n->x, Wq(n, 0), 0) &&
+                   conv_prepare<16, 32, false, EPI_POOL>(n, 1, n->p0, Wq(n, 1), 1) &&
+                   conv_prepare<32, 64, false, EPI_POOL>(n, 2, n->p1, Wq(n, 2), 2) &&
                    conv_prepare<64, 64, false, EPI_FWD>(n, 3, n->p2, Wq(n, 3), 3) &&
                    conv_prepare<64, 64, true, EPI_FWD>(n, 4, n->e3, Wq(n, 4), 2) &&
                    conv_prepare<64, 32, true, EPI_FWD>(n, 5, n->d2, Wq(n, 5), 1) &&
@@ -1576,16 +1612,14 @@ void forward(hca_net* n, cudaStream_t s, bool keep_d0) {
   const int* D = n->Ld;
   const int* H = n->Lh;
   const int* W = n->Lw;
-  if (n->use_tc)
+  if (n->use_tc) {
     conv_tc<16, 16, 4, false, EPI_FWD>(s, n->status, n->x, Wq(n, 0), Bias(n, 0), nullptr, n->e0, nullptr, nullptr,
                                        nullptr, D[0], H[0], W[0]);
-  else
-    conv<16, 16, false, EPI_FWD>(n, s, 0, Bias(n, 0), nullptr, n->e0, nullptr, nullptr, nullptr, 0);
-  pool<16>(n, s, n->e0, n->p0, 0);
-  conv<16, 32, false, EPI_FWD>(n, s, 1, Bias(n, 1), nullptr, n->e1, nullptr, nullptr, nullptr, 1);
-  pool<32>(n, s, n->e1, n->p1, 1);
-  conv<32, 64, false, EPI_FWD>(n, s, 2, Bias(n, 2), nullptr, n->e2, nullptr, nullptr, nullptr, 2);
-  pool<64>(n, s, n->e2, n->p2, 2);
+    pool<16>(n, s, n->e0, n->p0, 0);
+  } else
+    conv<16, 16, false, EPI_POOL>(n, s, 0, Bias(n, 0), nullptr, n->e0, nullptr, nullptr, nullptr, 0, n->p0);
+  conv<16, 32, false, EPI_POOL>(n, s, 1, Bias(n, 1), nullptr, n->e1, nullptr, nullptr, nullptr, 1, n->p1);
+  conv<32, 64, false, EPI_POOL>(n, s, 2, Bias(n, 2), nullptr, n->e2, nullptr, nullptr, nullptr, 2, n->p2);
   conv<64, 64, false, EPI_FWD>(n, s, 3, Bias(n, 3), nullptr, n->e3, nullptr, nullptr, nullptr, 3);
   conv<64, 64, true, EPI_FWD>(n, s, 4, Bias(n, 4), n->e2, n->d2, nullptr, nullptr, nullptr, 2);
   conv<64, 32, true, EPI_FWD>(n, s, 5, Bias(n, 5), n->e1, n->d1, nullptr, nullptr, nullptr, 1);

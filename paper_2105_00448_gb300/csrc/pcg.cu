@@ -15,16 +15,14 @@
 //   pass B: x += alpha p;  z -= alpha q / d;  rho = r.z = sum d z^2,
 //           |r|^2 = sum (d z)^2  (multigrid form: r -= alpha q, |r|^2; the
 //           V-cycle then forms z = M r and rho)
-// HBM traffic per site and iteration: pass A reads z, p, d and writes p and
-// q (20 B, FP32); pass B reads p, q, x, z (+ d, Jacobi form) and writes x, z
-// (24-28 B): 44 B, against the two-pass minimum of 40 B in which pass B
-// re-forms A p from p's neighbour rows instead of streaming q.
-// Neighbour rows are re-read through L1/L2.  Pass A rebuilds the new
-// direction at neighbour sites from the old one, so the old and new
-// directions live in two buffers that swap roles every iteration (an in-place
-// update would let one block read a neighbour row another block has already
-// overwritten); a parity bit in device memory, flipped by pass B, names the
-// current buffer, so the same two kernels form the body of a graph loop.
+// The row kernels here are the FP64 passes (FP32: cg.cu), the set-up, the
+// residual of a finished solve, and what FP32's defect correction does
+// besides its residual sweep (dc.cu).  Pass A rebuilds the new direction at
+// neighbour sites from the old one, so the old and new directions live in two
+// buffers that swap roles every iteration (an in-place update would let one
+// block read a neighbour row another block has already overwritten); a parity
+// bit in device memory, flipped by pass B, names the current buffer, so the
+// same two kernels form the body of a graph loop.
 #include <vector>
 
 #include <cstdlib>
