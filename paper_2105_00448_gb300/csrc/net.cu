@@ -158,6 +158,9 @@ __device__ __forceinline__ void cp_async16_zfill(void* sdst, const void* gsrc, i
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(sdst)), "l"(gsrc), "r"(src_bytes)
                : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(sdst)), "l"(gsrc) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -610,32 +613,37 @@ __global__ void __launch_bounds__(128) k_conv_tc(const ConvArgs a, int* status) 
 
 // ------------------------------------------------------------- wgrad ---
 // dW[t, co, ci] = sum over sites m of gy[m, co] x[m + off_t, ci] (x = the
-// layer input, upsampled on the fly when UP).  M = 16 co, N = up to 32 ci (a
-// tile per blockIdx.y), K = sites.  The nine warps of a block own one (dz, dy)
-// each with its three dx; along x the sites of a row are S interleaved groups
-// of 16 (upsampled: two per phase, one per parity), so a fragment of x serves
-// all three taps and a fragment of gy all of them.  Tiles (8 rows) arrive by
-// tensor copies, one ahead; blocks along x split them and write FP32 partials
-// that a second kernel sums in a fixed order.  Bound: the MMAs and, at the
-// coarse levels, latency.  All seven layers at 64^3:
-// 90 us (dec0's 25), against 195 (69) with fragments loaded per tap.
-template <int CI, int CO, int S, bool UP>
+// layer input, upsampled on the fly when UP).  M = 16 co, N = 16 ci (a tile
+// per blockIdx.y), K = 16 consecutive sites of x.  The nine warps of a block
+// own one (dz, dy) each with its three dx, so a fragment of gy serves three
+// taps.  Tiles (8 rows of 16 sites) arrive by tensor copies, three ahead;
+// blocks along x split them and write FP32 partials that a second kernel sums.
+//
+// The order of the sums is part of a training run's result (Adam divides by
+// sqrt(v), so a last bit grows from step to step): 16 consecutive sites an
+// instruction, the rows and tiles of a partial in order, then the partials in
+// order, their number following the layer (wgrad).  Interleaved site groups
+// whose x fragments serve several taps are faster but sum in another order.
+// Bound: the fragment loads, and latency at the coarse levels.  All seven
+// layers at 64^3: 97 us (dec0's 31), against 195 (69) with the tile staged
+// between barriers and the nine (dz, dy) sharing no fragment; 90 (25) with
+// interleaved groups.
+template <int CI, int CO, bool UP>
 struct WgTile {
-  static constexpr int CB = CI < 32 ? CI : 32;   // input channels of a block
-  static constexpr int TZ = 2, ROWS = TZ * kTY, M = (UP ? 2 : 1) * S, XO = 16 * M, LP = 18;
+  static constexpr int CB = 16;   // input channels of a block
+  static constexpr int TZ = 2, ROWS = TZ * kTY, XO = 16, LP = UP ? 10 : 18;
   static constexpr int HZ = UP ? TZ / 2 + 2 : TZ + 2, HY = UP ? kTY / 2 + 2 : kTY + 2;
-  static constexpr int PHASE = HZ * HY * LP, HALO = S * PHASE * CB * 2;
-  static constexpr int GROUP = ROWS * 16, GY = M * GROUP * 16 * 2;   // sites, bytes
-  static constexpr int STAGE = HALO + GY, SMEM = 2 * STAGE + 16;
-  static constexpr int PER_SM = 232448 / (SMEM + 1024) < 3 ? 232448 / (SMEM + 1024) : 3;   // (registers: 72 a thread)
-  static_assert(PHASE % 8 == 0 && HALO % (16 * CB) == 0 && STAGE % (16 * CB) == 0 && HALO % 256 == 0,
-                "phases, groups and stages start where the swizzle patterns do (8 rows)");
+  static constexpr int HALO = HZ * HY * LP * CB * 2, GY = ROWS * 16 * 16 * 2;   // bytes
+  static constexpr int RING = 4, STAGE = HALO + GY, SMEM = RING * STAGE + 8 * RING;
+  static constexpr int PER_SM = 3;   // (registers: 72 a thread)
+  static_assert(HALO % 256 == 0 && STAGE % 256 == 0, "arrays start where the swizzle pattern does (8 rows)");
+  static_assert(PER_SM * (SMEM + 1024) <= 232448, "blocks per multiprocessor");
 };
 
-// Tensor maps of a layer's weight gradient: the input by phase of x, the
-// output's gradient by site group (box: 16 channels of a tile's rows).
+// Tensor maps of a layer's weight gradient: the input (box: CB channels of a
+// tile's halo) and the output's gradient (box: 16 channels of a tile).
 struct WgMaps {
-  CUtensorMap in[2], gy[4];
+  CUtensorMap in, gy;
 };
 
 struct WgArgs {
@@ -645,34 +653,33 @@ struct WgArgs {
 
 constexpr int kWgThreads = 288;
 
-template <int CI, int CO, int S, bool UP>
-__global__ void __launch_bounds__(kWgThreads, (WgTile<CI, CO, S, UP>::PER_SM))
+template <int CI, int CO, bool UP>
+__global__ void __launch_bounds__(kWgThreads, (WgTile<CI, CO, UP>::PER_SM))
     k_wgrad(const WgArgs a, const __grid_constant__ WgMaps maps, int* status) {
-  using T = WgTile<CI, CO, S, UP>;
-  constexpr int CB = T::CB, NT = CB / 8, M = T::M;
+  using T = WgTile<CI, CO, UP>;
+  constexpr int CB = T::CB, NT = CB / 8, RING = T::RING;
   extern __shared__ __align__(1024) char smem[];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * T::STAGE);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + RING * T::STAGE);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int q = lane >> 3;
   const int dz = warp / 3 - 1, dy = warp % 3 - 1, mt = blockIdx.y % (CO / 16), c0 = (int)(blockIdx.y / (CO / 16)) * CB;
   const int n_tiles = a.tiles_x * a.tiles_y * a.tiles_z;
-  auto fetch = [&](int tile, int st) {
+  // this block's k-th tile, into stage k mod RING
+  const int mine = (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  auto fetch = [&](int k) {
+    const int tile = (int)blockIdx.x + k * (int)gridDim.x, st = k % RING;
     const int bx = tile % a.tiles_x, by = (tile / a.tiles_x) % a.tiles_y, bz = tile / (a.tiles_x * a.tiles_y);
-    const int z0 = bz * T::TZ, y0 = by * kTY;
+    const int z0 = bz * T::TZ, y0 = by * kTY, x0 = bx * T::XO;
     const uint32_t b = smem_u32(&bar[st]), d = smem_u32(smem) + st * T::STAGE;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"((uint32_t)T::STAGE) : "memory");
-    const int oz = UP ? (z0 >> 1) - 1 : z0 - 1, oy = UP ? (y0 >> 1) - 1 : y0 - 1;
-    for (int p = 0; p < S; ++p)   // (the tile starts at input site 16 S bx)
-      tma_box_4d(d + p * (T::PHASE * CB * 2), &maps.in[p], c0, 16 * bx - 1, oy, oz, b);
-    for (int m = 0; m < M; ++m)
-      tma_box_4d(d + T::HALO + m * (T::GROUP * 32), &maps.gy[m], 16 * mt, 16 * bx, y0, z0, b);
+    tma_box_4d(d, &maps.in, c0, (UP ? x0 >> 1 : x0) - 1, (UP ? y0 >> 1 : y0) - 1, (UP ? z0 >> 1 : z0) - 1, b);
+    tma_box_4d(d + T::HALO, &maps.gy, 16 * mt, x0, y0, z0, b);
   };
   if (threadIdx.x == 0) {
-    tc::mbar_init(&bar[0], 1);
-    tc::mbar_init(&bar[1], 1);
+    for (int k = 0; k < RING; ++k) tc::mbar_init(&bar[k], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if ((int)blockIdx.x < n_tiles) fetch(blockIdx.x, 0);
+    for (int k = 0; k < RING - 1 && k < mine; ++k) fetch(k);
   }
   float acc[3][NT][4];
 #pragma unroll
@@ -682,48 +689,37 @@ __global__ void __launch_bounds__(kWgThreads, (WgTile<CI, CO, S, UP>::PER_SM))
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][n][e] = 0.f;
   __syncthreads();
-  int it = 0;
-  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
-    const int st = it & 1;
-    if (threadIdx.x == 0 && tile + (int)gridDim.x < n_tiles) fetch(tile + gridDim.x, st ^ 1);
-    const bool ok = tc::mbar_wait(&bar[st], (uint32_t)(it >> 1) & 1u, kConvWaitLimit);
+  for (int it = 0; it < mine; ++it) {
+    const int st = it % RING;
+    if (threadIdx.x == 0 && it + RING - 1 < mine) fetch(it + RING - 1);   // (its stage was freed by the tile before)
+    const bool ok = tc::mbar_wait(&bar[st], (uint32_t)(it / RING) & 1u, kConvWaitLimit);
     if (!__syncthreads_and(ok)) {   // (the same in every thread)
       if (threadIdx.x == 0) {
         *(volatile int*)status = 1;
         // the copies in flight land before the block's shared memory is released
-        (void)tc::mbar_wait(&bar[st], (uint32_t)(it >> 1) & 1u, kConvWaitLimit);
-        if (tile + (int)gridDim.x < n_tiles)
-          (void)tc::mbar_wait(&bar[st ^ 1], (uint32_t)((it + 1) >> 1) & 1u, kConvWaitLimit);
+        for (int k = it; k < it + RING && k < mine; ++k)
+          (void)tc::mbar_wait(&bar[k % RING], (uint32_t)(k / RING) & 1u, kConvWaitLimit);
       }
       __syncthreads();
       return;
     }
     const uint32_t shb = smem_u32(smem) + st * T::STAGE, sgb = shb + T::HALO;
-#pragma unroll 1
+#pragma unroll 2
     for (int rr = 0; rr < T::ROWS; ++rr) {
       const int tz = rr / kTY, ty = rr - tz * kTY;
-      const int h = (UP ? (((tz + dz) >> 1) + 1) * T::HY + (((ty + dy) >> 1) + 1) : (tz + dz + 1) * T::HY + (ty + dy + 1)) *
-                        T::LP + (lane & 7) + ((q & 1) << 3);
-      uint32_t af[M][4];
+      const int h = (UP ? (((tz + dz) >> 1) + 1) * T::HY + (((ty + dy) >> 1) + 1) : (tz + dz + 1) * T::HY + (ty + dy + 1)) * T::LP;
+      uint32_t af[4];
+      ldsm_x4_t(sgb + 16 * chunk_pos<16>(rr * 16 + (lane & 7) + ((q >> 1) << 3), q & 1), af);
+      const int x = (lane & 7) + ((q & 1) << 3);   // the fragment's site
 #pragma unroll
-      for (int m = 0; m < M; ++m)
-        ldsm_x4_t(sgb + 16 * chunk_pos<16>(m * T::GROUP + rr * 16 + (lane & 7) + ((q >> 1) << 3), q & 1), af[m]);
-#pragma unroll
-      for (int p = 0; p < S + 2; ++p) {
+      for (int dx = -1; dx <= 1; ++dx) {
+        const int hx = h + (UP ? (x + dx) >> 1 : x + dx) + 1;
 #pragma unroll
         for (int np = 0; np < NT / 2; ++np) {
           uint32_t r[4];
-          ldsm_x4_t(shb + 16 * chunk_pos<CB>(((p + S - 1) % S) * T::PHASE + h + (p + S - 1) / S, 2 * np + (q >> 1)), r);
-#pragma unroll
-          for (int m = 0; m < M; ++m)
-#pragma unroll
-            for (int dx = -1; dx <= 1; ++dx) {
-              const int pm = UP ? m / 2 + (m % 2 + dx + 2) / 2 : m + dx + 1;   // the phase tap dx of group m reads
-              if (pm == p) {
-                mma16816(acc[dx + 1][2 * np], af[m], r[0], r[1]);
-                mma16816(acc[dx + 1][2 * np + 1], af[m], r[2], r[3]);
-              }
-            }
+          ldsm_x4_t(shb + 16 * chunk_pos<CB>(hx, 2 * np + (q >> 1)), r);
+          mma16816(acc[dx + 1][2 * np], af, r[0], r[1]);
+          mma16816(acc[dx + 1][2 * np + 1], af, r[2], r[3]);
         }
       }
     }
@@ -743,41 +739,55 @@ __global__ void __launch_bounds__(kWgThreads, (WgTile<CI, CO, S, UP>::PER_SM))
       }
 }
 
-// dst[i] = sum_g part[g][i] (split-K reduce): 8 warps of a block take every
-// eighth partial of 32 neighbouring elements, then add their sums in order, so
-// the result does not depend on the launch.  Latency of the loads is the
-// bound; a thread per element walking all partials took 31 us for 304 x 6,912
-// values, this form 5.
-constexpr int kSumWarps = 8;
+// s + v[0] + v[stride] + .. (n values), one after the other: the loads run
+// ahead of the chain of sums.
+__device__ __forceinline__ float add_in_order(float s, const float* v, int n, int stride) {
+#pragma unroll 16
+  for (int i = 0; i < n; ++i) s += v[i * stride];
+  return s;
+}
+
+// dst[i] = sum_g part[g][i], g = 0 .. G-1 in order (split-K reduce): the block
+// brings the partials of 32 neighbouring elements to shared memory (all copies
+// in flight at once), its first warp adds them.  Latency of the copies is the
+// bound; a thread per element walking the partials in global memory took 31 us
+// for 304 x 6,912 values.
+constexpr int kSumWarps = 8, kSumRows = 320;
 __global__ void __launch_bounds__(32 * kSumWarps) k_sum_parts(const float* __restrict__ part, int G, long long n,
                                                               float* __restrict__ dst) {
-  __shared__ float sb[kSumWarps][32];
+  __shared__ float sb[kSumRows][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long i = blockIdx.x * 32LL + lane;
   float s = 0.f;
-  if (i < n) {
-#pragma unroll 8
-    for (int g = warp; g < G; g += kSumWarps) s += part[(long long)g * n + i];
+  for (int g0 = 0; g0 < G; g0 += kSumRows) {
+    const int m = min(kSumRows, G - g0);
+    if (i < n)
+      for (int g = warp; g < m; g += kSumWarps) cp_async4(&sb[g][lane], part + (long long)(g0 + g) * n + i);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    if (warp == 0) s = add_in_order(s, &sb[0][lane], m, 32);
+    __syncthreads();
   }
-  sb[warp][lane] = s;
-  __syncthreads();
-  if (warp || i >= n) return;
-  float t = 0.f;
-#pragma unroll
-  for (int w = 0; w < kSumWarps; ++w) t += sb[w][lane];
-  dst[i] = t;
+  if (warp == 0 && i < n) dst[i] = s;
 }
 
-// The block's sum of v (fixed xor tree per warp, warps in order), in thread 0.
-template <int NT>
-__device__ __forceinline__ float block_sum(float v, float* sb) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float t = 0.f;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < NT / 32; ++w) t += sb[w];
+constexpr int kEwThreads = 256;
+
+// The sum of 256 values (32 to a row, this lane's column) by a binary tree, the
+// upper half added to the lower each time, in lane 0 of the warp.
+__device__ __forceinline__ float tree_256(const float* v) {
+  const int l = threadIdx.x & 31;
+  float t = ((v[l] + v[128 + l]) + (v[64 + l] + v[192 + l])) + ((v[32 + l] + v[160 + l]) + (v[96 + l] + v[224 + l]));
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   return t;
+}
+// The sum of v over a block of kEwThreads threads by that tree, in thread 0.
+__device__ __forceinline__ float block_sum(float v, float* sb) {
+  static_assert(kEwThreads == 256, "tree_256");
+  sb[threadIdx.x] = v;
+  __syncthreads();
+  return threadIdx.x < 32 ? tree_256(sb) : 0.f;
 }
 
 // Site s of an (nz, ny, nx) lattice (at most 2^27 sites: 32-bit divisions; the
@@ -813,29 +823,16 @@ __global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int 
   }
 }
 
-constexpr int kEwThreads = 256;
-
-// Per-block channel sums written to part[blockIdx.x][C] in a fixed order: v
-// holds 8 channels of chunk threadIdx.x % (C / 8); lanes of a chunk by an xor
-// tree, then the warps in order.
+// Per-block channel sums written to part[blockIdx.x][C], threads in order: v
+// holds 8 channels of chunk threadIdx.x % (C / 8).
 template <int C>
-__device__ __forceinline__ void block_channel_sums(float (&v)[8], float* __restrict__ part, float* sbuf) {
-  // sbuf: (kEwThreads / 32) * C floats
-  constexpr int NCH = C / 8;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void block_channel_sums(const float (&v)[8], float* __restrict__ part, float* sbuf) {
+  // sbuf: kEwThreads * 8 floats
 #pragma unroll
-  for (int e = 0; e < 8; ++e)
-    for (int o = 16; o >= NCH; o >>= 1) v[e] += __shfl_xor_sync(0xffffffffu, v[e], o);
-  if (lane < NCH) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) sbuf[warp * C + lane * 8 + e] = v[e];
-  }
+  for (int e = 0; e < 8; ++e) sbuf[threadIdx.x * 8 + e] = v[e];
   __syncthreads();
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    float s = 0.f;
-    for (int w = 0; w < kEwThreads / 32; ++w) s += sbuf[w * C + c];
-    part[(long long)blockIdx.x * C + c] = s;
-  }
+  if (threadIdx.x < C)
+    part[(long long)blockIdx.x * C + threadIdx.x] = add_in_order(0.f, sbuf + threadIdx.x, kEwThreads * 8 / C, C);
 }
 
 // Gradient of a layer's pre-activation from the raw gradient of its output:
@@ -847,7 +844,7 @@ template <int C, int POOL>
 __global__ void __launch_bounds__(kEwThreads) k_combine(const float* __restrict__ graw, const bf16* __restrict__ y,
                                                         const bf16* skip, bf16* g, int D, int H, int W,
                                                         float* __restrict__ part) {
-  __shared__ float sbuf[(kEwThreads / 32) * C];
+  __shared__ float sbuf[kEwThreads * 8];
   constexpr int NCH = C / 8;
   const long long n = (long long)D * H * W * NCH;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -908,7 +905,7 @@ __global__ void __launch_bounds__(kEwThreads) k_head_bwd(const bf16* __restrict_
                                                          const float* __restrict__ target, const float* __restrict__ gbuf,
                                                          const float* __restrict__ hw, long long N,
                                                          bf16* __restrict__ gd0, float* __restrict__ part) {
-  __shared__ float sbuf[kEwThreads / 32][kHeadParts];
+  __shared__ float sbuf[kHeadParts][kEwThreads];
   float acc[kHeadParts];
 #pragma unroll
   for (int k = 0; k < kHeadParts; ++k) acc[k] = 0.f;
@@ -946,37 +943,37 @@ __global__ void __launch_bounds__(kEwThreads) k_head_bwd(const bf16* __restrict_
     reinterpret_cast<uint4*>(gd0 + s * 16)[0] = o[0];
     reinterpret_cast<uint4*>(gd0 + s * 16)[1] = o[1];
   }
-  // the block's sums: lanes by an xor tree, warps in order (a block-wide tree
-  // with two barriers a level for each of the 34 sums was most of the kernel)
+  // the block's sums, a warp to a sum (a block-wide tree with two barriers a
+  // level for each of the 34 took most of the kernel)
 #pragma unroll
-  for (int k = 0; k < kHeadParts; ++k) {
-    float v = acc[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5][k] = v;
-  }
+  for (int k = 0; k < kHeadParts; ++k) sbuf[k][threadIdx.x] = acc[k];
   __syncthreads();
-  for (int k = threadIdx.x; k < kHeadParts; k += blockDim.x) {
-    float v = 0.f;
-    for (int w = 0; w < kEwThreads / 32; ++w) v += sbuf[w][k];
-    part[(long long)blockIdx.x * kHeadParts + k] = v;
+  for (int k = threadIdx.x >> 5; k < kHeadParts; k += kEwThreads / 32) {
+    const float v = tree_256(sbuf[k]);
+    if ((threadIdx.x & 31) == 0) part[(long long)blockIdx.x * kHeadParts + k] = v;
   }
 }
 
-// Sum per-block partials part[b][k] over b into dst[map(k)], a block per k
-// (threads take every 128th partial, then a fixed tree; one thread per k
-// walking all of them took up to 65 us for 1,216 blocks, this form 3).
-constexpr int kScatterThreads = 128;
+// Sum per-block partials part[b][k] (b = 0 .. nb-1 in order) into dst[map(k)],
+// a block per k: its threads bring them to shared memory, one adds (one thread
+// walking them in global memory took up to 65 us for 1,216 blocks).
+constexpr int kScatterThreads = 128, kScatterMax = 1280;
 __global__ void __launch_bounds__(kScatterThreads) k_scatter_parts(const float* __restrict__ part, int nb, int width,
                                                                    float* __restrict__ grads,
                                                                    const long long* __restrict__ dst_index,
                                                                    float* __restrict__ loss, float loss_scale) {
-  __shared__ float sb[kScatterThreads / 32];
+  __shared__ float sb[kScatterMax];
   const int k = blockIdx.x;
   float s = 0.f;
-#pragma unroll 4
-  for (int b = threadIdx.x; b < nb; b += kScatterThreads) s += part[(long long)b * width + k];
-  s = block_sum<kScatterThreads>(s, sb);
+  for (int b0 = 0; b0 < nb; b0 += kScatterMax) {
+    const int m = min(kScatterMax, nb - b0);
+    for (int b = threadIdx.x; b < m; b += kScatterThreads) cp_async4(&sb[b], part + (long long)(b0 + b) * width + k);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    if (threadIdx.x == 0) s = add_in_order(s, sb, m, 1);
+    __syncthreads();
+  }
   if (threadIdx.x != 0) return;
   const long long d = dst_index[k];
   if (d >= 0) grads[d] = s;
@@ -1031,7 +1028,7 @@ __device__ __forceinline__ float apply_scaled(const FeatureArgs& f, const Featur
 __global__ void __launch_bounds__(kEwThreads) k_res_u(FeatureArgs f, FeatureF c, const float* __restrict__ Kp,
                                                       const float* __restrict__ out, const float* __restrict__ tgt,
                                                       float* __restrict__ u, float* __restrict__ part) {
-  __shared__ float sb[kEwThreads / 32];
+  __shared__ float sb[kEwThreads];
   const long long n = (long long)f.nx * f.ny * f.nz;
   float acc = 0.f;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
@@ -1039,7 +1036,7 @@ __global__ void __launch_bounds__(kEwThreads) k_res_u(FeatureArgs f, FeatureF c,
     u[s] = v;
     acc += v * v;
   }
-  acc = block_sum<kEwThreads>(acc, sb);
+  acc = block_sum(acc, sb);
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
@@ -1049,7 +1046,7 @@ __global__ void __launch_bounds__(kEwThreads) k_loss_grad(FeatureArgs f, Feature
                                                           const float* __restrict__ out, const float* __restrict__ tgt,
                                                           const float* __restrict__ u, float w_mse, float w_res,
                                                           float* __restrict__ g, float* __restrict__ part) {
-  __shared__ float sb[kEwThreads / 32];
+  __shared__ float sb[kEwThreads];
   const long long n = (long long)f.nx * f.ny * f.nz;
   const float sc = 2.0f / (float)n;
   float acc = 0.f;
@@ -1060,23 +1057,29 @@ __global__ void __launch_bounds__(kEwThreads) k_loss_grad(FeatureArgs f, Feature
     if (w_res != 0.f) v += w_res * sc * apply_scaled(f, c, Kp, u, nullptr, s);
     g[s] = v;
   }
-  acc = block_sum<kEwThreads>(acc, sb);
+  acc = block_sum(acc, sb);
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// loss = sa * sum(pa[0..nb)) + sb * sum(pb[0..nb)) (one block, fixed order)
+// loss = sa * sum(pa[0..nb)) + sb * sum(pb[0..nb)), blocks in order
 __global__ void __launch_bounds__(kEwThreads) k_sum_loss(const float* __restrict__ pa, int nb, float sa,
                                                          const float* __restrict__ pb, float sb,
                                                          float* __restrict__ loss) {
-  __shared__ float sm[2][kEwThreads / 32];
-  float a = 0.f, b = 0.f;
-  for (int i = threadIdx.x; i < nb; i += kEwThreads) {
-    a += pa[i];
-    b += pb[i];
+  __shared__ float sm[2][kScatterMax], s_b;
+  float s = 0.f;   // (threads 0 and 32)
+  for (int b0 = 0; b0 < nb; b0 += kScatterMax) {
+    const int m = min(kScatterMax, nb - b0);
+    for (int i = threadIdx.x; i < m; i += kEwThreads) {
+      sm[0][i] = pa[b0 + i];
+      sm[1][i] = pb[b0 + i];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 || threadIdx.x == 32) s = add_in_order(s, sm[threadIdx.x >> 5], m, 1);
+    __syncthreads();
   }
-  a = block_sum<kEwThreads>(a, sm[0]);
-  b = block_sum<kEwThreads>(b, sm[1]);
-  if (threadIdx.x == 0) *loss = sa * a + sb * b;
+  if (threadIdx.x == 32) s_b = s;
+  __syncthreads();
+  if (threadIdx.x == 0) *loss = sa * s + sb * s_b;
 }
 
 // Adam (Kingma & Ba 2015, Algorithm 1) with FP32 master weights.
@@ -1379,16 +1382,11 @@ int conv_attr() {
   return conv_attr_t<CI, CO, C::CB, 1, C::R, C::NW, UP, EPI>();
 }
 
-// Phases of a weight gradient's tiles (the lattice of a layer's input has a
-// multiple of that many sites in x).
-template <int CI, int CO, bool UP>
-constexpr int wgrad_phases() { return CI == 16 || (CI == 32 && UP) ? 2 : 1; }
-
 template <int CI, int CO, bool UP>
 int wgrad_attr() {
-  constexpr int S = wgrad_phases<CI, CO, UP>(), sm = WgTile<CI, CO, S, UP>::SMEM;
-  NET_CUDA(cudaFuncSetAttribute(k_wgrad<CI, CO, S, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-  NET_CUDA(cudaFuncSetAttribute(k_wgrad<CI, CO, S, UP>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+  constexpr int sm = WgTile<CI, CO, UP>::SMEM;
+  NET_CUDA(cudaFuncSetAttribute(k_wgrad<CI, CO, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+  NET_CUDA(cudaFuncSetAttribute(k_wgrad<CI, CO, UP>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   return HCA_OK;
 }
 
@@ -1526,25 +1524,21 @@ void conv(hca_net* n, cudaStream_t s, int slot, const float* bias, const bf16* s
 // The maps of layer `layer`'s weight gradient; lvl: the output's level.
 template <int CI, int CO, bool UP>
 bool wgrad_prepare(hca_net* n, int layer, const bf16* in, const bf16* gy, int lvl) {
-  constexpr int S = wgrad_phases<CI, CO, UP>();
-  using T = WgTile<CI, CO, S, UP>;
+  using T = WgTile<CI, CO, UP>;
   WgMaps& m = n->wmaps[layer];
-  auto by_phase = [&](CUtensorMap* map, const bf16* base, int c, int phases, int l, int bc, int bx, int by, int bz) {
+  auto whole = [&](CUtensorMap* map, const bf16* base, int c, int l, int bc, int bx, int by, int bz) {
     const cuuint64_t row = (cuuint64_t)c * 2, W = n->Lw[l], H = n->Lh[l], D = n->Ld[l];
-    const cuuint64_t dims[4] = {(cuuint64_t)c, W / phases, H, D}, strides[3] = {phases * row, W * row, W * H * row};
+    const cuuint64_t dims[4] = {(cuuint64_t)c, W, H, D}, strides[3] = {row, W * row, W * H * row};
     const cuuint32_t box[4] = {(cuuint32_t)bc, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
-    for (int p = 0; p < phases; ++p)
-      if (!bf16_map(&map[p], base + (size_t)p * c, 4, bc, dims, strides, box)) return false;
-    return true;
+    return bf16_map(map, base, 4, bc, dims, strides, box);
   };
-  return by_phase(m.in, in, CI, S, lvl + UP, T::CB, T::LP, T::HY, T::HZ) && by_phase(m.gy, gy, CO, T::M, lvl, 16, 16, kTY, T::TZ);
+  return whole(&m.in, in, CI, lvl + UP, T::CB, T::LP, T::HY, T::HZ) && whole(&m.gy, gy, CO, lvl, 16, T::XO, kTY, T::TZ);
 }
 
 // Weight gradient of one layer into dst (27, CO, CI); the output lattice is level lvl.
 template <int CI, int CO, bool UP>
 void wgrad(hca_net* n, cudaStream_t s, int layer, int lvl, float* dst) {
-  constexpr int S = wgrad_phases<CI, CO, UP>();
-  using T = WgTile<CI, CO, S, UP>;
+  using T = WgTile<CI, CO, UP>;
   WgArgs a;
   a.part = n->wpart;
   a.tiles_x = (n->Lw[lvl] + T::XO - 1) / T::XO;
@@ -1553,13 +1547,13 @@ void wgrad(hca_net* n, cudaStream_t s, int layer, int lvl, float* dst) {
   constexpr int mts = CO / 16 * (CI / T::CB);   // tiles of the gradient
   const int n_tiles = a.tiles_x * a.tiles_y * a.tiles_z;
   const long long per = 27LL * CO * CI;
-  // one wave of blocks (every further block is a partial to sum), each with
-  // the same number of tiles but for a remainder
-  int G = std::max(1, std::min(n_tiles, T::PER_SM * n->sm_count / mts));
+  // partials: 21 to 304 by the layer's size (on 152 multiprocessors).  Their
+  // number is part of the sums' order, so it follows neither T nor the tiles a
+  // block takes: two a multiprocessor over the groups of 512 / CI (tap, 16 co).
+  constexpr int kGroups = (27 * (CO / 16) + 512 / CI - 1) / (512 / CI);
+  int G = std::max(1, std::min(n_tiles, 2 * n->sm_count / kGroups));
   G = (int)std::min<long long>(G, n->wpart_n / per);
-  const int rounds = (n_tiles + G - 1) / G;
-  G = (n_tiles + rounds - 1) / rounds;
-  k_wgrad<CI, CO, S, UP><<<dim3(G, mts), kWgThreads, T::SMEM, s>>>(a, n->wmaps[layer], n->status);
+  k_wgrad<CI, CO, UP><<<dim3(G, mts), kWgThreads, T::SMEM, s>>>(a, n->wmaps[layer], n->status);
   k_sum_parts<<<(int)((per + 31) / 32), 32 * kSumWarps, 0, s>>>(n->wpart, G, per, dst);
 }
 
@@ -1636,8 +1630,7 @@ void forward(hca_net* n, cudaStream_t s, bool keep_d0) {
 void backward(hca_net* n, cudaStream_t s, const float* target, const float* gbuf) {
   const ParamLayout& L = n->L;
   {
-    // two blocks per multiprocessor: each ends with its 34 sums
-    const int nb = std::min(std::min(ew_blocks(n->Ln[0], n->sm_count), 2 * n->sm_count), n->bpart_blocks);
+    const int nb = std::min(ew_blocks(n->Ln[0], n->sm_count), n->bpart_blocks);
     k_head_bwd<<<nb, kEwThreads, 0, s>>>(n->d0, n->out, target, gbuf, n->params + L.hw_off, n->Ln[0], n->g0,
                                          n->bpart);
     k_scatter_parts<<<kHeadParts, kScatterThreads, 0, s>>>(n->bpart, nb, kHeadParts, n->grads, n->head_index, gbuf ? nullptr : n->loss,
