@@ -448,7 +448,7 @@ void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int s
     bool ok = true, more = false;
     for (MGLevel* L : lv) {
       const int z = slab(*L, zs), ns = (L->nz + z - 1) / z;
-      if (z / L->seg > kMaxSeg) ok = false;
+      if ((z + L->seg - 1) / L->seg > kMaxSeg) ok = false;   // a slab's last segment may be partial
       if (z < L->nz) more = true;
       nb += (long long)ns * L->tx * L->ty;
       work += (double)ns * L->tx * L->ty * (z + extra);
