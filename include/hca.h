@@ -409,11 +409,14 @@ int hca_get_profile(hca_handle* h, hca_profile* out);
  * the library (about 33 KB per GPU, kept until the process exits), so the
  * lattice is limited to ny*nz <= 65536 rows (HCA_ERR_ARG beyond that).  Each
  * call looks up that array's device address in the context of the current
- * device (a host-side lookup that allocates nothing), then queues a memset of
- * its ticket, one kernel and a copy of the result to host memory on `stream`
- * (a cudaStream_t, NULL = the default stream), and synchronises `stream`
- * before it returns.  Every call shares the array: calls that overlap on the
- * GPU race and must be serialised by the caller.  Returns HCA_ERR_ARG for
+ * device (a host-side lookup that allocates nothing), then queues one kernel
+ * on `stream` (a cudaStream_t, NULL = the default stream) and synchronises
+ * `stream` before it returns.  Where the GPU can write pageable host memory
+ * the kernel stores the result in the calling thread's stack; elsewhere a copy
+ * to host memory follows it.  Every call shares the array: calls that overlap
+ * on the GPU race and must be serialised by the caller.  An overlapped call may
+ * launch its kernel a second time, return a wrong residual or HCA_ERR_CUDA; it
+ * leaves nothing behind that a later call would read.  Returns HCA_ERR_ARG for
  * bad arguments, HCA_ERR_CUDA for a failed CUDA call, HCA_ERR_NONFINITE for a
  * non-finite result. */
 int hca_o2_residual_noalloc(const hca_config* cfg, const uint8_t* state, const double* K_prev,

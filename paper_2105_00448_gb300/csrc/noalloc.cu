@@ -12,7 +12,7 @@
 // This entry point answers that with the same arithmetic as the handle's
 // true-residual kernel: per site r = b - A(K_prev) K with the 7-point
 // Neumann operator, summed per chunk of rows (1 to 32, by the lattice's size)
-// and then over chunks in a fixed order.  The per-chunk partial sums, the finishing ticket and the result
+// and then over chunks in a fixed order.  The per-chunk partial sums, the arrival count and the result
 // live in the file-scope device array `g_noalloc` below instead of memory
 // the caller or the library would allocate.  Its size is fixed at compile
 // time (kNoAllocMaxChunks chunks: ny * nz <= 65536 rows, e.g. 256 x 256 in
@@ -34,6 +34,8 @@
 // stack instead of through a copy.  48^3: 42 -> 28 us a call.
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "hca_internal.cuh"
 
 namespace {
@@ -44,17 +46,23 @@ constexpr int kNoAllocThreads = 256;   // fixed: the reduction order depends on 
 
 struct NoAllocScratch {
   double partial[kNoAllocMaxChunks][2];  // per chunk: |r|^2, |b|^2
-  double result[2];                      // |r| / |b|, |b|^2
-  unsigned int ticket;
-  unsigned int pad[3];
+  double result[2];                      // |r| / |b|, the number of the call it belongs to
+  // the call's number (upper bits) and the chunks it has finished (lower 16):
+  // every block raises the number to its own call's before it counts itself,
+  // so what an earlier call left (one that overlapped another, or was cut
+  // short) drops out, and no memset has to come before the kernel
+  unsigned long long ticket;
+  unsigned long long pad;
 };
+constexpr int kArrivalBits = 16;
+static_assert(kNoAllocMaxChunks < 1 << kArrivalBits, "a call's arrivals fit their bits");
 
 static __device__ __align__(256) NoAllocScratch g_noalloc;
 
 // out: where the result goes besides the scratch array (host memory the GPU
 // can write, or null).
 __global__ void __launch_bounds__(kNoAllocThreads) k_o2_residual_noalloc(
-    NoAllocScratch* __restrict__ sc, int nx, int ny, int nz, int chunk_rows, double c, double phi_K, double K1, double b0,
+    NoAllocScratch* __restrict__ sc, unsigned long long call, int nx, int ny, int nz, int chunk_rows, double c, double phi_K, double K1, double b0,
     double r_K, const uint8_t* __restrict__ state, const double* __restrict__ K_prev,
     const double* __restrict__ K, double* out) {
   __shared__ double s_cn[7];   // c times a neighbour count
@@ -101,7 +109,7 @@ __global__ void __launch_bounds__(kNoAllocThreads) k_o2_residual_noalloc(
     s_w[warp][1] = bb;
   }
   __syncthreads();
-  __shared__ unsigned int s_ticket;
+  __shared__ bool s_last;
   if (threadIdx.x == 0) {
     double a0 = 0.0, a1 = 0.0;
     for (int w = 0; w < kNoAllocThreads / 32; ++w) {
@@ -111,10 +119,11 @@ __global__ void __launch_bounds__(kNoAllocThreads) k_o2_residual_noalloc(
     sc->partial[blockIdx.x][0] = a0;
     sc->partial[blockIdx.x][1] = a1;
     __threadfence();
-    s_ticket = atomicAdd(&sc->ticket, 1u);
+    atomicMax(&sc->ticket, call << kArrivalBits);
+    s_last = atomicAdd(&sc->ticket, 1ull) == (call << kArrivalBits) + gridDim.x - 1;
   }
   __syncthreads();
-  if (s_ticket != gridDim.x - 1) return;
+  if (!s_last) return;
   // last block: chunk partials in a fixed order (thread t takes t, t + 256, ...)
   __threadfence();
   double p0 = 0.0, p1 = 0.0;
@@ -140,8 +149,7 @@ __global__ void __launch_bounds__(kNoAllocThreads) k_o2_residual_noalloc(
     }
     const double rel = a1 > 0.0 ? sqrt(a0 / a1) : 0.0;
     sc->result[0] = rel;
-    sc->result[1] = a1;
-    sc->ticket = 0u;
+    sc->result[1] = (double)call;
     if (out) *out = rel;
   }
 }
@@ -182,27 +190,25 @@ extern "C" int hca_o2_residual_noalloc(const hca_config* cfg, const uint8_t* sta
     return HCA_ERR_CUDA;
   }
   const double c = cfg->D_K / (cfg->dx * cfg->dx), b0 = cfg->r_K * cfg->K0;
-  // The kernel's last block leaves the ticket at zero.  A call cut short (or
-  // two that overlapped) may have left it otherwise, so that no block finds
-  // itself last: then the result still reads as the mark, the ticket is
-  // cleared and the check runs once more.
+  // A call that overlaps another may find no last block, as the two count in
+  // one place: then the result still reads as the mark (or belongs to another
+  // call) and the check runs once more.
+  static std::atomic<unsigned long long> calls{0};
   const double mark = -1.0;
   volatile double res = mark;
   for (int attempt = 0; attempt < 2 && res == mark; ++attempt) {
-    if ((attempt || !ats) && cudaMemsetAsync(&sc->ticket, 0, sizeof(unsigned int), s) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return HCA_ERR_CUDA;
-    }
+    const unsigned long long call = ++calls;   // (2^48 of them)
     k_o2_residual_noalloc<<<(unsigned)chunks, kNoAllocThreads, 0, s>>>(
-        sc, cfg->nx, cfg->ny, cfg->nz, chunk_rows, c, cfg->phi_K, cfg->K1, b0, cfg->r_K, state, K_prev, K,
+        sc, call, cfg->nx, cfg->ny, cfg->nz, chunk_rows, c, cfg->phi_K, cfg->K1, b0, cfg->r_K, state, K_prev, K,
         ats ? const_cast<double*>(&res) : nullptr);
+    double got[2] = {mark, 0.0};
     if (cudaGetLastError() != cudaSuccess ||
-        (!ats && cudaMemcpyAsync(const_cast<double*>(&res), sc->result, sizeof(double), cudaMemcpyDeviceToHost, s) !=
-                     cudaSuccess) ||
+        (!ats && cudaMemcpyAsync(got, sc->result, sizeof(got), cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
         cudaStreamSynchronize(s) != cudaSuccess) {
       (void)cudaGetLastError();
       return HCA_ERR_CUDA;
     }
+    if (!ats && got[1] == (double)call) res = got[0];
   }
   if (!isfinite(res)) return HCA_ERR_NONFINITE;
   if (res == mark) return HCA_ERR_CUDA;
