@@ -150,6 +150,7 @@ struct ConvArgs {
   const float* head_b; // 1 (EPI_HEAD)
   int D, H, W;         // output lattice
   int Di, Hi, Wi;      // input lattice (D/2.. when UP)
+  int z0;              // k_conv: the launch's first plane
 };
 
 // 16-byte copy from global to shared memory; src_bytes = 0 writes zeros
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(32 * NW, (ConvTile<CI, CO, CB, S, R, NW, UP, E
   char* sw = smem + T::SMEM - 16 - 2 * T::WPLANE;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + T::SMEM - 16);
   const int cg = blockIdx.x % (CO / CB), co0 = cg * CB;
-  const int z0 = blockIdx.z * T::TZ, y0 = blockIdx.y * kTY, x0 = (int)(blockIdx.x / (CO / CB)) * T::XO;
+  const int z0 = a.z0 + blockIdx.z * T::TZ, y0 = blockIdx.y * kTY, x0 = (int)(blockIdx.x / (CO / CB)) * T::XO;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // the halo and the first two planes of taps; the third follows the first
   auto stage_w = [&](int plane) {
@@ -1493,13 +1494,18 @@ bool conv_prepare(hca_net* n, int slot, const bf16* in, const bf16* w, int lvl) 
 }
 
 template <int CI, int CO, int CB, int S, int R, int NW, bool UP, int EPI>
-void conv_launch(cudaStream_t s, const ConvArgs& a, const ConvMaps& maps, int* status) {
+void conv_launch(cudaStream_t s, ConvArgs a, const ConvMaps& maps, int* status) {
   using T = ConvTile<CI, CO, CB, S, R, NW, UP, EPI>;
-  const dim3 grid((a.W + T::XO - 1) / T::XO * (CO / CB), (a.H + kTY - 1) / kTY, (a.D + T::TZ - 1) / T::TZ);
-  k_conv<CI, CO, CB, S, R, NW, UP, EPI><<<grid, 32 * NW, T::SMEM, s>>>(a, maps, status);
+  // a grid has at most 65,535 blocks along z: a longer lattice takes further launches
+  const int tiles_z = (a.D + T::TZ - 1) / T::TZ;
+  for (int t = 0; t < tiles_z; t += 65535) {
+    a.z0 = t * T::TZ;
+    const dim3 grid((a.W + T::XO - 1) / T::XO * (CO / CB), (a.H + kTY - 1) / kTY, std::min(65535, tiles_z - t));
+    k_conv<CI, CO, CB, S, R, NW, UP, EPI><<<grid, 32 * NW, T::SMEM, s>>>(a, maps, status);
+  }
 }
 
-// One convolution launch on the inputs of maps[slot]; the output lattice is level lvl.
+// One convolution on the inputs of maps[slot]; the output lattice is level lvl.
 template <int CI, int CO, bool UP, int EPI>
 void conv(hca_net* n, cudaStream_t s, int slot, const float* bias, const bf16* skip, bf16* out, float* out_f,
           const float* hw, const float* hb, int lvl, bf16* out_p = nullptr) {
