@@ -532,42 +532,13 @@ __device__ __forceinline__ void level_up(const Slab& s, const float* ca, const f
 }
 
 // The coarsest level: MG_NU_COARSE sweeps of weight MG_OMEGA_COARSE; the
-// result ends in a.  At most MG_MIN_SITES sites are at most one group a
-// thread, whose right-hand side and diagonal stay in registers; a hierarchy
-// that ran out of levels (a chain of millions of sites) has more.
+// result ends in a.  At most MG_MIN_SITES sites (the hierarchies end there:
+// MG_MAXLEV) are at most one group a thread, whose right-hand side and diagonal
+// stay in registers.
 static_assert(MG_MIN_SITES <= kCT, "a thread holds at most one group of the coarsest level");
-__device__ __noinline__ void coarsest_large(const Slab& s, bool zp) {
-  const int pitch = 4 * s.gpr, ps = pitch * s.nr, n = s.np * s.nr * s.gpr;
-  for (int it = 0; it < MG_NU_COARSE; ++it) {
-    float* dst = ((MG_NU_COARSE - 1 - it) & 1) ? s.b : s.a;
-    const float* src = dst == s.a ? s.b : s.a;
-    Walk3 k(threadIdx.x, s.gpr, s.nr, s.mg, s.mr);
-    for (int t = threadIdx.x; t < n; t += kCT, k.next()) {
-      const int e = k.lp * ps + k.q * pitch + 4 * k.g;
-      const Q4 d = ldq(s.d + k.lp * s.dplane + k.q * s.drow + 4 * k.g), w = invq(d),
-               r = ldq(s.r + k.lp * s.rplane + k.q * s.rrow + 4 * k.g);
-      Q4 o, S = zeroq(), x = zeroq();
-      if (it > 0) {
-        x = ldq(src + e);
-        S = nb_group(s, src, nullptr, nullptr, k.lp, k.q, k.g, zp, x);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float2 res = __ffma2_rn(make_float2(-d.v[h].x, -d.v[h].y), x.v[h], __ffma2_rn(dup(s.c), S.v[h], r.v[h]));
-        o.v[h] = __ffma2_rn(__fmul2_rn(dup(kWC), w.v[h]), res, x.v[h]);
-      }
-      stq(dst + e, o);
-    }
-    __syncthreads();
-  }
-}
 // zero: 16 bytes of zeros in shared memory.
 __device__ __forceinline__ void coarsest(const Slab& shared_s, bool zp, const float4* zero) {
   const int n = shared_s.np * shared_s.nr * shared_s.gpr;
-  if (n > kCT) {
-    coarsest_large(shared_s, zp);
-    return;
-  }
   const Slab s = shared_s;
   const int nt = (n + 31) & ~31;   // the warps with groups
   if ((int)threadIdx.x < nt) {

@@ -1200,7 +1200,7 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
         // coarsen while the level is large and some extent exceeds 1; the
         // coupling grows by 2^k / 4 for the k extents above 1 (2 on a 3-D
         // lattice, 1 on a flat one)
-        while (nn > hca::MG_MIN_SITES && std::max(nx, std::max(ny, nz)) > 1 && nl < hca::MG_MAXLEV) {
+        while (nn > hca::MG_MIN_SITES && std::max(nx, std::max(ny, nz)) > 1 && nl < (h->fp64 ? hca::MG_MAXLEV_FP64 : hca::MG_MAXLEV)) {
           const int k = (nx > 1) + (ny > 1) + (nz > 1);
           cs *= std::ldexp(1.0, k - 2);
           nx = (nx + 1) / 2;

@@ -341,7 +341,10 @@ constexpr long long MG_MIN_SITES = 512;     // coarsening stops at or below this
 constexpr long long MG_SMALL_SITES = 4096;  // levels this small run inside one block
 
 constexpr long long kClusterSites = 4096;   // most sites per block of a cluster's first level
-constexpr int MG_MAXLEV = 16;
+// Most levels of a hierarchy.  FP32: enough to end at MG_MIN_SITES for any
+// lattice of fewer than 2^31 sites, also one that coarsens along one axis alone
+// (the clusters hold the last levels in shared memory); FP64: 16.
+constexpr int MG_MAXLEV = 24, MG_MAXLEV_FP64 = 16;
 constexpr int kVcycleParts = 6;   // launch groups of a V-cycle (see launch_vcycle)
 
 // Host summary of the hierarchies of a handle's replicates (launch geometry).
