@@ -353,10 +353,11 @@ int hca_apply_operator(hca_handle* h, int32_t rep, int32_t which, const void* u,
 
 /* The launch shape the handle uses: threads per block of the row kernels and
  * the register cap of the CG passes.  With threads_per_block = 0 in the
- * config the library picks the threads at creation: FP64 handles by timing
- * the oxygen CG passes on the handle's own lattices (set HCA_NO_TUNE=1 to
- * keep 128), FP32 handles from the lattices' shapes.  Results do not depend
- * on the choice. */
+ * config the library picks the threads at creation: FP64 handles whose solves
+ * use the CG passes by timing them on the handle's own lattices (set
+ * HCA_NO_TUNE=1 to keep 128), FP32 handles and FP64 handles whose solves are
+ * all one launch each (Jacobi, up to about 300 000 sites a lattice) from the
+ * lattices' shapes.  Results do not depend on the choice. */
 int hca_get_launch_config(hca_handle* h, int32_t* threads_per_block, int32_t* pass_regs);
 
 /* z = M r for replicate rep, with M the multigrid V-cycle (HCA_PC_MG) built

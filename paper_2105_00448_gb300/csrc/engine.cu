@@ -930,7 +930,7 @@ int check_convergence(hca_handle* h) {
   return HCA_OK;
 }
 
-// Launch-shape autotuner (FP64 handles): times the oxygen CG passes (the hot
+// Launch-shape autotuner (FP64 handles whose solves use the CG passes): times the oxygen CG passes (the hot
 // pair) for each candidate block size on the handle's own lattices, best of
 // three timed runs each, and keeps the fastest.  It runs at creation, on the
 // solver's scratch vectors (x = aux), before anything depends on them; the
@@ -1133,8 +1133,10 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
   // chunks (a flat one of 200 rows has 25) get more warps a chunk instead of
   // idle multiprocessors (its ODEs: 0.30 ms at 128 threads, 0.13 at 512)
   c.threads = cfgs[0].threads_per_block ? cfgs[0].threads_per_block : 128;
-  if (!cfgs[0].threads_per_block && !h->fp64)
+  auto threads_of_shape = [&] {
     while (c.threads < 512 && (long long)chunk0 * c.threads < 512LL * c.sm_count) c.threads *= 2;
+  };
+  if (!cfgs[0].threads_per_block && !h->fp64) threads_of_shape();
   c.stream = h->stream;
   const size_t es = elem_size(h);
   const size_t fbytes = (size_t)h->total * es;
@@ -1654,7 +1656,12 @@ int create_impl(int n, const hca_config* cfgs, const float* const* p_cell, const
     // (the FP32 passes have one launch shape, chosen from the lattices)
     if (!cfgs[0].threads_per_block && h->fp64) {
       const char* nt = std::getenv("HCA_NO_TUNE");
-      if (!(nt && nt[0] == '1')) {
+      if (c.rounds64 && !h->large64) {
+        // no solve launches the passes that the tuner times: the row kernels'
+        // rule (a 64^3 step: 8.9 ms at its 512 threads; timing the unused passes
+        // picked 128 or 256 from run to run, 9.7 to 9.9 ms)
+        threads_of_shape();
+      } else if (!(nt && nt[0] == '1')) {
         rc = autotune(h);
         if (rc) goto fail;
       }
