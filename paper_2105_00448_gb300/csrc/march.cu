@@ -401,6 +401,11 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_mg_up(Ctx c, int whic
 }  // namespace
 
 // ---------------------------------------------------------- configuration --
+int march_threads(const std::vector<MGLevel*>& lv);
+// Segments below which a lattice's segments are cut shorter: near the number of
+// multiprocessors, but the same on every chip, as segments shape the sums.
+constexpr int kFewSegs = 128;
+
 // Tiling of a level: the fewest tiles of kMT patches (every halo patch is
 // redundant work).  It depends on the level's shape alone, as do the segment
 // sums, so results do not depend on slabs, batches or launch forms.
@@ -427,8 +432,12 @@ void march_tile(MGLevel& L, int halo_rows) {
     }
     if (cols <= 6) break;
   }
-  // planes per reduction segment (even, so a slab starts on a coarse plane)
+  // planes per reduction segment (even, so a slab starts on a coarse plane);
+  // shorter on lattices of few tiles, whose slabs of whole segments would leave
+  // multiprocessors idle (oxygen solve with Jacobi, 43 x 41 x 300: 1.46 ms, 2.06
+  // with 16 planes a segment, 1.75 with the row kernels before)
   L.seg = L.nz > 256 ? 16 : L.nz > 128 ? 8 : L.nz > 64 ? 4 : 2;
+  while (L.seg > 2 && (long long)L.tx * L.ty * ((L.nz + L.seg - 1) / L.seg) < kFewSegs) L.seg /= 2;
   L.nseg = (L.nz + L.seg - 1) / L.seg;
 }
 
@@ -438,23 +447,22 @@ void march_tile(MGLevel& L, int halo_rows) {
 // multiprocessors.
 void march_blocks(std::vector<MGLevel*>& lv, const std::vector<int>& reps, int sm_count, int extra,
                   std::vector<int4>& out) {
-  const long long resident = 2LL * sm_count;
-  auto slab = [](const MGLevel& L, int zs) { return std::min(L.nz, (zs + L.seg - 1) / L.seg * L.seg); };
+  const long long resident = (long long)blocks_per_sm(march_threads(lv)) * sm_count;
+  // a block has slots for kMaxSeg segments (the last one may be partial)
+  auto slab = [](const MGLevel& L, int zs) { return std::min(L.nz, std::min((zs + L.seg - 1) / L.seg, kMaxSeg) * L.seg); };
   int best_zs = 0;
   double best = -1;
   for (int zs = 2; zs <= 1024; zs = zs < 64 ? zs + 2 : zs + 8) {
     long long nb = 0;
     double work = 0, longest = 0;
-    bool ok = true, more = false;
+    bool more = false;
     for (MGLevel* L : lv) {
       const int z = slab(*L, zs), ns = (L->nz + z - 1) / z;
-      if ((z + L->seg - 1) / L->seg > kMaxSeg) ok = false;   // a slab's last segment may be partial
-      if (z < L->nz) more = true;
+      if (z < L->nz && z < kMaxSeg * L->seg) more = true;
       nb += (long long)ns * L->tx * L->ty;
       work += (double)ns * L->tx * L->ty * (z + extra);
       longest = std::max(longest, z + (double)extra);
     }
-    if (!ok) break;
     // whole waves while there are few, an even share plus a tail beyond
     const double waves = (double)nb / resident;
     const double t = waves <= 4 ? std::max(1.0, std::ceil(waves)) * longest : work / resident + 0.5 * longest;
