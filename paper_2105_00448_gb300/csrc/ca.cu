@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(256) k_ca_colour(Ctx c, int colour) {
 // (the cell, its kill test, the neighbours' K) is read before the barrier, so
 // that one load, the neighbour's state, is left after it.  Measured: 0.42 ->
 // 0.17 ms at 256^3 (2300 cells a colour), 0.26 -> 0.13 ms at 64^3, 16 uneven
-// replicates 5.9 -> 0.43 ms (one replicate after the other before).
+// replicates 5.9 -> 0.30 ms (one replicate after the other before).
 constexpr int kCaThreads = 512;
 constexpr int kCaReps = 512;   // most replicates of the cooperative form
 

@@ -21,7 +21,7 @@
 // switch between them and those kernels cost ~12 us (with the split pinned
 // for all of them, pass A 102 us and pass B 89 us).  Measured at 256^3: pass
 // A 75 us (an average of 22 B a site; 87 with per-thread copies), pass B 48 us;
-// a step 15.2 -> 13.0 ms by the passes themselves.
+// a step 15.2 -> 13.6 ms by the passes themselves.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

@@ -11,6 +11,10 @@
 // at 1/64 of the FP32 rate on this GPU (measured: a warp instruction occupies
 // its quarter of the multiprocessor for 76 cycles, 64 to its result), so
 // operations count, 15 a site and iteration, and chains of them in the sums.
+// S(p) by recurrence drifts from the neighbour sum of p by rounding, and z is a
+// product with a rounded 1 / d, beta one with a rounded reciprocal: the solve
+// stops on the recurred residual, as CG does, and the residual that the
+// statistics report is recomputed from x.
 // Measured at 48^3 (379 iterations a step): 41 -> 12.3 us an iteration, a
 // third of it FP64 arithmetic, the rest the two exchanges (four trips through
 // L2); a step 15.3 -> 5.9 ms.

@@ -22,7 +22,7 @@
 // float-float chains' latency at 16 warps per multiprocessor (ncu at 256^3:
 // 51 % of issue slots, 3 TB/s).  Measured, an average of first and later
 // sweeps (FP32, V-cycle form): 137 us at 256^3 against 170 us of the row kernel
-// it replaced, 360 against 859 us on 16 uneven replicates (59 M sites).
+// it replaced, 384 against 859 us on 16 uneven replicates (59 M sites).
 #include <algorithm>
 #include <type_traits>
 #include <vector>

@@ -34,7 +34,7 @@
 // per-thread cp.async of each patch), against 110 us for the pre-sweep and
 // restriction kernels and 118 us for the two post-sweep kernels they replaced
 // (28.5 B a site each); on 16 uneven replicates (59 M sites, all levels'
-// launches apart) 137 and 145 us, against 449 and 495 us.
+// launches apart) 124 and 131 us, against 449 and 495 us.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

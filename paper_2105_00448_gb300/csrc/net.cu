@@ -22,7 +22,8 @@
 //
 // Bound (forward at 128^3, 135 GFLOP, 414 us): the mma.sync pipe, which peaks
 // at 600 TFLOP/s on this chip (225 us), with the halo's traffic exposed where
-// two or three blocks fit a multiprocessor: dec0 129 us, enc0 83, dec1 68.
+// two or three blocks fit a multiprocessor: dec0 131 us, enc0 with its pooling
+// 96, dec1 69.
 // (One ldmatrix of the input per tap and tile, weights staged between barriers
 // and 128-thread blocks took 192, 115 and 88 us, 585 us in all.)
 
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(const ConvArgs a, int* status) 
 // order, their number following the layer (wgrad).  Interleaved site groups
 // whose x fragments serve several taps are faster but sum in another order.
 // Bound: the fragment loads, and latency at the coarse levels.  All seven
-// layers at 64^3: 97 us (dec0's 31), against 195 (69) with the tile staged
+// layers at 64^3: 96 us (dec0's 31), against 195 (69) with the tile staged
 // between barriers and the nine (dz, dy) sharing no fragment; 90 (25) with
 // interleaved groups.
 template <int CI, int CO, bool UP>
