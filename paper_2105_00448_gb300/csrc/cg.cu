@@ -41,6 +41,18 @@ constexpr int kARing = 3;             // planes k .. k + 2 of z, p_old and dx, k
 constexpr size_t a_smem(int nt) { return (size_t)(kARing * 8 + 4) * nt * 16 + (size_t)kMaxSeg * (nt / 32) * 8 + 128; }
 
 // ----------------------------------------------------------------- pass A --
+// One thread, with sigma = p.q of replicate rep.
+__device__ __forceinline__ void alpha_of(const Ctx& c, int rep, double sigma) {
+  RepSolve& s = c.solve[rep];
+  if (!(sigma > 0.0) || !isfinite(sigma)) {
+    if (!isfinite(sigma)) c.sync->error = 1;
+    s.active = 0;
+    s.pend = 0;   // this launch added the last step
+    return;
+  }
+  s.alpha = s.rho / sigma;
+}
+
 template <int NT, bool DEFER>
 __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which) {
   extern __shared__ __align__(16) float4 msm[];
@@ -179,16 +191,143 @@ __global__ void __launch_bounds__(NT, blocks_per_sm(NT)) k_cg_a(Ctx c, int which
     }
     slots[s] = t;
   }
-  march_finish(c, rep, L.nblk, c.mslot + L.slot0, L.tx * L.ty * L.nseg, [&](double sigma) {
-    RepSolve& s = c.solve[rep];
-    if (!(sigma > 0.0) || !isfinite(sigma)) {
-      if (!isfinite(sigma)) c.sync->error = 1;
-      s.active = 0;
-      s.pend = 0;   // this launch added the last step
-      return;
+  march_finish(c, rep, L.nblk, c.mslot + L.slot0, L.tx * L.ty * L.nseg, [&](double sigma) { alpha_of(c, rep, sigma); });
+}
+
+// Pass A on flat lattices (every lattice of the handle has one plane).  There
+// is nothing to march over: a block of the marching form would hold one tile
+// for two planes' steps, and its start, fence and arrival took 7 us a tile
+// (4000 x 4000 x 1: 240 us a launch).  Here a block walks over a run of the
+// same tiles, reads rows and their neighbours through the caches, without
+// barriers, and arrives once for all of them: 85 us, bound by HBM (an oxygen
+// solve with Jacobi 21.1 -> 11.7 ms, 11.8 with the row kernels before the
+// marching form; with the V-cycle 8.2 -> 7.1).  Sites, patches, lanes and sums
+// are those of the marching form, so the results are the same bits.
+constexpr int kFlatTiles = 32;   // tiles whose sums a block holds
+constexpr int flat_blocks(int nt) { return 768 / nt; }   // resident: registers for 24 warps
+
+template <int NT, bool DEFER>
+__global__ void __launch_bounds__(NT, flat_blocks(NT)) k_cg_a_flat(Ctx c, int which) {
+  constexpr int NW = NT / 32;
+  __shared__ float2 segs[kFlatTiles * NW];
+  HCA_COUNT_KERNEL(c);
+  const int par = c.sync->parity;
+  const int e0 = (int)((long long)c.n_ablk * blockIdx.x / gridDim.x), e1 = (int)((long long)c.n_ablk * (blockIdx.x + 1) / gridDim.x);
+  const float2 zero = make_float2(0.f, 0.f);
+  for (int e = e0; e < e1;) {
+    // a run of tiles of one replicate
+    const int rep = c.ablk[e].x, first = c.ablk[e].y;
+    const MGLevel& L = c.cg_lv[rep];
+    const int n = min(min(e1 - e, L.nblk - first), kFlatTiles);
+    e += n;
+    const RepSolve sv = c.solve[rep];
+    if (!sv.active) continue;
+    const RepDesc& rd = c.reps[rep];
+    const float cpl = rd.cpl32[which];
+    const long long off = rd.off;
+    const float* __restrict__ zz = (const float*)c.z + off;
+    const float* __restrict__ dd = (const float*)c.d + off;
+    const float* __restrict__ po = (const float*)(par ? c.p_alt : c.p) + off;
+    float* __restrict__ pn = (float*)(par ? c.p : c.p_alt) + off;
+    float* __restrict__ qq = (float*)c.q + off;
+    float* __restrict__ xx = (float*)c.dx + off;
+    const float2 beta = dup((float)sv.beta), alpha = dup((float)sv.alpha);
+    const bool add = DEFER && sv.pend, use_p = sv.beta != 0.0 || add, use_x = add && sv.iters > 1;
+    const float2 zs = dup((sv.iters == 0 && !c.mg) ? (float)sv.scale : 1.f);
+    const int ny = L.ny;
+    for (int t = 0; t < n; ++t) {
+      const Patch p = patch_of<NT, 1>(L, make_int4(rep, first + t, 0, 1));
+      const int col = p.tid % L.cols, pr = p.tid / L.cols;
+      const bool gok = p.x0 >= 0 && p.x0 < p.nx && pr < L.pairs, cin = col >= 1 && col <= L.ox;
+      // rows y0 - 1 .. y0 + 2 of z and p_old; the outer two where an interior row needs them
+      float2 u[4][2], o[4][2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int y = p.y0 - 1 + i;
+        const bool ok = gok && y >= 0 && y < ny && (i == 0 ? p.in[0] : i == 3 ? p.in[1] : true);
+        u[i][0] = u[i][1] = o[i][0] = o[i][1] = zero;
+        const unsigned a = ok ? (unsigned)p.x0 + p.sy * (unsigned)y : 0u;
+        if (ok) get_row(u[i], reinterpret_cast<const float4*>(zz + a));
+        if (ok && use_p) get_row(o[i], reinterpret_cast<const float4*>(po + a));
+      }
+      // left and right neighbours that another warp holds
+      float zl[2] = {0.f, 0.f}, pl[2] = {0.f, 0.f}, zr[2] = {0.f, 0.f}, pq[2] = {0.f, 0.f};
+      float2 d[2][2], x[2][2];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        d[a][0] = d[a][1] = x[a][0] = x[a][1] = zero;
+        if (!p.in[a]) continue;
+        const unsigned ea = p.e + a * p.sy;
+        get_row(d[a], reinterpret_cast<const float4*>(dd + ea));
+        if (use_x) get_row(x[a], reinterpret_cast<const float4*>(xx + ea));
+        if (p.l0 && p.x0 > 0) {
+          zl[a] = zz[ea - 1];
+          if (use_p) pl[a] = po[ea - 1];
+        }
+        if (p.l31 && p.x0 + 4 < p.nx) {
+          zr[a] = zz[ea + 4];
+          if (use_p) pq[a] = po[ea + 4];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          u[i][h] = __ffma2_rn(beta, o[i][h], __fmul2_rn(zs, u[i][h]));
+          if (p.part) {   // padding sites count as zeros
+            if (p.x0 + 2 * h >= p.nx) u[i][h].x = 0.f;
+            if (p.x0 + 2 * h + 1 >= p.nx) u[i][h].y = 0.f;
+          }
+        }
+      FF acc{0.f, 0.f};
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const float2 u0 = u[a + 1][0], u1 = u[a + 1][1];
+        float lft = __shfl_up_sync(0xffffffffu, u1.y, 1), rgt = __shfl_down_sync(0xffffffffu, u0.x, 1);
+        if (!p.in[a]) continue;
+        if (p.l0) lft = __fmaf_rn(beta.x, pl[a], __fmul_rn(zs.x, zl[a]));
+        if (p.l31) rgt = __fmaf_rn(beta.x, pq[a], __fmul_rn(zs.x, zr[a]));
+        const float2 xs[2] = {make_float2(lft + u0.y, u0.x + u1.x), make_float2(u0.y + u1.y, u1.x + rgt)};
+        float2 q[2];
+        float g_s = 0.f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float2 S = __fadd2_rn(__fadd2_rn(__fadd2_rn(xs[h], __fadd2_rn(u[a][h], u[a + 2][h])), zero), zero);
+          const float2 m = __fmul2_rn(dup(cpl), S);
+          const float2 w = u[a + 1][h];
+          q[h] = __ffma2_rn(d[a][h], w, make_float2(-m.x, -m.y));
+          if (p.part) {
+            if (p.x0 + 2 * h >= p.nx) q[h].x = 0.f;
+            if (p.x0 + 2 * h + 1 >= p.nx) q[h].y = 0.f;
+          }
+          g_s = cg_madd(w.x, q[h].x, g_s);
+          g_s = cg_madd(w.y, q[h].y, g_s);
+        }
+        const unsigned ea = p.e + a * p.sy;
+        if (add) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) x[a][h] = __ffma2_rn(alpha, o[a + 1][h], x[a][h]);
+          *reinterpret_cast<float4*>(xx + ea) = make_float4(x[a][0].x, x[a][0].y, x[a][1].x, x[a][1].y);
+        }
+        *reinterpret_cast<float4*>(pn + ea) = make_float4(u0.x, u0.y, u1.x, u1.y);
+        *reinterpret_cast<float4*>(qq + ea) = make_float4(q[0].x, q[0].y, q[1].x, q[1].y);
+        acc = ff_add(acc, g_s);
+      }
+      const FF s = row_reduce_ff(acc, 32);
+      if (p.lane == 0) segs[t * NW + (p.tid >> 5)] = make_float2(s.hi, s.lo);
     }
-    s.alpha = s.rho / sigma;
-  });
+    __syncthreads();
+    double* slots = c.mslot + L.slot0 + first;
+    for (int t = threadIdx.x; t < n; t += NT) {
+      double v = 0.0;
+      for (int w = 0; w < NW; ++w) {
+        const float2 f = segs[t * NW + w];
+        v += (double)f.x + (double)f.y;
+      }
+      slots[t] = v;
+    }
+    march_finish(c, rep, L.nblk, c.mslot + L.slot0, L.tx * L.ty, [&](double sigma) { alpha_of(c, rep, sigma); }, n);
+  }
 }
 
 // ----------------------------------------------------------------- pass B --
@@ -394,7 +533,14 @@ bool b_init() {
 }
 template <int NT>
 void a_launch(const Ctx& c, int which, bool defer) {
-  const dim3 g(c.n_ablk), t(NT);
+  const dim3 t(NT);
+  if (c.flat) {
+    const dim3 gf(std::min(c.n_ablk, flat_blocks(NT) * c.sm_count));
+    if (defer) launch_k(c.pdl != 0, k_cg_a_flat<NT, true>, gf, t, 0, c.stream, c, which);
+    else launch_k(c.pdl != 0, k_cg_a_flat<NT, false>, gf, t, 0, c.stream, c, which);
+    return;
+  }
+  const dim3 g(c.n_ablk);
   if (defer) launch_k(c.pdl != 0, k_cg_a<NT, true>, g, t, a_smem(NT), c.stream, c, which);
   else launch_k(c.pdl != 0, k_cg_a<NT, false>, g, t, a_smem(NT), c.stream, c, which);
 }

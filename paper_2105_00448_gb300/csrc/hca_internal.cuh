@@ -415,6 +415,7 @@ struct Ctx {
   const int4* bblk;       // blocks of the streaming pass B: (replicate, first chunk, end chunk, blocks of the replicate)
   const int4* bgeo;       // [rep] pass B: groups, groups per chunk, chunks, first slot
   int n_ablk, n_bblk, a_nt;
+  int flat;               // 1: pass A takes its form for flat lattices
   const Cg64Block* blk64;   // FP64 Jacobi: [round][block] of the small replicates' one-launch solves
   ulonglong2* slot64;       // their blocks' partial sums
   unsigned* epoch64;        // [rep] their exchanges so far

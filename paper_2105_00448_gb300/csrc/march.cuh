@@ -195,14 +195,16 @@ __device__ __forceinline__ void zero_patch(P8& u) {
 // The end of a marching kernel that sums into slots: the last block of the
 // replicate (nblk blocks) to arrive adds its n slots in an order that is the
 // same whatever the launch (64 lanes take every 64th slot, then a fixed
-// tree) and hands the sum to fin, called by one thread.
+// tree) and hands the sum to fin, called by one thread.  count: how many of
+// the nblk blocks this one stands for.
 template <class Fin>
-__device__ __forceinline__ void march_finish(const Ctx& c, int rep, int nblk, const double* slots, int n, Fin fin) {
+__device__ __forceinline__ void march_finish(const Ctx& c, int rep, int nblk, const double* slots, int n, Fin fin,
+                                             int count = 1) {
   __shared__ int s_last;
   __shared__ double s_half[2];
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&c.mcnt[rep], 1) == nblk - 1;
+  if (threadIdx.x == 0) s_last = atomicAdd(&c.mcnt[rep], count) == nblk - count;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
